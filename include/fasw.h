@@ -161,14 +161,14 @@ int fasw_use_graphs(fasw_ctx* ctx, int enable);
  * 4 = with 16 rows per strip, 5 = hyperplane-staged (mixed precision only, nj <= 256: blocks
  * stored hyperplane-major and staged through shared memory by cp.async; elsewhere as 0), 6 / 7 =
  * hyperplane-staged with a staging ring of 4 / 8 steps, 8 = strip-pipelined with 4 rows per
- * strip, 9 = warp strips: one warp per strip of 32 rows, each lane a row holding all four
- * components of its cell, operands staged into shared memory by bulk asynchronous copies, the
- * strips of one sweep launched as one thread-block cluster, each strip storing its boundary row
+ * strip, 9 = warp strips: one computing warp per strip of 8 rows, four lanes per cell, its operands
+ * staged into shared memory and its results taken out by bulk asynchronous copies, the strips of
+ * one sweep (two per CTA) launched as one thread-block cluster, each strip's boundary row stored
  * straight into the shared memory of the strip that reads it; its recurrence runs in FP32, and in
  * FP64 contexts it is followed by one FP64 defect correction (the FP64 residual of the SGS system
  * at the FP32 result, solved by a second FP32 sweep and added), which brings the result to FP64
- * accuracy; 10 = as 9, with operand chunks of 8 steps instead of 16 staged in shared memory (half
- * the shared memory per strip, so that strips of different batch cases can share an SM).  All
+ * accuracy; 10 = as 9, with a ring of three stages of operands instead of five in shared memory (so
+ * that strips of different batch cases can share an SM).  All
  * give the same Gauss-Seidel result up to rounding.  Synchronizes the stream; drops captured
  * cycles. */
 int fasw_set_sweep(fasw_ctx* ctx, int kind);

@@ -231,8 +231,9 @@ int level_sweep_kind(const fasw_ctx* c, const LevelDev& L) {
   int k = c->sweep_kind;
   if (k == SWEEP_AUTO) {
     // measured per level on GB300: the warp strips win on every level in both precisions (mixed,
-    // one application: 64x16 28.6 against 32.3 us for the one-CTA hyperplane-staged sweep,
-    // 128x32 41.9 against 58.3 us)
+    // one application, before their strips went from 32 to 8 rows: 64x16 28.6 against 32.3 us for
+    // the one-CTA hyperplane-staged sweep, 128x32 41.9 against 58.3 us; the sweep alone is a quarter
+    // faster since)
     if (L.wsF) return SWEEP_WS;
     return c->mixed ? (L.hpF ? SWEEP_HP : SWEEP_CTA) : SWEEP_STRIPS;
   }

@@ -38,9 +38,9 @@ __device__ __forceinline__ bool on_cut(const LevelDev& L, int i) { return L.nw >
 // go to the hyperplane-major arrays of k_sweep_hp instead: entry h = (i + j) * nj + j holds
 // hpF[32h..] = G_W, G_S and hpB[32h..] = H_E, H_N (row-major 4x4 each); D^-1 stays in tb.
 // MODE 2 (WS): tb as MODE 0, and blocks 1-4 also in FP32 in the skewed layout of the warp-strip
-// sweep (kernels_sweep_ws.cu): forward rows G_W, G_S at strip j / 32, step i + j % 32, lane j % 32
+// sweep (kernels_sweep_ws.cu): forward rows G_W, G_S at strip j / 8, step i + j % 8, row j % 8
 // (G_S zero on row 0 except the upper wake, whose mirror precedes it), backward rows H_E, H_N at
-// step Mp - 1 - i - j % 32; the lower wake's G_S (the backward coupling to its mirror) to wsCut.
+// step Mp - 1 - i - j % 8; the lower wake's G_S (the backward coupling to its mirror) to wsCut.
 template <typename T, int MODE>
 __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
   constexpr bool HP = MODE == 1;
@@ -85,8 +85,8 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
   // MODE 2: this cell's forward / backward rows in the warp-strip layout
   const int jl = j % WS_ROWS, Mp = ws_steps(ni, nj);
   const bool cut = on_cut(L, i);
-  float4* wf = reinterpret_cast<float4*>(L.wsF) + ((size_t)(j / WS_ROWS) * Mp + (i + jl)) * WS_F4_STEP + jl;
-  float4* wb = reinterpret_cast<float4*>(L.wsB) + ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_F4_STEP + jl;
+  float4* wf = reinterpret_cast<float4*>(L.wsF) + ((size_t)(j / WS_ROWS) * Mp + (i + jl)) * WS_F4_STEP + 4 * jl;
+  float4* wb = reinterpret_cast<float4*>(L.wsB) + ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_F4_STEP + 4 * jl;
   const bool gs_fwd = j > 0 || (cut && ni - 1 - i < i);
   const bool cut_lower = j == 0 && cut && ni - 1 - i > i;
   // product helper: out = s * Di * B (B entry-major with stride sb at face f)
@@ -113,13 +113,13 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
       }
       if constexpr (MODE == 2) {
         const float4 f = make_float4(float(row[0]), float(row[1]), float(row[2]), float(row[3]));
-        if (slot == 1) wf[r * WS_ROWS] = f;
+        if (slot == 1) wf[r] = f;
         if (slot == 2) {
-          wf[(4 + r) * WS_ROWS] = gs_fwd ? f : make_float4(0.f, 0.f, 0.f, 0.f);
+          wf[WS_F4_STEP / 2 + r] = gs_fwd ? f : make_float4(0.f, 0.f, 0.f, 0.f);
           if (cut_lower) *reinterpret_cast<float4*>(L.wsCut + 16 * i + 4 * r) = f;
         }
-        if (slot == 3) wb[r * WS_ROWS] = f;
-        if (slot == 4) wb[(4 + r) * WS_ROWS] = f;
+        if (slot == 3) wb[r] = f;
+        if (slot == 4) wb[WS_F4_STEP / 2 + r] = f;
       }
     }
   };
@@ -776,7 +776,7 @@ int launch_sweep(const LevelDev& L, int mixed, int kind, int do_update, int aw, 
                  long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters) {
   if (is_ws(kind) && L.wsF)
     return launch_ws_sweep(L, mixed, 1, do_update, aw, alpha, rhs, prog, err, limit, st, exact_iters,
-                           kind == SWEEP_WS8 ? 8 : WS_K);
+                           kind != SWEEP_WS8);
   if (is_ws(kind)) kind = mixed ? SWEEP_AUTO : SWEEP_STRIPS;
   if (is_hp(kind) && mixed && L.hpF) {
     launch_pdl(k_hp_cy, (L.n + 127) / 128, 128, 0, st, L, reinterpret_cast<const float*>(L.tb), rhs);

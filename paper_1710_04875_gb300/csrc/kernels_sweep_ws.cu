@@ -6,23 +6,38 @@
 //   forward  y_c = D_c^-1 r_c + G_W y_W + G_S y_S            (y_S: the wake-cut mirror on row 0
 //                                                             of the upper wake),
 //   backward z_c = y_c + H_E z_E + H_N z_N (+ G_S z_mirror on row 0 of the lower wake).
-// Rows are cut into strips of 32, one warp each (lane = row); a lane holds all four components
-// of its cell, so a step of the recurrence is its own previous vector (the west / east
-// neighbour), the neighbour row's previous vector by one shuffle (south / north), and 32 FMAs.
-// There is no barrier inside a step: a strip is one warp.  A strip's operands are laid out in
-// the order the warp consumes them (strip-major, step by step; "skewed" so that lane jl at
-// step s holds cell i = s - jl, with zero padding where that cell does not exist), so that the
-// operands of CHUNK steps are one contiguous block: one elected lane moves it into shared
-// memory with one cp.async.bulk per chunk and array, completion tracked by an mbarrier, double
-// buffered, the first step's operands of the next chunk loaded before the last step of this one.
+// Rows are cut into strips of 8, one warp each, four lanes per cell (one per component): lane
+// 4 r + q holds component q of row r.  Step s of a strip takes cell i = s - r of row r, so that a
+// step needs only what the step before left: the cell's own previous vector (the west / east
+// neighbour) and the neighbour row's (south / north).
+//
+// What bounds it: the latency of one step, not bandwidth (about 5 % of the DRAM rate).  A step is
+// a store of the previous result to shared memory, two 16-byte loads of it (own vector and
+// neighbour row) and a chain of eight FMAs; at 1024x256 the chain is walked 2 x 1,032 times.
+// Measured per step on one SM, operands in shared memory: one lane per cell (32 rows, shuffles,
+// nine 16-byte operand loads per lane) 96 cycles and 124 with its 16-byte result store; two lanes
+// per cell 108; four lanes with eight shuffles 85; four lanes exchanging through shared memory 67.
+// The operand and result instructions of a step queue ahead of the next step's exchange in the
+// same in-order pipe, so fewer of them per lane is what shortens the step.
+//
+// A strip's operands are laid out in the order its warp consumes them (strip-major, step by step,
+// zero where a step has no cell).  A second warp per strip moves them: stages of eight steps by
+// cp.async.bulk into a ring in shared memory, and the results back by one bulk store per stage, so
+// that the computing warp issues no global access at all; a third warp watches for what a stage
+// needs.  Two strips share a CTA (each strip's computing warp has a scheduler of its own; one strip
+// per CTA is 1-3 % faster alone and takes twice the SMs).
+//
 // The strips of a sweep form one thread-block cluster.  Strip b follows strip b-1 (forward; b+1
-// backward) through the neighbour's boundary row: the neighbour's out lane stores its vector of
-// every step straight into this strip's shared memory (a remote store inside the cluster), into
-// a buffer that holds a sentinel bit pattern until the value lands; this strip polls its own
-// shared memory once per chunk.  No fence or flag is needed: each 32-bit word arrives whole, and
-// the sentinel (a NaN payload that no arithmetic produces) marks the words not yet written.
-// Every wait is bounded; on timeout the kernel sets the error word, waits (bounded) for its own
-// copies in flight, and still meets the cluster's barriers, so that no strip waits forever.
+// backward) through the neighbour's boundary row: each stage of the neighbour's out row is stored
+// straight into this strip's edge buffer (remote stores inside the cluster), which holds a
+// sentinel bit pattern until the value lands.  No fence or flag is needed: each 32-bit word arrives
+// whole, and the sentinel (a NaN payload that no arithmetic produces) marks the words not yet
+// written.  Every wait is bounded; on timeout the kernel sets the error word, waits (bounded) for its
+// own copies in flight, and still meets the cluster's barriers, so that no strip waits forever.
+//
+// One sweep pair (launches back to back), against strips of 32 rows with a lane per cell that staged
+// and stored for themselves: 64x16 17.7 -> 13.3 us, 128x32 30.8 -> 24.2, 256x64 62.5 -> 45.3,
+// 1024x256 246 -> 171; about 45 ns a step (about 80 before) and 1.3 us from strip to strip.
 #include <atomic>
 #include <cstdint>
 #include <type_traits>
@@ -34,9 +49,12 @@ namespace fasw {
 
 namespace {
 
-constexpr int WS_STAGES = 2;   // chunk buffers (one in use, one in flight)
-constexpr int WS_U = 8;        // steps unrolled together (a chunk of KC steps is KC / WS_U such blocks)
 constexpr unsigned WS_SENT = 0xFFFFFFFFu;  // "not yet written": a NaN payload no FP32 operation returns
+constexpr unsigned WS_ALL = 0xFFFFFFFFu;   // every lane of a warp
+constexpr int WS_STEP_BYTES = 16 * WS_F4_STEP, WS_VEC_BYTES = 16 * WS_ROWS;  // one step's blocks / vectors
+constexpr int WS_HEAD = 512;               // barriers and the two strips' give-up words
+constexpr int WS_STAGES = 5, WS_SHALLOW = 3;  // ring depth; of kind 10
+constexpr int WS_TAIL = 16;                // zero entries after the edge buffer's last step
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -66,6 +84,14 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned b
                : "memory");
 }
 
+// shared -> global bulk copy (same rules), and the wait until its source may be overwritten
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_addr(src)),
+               "r"(bytes)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
 // address of the same shared-memory variable in CTA `rank` of this cluster
 __device__ __forceinline__ unsigned cluster_addr(const void* p, unsigned rank) {
   unsigned r;
@@ -73,103 +99,125 @@ __device__ __forceinline__ unsigned cluster_addr(const void* p, unsigned rank) {
   return r;
 }
 
-// predicated in the instruction itself (no branch around it: one lane of the warp stores)
-__device__ __forceinline__ void st_cluster4_if(bool pred, unsigned addr, float4 v) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n"
-      " @p st.relaxed.cluster.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n}\n" ::"r"(addr),
-      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"((unsigned)pred)
-      : "memory");
+__device__ __forceinline__ float4 lds4(unsigned a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
 }
 
-__device__ __forceinline__ uint4 ld_cluster4(const float4* p) {
+__device__ __forceinline__ float lds1(unsigned a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void sts1(unsigned a, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+// predicated in the instruction itself (no branch around it)
+__device__ __forceinline__ void sts1_if(bool pred, unsigned a, float v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n @p st.shared.f32 [%0], %1;\n}\n" ::"r"(a), "f"(v),
+               "r"((unsigned)pred)
+               : "memory");
+}
+
+__device__ __forceinline__ void sts4(unsigned a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
+__device__ __forceinline__ void st_cluster4(unsigned a, float4 v) {
+  asm volatile("st.relaxed.cluster.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_if(bool pred, uint64_t* bar) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %1, 0;\n @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n" ::"r"(
+                   smem_addr(bar)),
+               "r"((unsigned)pred)
+               : "memory");
+}
+
+__device__ __forceinline__ uint4 ld_cluster4(unsigned a) {
   uint4 v;
   asm volatile("ld.relaxed.cluster.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "r"(smem_addr(p))
+               : "r"(a)
                : "memory");
   return v;
+}
+
+__device__ __forceinline__ unsigned ld_acquire(unsigned a) {
+  unsigned v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ unsigned ld_relaxed(unsigned a) {
+  unsigned v;
+  asm volatile("ld.relaxed.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_release(unsigned a, unsigned v) {
+  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ bool unwritten(uint4 v) {
   return v.x == WS_SENT || v.y == WS_SENT || v.z == WS_SENT || v.w == WS_SENT;
 }
 
-// A lone strip (a cluster of one CTA, one warp) shares its shared memory with no one: a warp
-// barrier orders its own accesses, and the cluster barrier is skipped.
-__device__ __forceinline__ void cluster_sync() {
-  __syncwarp();
-  if (gridDim.x > 1)
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  else
-    __syncwarp();
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-__device__ __forceinline__ float4 shfl_up4(float4 v) {
-  v.x = __shfl_up_sync(0xffffffffu, v.x, 1);
-  v.y = __shfl_up_sync(0xffffffffu, v.y, 1);
-  v.z = __shfl_up_sync(0xffffffffu, v.z, 1);
-  v.w = __shfl_up_sync(0xffffffffu, v.w, 1);
-  return v;
-}
-
-__device__ __forceinline__ float4 shfl_down4(float4 v) {
-  v.x = __shfl_down_sync(0xffffffffu, v.x, 1);
-  v.y = __shfl_down_sync(0xffffffffu, v.y, 1);
-  v.z = __shfl_down_sync(0xffffffffu, v.z, 1);
-  v.w = __shfl_down_sync(0xffffffffu, v.w, 1);
-  return v;
-}
-
-// out = c + A x + B w for row-major 4x4 blocks given as block rows A[0..3], B[0..3]
-__device__ __forceinline__ float4 two_blocks(float4 c, const float4* A, float4 x, const float4* B, float4 w) {
-  float o[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    // x (this lane's previous vector) is ready a shuffle earlier than w: one chain of eight FMAs,
-    // the A-part first (measured faster than splitting the w-part into two shorter chains joined
-    // by an add: four instructions fewer per step outweigh one FMA more of latency after the
-    // shuffle; 64x16 sweep pair 20.6 -> 18.6 us, 1024x256 243.8 -> 237.7 us)
-    const float4 a = A[q], b = B[q];
-    float s = (q == 0 ? c.x : q == 1 ? c.y : q == 2 ? c.z : c.w);
-    s = fmaf(a.x, x.x, s);
-    s = fmaf(a.y, x.y, s);
-    s = fmaf(a.z, x.z, s);
-    s = fmaf(a.w, x.w, s);
-    o[q] = fmaf(b.w, w.w, fmaf(b.z, w.z, fmaf(b.y, w.y, fmaf(b.x, w.x, s))));
-  }
-  return make_float4(o[0], o[1], o[2], o[3]);
-}
-
-__device__ __forceinline__ float4 add_block(float4 v, const float* G, float4 x) {
-  v.x += G[0] * x.x + G[1] * x.y + G[2] * x.z + G[3] * x.w;
-  v.y += G[4] * x.x + G[5] * x.y + G[6] * x.z + G[7] * x.w;
-  v.z += G[8] * x.x + G[9] * x.y + G[10] * x.z + G[11] * x.w;
-  v.w += G[12] * x.x + G[13] * x.y + G[14] * x.z + G[15] * x.w;
-  return v;
-}
-
-// Shared memory of the sweep: [mbarriers][ring of blocks][ring of vectors][stage][edge][cut vectors][cut blocks]
+// Shared memory of one strip (byte addresses): the barriers of its ring, the ring (blocks, right
+// hand sides, results), the exchange vectors of the last step, the edge buffers of the two passes
+// (one buffer, cleared between them, on grids too long for two); and, shared by the CTA, the wake
+// cut's vectors and coupling blocks (strip 0 only).
 struct WsSmem {
-  uint64_t* bar;
-  float4* ringF;  // WS_STAGES x KC x WS_F4_STEP
-  float4* ringC;  // WS_STAGES x KC x 32
-  float4* stage;  // KC: the neighbour's boundary vectors of the current chunk, checked
-  float4* edge;   // Mp + 32: the neighbour's out-lane vector of its step t (t >= Mp: zero)
-  float4* cutv;   // nw
-  float* cutG;    // nw x 16
+  uint64_t *full, *empty;    // per ring slot: operands landed; slot consumed, its results complete
+  // counters: ring uses whose operands and edge entries have landed; passes whose first right-hand
+  // sides are in place
+  unsigned char *ready, *primed;
+  volatile int* gave_up;     // a warp of this strip gave up
+  unsigned char *F, *C, *H;  // NS stages of blocks / right-hand sides / results
+  unsigned char* X;          // [row][component] of the last step
+  unsigned char *Ef, *Eb;    // Mp + WS_TAIL vectors: the neighbour's out row by its step (t >= Mp: zero)
+  unsigned char *cutv, *cutG;
 };
 
-template <int KC>
-__device__ __forceinline__ WsSmem ws_carve(unsigned char* base, int Mp, int nw) {
+template <int NS, bool TWO>
+__host__ __device__ constexpr size_t ws_strip_bytes(int Mp) {
+  return (size_t)NS * WS_U * (WS_STEP_BYTES + 2 * WS_VEC_BYTES) + WS_VEC_BYTES +
+         (TWO ? 2 : 1) * (size_t)(Mp + WS_TAIL) * 16;
+}
+
+template <int NS, bool TWO>
+__host__ __device__ constexpr size_t ws_cta_bytes(int Mp, int nw) {
+  return WS_HEAD + 2 * ws_strip_bytes<NS, TWO>(Mp) + 80 * (size_t)(nw > 0 ? nw : 1);
+}
+
+template <int NS, bool TWO>
+__device__ __forceinline__ WsSmem ws_carve(unsigned char* base, int w, int Mp, int nw) {
+  static_assert(32 * NS + 32 <= WS_HEAD, "the barriers fit the head");
   WsSmem S;
-  S.bar = reinterpret_cast<uint64_t*>(base);
-  S.ringF = reinterpret_cast<float4*>(base + 128);
-  S.ringC = S.ringF + WS_STAGES * KC * WS_F4_STEP;
-  S.stage = S.ringC + WS_STAGES * KC * WS_ROWS;
-  S.edge = S.stage + KC;
-  S.cutv = S.edge + Mp + 32;
-  S.cutG = reinterpret_cast<float*>(S.cutv + (nw > 0 ? nw : 1));
+  S.full = reinterpret_cast<uint64_t*>(base) + w * 2 * NS;
+  S.empty = S.full + NS;
+  S.ready = base + WS_HEAD - 8 + 4 * w;
+  S.primed = S.ready - 16;
+  S.gave_up = reinterpret_cast<volatile int*>(base + WS_HEAD - 16) + w;
+  S.F = base + WS_HEAD + w * ws_strip_bytes<NS, TWO>(Mp);
+  S.C = S.F + NS * WS_U * WS_STEP_BYTES;
+  S.H = S.C + NS * WS_U * WS_VEC_BYTES;
+  S.X = S.H + NS * WS_U * WS_VEC_BYTES;
+  S.Ef = S.X + WS_VEC_BYTES;
+  S.Eb = TWO ? S.Ef + (size_t)(Mp + WS_TAIL) * 16 : S.Ef;
+  S.cutv = base + WS_HEAD + 2 * ws_strip_bytes<NS, TWO>(Mp);
+  S.cutG = S.cutv + 16 * (size_t)(nw > 0 ? nw : 1);
   return S;
 }
 
@@ -177,251 +225,346 @@ __device__ __forceinline__ WsSmem ws_carve(unsigned char* base, int Mp, int nw) 
 
 int ws_strips(int nj) { return (nj + WS_ROWS - 1) / WS_ROWS; }
 
-size_t ws_smem_bytes(int ni, int nj, int nw, int KC) {
-  const int m = nw > 0 ? nw : 1;
-  return 128 + 16 * ((size_t)WS_STAGES * KC * (WS_F4_STEP + WS_ROWS) + KC + ws_steps(ni, nj) + 32 + m) +
-         64 * (size_t)m;
-}
-
 namespace {
 
 // Skewed index of cell (i, j) in the backward order (the layout of y as the backward pass reads
-// it and of its result z): strip j / 32, step Mp - 1 - i - jl, lane jl.
+// it and of its result z): strip j / WS_ROWS, step Mp - 1 - i - r, row r.
 __device__ __forceinline__ size_t ws_bpos(int i, int j, int Mp) {
   const int jl = j & (WS_ROWS - 1);
   return ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_ROWS + jl;
 }
 
-// One pass (forward: FWD, else backward) of one strip.  Returns false on a timeout.
-// F: blocks of the pass, C: its right-hand side vectors (forward: D^-1 r; backward: y), both
-// skewed; Out: the pass's result, skewed in the backward order (forward: y; backward: z).
-// has_in: a neighbour strip feeds this one's edge lane (below forward, above backward) through
-// S.edge; redge: the cluster address of the edge buffer of the strip this one feeds (0: none).
-// Lane jl at step s holds cell i = s - jl (forward) or Mp - 1 - s - jl (backward); the edge lane
-// needs the neighbour's out-lane vector of the same column, which the neighbour computed at its
-// step s + 31: edge entry s + 31 (entries Mp .. Mp + 31 are zero).
-template <bool FWD, int KC>
-__device__ bool ws_pass(const LevelDev& L, const WsSmem& S, int b, const float4* F, const float4* C, float4* Out,
-                        bool has_in, unsigned redge, int* err, long long limit, unsigned& phase_bits) {
-  const int lane = threadIdx.x;
-  const int ni = L.ni, nw = L.nw;
-  const int Mp = ws_steps(ni, L.nj);        // steps that hold a cell, padded to whole chunks
-  const int nch = Mp / KC;
-  const int edge_lane = FWD ? 0 : WS_ROWS - 1;      // lane that reads the neighbour's row
-  const int out_lane = FWD ? WS_ROWS - 1 : 0;       // lane whose row the other neighbour reads
-  const float4* Fs = F + (size_t)b * Mp * WS_F4_STEP;
-  const float4* Cs = C + (size_t)b * Mp * WS_ROWS;
-  float4* Os = Out + (size_t)b * Mp * WS_ROWS + lane;
-  const unsigned bytesF = KC * WS_F4_STEP * 16, bytesC = KC * WS_ROWS * 16;
-  const bool feeds = redge != 0 && lane == out_lane;
+// Ring bookkeeping: stage ch of a pass that starts at ring count `base` (0 forward, the number of
+// stages backward) is ring use n = base + ch: slot n % NS, phase n / NS.
+template <int NS>
+__device__ __forceinline__ bool ws_landed(uint64_t* bar, unsigned n) {
+  return mbar_test(&bar[n % NS], (n / NS) & 1u);
+}
 
-  // Refill of a slot by the async proxy: the slot's previous contents were only read (no generic
-  // writes), and every one of those reads has completed, its value used by an earlier step of
-  // this warp, so no proxy fence is needed before the copy overwrites them.
-  auto issue = [&](int ch) {  // lane 0 only
-    const int slot = ch % WS_STAGES;
-    mbar_expect_tx(&S.bar[slot], bytesF + bytesC);
-    bulk_copy(S.ringF + (size_t)slot * KC * WS_F4_STEP, Fs + (size_t)ch * KC * WS_F4_STEP, bytesF, &S.bar[slot]);
-    bulk_copy(S.ringC + (size_t)slot * KC * WS_ROWS, Cs + (size_t)ch * KC * WS_ROWS, bytesC, &S.bar[slot]);
-  };
-  int waited = 0;  // chunks whose copies have landed (and been accounted for)
-  // bounded wait for the chunk in a slot; false on timeout
-  auto wait_slot = [&](int slot) -> bool {
-    const unsigned par = (phase_bits >> slot) & 1u;
-    long long spins = 0;
-    bool ok = true;
-    while (!mbar_test(&S.bar[slot], par)) {
-      if (++spins > limit) {
-        ok = false;
-        break;
-      }
-    }
-    ok = __all_sync(0xffffffffu, ok);
-    if (ok) {
-      phase_bits ^= 1u << slot;
-      ++waited;
-    }
-    return ok;
-  };
-  int issued = 0;
-  // after a timeout: wait for every copy still in flight into this CTA's shared memory before
-  // returning.  These copies depend on no other CTA and finish within microseconds, so their
-  // bound is fixed and generous, independent of the caller's (possibly tiny) spin limit.
-  auto fail = [&]() {
-    if (lane == 0) atomicExch(err, 1);
-    for (int ch = waited; ch < issued; ++ch) {
-      const int slot = ch % WS_STAGES;
-      const unsigned par = (phase_bits >> slot) & 1u;
-      long long spins = 0;
-      while (!mbar_test(&S.bar[slot], par) && ++spins <= (1LL << 26)) {
-      }
-      phase_bits ^= 1u << slot;
-    }
-    __syncwarp();
-    return false;
-  };
-  // the neighbour's boundary vectors of steps s0 .. s0 + KC - 1 into S.stage: lane k polls
-  // edge entry s0 + 31 + k until the neighbour's store has landed (bounded; a neighbour that
-  // gave up has set the error word)
-  // The loop is warp-uniform (a vote decides whether any lane still waits), so that the warp
-  // leaves it converged.
-  auto poll_edge = [&](int s0) -> bool {
-    const float4* e = S.edge + s0 + (WS_ROWS - 1) + (lane & (KC - 1));
-    uint4 v = ld_cluster4(e);
-    long long spins = 0;
-    while (__any_sync(0xffffffffu, unwritten(v))) {
-      if (++spins > limit || ((spins & 255) == 0 && *((volatile int*)err) != 0)) return false;
-      v = ld_cluster4(e);
-    }
-    if (lane < KC)
-      S.stage[lane] = make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z),
-                                  __uint_as_float(v.w));
-    __syncwarp();
-    return true;
-  };
+__device__ __forceinline__ void ws_give_up(const WsSmem& S, int* err) {
+  atomicExch(err, 1);
+  *S.gave_up = 1;
+}
 
-  if (lane == 0)
-    for (int ch = 0; ch < WS_STAGES && ch < nch; ++ch) issue(ch);
+// What the copying warp of a strip moves: blocks and right-hand sides in, results out.
+struct WsGlobal {
+  const unsigned char *F, *B, *C;  // forward / backward blocks, forward right-hand sides
+  unsigned char *Y, *Z;            // forward result (the backward right-hand sides), backward result
+  int nch;                         // stages of a pass
+};
+
+// Fills the slot of ring use n (the copying lane).  The right-hand sides of the first NS backward
+// stages are not fetched: they are the last forward stages' results, still in shared memory.
+template <int NS>
+__device__ __forceinline__ void ws_fill(const WsSmem& S, const WsGlobal& G, unsigned n) {
+  constexpr unsigned FB = WS_U * WS_STEP_BYTES, CB = WS_U * WS_VEC_BYTES;
+  const unsigned sl = n % NS;
+  const bool fwd = n < (unsigned)G.nch;
+  const size_t ch = fwd ? n : n - G.nch;
+  const bool rhs = fwd || ch >= NS;
+  mbar_expect_tx(&S.full[sl], rhs ? FB + CB : FB);
+  bulk_copy(S.F + sl * FB, (fwd ? G.F : G.B) + ch * FB, FB, &S.full[sl]);
+  if (rhs) bulk_copy(S.C + sl * CB, (fwd ? G.C : G.Y) + ch * CB, CB, &S.full[sl]);
+}
+
+// The helper warps' loops are warp-uniform (a vote decides whether any lane still waits), so that a
+// warp leaves them converged; each ends when the strip gives up, or after WS_LONG rounds (helpers
+// outwait the computing warp and the edge entries, whose limit is the caller's).
+constexpr long long WS_LONG = 1LL << 26;
+
+template <class Ready>
+__device__ __forceinline__ bool ws_wait(const WsSmem& S, Ready ready) {
+  long long spins = 0;
+  while (!__all_sync(WS_ALL, ready()))
+    if (__any_sync(WS_ALL, *S.gave_up || ++spins > WS_LONG)) return false;
+  return true;
+}
+
+// One pass of the copying warp: a consumed slot's boundary row goes to the strip this one feeds
+// (feeds: the cluster address of its edge buffer, 0: none), its results to global memory, then the
+// slot is filled again (backward stages too: their blocks are on their way while the forward pass
+// ends).  A slot's operands were only read by the computing warp, its results written by it before
+// it arrived on `empty`.  Returns false if the strip gave up, after waiting (bounded: its copies
+// depend on no other CTA) for the copies in flight into this CTA's shared memory.
+template <bool FWD, int NS>
+__device__ __forceinline__ bool ws_copies(const WsSmem& S, const WsGlobal& G, unsigned feeds) {
+  constexpr unsigned CB = WS_U * WS_VEC_BYTES;
+  const int lane = threadIdx.x & 31;
+  const unsigned nch = G.nch, all = 2 * nch, base = FWD ? 0 : nch, end = base + nch;
+  if (FWD) {
+    if (lane == 0)
+      for (unsigned n = 0; n < NS && n < all; ++n) ws_fill<NS>(S, G, n);
+  } else {
+    // results of stage nch - 1 - k: right-hand sides of ring use nch + k
+    for (int k = min(NS, G.nch) - 1; k >= 0; --k) {
+      const unsigned from = smem_addr(S.H) + ((nch - 1 - k) % NS) * CB, to = smem_addr(S.C) + ((nch + k) % NS) * CB;
+      for (unsigned x = 16 * lane; x < CB; x += 512) sts4(to + x, lds4(from + x));
+    }
+  }
   __syncwarp();
-  issued = nch < WS_STAGES ? nch : WS_STAGES;
-  if (!has_in && lane < KC) S.stage[lane] = make_float4(0.f, 0.f, 0.f, 0.f);  // no neighbour: zero
-  __syncwarp();
-
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // this lane's vector at the previous step
-  // Operands of one step: this lane's rows of the two blocks and its right-hand side vector,
-  // loaded one step ahead of their use (across chunk boundaries too: the next chunk's first
-  // step is loaded before this chunk's last), and the edge value, loaded one step ahead inside
-  // a chunk, so that shared-memory latency stays off the chain.
-  struct Ops {
-    float4 A[4], B[4], c;
-  };
-  auto load = [&](Ops& o, int slot, int k) {
-    const float4* rF = S.ringF + (size_t)slot * KC * WS_F4_STEP;
-    const float4* rC = S.ringC + (size_t)slot * KC * WS_ROWS;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      o.A[q] = rF[k * WS_F4_STEP + q * WS_ROWS + lane];
-      o.B[q] = rF[k * WS_F4_STEP + (4 + q) * WS_ROWS + lane];
-    }
-    o.c = rC[k * WS_ROWS + lane];
-  };
-  // One step.  Padded positions (no cell) carry zero blocks and vectors, so they compute zero
-  // and need no test: every step writes its result.  Only the wake-cut coupling of row 0
-  // (strip 0, lane 0) is special, and chunks that hold no cut cell run the step without it
-  // (CUT false).
-  auto step = [&](const Ops& o, float4 e, int s, auto cut_tag) {
-    constexpr bool CUT = decltype(cut_tag)::value;
-    float4 w = FWD ? shfl_up4(v) : shfl_down4(v);  // the row below (forward) / above (backward)
-    if (lane == edge_lane) w = e;                   // neighbour strip's row, or zero
-    const int i = FWD ? s - lane : Mp - 1 - s - lane;  // this lane's cell (i, j)
-    if constexpr (CUT && FWD)
-      if (lane == 0 && i >= ni - nw && i < ni) w = S.cutv[ni - 1 - i];  // upper wake: its mirror
-    float4 y = two_blocks(o.c, o.A, v, o.B, w);
-    if constexpr (CUT && !FWD)
-      if (lane == 0 && i >= 0 && i < nw) y = add_block(y, S.cutG + 16 * i, S.cutv[i]);  // lower wake
-    if constexpr (CUT) {
-      if (lane == 0 && FWD && i >= 0 && i < nw) S.cutv[i] = y;                   // read by its mirror
-      if (lane == 0 && !FWD && i >= ni - nw && i < ni) S.cutv[ni - 1 - i] = y;   // read by its mirror
-    }
-    Os[(size_t)(FWD ? Mp - 1 - s : s) * WS_ROWS] = y;
-    st_cluster4_if(feeds, redge + 16u * (unsigned)s, y);  // the fed strip's edge entry s
-    v = y;
-  };
-  // o[0] holds the next step's operands between chunks: the last step of a chunk loads the next
-  // chunk's first step into it.  A chunk runs as KC / WS_U blocks of WS_U unrolled steps, which
-  // keeps the code of a pass small enough for the instruction cache.
-  Ops o[2];
-  float4 e[2];
-  bool late = false;  // the next chunk's wait gave up
-  auto run_chunk = [&](int slot, int ch, int s0, auto cut_tag) {
-    e[0] = S.stage[0];
-#pragma unroll 1
-    for (int kk = 0; kk < KC; kk += WS_U) {
-#pragma unroll
-      for (int u = 0; u < WS_U; ++u) {
-        const int k = kk + u;
-        if (u + 1 < WS_U || kk + WS_U < KC) {
-          load(o[(u + 1) & 1], slot, k + 1);
-          e[(u + 1) & 1] = S.stage[k + 1];
-        } else if (ch + 1 < nch) {
-          if (wait_slot((ch + 1) % WS_STAGES))
-            load(o[0], (ch + 1) % WS_STAGES, 0);
-          else
-            late = true;
+  if (lane == 0) st_release(smem_addr(S.primed), FWD ? 1 : 2);
+  for (unsigned n = base; n < end; ++n) {
+    if (!ws_wait(S, [&] { return ws_landed<NS>(S.empty, n); })) {
+      for (unsigned k = n; k < n + NS && k < all; ++k) {
+        long long m = 0;
+        while (!ws_landed<NS>(S.full, k) && ++m <= WS_LONG) {
         }
-        step(o[u & 1], e[u & 1], s0 + k, cut_tag);
+      }
+      asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+      __syncwarp();
+      return false;
+    }
+    const unsigned d = n - base;
+    const unsigned char* H = S.H + (n % NS) * CB;
+    if (feeds && lane < WS_U)  // the out row at step d WS_U + lane
+      st_cluster4(feeds + 16 * (d * WS_U + lane),
+                  lds4(smem_addr(H) + (FWD ? WS_U - 1 - lane : lane) * WS_VEC_BYTES + (FWD ? 16 * (WS_ROWS - 1) : 0)));
+    if (lane == 0) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the results just acquired
+      bulk_store((FWD ? G.Y : G.Z) + (size_t)(FWD ? nch - 1 - d : d) * CB, H, CB);
+      if (n + NS < all) {
+        if (n == nch)  // from here on y comes back from global memory: its stores have completed
+          asm volatile("cp.async.bulk.wait_group 1;\n\tfence.proxy.async.global;" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        ws_fill<NS>(S, G, n + NS);
       }
     }
-  };
+    __syncwarp();
+  }
+  if (!FWD) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  __syncwarp();
+  return true;
+}
 
-  if (!wait_slot(0)) return fail();
-  load(o[0], 0, 0);
+// One pass of the watching warp: a stage is ready when its operands have landed and, where a
+// neighbour feeds this strip, its edge entries (lane k: entry s0 + 7 + k): none of their words holds
+// the sentinel.
+template <int NS>
+__device__ __forceinline__ bool ws_watch(const WsSmem& S, int nch, unsigned base, bool fed, const unsigned char* Eb,
+                                         int* err, long long limit) {
+  const int lane = threadIdx.x & 31;
+  const unsigned E = smem_addr(Eb) + 16 * (WS_ROWS - 1 + (lane & (WS_U - 1)));
+  if (!ws_wait(S, [&] { return ld_acquire(smem_addr(S.primed)) > (base ? 1u : 0u); })) return false;
   for (int ch = 0; ch < nch; ++ch) {
-    const int s0 = ch * KC;
-    if (has_in && !poll_edge(s0)) return fail();
-    const int slot = ch % WS_STAGES;
-    // does lane 0 of strip 0 meet a wake-cut cell in this chunk?
-    const int ilo = FWD ? s0 : Mp - s0 - KC, ihi = FWD ? s0 + KC - 1 : Mp - 1 - s0;
-    const bool cut = b == 0 && nw > 0 && (ilo < nw || ihi >= ni - nw);
-    if (cut)
-      run_chunk(slot, ch, s0, std::true_type{});
-    else
-      run_chunk(slot, ch, s0, std::false_type{});
+    if (!ws_wait(S, [&] { return ws_landed<NS>(S.full, base + ch); })) return false;
+    long long spins = 0;
+    while (fed && __any_sync(WS_ALL, unwritten(ld_cluster4(E + 16 * WS_U * ch)))) {
+      ++spins;
+      const bool stop = spins > limit || ((spins & 255) == 0 && (*S.gave_up || *((volatile int*)err) != 0));
+      if (__any_sync(WS_ALL, stop)) {
+        if (lane == 0) ws_give_up(S, err);
+        __syncwarp();
+        return false;
+      }
+    }
     __syncwarp();
-    if (late) return fail();
-    // this chunk's slot is free again (its operands are all in registers or consumed)
-    if (lane == 0 && issued < nch) issue(issued);
-    if (issued < nch) ++issued;
-    __syncwarp();
+    if (lane == 0) st_release(smem_addr(S.ready), base + ch + 1);
   }
   return true;
 }
 
-// the edge buffer before a pass: entries the neighbour will write hold the sentinel, the
-// entries past the last step zero
-__device__ __forceinline__ void ws_clear_edge(const WsSmem& S, int Mp) {
-  const float sent = __uint_as_float(WS_SENT);
-  for (int t = threadIdx.x; t < Mp + 32; t += 32)
-    S.edge[t] = t < Mp ? make_float4(sent, sent, sent, sent) : make_float4(0.f, 0.f, 0.f, 0.f);
+// One pass (forward: FWD, else backward) of one strip by its computing warp.  Returns false on a
+// timeout.  Row r at step s holds cell i = s - r (forward) or Mp - 1 - s - r (backward); the edge
+// row needs the neighbour's out row of the same column, which the neighbour computed at its step
+// s + 7: edge entry s + 7 (entries Mp ... are zero).  On row 0 of the upper wake the entry is the
+// mirror cell's vector, stored there by this strip's own row 0 when it passed that cell.
+// zero: always 0, unknown to the compiler.
+//
+// A taken branch costs this warp about 35 cycles and each test or vote as much as half a step, so
+// a stage is straight-line code: eight unrolled steps, one wait, asked for two steps ahead, and one
+// loop branch; everything else is the other warps' work.
+template <bool FWD, int NS>
+__device__ __forceinline__ bool ws_pass(const LevelDev& L, const WsSmem& S, int b, int Mp, unsigned base, int* err,
+                                        long long limit, unsigned zero) {
+  constexpr unsigned FB = WS_U * WS_STEP_BYTES, CB = WS_U * WS_VEC_BYTES;
+  const int lane = threadIdx.x & 31, r = lane >> 2, q = lane & 3;
+  const int ni = L.ni, nw = L.nw, nch = Mp / WS_U;
+  const bool edge_row = r == (FWD ? 0 : WS_ROWS - 1);
+  const unsigned x_own = smem_addr(S.X) + 16 * r, x_put = smem_addr(S.X) + 4 * lane;
+  const unsigned E = smem_addr(FWD ? S.Ef : S.Eb), ready = smem_addr(S.ready);
+  const unsigned fa = smem_addr(S.F) + 16 * lane, ca = smem_addr(S.C) + 4 * lane, ha = smem_addr(S.H) + 4 * lane;
+  const unsigned cutv = smem_addr(S.cutv), cutG = smem_addr(S.cutG) + 16 * q;
+  // the row below (forward) / above (backward); the edge row's moves on by an entry a step
+  const unsigned nb0 = edge_row ? E + 16 * (WS_ROWS - 1) : FWD ? x_own - 16 : x_own + 16;
+  const unsigned nb_step = edge_row ? 16 : 0;
+
+  auto wait_stage = [&](unsigned n) -> bool {  // the rare path: the stage has not landed yet
+    long long spins = 0;
+    while (!__all_sync(WS_ALL, ld_acquire(ready) > n)) {
+      ++spins;
+      const bool stop = spins > limit || ((spins & 255) == 0 && *S.gave_up);
+      if (__any_sync(WS_ALL, stop)) {
+        if (lane == 0) ws_give_up(S, err);
+        __syncwarp();
+        return false;
+      }
+    }
+    return true;
+  };
+  // Operands of one step: this lane's row of the two blocks and its right-hand side component,
+  // loaded one step ahead of their use (across stages too).
+  float4 A[2], B[2];
+  float c[2];
+  auto load = [&](int z, unsigned sl, int u) {
+    A[z] = lds4(fa + sl * FB + u * WS_STEP_BYTES);
+    B[z] = lds4(fa + sl * FB + u * WS_STEP_BYTES + WS_STEP_BYTES / 2);
+    c[z] = lds1(ca + sl * CB + u * WS_VEC_BYTES);
+  };
+  float y = 0.f;            // this lane's component at the previous step
+  unsigned sl = base % NS;  // ring slot
+  bool ok = true;
+  // Stages ch0 .. ch1 - 1.  Padded positions (no cell) carry zero blocks and vectors, so they
+  // compute zero and need no test.  Only the wake-cut coupling of row 0 (strip 0) is special; stages
+  // that hold no cut cell run without it (CUT false).
+  auto stages = [&](int ch0, int ch1, auto cut_tag) {
+    constexpr bool CUT = decltype(cut_tag)::value;
+#pragma unroll 1
+    for (int ch = ch0; ch < ch1; ++ch) {
+      const int s = ch * WS_U;
+      const unsigned nb = nb0 + ch * WS_U * nb_step, h = ha + sl * CB;
+      const unsigned nsl = sl + 1 == NS ? 0 : sl + 1;
+      const unsigned next = base + min(ch + 1, nch - 1);  // the last stage waits for itself
+      unsigned landed = 0;
+#pragma unroll
+      for (int u = 0; u < WS_U; ++u) {
+        // The address depends (by an AND with zero) on the operands loaded during the last step:
+        // without it they are scheduled right before this store and delay the exchange behind them
+        // (67 -> 80 cycles per step).
+        sts1(x_put | (__float_as_uint(c[u & 1]) & zero), y);
+        __syncwarp();
+        const float4 x = lds4(x_own), w = lds4(nb + u * nb_step);
+        if (u > 0) sts1(h + (FWD ? WS_U - u : u - 1) * WS_VEC_BYTES, y);  // the previous step's result
+        if (u == WS_U - 2) landed = ld_relaxed(ready);
+        if (u == WS_U - 1 && __builtin_expect(landed <= next, 0) && !wait_stage(next)) {
+          ok = false;
+          return;
+        }
+        if (u == WS_U - 1) asm volatile("fence.acq_rel.cta;" ::: "memory");  // the counter was read relaxed
+        load((u + 1) & 1, u + 1 < WS_U ? sl : nsl, (u + 1) % WS_U);
+        // the west / east part first: its vector is this row's own
+        float a = c[u & 1];
+        a = fmaf(A[u & 1].x, x.x, a);
+        a = fmaf(A[u & 1].y, x.y, a);
+        a = fmaf(A[u & 1].z, x.z, a);
+        a = fmaf(A[u & 1].w, x.w, a);
+        a = fmaf(B[u & 1].x, w.x, a);
+        a = fmaf(B[u & 1].y, w.y, a);
+        a = fmaf(B[u & 1].z, w.z, a);
+        a = fmaf(B[u & 1].w, w.w, a);
+        if constexpr (CUT) {
+          const int i = FWD ? s + u : Mp - 1 - s - u, m = ni - 1 - i;  // row 0's cell and its mirror
+          if (FWD) {  // lower wake: read by its mirror as that cell's edge entry
+            sts1_if(r == 0 && i < nw, E + 16 * (unsigned)(m + WS_ROWS - 1) + 4 * q, a);
+          } else {
+            const int ic = min(max(i, 0), nw - 1);
+            const float4 g = lds4(cutG + 64 * ic), v = lds4(cutv + 16 * ic);
+            const float t = fmaf(g.w, v.w, fmaf(g.z, v.z, fmaf(g.x, v.x, __fmul_rn(g.y, v.y))));
+            if (r == 0 && i >= 0 && i < nw) a = __fadd_rn(a, t);                              // lower wake
+            sts1_if(r == 0 && i < ni && m < nw, cutv + 16 * (unsigned)max(m, 0) + 4 * q, a);  // read by its mirror
+          }
+        }
+        y = a;
+      }
+      sts1(h + (FWD ? 0 : WS_U - 1) * WS_VEC_BYTES, y);
+      // the slot's operands are consumed and its results complete: over to the copying warp
+      __syncwarp();
+      mbar_arrive_if(lane == 0, &S.empty[sl]);
+      sl = nsl;
+    }
+  };
+  if (!wait_stage(base)) return false;
+  load(0, sl, 0);
+  // stages with a cut cell of row 0 whose coupling is its own: forward the lower wake (the first
+  // nw columns); backward the upper wake (whose vectors are kept) and the lower one
+  const bool cut = b == 0 && nw > 0;
+  const int lo = cut ? min((nw + WS_U - 1) / WS_U, nch) : 0;               // stages 0 .. lo - 1: columns < nw
+  const int hi = cut ? min((Mp - (ni - nw) + WS_U - 1) / WS_U, nch) : 0;   // backward: columns >= ni - nw
+  const int mid = cut && !FWD ? min(max(hi, (Mp - nw) / WS_U), nch) : nch;  // backward, from here: columns < nw
+  stages(0, FWD ? lo : hi, std::true_type{});
+  if (ok) stages(FWD ? lo : hi, mid, std::false_type{});
+  if (ok) stages(mid, nch, std::true_type{});
+  return ok;
 }
 
-// One launch: forward then backward pass of strip b (one warp per CTA, the nb strips one
-// cluster).  Every strip meets the cluster barriers (set-up, between the passes, at the end)
-// whatever happened in its passes, so that a strip that gave up leaves no other one waiting on
-// a barrier; the last barrier also keeps every strip's shared memory alive until the
-// neighbours' remote stores into it have completed.
-template <int KC>
-__global__ void __launch_bounds__(32) k_sweep_ws(LevelDev L, const float4* Fb, const float4* Bb, const float4* C,
-                                                 float4* Y, const float* cutG, float4* Z, int* err, long long limit) {
-  pdl_entry();
+__device__ __forceinline__ void ws_clear(unsigned char* E, int Mp, bool fed, int t0, int dt) {
+  const float sent = __uint_as_float(WS_SENT);
+  for (int t = t0; t < Mp + WS_TAIL; t += dt) {
+    const float v = t < Mp && fed ? sent : 0.f;
+    reinterpret_cast<float4*>(E)[t] = make_float4(v, v, v, v);
+  }
+}
+
+// One launch: forward then backward pass of every strip.  Warps 0 and 1 of a CTA compute strips
+// 2 blockIdx and 2 blockIdx + 1, on schedulers 0 and 1; their helpers (copying: warps 2, 3; watching:
+// 6, 7) are the warps of schedulers 2 and 3, so that no helper takes an issue slot of a computing
+// warp, and warps 4 and 5 only meet the barriers.  Every thread meets the cluster barriers (set-up,
+// two between the passes where they share an edge buffer, at the end) whatever happened in its
+// passes, so that a strip that gave up leaves no other one waiting on a barrier; the last barrier
+// also keeps every CTA's shared memory alive until the neighbours' remote stores into it have
+// completed.
+constexpr int WS_THREADS = 256;
+
+template <int NS, bool TWO>
+__global__ void __launch_bounds__(WS_THREADS)
+    k_sweep_ws(LevelDev L, const float4* Fb, const float4* Bb, const float4* C, float4* Y, const float* cutG, float4* Z,
+               int* err, long long limit, unsigned zero) {
   extern __shared__ __align__(128) unsigned char ws_raw[];
-  const int nw = L.nw;
-  const int Mp = ws_steps(L.ni, L.nj);
-  WsSmem S = ws_carve<KC>(ws_raw, Mp, nw);
-  const int b = blockIdx.x, nb = gridDim.x, lane = threadIdx.x;
-  if (lane == 0) {
-    for (int k = 0; k < WS_STAGES; ++k) mbar_init(&S.bar[k], 1);
+  const int nw = L.nw, Mp = ws_steps(L.ni, L.nj), nst = (L.nj + WS_ROWS - 1) / WS_ROWS;
+  const int warp = threadIdx.x >> 5, w = warp & 1, b = 2 * blockIdx.x + w, lane = threadIdx.x & 31;
+  const bool compute = warp < 2, copier = (warp & ~1) == 2, watcher = (warp & ~1) == 6;
+  const bool below = b > 0, above = b < nst - 1;  // neighbour strips
+  const WsSmem S = ws_carve<NS, TWO>(ws_raw, w, Mp, nw);
+  // set-up that touches this CTA's shared memory only, before the wait for the kernel before
+  if (copier && lane == 0) {
+    for (int k = 0; k < NS; ++k) {
+      mbar_init(&S.full[k], 1);
+      mbar_init(&S.empty[k], 1);
+    }
+    *S.gave_up = 0;
+    st_release(smem_addr(S.ready), 0);
+    st_release(smem_addr(S.primed), 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  const int part = (warp >> 1) * 32 + lane;  // of the threads of this strip
+  ws_clear(S.Ef, Mp, below, part, WS_THREADS / 2);
+  if (TWO) ws_clear(S.Eb, Mp, above, part, WS_THREADS / 2);
+  pdl_entry();
+  const size_t blk = (size_t)b * Mp * WS_STEP_BYTES, vec = (size_t)b * Mp * WS_VEC_BYTES;
+  const WsGlobal G{reinterpret_cast<const unsigned char*>(Fb) + blk, reinterpret_cast<const unsigned char*>(Bb) + blk,
+                   reinterpret_cast<const unsigned char*>(C) + vec,  reinterpret_cast<unsigned char*>(Y) + vec,
+                   reinterpret_cast<unsigned char*>(Z) + vec,        Mp / WS_U};
   if (b == 0)
-    for (int x = lane; x < 16 * nw; x += 32) S.cutG[x] = cutG[x];
-  ws_clear_edge(S, Mp);
+    for (int x = part; x < 16 * nw; x += WS_THREADS / 2) reinterpret_cast<float*>(S.cutG)[x] = cutG[x];
   // every strip's edge buffer holds its sentinels before any neighbour stores into it
-  cluster_sync();
-  unsigned phase_bits = 0;
-  // forward: strip b feeds b + 1 (lane 31) and is fed by b - 1; backward the other way round
-  const unsigned up = b < nb - 1 ? cluster_addr(S.edge, (unsigned)(b + 1)) : 0u;
-  const unsigned down = b > 0 ? cluster_addr(S.edge, (unsigned)(b - 1)) : 0u;
-  bool ok = ws_pass<true, KC>(L, S, b, Fb, C, Y, b > 0, up, err, limit, phase_bits);
-  // the backward pass reads, through the async proxy, the y this warp has just written
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-  // every strip has read its edge buffer to the end before it is cleared for the backward pass,
-  // and cleared before a neighbour stores into it again
-  cluster_sync();
-  ws_clear_edge(S, Mp);
-  cluster_sync();
-  if (ok) ws_pass<false, KC>(L, S, b, Bb, Y, Z, b < nb - 1, down, err, limit, phase_bits);
-  cluster_sync();
+  cluster_arrive();
+  cluster_wait();
+  bool ok = b < nst;
+  const WsSmem other = ws_carve<NS, TWO>(ws_raw, w ^ 1, Mp, nw);
+  if (compute) {
+    ok = ok && ws_pass<true, NS>(L, S, b, Mp, 0, err, limit, zero);
+  } else if (copier) {
+    ok = ok && ws_copies<true, NS>(S, G, above ? cluster_addr(other.Ef, (unsigned)(b + 1) >> 1) : 0u);
+  } else if (watcher) {
+    ok = ok && ws_watch<NS>(S, G.nch, 0, below, S.Ef, err, limit);
+  }
+  __syncwarp();
+  if (!TWO) {  // every strip has read its edge buffer to the end; cleared before a neighbour stores into it again
+    cluster_arrive();
+    cluster_wait();
+    ws_clear(S.Eb, Mp, above, part, WS_THREADS / 2);
+    cluster_arrive();
+    cluster_wait();
+  }
+  if (compute) {
+    if (ok) ws_pass<false, NS>(L, S, b, Mp, G.nch, err, limit, zero);
+  } else if (copier) {
+    if (ok) ws_copies<false, NS>(S, G, below ? cluster_addr(other.Eb, (unsigned)(b - 1) >> 1) : 0u);
+  } else if (watcher) {
+    if (ok) ws_watch<NS>(S, G.nch, G.nch, above, S.Eb, err, limit);
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
 }
 
 // ---------------------------------------------------------------- operand layout
@@ -640,32 +783,27 @@ __global__ void k_ws_finish_x(LevelDev L, const double* x, int do_update, int aw
 }
 
 constexpr size_t kWsSmemMax = 227 * 1024;
+constexpr int kWsPortable = 8, kWsCluster = 16;  // CTAs of a cluster: portable, and the most sm_103 allows
 
-}  // namespace
-
-bool ws_fits(int ni, int nj, int nw) {
-  return ws_strips(nj) <= 8 && ws_smem_bytes(ni, nj, nw, WS_K) <= kWsSmemMax;  // one portable cluster per sweep
+// The kernel's per-device attributes, set once on each device (idempotent if two host threads race
+// on the first launch).
+template <int NS, bool TWO>
+void ws_attributes() {
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || (done.load() & (1ull << dev))) return;
+  if (cudaFuncSetAttribute(k_sweep_ws<NS, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWsSmemMax) ==
+          cudaSuccess &&
+      cudaFuncSetAttribute(k_sweep_ws<NS, TWO>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+    done.fetch_or(1ull << dev);
 }
 
-
-namespace {
-template <int KC>
-cudaError_t ws_sweep_launch(const LevelDev& L, float4* zout, int* err, long long limit, cudaStream_t st) {
-  const int nb = ws_strips(L.nj);
-  const size_t sm = ws_smem_bytes(L.ni, L.nj, L.nw, KC);
-  // the shared-memory limit is a per-device attribute of each instance: set once on each device
-  // (idempotent if two host threads race on the first launch)
-  static std::atomic<unsigned long long> attr_done{0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !(attr_done.load() & (1ull << dev))) {
-    if (cudaFuncSetAttribute(k_sweep_ws<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWsSmemMax) ==
-        cudaSuccess)
-      attr_done.fetch_or(1ull << dev);
-  }
-  // The strips of one sweep wait on one another, so they are launched as one thread-block
-  // cluster (nb <= 8 CTAs): the hardware schedules a cluster's CTAs together, so every strip is
-  // resident whatever else runs beside it (concurrent cases of a batch included).
-  cudaLaunchAttribute at[2];
+// The strips of one sweep wait on one another, so they are launched as one thread-block cluster
+// (two strips per CTA): the hardware schedules a cluster's CTAs together, so every strip is
+// resident whatever else runs beside it (concurrent cases of a batch included).
+template <int NS, bool TWO>
+cudaLaunchConfig_t ws_config(const LevelDev& L, cudaLaunchAttribute* at, cudaStream_t st) {
+  const int nb = (ws_strips(L.nj) + 1) / 2;
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   at[1].id = cudaLaunchAttributeClusterDimension;
@@ -674,23 +812,65 @@ cudaError_t ws_sweep_launch(const LevelDev& L, float4* zout, int* err, long long
   at[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nb);
-  cfg.blockDim = dim3(32);
-  cfg.dynamicSmemBytes = sm;
+  cfg.blockDim = dim3(WS_THREADS);
+  cfg.dynamicSmemBytes = ws_cta_bytes<NS, TWO>(ws_steps(L.ni, L.nj), L.nw);
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k_sweep_ws<KC>, L, reinterpret_cast<const float4*>(L.wsF),
-                            reinterpret_cast<const float4*>(L.wsB), reinterpret_cast<const float4*>(L.wsC),
-                            reinterpret_cast<float4*>(L.wsY), static_cast<const float*>(L.wsCut), zout, err,
-                            limit);
+  return cfg;
 }
+
+template <int NS, bool TWO>
+cudaError_t ws_sweep_launch(const LevelDev& L, float4* zout, int* err, long long limit, cudaStream_t st) {
+  ws_attributes<NS, TWO>();
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t cfg = ws_config<NS, TWO>(L, at, st);
+  return cudaLaunchKernelEx(&cfg, k_sweep_ws<NS, TWO>, L, reinterpret_cast<const float4*>(L.wsF),
+                            reinterpret_cast<const float4*>(L.wsB), reinterpret_cast<const float4*>(L.wsC),
+                            reinterpret_cast<float4*>(L.wsY), static_cast<const float*>(L.wsCut), zout, err, limit, 0u);
+}
+
+template <int NS, bool TWO>
+bool ws_smem_fits(int ni, int nj, int nw) {
+  return ws_cta_bytes<NS, TWO>(ws_steps(ni, nj), nw) <= kWsSmemMax;
+}
+
 }  // namespace
 
+// One cluster per sweep: at most 16 CTAs of two strips, a ring and an edge buffer that fit in shared
+// memory, and (beyond the portable 8 CTAs) a device that can hold such a cluster.
+bool ws_fits(int ni, int nj, int nw) {
+  const int nb = (ws_strips(nj) + 1) / 2;
+  if (nb > kWsCluster || !ws_smem_fits<WS_SHALLOW, false>(ni, nj, nw)) return false;
+  if (nb <= kWsPortable) return true;
+  LevelDev L = {};
+  L.ni = ni;
+  L.nj = nj;
+  L.nw = nw;
+  ws_attributes<WS_SHALLOW, false>();
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t cfg = ws_config<WS_SHALLOW, false>(L, at, nullptr);
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k_sweep_ws<WS_SHALLOW, false>, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();  // not this call's error: the level takes another sweep
+  return e == cudaSuccess && n >= 1;
+}
+
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,
-                    long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, int chunk) {
+                    long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, bool deep) {
   (void)prog;  // the warp strips exchange their boundary rows in shared memory, not through progress words
   auto sweep = [&](float4* zout) {
-    return chunk == 8 ? ws_sweep_launch<8>(L, zout, err, limit, st) : ws_sweep_launch<WS_K>(L, zout, err, limit, st);
+    // An edge buffer per pass where two fit (1024x256 pair 171 us; with one, cleared between the
+    // passes, 177 us), a ring of five stages where it fits (three: 1-3 % slower).
+    const auto fits = [&](auto deep, auto two) {
+      return ws_smem_fits<decltype(deep)::value ? WS_STAGES : WS_SHALLOW, decltype(two)::value>(L.ni, L.nj, L.nw);
+    };
+    constexpr std::true_type yes{};
+    constexpr std::false_type no{};
+    if (deep && fits(yes, yes)) return ws_sweep_launch<WS_STAGES, true>(L, zout, err, limit, st);
+    if (deep && fits(yes, no)) return ws_sweep_launch<WS_STAGES, false>(L, zout, err, limit, st);
+    if (fits(no, yes)) return ws_sweep_launch<WS_SHALLOW, true>(L, zout, err, limit, st);
+    return ws_sweep_launch<WS_SHALLOW, false>(L, zout, err, limit, st);
   };
   const int g = (L.n + 127) / 128;
   float4* z0 = reinterpret_cast<float4*>(L.wsZ);

@@ -451,6 +451,12 @@ long long fasw_batch_launch_count(fasw_batch* batch);
  * FASW_ERR_OOM / FASW_ERR_CUDA on device failures. */
 int fasw_check_math(int n, const double* a, const double* b, double* out, int on_device);
 
+/* Verification hook for the FP64 helpers that keep off the FP64 pipe: for t < n, out[4t..4t+3] = (the
+ * library's 1/a[t], the division 1/a[t], a[t] rounded to FP32 by the library's bit-pattern conversion,
+ * its inverse conversion of (float)a[t]).  a: n doubles, out: 4n doubles, host pointers.  Synchronous.
+ * FASW_ERR_ARG for n < 0 or null pointers, FASW_ERR_OOM / FASW_ERR_CUDA on device failures. */
+int fasw_check_fp64(int n, const double* a, double* out);
+
 /* Coefficients of the stage loop of a scheme, Table "RK smoothers" (section 4.1): *nstages
  * (3 or 5) and alpha[k], beta[k] for k < *nstages (alpha, beta nullable, 5 doubles each).  The
  * W methods use the ARK coefficients of the same name; AW51/AW52 and ARK51/ARK52 take the

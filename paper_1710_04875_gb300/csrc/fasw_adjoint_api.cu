@@ -11,6 +11,17 @@
 
 using namespace fasw;
 
+namespace {
+// The adjoint differences residuals (coarse Jacobians, grid derivatives), which multiplies their
+// rounding by 1e6: its evaluations keep the one order of operations of mixed contexts.
+PhysParams adj_ph(const fasw_ctx* c) {
+  PhysParams p = c->ph;
+  p.fast = 0;
+  return p;
+}
+}  // namespace
+
+
 extern "C" {
 
 // ---- discrete adjoint (steady finest level, eddy viscosity frozen)
@@ -34,13 +45,13 @@ static int adj_ready(fasw_ctx* c) {
 // The finest level's Jacobian and, for the transposed FAS cycle, those of the coarse levels at
 // the restricted state.
 static int adj_assemble_all(fasw_ctx* c, double h_rel) {
-  int r = adj_assemble(c->adj, c->lev[c->L()], c->ph, h_rel, c->st, c->launches);
+  int r = adj_assemble(c->adj, c->lev[c->L()], adj_ph(c), h_rel, c->st, c->launches);
   if (r) return r;
   const int kind = c->adj.precond_kind;
   if ((kind == ADJ_FAS_CYCLE_T || kind == ADJ_FAS_VCYCLE_T) && c->L() > 0) {
     const int gamma = kind == ADJ_FAS_VCYCLE_T ? 1 : c->prm.gamma_cycle;
     if ((r = adj_mg_setup(c->adj, c->lev, gamma, c->prm.nu1, c->allocs, c->st))) return r;
-    if ((r = adj_mg_assemble(c->adj, c->lev, c->ph, c->prm.turb, h_rel, c->st, c->launches))) return r;
+    if ((r = adj_mg_assemble(c->adj, c->lev, adj_ph(c), c->prm.turb, h_rel, c->st, c->launches))) return r;
   }
   return FASW_OK;
 }
@@ -52,7 +63,7 @@ int fasw_force_coefficients(fasw_ctx* c, double* cl, double* cd) {
   if (!c || !cl || !cd) return FASW_ERR_ARG;
   int r = adj_ready(c);
   if (r) return r;
-  return adj_force_coefficients(c->adj, c->lev[c->L()], c->ph, c->st, cl, cd, c->launches);
+  return adj_force_coefficients(c->adj, c->lev[c->L()], adj_ph(c), c->st, cl, cd, c->launches);
 }
 
 int fasw_adjoint_jacobian(fasw_ctx* c, double h_rel) {
@@ -92,7 +103,7 @@ int fasw_adjoint_precond_apply(fasw_ctx* c, double cfl, int steps, const double*
   const size_t m = 4 * (size_t)c->adj.n;
   if ((e = copy_in(c, c->d_tmp, r, m, on_device))) return e;
   err_clear(c);
-  adj_build_precond(c->adj, c->lev[c->L()], c->ph, c->sc, cfl, c->st, c->launches);
+  adj_build_precond(c->adj, c->lev[c->L()], adj_ph(c), c->sc, cfl, c->st, c->launches);
   adj_steps_apply(c->adj, steps, c->d_tmp, c->d_tmp2, c->st);
   c->launches += 2;
   if ((e = adj_err_check(c))) return e;
@@ -114,8 +125,8 @@ int fasw_tangent_residual(fasw_ctx* c, const double* v, double* dF, double* F, i
   LevelDev& L = c->lev[c->L()];
   const size_t m = 4 * (size_t)L.n;
   if ((r = copy_in(c, c->d_tmp, v, m, on_device))) return r;
-  launch_bc_aux(L, c->ph, 1.0, 0, c->st);
-  launch_tangent(L, c->adj.tan, c->ph, c->d_tmp, nullptr, 0, -1, 0.0, c->adj.Fp, nullptr, F ? c->adj.Fm : nullptr,
+  launch_bc_aux(L, adj_ph(c), 1.0, 0, c->st);
+  launch_tangent(L, c->adj.tan, adj_ph(c), c->d_tmp, nullptr, 0, -1, 0.0, c->adj.Fp, nullptr, F ? c->adj.Fm : nullptr,
                  nullptr, nullptr, c->st);
   c->launches += 6;
   if ((r = copy_out(c, dF, c->adj.Fp, m, on_device))) return r;
@@ -144,9 +155,9 @@ int fasw_adjoint_cycle_apply(fasw_ctx* c, double cfl, int kind, int transpose, c
   int e = copy_in(c, c->d_tmp, r, m, on_device);
   if (e) return e;
   err_clear(c);
-  adj_build_precond(c->adj, c->lev[c->L()], c->ph, c->sc, cfl, c->st, c->launches);
+  adj_build_precond(c->adj, c->lev[c->L()], adj_ph(c), c->sc, cfl, c->st, c->launches);
   if (kind == 2) {
-    adj_mg_build_precond(c->adj, c->lev, c->ph, c->sc, cfl, c->st, c->launches);
+    adj_mg_build_precond(c->adj, c->lev, adj_ph(c), c->sc, cfl, c->st, c->launches);
     adj_mg_apply(c->adj, transpose, c->d_tmp, c->d_tmp2, c->st);
   } else {
     adj_smoother_apply(c->adj, c->adj.smooth_steps, transpose, c->d_tmp, c->d_tmp2, c->st);
@@ -170,7 +181,7 @@ int fasw_adjoint_solve(fasw_ctx* c, int which, const double* g, double* lam, dou
   }
   const double pcfl = cfl > 0.0 ? cfl : c->prm.cfl;
   err_clear(c);
-  const int code = adj_solve(c->adj, c->lev, c->ph, c->sc, pcfl, rhs, c->d_tmp2, tol, max_iters, restart,
+  const int code = adj_solve(c->adj, c->lev, adj_ph(c), c->sc, pcfl, rhs, c->d_tmp2, tol, max_iters, restart,
                              c->allocs, c->st, iters, rel_res, c->launches);
   if (code != FASW_OK && code != FASW_ERR_NOT_CONVERGED) return code;
   int r = adj_err_check(c);
@@ -201,11 +212,11 @@ int shape_term(fasw_ctx* c, int which, const double* d_lam, const double* vk, do
   for (int sgn = 0; sgn < 2; ++sgn) {
     adj_lincomb((int)nv, c->d_y0, sgn == 0 ? h_x : -h_x, vk, ytmp, c->st);
     launch_metrics_fine(F, c->d_x0, ytmp, c->st, rotate, phi, phidot, xc, yc);
-    launch_bc_aux(F, c->ph, 1.0, 0, c->st);
+    launch_bc_aux(F, adj_ph(c), 1.0, 0, c->st);
     a.F = sgn == 0 ? c->adj.Fp : c->adj.Fm;
-    launch_residual(F, c->ph, a, c->st);
+    launch_residual(F, adj_ph(c), a, c->st);
     c->launches += 4;
-    int r = adj_force_coefficients(c->adj, F, c->ph, c->st, &cl[sgn], &cd[sgn], c->launches);
+    int r = adj_force_coefficients(c->adj, F, adj_ph(c), c->st, &cl[sgn], &cd[sgn], c->launches);
     if (r) return r;
   }
   adj_lincomb((int)m, c->adj.Fp, -1.0, c->adj.Fm, c->d_tmp2, c->st);  // F+ - F-
@@ -234,7 +245,7 @@ int fasw_adjoint_shape_gradient(fasw_ctx* c, int which, const double* lam, int n
     grad[k] = (dJ - dot) / (2.0 * h_x);
   }
   launch_metrics_fine(F, c->d_x0, c->d_y0, c->st);
-  launch_bc_aux(F, c->ph, 1.0, 0, c->st);
+  launch_bc_aux(F, adj_ph(c), 1.0, 0, c->st);
   c->launches += 2;
   return sync(c);
 }
@@ -307,7 +318,7 @@ void unsteady_reset(fasw_ctx* c, const double* u0) {
   cudaMemsetAsync(F.src, 0, 4 * (size_t)F.n * sizeof(double), c->st);
   if (u0) {
     launch_pack(F, u0, 1, nullptr, c->st);
-    launch_bc(F, c->ph, c->st);
+    launch_bc(F, adj_ph(c), c->st);
   }
   c->launches += nl + (u0 ? 2 : 0);
   c->steps_done = 0;
@@ -378,7 +389,7 @@ int fasw_unsteady_adjoint(fasw_ctx* c, double amp, double omega, double xc, doub
         else if (r) return fail(r);
         if (n > reached) {  // the first sweep: the objective
           double cl = 0.0, cd = 0.0;
-          if ((r = adj_force_coefficients(c->adj, F, c->ph, c->st, &cl, &cd, c->launches))) return fail(r);
+          if ((r = adj_force_coefficients(c->adj, F, adj_ph(c), c->st, &cl, &cd, c->launches))) return fail(r);
           J += w * (which == 0 ? cl : cd);
           reached = n;
         }
@@ -408,7 +419,7 @@ int fasw_unsteady_adjoint(fasw_ctx* c, double amp, double omega, double xc, doub
         cudaMemcpyAsync(c->d_unm1, s + m, m * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
         c->steps_done = act.arg;
       }
-      launch_bc(F, c->ph, c->st);
+      launch_bc(F, adj_ph(c), c->st);
       c->launches += 2;
       pos = act.arg;
     } else {  // CK_CONSUME: adjoint step of level n = pos
@@ -425,8 +436,8 @@ int fasw_unsteady_adjoint(fasw_ctx* c, double amp, double omega, double xc, doub
       }
       cudaMemsetAsync(F.src, 0, m * sizeof(double), c->st);
       if (c->prm.turb && !c->mut_frozen) {  // eddy viscosity frozen at its value for u^n
-        launch_bc_aux(F, c->ph, 1.0, 0, c->st);
-        launch_bl(F, c->ph, c->st);
+        launch_bc_aux(F, adj_ph(c), 1.0, 0, c->st);
+        launch_bl(F, adj_ph(c), c->st);
         c->launches += 2;
       }
       if ((r = adj_assemble_all(c, h_rel))) return fail(r);
@@ -438,7 +449,7 @@ int fasw_unsteady_adjoint(fasw_ctx* c, double amp, double omega, double xc, doub
       int it = 0;
       double rr = 0.0;
       err_clear(c);
-      r = adj_solve(c->adj, c->lev, c->ph, c->sc, pcfl, rhs, lamn, tol, max_iters, restart, c->allocs, c->st, &it, &rr,
+      r = adj_solve(c->adj, c->lev, adj_ph(c), c->sc, pcfl, rhs, lamn, tol, max_iters, restart, c->allocs, c->st, &it, &rr,
                     c->launches);
       if (r == FASW_ERR_NOT_CONVERGED) soft = true;
       else if (r) return fail(r);
@@ -514,17 +525,17 @@ int fasw_adjoint_vertex_gradient(fasw_ctx* c, int which, const double* lam, doub
       for (int sgn = 0; sgn < 2; ++sgn) {
         adj_vertex_perturb(A, k, dir, sgn == 0 ? h_x : -h_x, c->d_x0, c->d_y0, xo, yo, c->st);
         launch_metrics_fine(Fz, xo, yo, c->st);
-        launch_bc_aux(Fz, c->ph, 1.0, 0, c->st);
+        launch_bc_aux(Fz, adj_ph(c), 1.0, 0, c->st);
         a.F = sgn == 0 ? A.Fp : A.Fm;
-        launch_residual(Fz, c->ph, a, c->st);
-        launch_wall_force(Fz, c->ph, A.fw + 2 * sgn * A.ni, A.fw + (2 * sgn + 1) * A.ni, c->st);
+        launch_residual(Fz, adj_ph(c), a, c->st);
+        launch_wall_force(Fz, adj_ph(c), A.fw + 2 * sgn * A.ni, A.fw + (2 * sgn + 1) * A.ni, c->st);
         c->launches += 5;
       }
       adj_vertex_accumulate(A, k, which, sa, ca, c->d_tmp, A.Fp, A.Fm, A.fw, h_x, g + dir * nv, c->st);
       ++c->launches;
     }
   launch_metrics_fine(F, c->d_x0, c->d_y0, c->st);
-  launch_bc_aux(F, c->ph, 1.0, 0, c->st);
+  launch_bc_aux(F, adj_ph(c), 1.0, 0, c->st);
   c->launches += 2;
   if ((r = copy_out(c, gx, g, nv, on_device)) || (r = copy_out(c, gy, g + nv, nv, on_device))) return r;
   return sync(c);

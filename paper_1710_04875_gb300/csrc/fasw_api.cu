@@ -156,6 +156,9 @@ int alloc_level(fasw_ctx* c, LevelDev& L) {
   A(L.sxi, 2 * nfx);
   A(L.seta, 2 * nfe);
   A(L.vol, n);
+  A(L.rvol, n);
+  A(L.clen, 2 * n);
+  A(L.rvf, nfe);
   A(L.mut, n);
   A(L.wdist, n);
   A(L.omega, n);
@@ -304,7 +307,7 @@ void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm) {
   ResArgs a{};
   a.mode = RES_FASRES;
   { Prof p(c, FASW_K_RESIDUAL); launch_residual(F, c->ph, a, c->st); }
-  { Prof p(c, FASW_K_RESTRICT); launch_restrict(F, C, c->prm.turb, c->st); }
+  { Prof p(c, FASW_K_RESTRICT); launch_restrict(F, C, c->prm.turb, c->ph.fast, c->st); }
   c->launches += 2;
   bc_aux(c, l - 1, cfl, 0);
   ResArgs b{};
@@ -448,6 +451,7 @@ int fasw_create(int ni, int nj, int n_wake, const double* x, const double* y, in
   c->ph.sensor = p->sensor;
   c->ph.flux = p->flux;
   c->ph.d_cut = p->d_cut;
+  c->ph.fast = !c->mixed;
   free_stream(p->mach, p->alpha_deg, c->ph.uinf);
   set_free_stream_prims(c->ph);
   const Coef& cf = kCoef[p->scheme % 4];
@@ -884,6 +888,22 @@ int fasw_check_math(int n, const double* a, const double* b, double* out, int on
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpy(out, d + 2 * m, 4 * m * sizeof(double), cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? FASW_OK : cuda_fail(e);
+}
+
+int fasw_check_fp64(int n, const double* a, double* out) {
+  if (n < 0 || (n > 0 && (!a || !out))) return FASW_ERR_ARG;
+  if (n == 0) return FASW_OK;
+  const size_t m = (size_t)n;
+  double* d = nullptr;
+  if (cudaMalloc(&d, 5 * m * sizeof(double)) != cudaSuccess) return FASW_ERR_OOM;
+  cudaError_t e = cudaMemcpy(d, a, m * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    launch_check_fp64(n, d, d + m, 0);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(out, d + m, 4 * m * sizeof(double), cudaMemcpyDeviceToHost);
   cudaFree(d);
   return e == cudaSuccess ? FASW_OK : cuda_fail(e);
 }

@@ -1,0 +1,67 @@
+// FP64 operations that keep off the FP64 pipe.  On this part a scheduler's FP64 pipe takes one warp
+// instruction per 64 clocks, whatever the number of active lanes, and the kernels around the sweeps
+// are bound by it (ncu: FP64 pipe active 70-85 % of the active cycles in every one of them).
+// Conversions between FP32 and FP64 and comparisons of FP64 values count as such instructions; the
+// integer pipe takes one per two clocks.  So exact conversions are done on the bit patterns, and a
+// reciprocal is four FP64 instructions instead of the nine of an IEEE division.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace fasw {
+
+// (double)x, exactly.  Subnormals, infinities and NaNs take the conversion instruction.
+__device__ __forceinline__ double f2d(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;
+  const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// (float)x, rounded to nearest even.  Results that are not normal numbers (zero, subnormal, values
+// that round past the largest float, infinities, NaNs) take the conversion instruction.
+__device__ __forceinline__ float d2f(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), m = hi & 0x7fffffffu;
+  if (m - 0x38100000u >= 0x0fd00000u) return (float)x;
+  unsigned f = ((m - 0x38000000u) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  f += rest > 0x10000000u || (rest == 0x10000000u && (f & 1u)) ? 1u : 0u;  // a carry moves into the exponent
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// 1/x for normal x whose reciprocal is normal: two Newton steps y <- y (2 - x y) from the hardware's
+// approximation (relative error below 2^-18), which leave an error of about one unit in the last
+// place.  Zero, subnormals, infinities and NaNs give a NaN.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
+
+// x in the precision of T
+template <typename T>
+__device__ __forceinline__ T from64(double x);
+template <>
+__device__ __forceinline__ double from64<double>(double x) {
+  return x;
+}
+template <>
+__device__ __forceinline__ float from64<float>(double x) {
+  return d2f(x);
+}
+__device__ __forceinline__ double to64(double x) { return x; }
+__device__ __forceinline__ double to64(float x) { return f2d(x); }
+
+// The larger of two non-negative values, the smaller of x and a positive c: on the bit patterns, whose
+// order as signed integers is that of the values.
+__device__ __forceinline__ double max_nn(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
+__device__ __forceinline__ double min_pos(double x, double c) {
+  return __double_as_longlong(x) < __double_as_longlong(c) ? x : c;
+}
+// max(x, 0)
+__device__ __forceinline__ double relu64(double x) { return __double2hiint(x) < 0 ? 0.0 : x; }
+__device__ __forceinline__ bool is_zero(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) == 0; }
+
+}  // namespace fasw

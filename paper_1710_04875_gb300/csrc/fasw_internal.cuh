@@ -68,6 +68,9 @@ struct LevelDev {
   double* sxi;  // 2*nfx  i-face area vectors (x plane, y plane), index j*(ni+1)+i
   double* seta; // 2*nfe  j-face area vectors, index j*ni+i
   double* vol;  // n
+  double* rvol; // n    1 / vol
+  double* clen; // 2*n  lengths of the cell's mean i- and j-face area vectors (xi plane, eta plane)
+  double* rvf;  // nfe  1 / mean volume of the two cells at a j-face
   double* mut;  // n    eddy viscosity
   double* wdist;// n    distance to the wall-face midpoint of the column (finest level)
   double* omega;// n    vorticity magnitude scratch (finest level)
@@ -115,6 +118,10 @@ struct PhysParams {
   int moving;  // grid in rigid motion: moving-wall ghosts
   int flux;    // residual face flux: 0 = JST, 1 = first-order flux-vector splitting
   double d_cut;  // eigenvalue cutoff of the flux-vector splitting (also the preconditioner's)
+  // FP64 contexts: regrouped sums and Newton reciprocals, which move a result by its last bits.  In
+  // mixed precision those bits decide the FP32 roundings of the sweeps that follow, so that states move
+  // by up to 1e-8 (the size of the FP32 error itself); mixed contexts keep one order of operations.
+  int fast;
 };
 
 // Primitive variables of the free stream for the far-field boundary, formed once on the host.
@@ -166,6 +173,8 @@ void launch_norm_final(const LevelDev& L, int nparts, int ncomp_cells, double* o
 void launch_bl(const LevelDev& L, const PhysParams& ph, cudaStream_t st);
 // the auxiliaries' FP64 powers beside pow()/cbrt(), n values (device pointers)
 void launch_check_math(int n, const double* a, const double* b, double* out, cudaStream_t st);
+// rcp64 and the exact conversions beside the instructions they stand for
+void launch_check_fp64(int n, const double* a, double* out, cudaStream_t st);
 // per-wall-face force on the body from the j = 0 face fluxes (ghosts and auxiliaries current)
 void launch_wall_force(const LevelDev& L, const PhysParams& ph, double* fx, double* fy, cudaStream_t st);
 
@@ -178,7 +187,8 @@ void launch_sgs(const LevelDev& L, const SchemeParams& sc, int mixed, int do_upd
 
 // ---- launchers (kernels_transfer.cu)
 void launch_copy_u0(const LevelDev& L, cudaStream_t st);
-void launch_restrict(const LevelDev& F, const LevelDev& C, int restrict_mut, cudaStream_t st);
+// fast: PhysParams::fast
+void launch_restrict(const LevelDev& F, const LevelDev& C, int restrict_mut, int fast, cudaStream_t st);
 void launch_prolong(const LevelDev& F, const LevelDev& C, cudaStream_t st);
 cudaError_t launch_pack(const LevelDev& L, const double* interior_in, int to_ghosted, double* out, cudaStream_t st);
 

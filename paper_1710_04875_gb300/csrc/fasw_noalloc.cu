@@ -45,10 +45,13 @@ size_t carve(LevelDev& L, double* base) {
   take(L.sxi, 2 * (size_t)L.nfx);
   take(L.seta, 2 * (size_t)L.nfe);
   take(L.vol, (size_t)L.n);
+  take(L.rvol, (size_t)L.n);
+  take(L.clen, 2 * (size_t)L.n);
+  take(L.rvf, (size_t)L.nfe);
   take(L.wdist, (size_t)L.n);
   take(L.mut, (size_t)L.n);
   take(L.s, 4 * (size_t)L.n);
-  take(L.src, 4 * (size_t)L.n);
+  L.src = L.s;  // both zero, and only read
   take(L.norm_part, (size_t)residual_blocks(L));
   take(L.vfx, (size_t)L.nfx);
   take(L.vfe, (size_t)L.nfe);
@@ -116,6 +119,7 @@ extern "C" int fasw_residual_noalloc(int ni, int nj, int n_wake, const double* x
   ph.sensor = p->sensor;
   ph.flux = p->flux == 1 ? 1 : 0;
   ph.d_cut = p->d_cut;
+  ph.fast = p->precision != FASW_MIXED;
   {
     const double al = p->alpha_deg * M_PI / 180.0;
     const double pinf = 1.0 / (GAM * p->mach * p->mach);
@@ -128,10 +132,9 @@ extern "C" int fasw_residual_noalloc(int ni, int nj, int n_wake, const double* x
   set_free_stream_prims(ph);
 
   // The scratch keeps the previous call's contents: clear what the residual reads as zero
-  // (eddy viscosity, forcing, dual-time source) before use.
+  // (eddy viscosity; forcing and dual-time source, one array) before use.
   if (cudaMemsetAsync(L.mut, 0, (size_t)L.n * sizeof(double), st) != cudaSuccess ||
-      cudaMemsetAsync(L.s, 0, 4 * (size_t)L.n * sizeof(double), st) != cudaSuccess ||
-      cudaMemsetAsync(L.src, 0, 4 * (size_t)L.n * sizeof(double), st) != cudaSuccess)
+      cudaMemsetAsync(L.s, 0, 4 * (size_t)L.n * sizeof(double), st) != cudaSuccess)
     return FASW_ERR_CUDA;
   ResArgs a;
   std::memset(&a, 0, sizeof(a));

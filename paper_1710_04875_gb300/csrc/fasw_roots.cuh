@@ -1,6 +1,7 @@
 // FP64 powers of the per-cell auxiliaries by Newton's method from FP32 estimates (shared by the
 // residual kernels and their forward-mode linearization).
 #pragma once
+#include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 
 namespace fasw {
@@ -12,8 +13,8 @@ namespace fasw {
 // 1.4, 8.9e-17 below 7/5, and differs from it by |ln rho| 8.9e-17 relative).
 static_assert(GAM == 1.4, "rho^-gamma is formed as the root of rho^7 z^5 = 1");
 __device__ __forceinline__ double pow_neg_gamma(double rho) {
-  const float rf = (float)rho;
-  double z = (double)exp2f(-1.4f * __log2f(rf));
+  const float rf = d2f(rho);
+  double z = f2d(exp2f(-1.4f * __log2f(rf)));
   const double r2 = rho * rho, r7 = (r2 * r2) * (r2 * rho);
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
@@ -28,10 +29,10 @@ __device__ __forceinline__ double pow_neg_gamma(double rho) {
 // from the FP32 cube root with the derivative's reciprocal 1/(3 den c^2) taken in FP32 (the
 // error contracts by ~1e-7 per step: two steps reach FP64 rounding).  No FP64 division.
 __device__ __forceinline__ double cbrt_ratio(double num, double den) {
-  const float nf = (float)num, df = (float)den;
+  const float nf = d2f(num), df = d2f(den);
   const float c0 = cbrtf(nf / df);
-  const double d = (double)(1.0f / (3.0f * df * c0 * c0));
-  double c = (double)c0;
+  const double d = f2d(1.0f / (3.0f * df * c0 * c0));
+  double c = f2d(c0);
 #pragma unroll
   for (int it = 0; it < 2; ++it) c = fma(-fma(den, (c * c) * c, -num), d, c);
   return c;

@@ -1085,7 +1085,7 @@ int adj_mg_assemble(AdjointDev& A, const std::vector<LevelDev>& lev, const PhysP
   if (!A.mg) return FASW_ERR_ARG;
   const int L = A.mg->L;
   for (int l = L; l >= 1; --l) {
-    launch_restrict(lev[l], lev[l - 1], turb, st);
+    launch_restrict(lev[l], lev[l - 1], turb, ph.fast, st);
     ++launches;
   }
   for (int l = L - 1; l >= 0; --l) {

@@ -188,8 +188,8 @@ __global__ void k_bc(LevelDev L, PhysParams ph) {
   store4(L, gidx(L, gi, gj), g);
 }
 
-// FP64 on this part issues one warp instruction per ~64 clocks per scheduler, and the library
-// pow() costs about 3.3 us of dependent chain per call (cbrt 0.54 us, a division 0.29 us, an
+// FP64 on this part issues one warp instruction per 64 clocks per scheduler (fasw_fp64.cuh), and the
+// library pow() costs about 3.3 us of dependent chain per call (cbrt 0.54 us, a division 0.29 us, an
 // FMA 32 ns): the per-cell auxiliaries are bound by that chain, not by memory.  The two powers
 // they need are computed as roots of polynomial equations by Newton's method in FP64 from an
 // FP32 estimate; both are checked against pow() and cbrt() by fasw_check_math.
@@ -198,7 +198,7 @@ __global__ void k_bc(LevelDev L, PhysParams ph) {
 // sensor quantity of one (ghosted) cell.
 __device__ __forceinline__ void cell_thermo(const LevelDev& L, const PhysParams& ph, int g, const double w[4],
                                             double& rr, double& u, double& v, double& p) {
-  rr = 1.0 / w[0];
+  rr = ph.fast ? rcp64(w[0]) : 1.0 / w[0];
   u = w[1] * rr;
   v = w[2] * rr;
   p = (GAM - 1.0) * (w[3] - 0.5 * (w[1] * u + w[2] * v));
@@ -242,16 +242,21 @@ __global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, 
   const double sy = 0.5 * (L.sxi[L.nfx + fw] + L.sxi[L.nfx + fw + 1]);
   const double ex = 0.5 * (L.seta[fs] + L.seta[fs + ni]);
   const double ey = 0.5 * (L.seta[L.nfe + fs] + L.seta[L.nfe + fs + ni]);
-  const double vx = 0.5 * (L.vfx[fw] + L.vfx[fw + 1]);
-  const double ve = 0.5 * (L.vfe[fs] + L.vfe[fs + ni]);
-  const double rxi = fabs(u * sx + v * sy - vx) + a * sqrt(sx * sx + sy * sy);
-  const double reta = fabs(u * ex + v * ey - ve) + a * sqrt(ex * ex + ey * ey);
+  double qx = u * sx + v * sy, qe = u * ex + v * ey;
+  if (ph.moving) {
+    qx -= 0.5 * (L.vfx[fw] + L.vfx[fw + 1]);
+    qe -= 0.5 * (L.vfe[fs] + L.vfe[fs + ni]);
+  }
+  const double rxi = fabs(qx) + a * L.clen[c], reta = fabs(qe) + a * L.clen[L.n + c];
   // Martinelli scaling: with cr = (r_eta/r_xi)^(1/3), r_xi (r_eta/r_xi)^(2/3) = r_xi cr^2 and
   // r_eta (r_xi/r_eta)^(2/3) = r_xi cr (one cube root, no division).
   const double cr = cbrt_ratio(reta, rxi);
   L.rt[c] = rxi + rxi * (cr * cr);
   L.rt[L.n + c] = reta + rxi * cr;
-  if (want_dts) L.dts[c] = cfl * L.vol[c] / (rxi + reta);
+  if (want_dts) {
+    const double cv = cfl * L.vol[c], r = rxi + reta;
+    L.dts[c] = ph.fast ? cv * rcp64(r) : cv / r;
+  }
 }
 
 // Martinelli radius of a possibly-ghost cell: ghosts take the adjacent interior cell's value,
@@ -267,8 +272,10 @@ __device__ __forceinline__ double rt_cell(const LevelDev& L, int i, int j, int d
   return L.rt[dir * L.n + j * L.ni + i];
 }
 
+template <bool FAST>
 __device__ __forceinline__ double sensor_val(double qm, double q0, double qp) {
-  return fabs(qp - 2.0 * q0 + qm) / (qp + 2.0 * q0 + qm + 0.001);
+  const double d = fabs(qp - 2.0 * q0 + qm), s = qp + 2.0 * q0 + qm + 0.001;
+  return FAST ? d * rcp64(s) : d / s;
 }
 
 // JST flux through a face with area vector (sx, sy) from L to R; stencil LL, L, R, RR
@@ -330,78 +337,97 @@ __device__ void fvs_face(const LevelDev& L, int gL, int gR, double sx, double sy
   }
 }
 
-__device__ void jst_face(const LevelDev& L, int gLL, int gL, int gR, int gRR, double sx, double sy, double vf,
-                         double rtL, double rtR, double s_coarse, double hc[4], double hd[4]) {
+// The factor 1/2 of the averages goes on the face vector, and on a fixed grid (moving 0) the terms in vf
+// are left out: both leave every bit as it is.  FAST (PhysParams::fast) takes the grid's flux off the
+// normal velocities once, sums the two cells' terms in chains, and forms the fourth differences as
+// (eps2 + 3 eps4) dw - eps4 (w_RR - w_LL): about 65 FP64 instructions a face against 80, and 105 before
+// either and with a sensor formed by each face that reads it; residual of the 1024x256 level 230 -> 160 us
+// in FP64, of the 64x16 level 10.6 -> 9.1.  s: the larger of the two cells' sensors (finest level).
+template <bool FAST>
+__device__ __forceinline__ void jst_face(const LevelDev& L, int gLL, int gL, int gR, int gRR, double sx, double sy,
+                                         double vf, int moving, double rtL, double rtR, double s, double s_coarse,
+                                         double hc[4], double hd[4]) {
   double uL[4], uR[4];
   load4(L, gL, uL);
   load4(L, gR, uR);
   const double pL = L.p[gL], pR = L.p[gR];
+  const double wL3 = uL[3] + pL, wR3 = uR[3] + pR;  // w = (rho, rho u, rho v, rho H)
   {
-    const double qnL = (uL[1] * sx + uL[2] * sy) * L.rinv[gL];
-    const double qnR = (uR[1] * sx + uR[2] * sy) * L.rinv[gR];
-    hc[0] = 0.5 * ((uL[0] * qnL - uL[0] * vf) + (uR[0] * qnR - uR[0] * vf));
-    hc[1] = 0.5 * (((uL[1] * qnL + pL * sx) - uL[1] * vf) + ((uR[1] * qnR + pR * sx) - uR[1] * vf));
-    hc[2] = 0.5 * (((uL[2] * qnL + pL * sy) - uL[2] * vf) + ((uR[2] * qnR + pR * sy) - uR[2] * vf));
-    hc[3] = 0.5 * (((uL[3] + pL) * qnL - uL[3] * vf) + ((uR[3] + pR) * qnR - uR[3] * vf));
+    const double hx = 0.5 * sx, hy = 0.5 * sy, hf = 0.5 * vf;
+    const double qL = (uL[1] * hx + uL[2] * hy) * L.rinv[gL];
+    const double qR = (uR[1] * hx + uR[2] * hy) * L.rinv[gR];
+    if (FAST) {
+      const double aL = moving ? qL - hf : qL, aR = moving ? qR - hf : qR, ps = pL + pR;
+      hc[0] = uL[0] * aL + uR[0] * aR;
+      hc[1] = uL[1] * aL + (uR[1] * aR + ps * hx);
+      hc[2] = uL[2] * aL + (uR[2] * aR + ps * hy);
+      hc[3] = uL[3] * aL + (uR[3] * aR + (pL * qL + pR * qR));
+    } else if (moving) {
+      const double qnL = (uL[1] * sx + uL[2] * sy) * L.rinv[gL];
+      const double qnR = (uR[1] * sx + uR[2] * sy) * L.rinv[gR];
+      hc[0] = 0.5 * ((uL[0] * qnL - uL[0] * vf) + (uR[0] * qnR - uR[0] * vf));
+      hc[1] = 0.5 * (((uL[1] * qnL + pL * sx) - uL[1] * vf) + ((uR[1] * qnR + pR * sx) - uR[1] * vf));
+      hc[2] = 0.5 * (((uL[2] * qnL + pL * sy) - uL[2] * vf) + ((uR[2] * qnR + pR * sy) - uR[2] * vf));
+      hc[3] = 0.5 * (((uL[3] + pL) * qnL - uL[3] * vf) + ((uR[3] + pR) * qnR - uR[3] * vf));
+    } else {
+      hc[0] = __dadd_rn(__dmul_rn(uL[0], qL), __dmul_rn(uR[0], qR));
+      hc[1] = __dadd_rn(uL[1] * qL + pL * hx, uR[1] * qR + pR * hx);
+      hc[2] = __dadd_rn(uL[2] * qL + pL * hy, uR[2] * qR + pR * hy);
+      hc[3] = __dadd_rn(__dmul_rn(wL3, qL), __dmul_rn(wR3, qR));
+    }
   }
-  const double r = fmax(rtL, rtR);
-  double eps2, eps4;
+  const double r = max_nn(rtL, rtR);
+  uL[3] = wL3;
+  uR[3] = wR3;
+  double e2 = s_coarse * r, e4 = 0.0;
   if (L.finest) {
-    const double qLL = L.q[gLL], qL = L.q[gL], qR = L.q[gR], qRR = L.q[gRR];
-    const double sL = sensor_val(qLL, qL, qR), sR = sensor_val(qL, qR, qRR);
-    const double s = fmin(0.25, fmax(sL, sR));
-    eps2 = s * r;
-    eps4 = fmax(0.0, r / 32.0 - 2.0 * eps2);
-  } else {
-    eps2 = s_coarse * r;
-    eps4 = 0.0;
+    e2 = min_pos(s, 0.25) * r;
+    e4 = relu64(fma(-2.0, e2, r * (1.0 / 32.0)));
   }
-  double uLL[4], uRR[4];
-  if (eps4 != 0.0) {
+  if (!is_zero(e4)) {
+    double uLL[4], uRR[4];
     load4(L, gLL, uLL);
     load4(L, gRR, uRR);
-  }
+    uLL[3] += L.p[gLL];
+    uRR[3] += L.p[gRR];
+    const double e = fma(3.0, e4, e2);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const double wL = k == 3 ? uL[3] + pL : uL[k];
-    const double wR = k == 3 ? uR[3] + pR : uR[k];
-    const double dw0 = wR - wL;
-    double d = eps2 * dw0;
-    if (eps4 != 0.0) {
-      const double wLL = k == 3 ? uLL[3] + L.p[gLL] : uLL[k];
-      const double wRR = k == 3 ? uRR[3] + L.p[gRR] : uRR[k];
-      const double dwm = wL - wLL, dwp = wRR - wR;
-      d -= eps4 * ((dwp + dwm) - 2.0 * dw0);
+    for (int k = 0; k < 4; ++k) {
+      const double dw0 = uR[k] - uL[k];
+      if (FAST) {
+        hd[k] = e * dw0 - e4 * (uRR[k] - uLL[k]);
+      } else {
+        const double dwm = uL[k] - uLL[k], dwp = uRR[k] - uR[k];
+        hd[k] = fma(-e4, fma(-2.0, dw0, dwp + dwm), __dmul_rn(e2, dw0));
+      }
     }
-    hd[k] = d;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) hd[k] = e2 * (uR[k] - uL[k]);
   }
 }
 
+// Sensor of the cell at ghosted index g along stride d (1: along i, the pitch: along j).
+template <bool FAST>
+__device__ __forceinline__ double cell_sensor(const LevelDev& L, int g, int d) {
+  return sensor_val<FAST>(L.q[g - d], L.q[g], L.q[g + d]);
+}
+
 // Thin-layer viscous flux through j-face (i, j): gradients = jump across the face times S over
-// the mean volume of the two cells (ghost volumes: interior neighbour; across the cut: mirror).
-__device__ void visc_face(const LevelDev& L, const PhysParams& ph, int i, int j, double sx, double sy, double hv[4]) {
+// the mean volume of the two cells.  FAST: with gradients (du, dv) S / Omega_f the stress on the face
+// is mu_eff / Omega_f times (du (4/3 Sx^2 + Sy^2) + dv Sx Sy / 3, dv (4/3 Sy^2 + Sx^2) + du Sx Sy / 3).
+template <bool FAST>
+__device__ __forceinline__ void visc_face(const LevelDev& L, const PhysParams& ph, int i, int j, double sx, double sy,
+                                          double hv[4]) {
   const int ni = L.ni, nj = L.nj;
-  double volL, volR, mutf;
-  if (j == 0) {
-    volR = L.vol[i];
-    if (on_cut(L, i)) {
-      const int m = ni - 1 - i;
-      volL = L.vol[m];
-      mutf = 0.5 * (L.mut[i] + L.mut[m]);
-    } else {
-      volL = volR;
-      mutf = 0.0;
-    }
-  } else if (j == nj) {
-    volL = L.vol[(nj - 1) * ni + i];
-    volR = volL;
+  double mutf;
+  if (j == 0)
+    mutf = on_cut(L, i) ? 0.5 * (L.mut[i] + L.mut[ni - 1 - i]) : 0.0;
+  else if (j == nj)
     mutf = L.mut[(nj - 1) * ni + i];
-  } else {
-    volL = L.vol[(j - 1) * ni + i];
-    volR = L.vol[j * ni + i];
+  else
     mutf = 0.5 * (L.mut[(j - 1) * ni + i] + L.mut[j * ni + i]);
-  }
-  const double rvf = 2.0 / (volL + volR);  // 1 / mean volume
+  const double rvf = L.rvf[j * ni + i];
   double wL[4], wR[4];
   const int gL = gidx(L, i, j - 1), gR = gidx(L, i, j);
   load4(L, gL, wL);
@@ -409,10 +435,21 @@ __device__ void visc_face(const LevelDev& L, const PhysParams& ph, int i, int j,
   const double rL = L.rinv[gL], rR = L.rinv[gR];
   const double uL = wL[1] * rL, vL = wL[2] * rL, uR = wR[1] * rR, vR = wR[2] * rR;
   constexpr double cp = GAM / (GAM - 1.0);
-  const double hL = cp * L.p[gL] * rL, hR = cp * L.p[gR] * rR;
   const double mu = ph.inv_re;
   const double mueff = mu + mutf;
   const double keff = mu * ph.inv_pr + mutf * ph.inv_prt;
+  hv[0] = 0.0;
+  if (FAST) {
+    const double du = uR - uL, dv = vR - vL, dh = L.p[gR] * rR - L.p[gL] * rL;
+    const double xx = sx * sx, yy = sy * sy, s2 = xx + yy, c3 = (1.0 / 3.0) * sx * sy, k = mueff * rvf;
+    const double fx = k * (du * fma(1.0 / 3.0, xx, s2) + dv * c3);
+    const double fy = k * (dv * fma(1.0 / 3.0, yy, s2) + du * c3);
+    hv[1] = fx;
+    hv[2] = fy;
+    hv[3] = 0.5 * ((uL + uR) * fx + (vL + vR) * fy) + (cp * keff * rvf) * (dh * s2);
+    return;
+  }
+  const double hL = cp * L.p[gL] * rL, hR = cp * L.p[gR] * rR;
   const double sxv = sx * rvf, syv = sy * rvf;
   const double gux = (uR - uL) * sxv, guy = (uR - uL) * syv;
   const double gvx = (vR - vL) * sxv, gvy = (vR - vL) * syv;
@@ -423,7 +460,6 @@ __device__ void visc_face(const LevelDev& L, const PhysParams& ph, int i, int j,
   const double txy = mueff * (guy + gvx);
   const double uf = 0.5 * (uL + uR), vf = 0.5 * (vL + vR);
   const double fx = txx * sx + txy * sy, fy = txy * sx + tyy * sy;
-  hv[0] = 0.0;
   hv[1] = fx;
   hv[2] = fy;
   hv[3] = uf * fx + vf * fy + keff * (ghx * sx + ghy * sy);
@@ -444,16 +480,36 @@ __device__ double block_sum(double v, double* wsum) {
 
 // One tile of TX x TY cells: every face of the tile is computed once into shared memory,
 // then each cell assembles F^c and F^v and writes what the mode asks for.
-template <int TY>
+template <int TY, bool FAST>
 __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysParams ph, ResArgs a) {
   pdl_entry();
   __shared__ double xc[4][TY][TX + 1], xd[4][TY][TX + 1];
   __shared__ double ec[4][TY + 1][TX], ed[4][TY + 1][TX];
   __shared__ double wsum[2 * TY + 1];
+  __shared__ double si[TY], sj[TY + 2][TX];  // sensors: along i of cell (i0 + TX, j0 + y), along j of rows j0 - 1 ..
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   const int ni = L.ni, nj = L.nj;
+  // Each cell's pressure switch is formed once (finest level): an i-face warp's lane takes cell
+  // i0 + lane - 1 of its row and passes it on, its last cell is the j-face warps' spare lane's; the
+  // j-face warps take a row each (the last one two).
+  double sl = 0.0;
+  const bool sensors = L.finest && !ph.flux;
+  if (sensors) {
+    if (warp < TY) {
+      if (i0 + lane <= ni + 1 && j0 + warp < nj) sl = cell_sensor<FAST>(L, gidx(L, i0 + lane - 1, j0 + warp), 1);
+    } else {
+      const int y = warp - TY;
+      const int i = i0 + lane, j = j0 + (lane < TX ? y - 1 : y);
+      if (lane < TX ? i < ni && j <= nj : y < TY && i < ni + 1 && j < nj)
+        (lane < TX ? sj[y][lane] : si[y]) =
+            cell_sensor<FAST>(L, gidx(L, i, j), lane < TX ? L.P : 1);
+      if (y == TY && lane < TX && i < ni && j0 + TY <= nj) sj[TY + 1][lane] = cell_sensor<FAST>(L, gidx(L, i, j0 + TY), L.P);
+    }
+    __syncthreads();
+  }
   if (warp < TY) {  // i-face (i0 + lane, j0 + warp)
+    const double sdn = __shfl_down_sync(0xffffffffu, sl, 1), sr = lane < TX ? sdn : si[warp];
     const int tx = lane, ty = warp;
     const int i = i0 + tx, j = j0 + ty;
     if (i <= ni && j < nj) {
@@ -462,8 +518,9 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
       if (ph.flux)
         fvs_face(L, gidx(L, i - 1, j), gidx(L, i, j), L.sxi[f], L.sxi[L.nfx + f], L.vfx[f], ph.d_cut, hc, hd);
       else
-        jst_face(L, gidx(L, i - 2, j), gidx(L, i - 1, j), gidx(L, i, j), gidx(L, i + 1, j), L.sxi[f],
-                 L.sxi[L.nfx + f], L.vfx[f], rt_cell(L, i - 1, j, 0), rt_cell(L, i, j, 0), ph.s_coarse, hc, hd);
+        jst_face<FAST>(L, gidx(L, i - 2, j), gidx(L, i - 1, j), gidx(L, i, j), gidx(L, i + 1, j), L.sxi[f],
+                 L.sxi[L.nfx + f], ph.moving ? L.vfx[f] : 0.0, ph.moving, rt_cell(L, i - 1, j, 0), rt_cell(L, i, j, 0),
+                 fmax(sl, sr), ph.s_coarse, hc, hd);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         xc[k][ty][tx] = hc[k];
@@ -480,13 +537,14 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
       if (ph.flux)
         fvs_face(L, gidx(L, i, j - 1), gidx(L, i, j), sx, sy, L.vfe[f], ph.d_cut, hc, hd);
       else
-        jst_face(L, gidx(L, i, j - 2), gidx(L, i, j - 1), gidx(L, i, j), gidx(L, i, j + 1), sx, sy, L.vfe[f],
-                 rt_cell(L, i, j - 1, 1), rt_cell(L, i, j, 1), ph.s_coarse, hc, hd);
+        jst_face<FAST>(L, gidx(L, i, j - 2), gidx(L, i, j - 1), gidx(L, i, j), gidx(L, i, j + 1), sx, sy,
+                 ph.moving ? L.vfe[f] : 0.0, ph.moving, rt_cell(L, i, j - 1, 1), rt_cell(L, i, j, 1),
+                 sensors ? fmax(sj[ty][tx], sj[ty + 1][tx]) : 0.0, ph.s_coarse, hc, hd);
       if (ph.viscous) {
         double hv[4];
-        visc_face(L, ph, i, j, sx, sy, hv);
+        visc_face<FAST>(L, ph, i, j, sx, sy, hv);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) hd[k] += hv[k];
+        for (int k = 1; k < 4; ++k) hd[k] += hv[k];
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -503,14 +561,16 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
     if (i < ni && j < nj) {
       const int c = j * ni + i;
       const int n = L.n;
-      const double rvol = 1.0 / L.vol[c];
+      const double rvol = L.rvol[c];
+      const bool timed = !is_zero(L.a_t);
       const int g = gidx(L, i, j);
       double Fc[4], Fv[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const double fc = (xc[k][ty][tx + 1] - xc[k][ty][tx]) + (ec[k][ty + 1][tx] - ec[k][ty][tx]);
-        const double fd = -((xd[k][ty][tx + 1] - xd[k][ty][tx]) + (ed[k][ty + 1][tx] - ed[k][ty][tx]));
-        double fcv = fc * rvol + L.a_t * L.u[k * L.Gn + g] + L.src[k * n + c];
+        const double fd = (xd[k][ty][tx] - xd[k][ty][tx + 1]) + (ed[k][ty][tx] - ed[k][ty + 1][tx]);
+        double fcv = timed ? fma(fc, rvol, __dmul_rn(L.a_t, L.u[k * L.Gn + g])) : fc * rvol;
+        if (L.finest) fcv += L.src[k * n + c];  // coarse levels have no history source
         if (a.mode != RES_FORCING) fcv -= L.s[k * n + c];
         Fc[k] = fcv;
         Fv[k] = fd * rvol;
@@ -574,11 +634,13 @@ __global__ void k_wall_force(LevelDev L, PhysParams ph, double* fx, double* fy) 
   if (ph.flux)
     fvs_face(L, gidx(L, i, -1), gidx(L, i, 0), sx, sy, L.vfe[i], ph.d_cut, hc, hd);
   else
-    jst_face(L, gidx(L, i, -2), gidx(L, i, -1), gidx(L, i, 0), gidx(L, i, 1), sx, sy, L.vfe[i],
-             rt_cell(L, i, -1, 1), rt_cell(L, i, 0, 1), ph.s_coarse, hc, hd);
+    jst_face<false>(L, gidx(L, i, -2), gidx(L, i, -1), gidx(L, i, 0), gidx(L, i, 1), sx, sy, L.vfe[i], ph.moving,
+             rt_cell(L, i, -1, 1), rt_cell(L, i, 0, 1),
+             L.finest ? fmax(cell_sensor<false>(L, gidx(L, i, -1), L.P), cell_sensor<false>(L, gidx(L, i, 0), L.P)) : 0.0,
+             ph.s_coarse, hc, hd);
   if (ph.viscous) {
     double hv[4];
-    visc_face(L, ph, i, 0, sx, sy, hv);
+    visc_face<false>(L, ph, i, 0, sx, sy, hv);
     for (int k = 0; k < 4; ++k) hd[k] += hv[k];
   }
   fx[i] = -(hc[1] - hd[1]);
@@ -699,7 +761,22 @@ __global__ void k_check_math(int n, const double* __restrict__ a, const double* 
   out[4 * t + 3] = cbrt(a[t] / b[t]);
 }
 
+// The FP64 helpers beside the instructions they stand for: out[4 t ..] = (rcp64(a), 1/a, d2f(a),
+// f2d((float)a)).
+__global__ void k_check_fp64(int n, const double* __restrict__ a, double* __restrict__ out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  out[4 * t + 0] = rcp64(a[t]);
+  out[4 * t + 1] = 1.0 / a[t];
+  out[4 * t + 2] = (double)d2f(a[t]);
+  out[4 * t + 3] = f2d((float)a[t]);
+}
+
 }  // namespace
+
+void launch_check_fp64(int n, const double* a, double* out, cudaStream_t st) {
+  if (n > 0) k_check_fp64<<<(n + 127) / 128, 128, 0, st>>>(n, a, out);
+}
 
 void launch_check_math(int n, const double* a, const double* b, double* out, cudaStream_t st) {
   if (n > 0) k_check_math<<<(n + 127) / 128, 128, 0, st>>>(n, a, b, out);
@@ -729,15 +806,22 @@ int residual_blocks(const LevelDev& L) {
   return ((L.ni + TX - 1) / TX) * ((L.nj + ty - 1) / ty);
 }
 
+namespace {
+template <bool FAST>
+cudaError_t residual_ty(int ty, dim3 grid, cudaStream_t st, const LevelDev& L, const PhysParams& ph, const ResArgs& a) {
+  switch (ty) {
+    case 8: return launch_pdl(k_residual<8, FAST>, grid, res_threads(8), 0, st, L, ph, a);
+    case 4: return launch_pdl(k_residual<4, FAST>, grid, res_threads(4), 0, st, L, ph, a);
+    case 2: return launch_pdl(k_residual<2, FAST>, grid, res_threads(2), 0, st, L, ph, a);
+    default: return launch_pdl(k_residual<1, FAST>, grid, res_threads(1), 0, st, L, ph, a);
+  }
+}
+}  // namespace
+
 cudaError_t launch_residual(const LevelDev& L, const PhysParams& ph, const ResArgs& a, cudaStream_t st) {
   const int ty = res_ty(L);
   const dim3 grid((L.ni + TX - 1) / TX, (L.nj + ty - 1) / ty);
-  switch (ty) {
-    case 8: return launch_pdl(k_residual<8>, grid, res_threads(8), 0, st, L, ph, a);
-    case 4: return launch_pdl(k_residual<4>, grid, res_threads(4), 0, st, L, ph, a);
-    case 2: return launch_pdl(k_residual<2>, grid, res_threads(2), 0, st, L, ph, a);
-    default: return launch_pdl(k_residual<1>, grid, res_threads(1), 0, st, L, ph, a);
-  }
+  return ph.fast ? residual_ty<true>(ty, grid, st, L, ph, a) : residual_ty<false>(ty, grid, st, L, ph, a);
 }
 
 int residual_blocks_max(const LevelDev& L) { return ((L.ni + TX - 1) / TX) * L.nj; }

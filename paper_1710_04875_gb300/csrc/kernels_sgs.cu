@@ -12,6 +12,7 @@
 // The sweeps follow the hyperplane order i + j = const; on a hyperplane the cells are
 // independent, and the lower/upper neighbour sets of every cell are those of the
 // lexicographic ordering, so the result equals the lexicographic Gauss-Seidel sweep.
+#include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 
 namespace fasw {
@@ -69,8 +70,52 @@ __device__ void split_blocks(const T w[4], T sx, T sy, T vf, T d, T Ap[16], T Am
   }
 }
 
+// The same in FP64 with one reciprocal each of length, density, sound speed and cutoff (rd = 1/d), the
+// length folded into the eigenvalues, and the zeros and ones of r0, r1, dp and dvn left out: about 175
+// FP64 instructions a face against 300 of the form above, which is what bounds the kernel (1024x256
+// level 305 -> 185 us at the pipe's rate).  FP32 keeps the form above, operation by operation.
+__device__ __forceinline__ void split_blocks64(const double w[4], double sx, double sy, double vf, int moving, double d,
+                                               double rd, double Ap[16], double Am[16]) {
+  constexpr double g1 = GAM - 1.0;
+  const double len = sqrt(sx * sx + sy * sy), rl = rcp64(len);
+  const double nx = sx * rl, ny = sy * rl;
+  const double rr = rcp64(w[0]), u = w[1] * rr, v = w[2] * rr;
+  const double q2 = u * u + v * v;
+  const double p = g1 * (w[3] - 0.5 * w[0] * q2);
+  const double a = sqrt(GAM * p * rr), ia = rcp64(a);
+  const double H = (w[3] + p) * rr;
+  const double vn = u * nx + v * ny, vr = moving ? vn - vf * rl : vn;
+  const double dp[3] = {0.5 * g1 * q2, -g1 * u, -g1 * v};  // dp[3] = g1; dvn = (-vn, nx, ny, 0)
+  const double lam[3] = {vr, vr + a, vr - a}, ad = a * d, iad = ia * rd, hl = 0.5 * len;
+  double P[3], Q[3];  // halves of the eigenvalues and of their cutoff moduli, times the length
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double al = fabs(lam[k]);
+    const bool cut = d > 0.0 && __double_as_longlong(al) <= __double_as_longlong(ad);
+    P[k] = hl * lam[k];
+    Q[k] = hl * (cut ? 0.5 * fma(lam[k] * lam[k], iad, ad) : al);
+  }
+#pragma unroll
+  for (int sgn = 0; sgn < 2; ++sgn) {
+    const double l1 = sgn ? P[0] - Q[0] : P[0] + Q[0], l3 = sgn ? P[1] - Q[1] : P[1] + Q[1],
+                 l4 = sgn ? P[2] - Q[2] : P[2] + Q[2];
+    const double c1 = fma(0.5, l3 + l4, -l1), c2a = 0.5 * (l3 - l4) * ia, c1a = c1 * (ia * ia);
+    const double g0[4] = {c1a * dp[0] - c2a * vn, c1a * dp[1] + c2a * nx, c1a * dp[2] + c2a * ny, c1a * g1};
+    const double gg[4] = {c2a * dp[0] - c1 * vn, c2a * dp[1] + c1 * nx, c2a * dp[2] + c1 * ny, c2a * g1};
+    double* M = sgn == 0 ? Ap : Am;
+    const double r0[4] = {1.0, u, v, H}, r1[4] = {0.0, nx, ny, vn};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) M[c] = c == 0 ? g0[0] + l1 : g0[c];
+#pragma unroll
+    for (int r = 1; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) M[4 * r + c] = fma(r1[r], gg[c], r == c ? fma(r0[r], g0[c], l1) : r0[r] * g0[c]);
+  }
+}
+
 // Thin-layer viscous Jacobian of j-face (i, j) in scalar form: nu |S|^2 / Omega_f with
 // nu = max(mu + mu_t, gamma (mu/Pr + mu_t/Pr_t)) / rho; added as +V I to A+ and -V I to A-.
+template <bool FAST>
 __device__ double visc_radius(const LevelDev& L, const PhysParams& ph, int i, int j, double rho) {
   const int ni = L.ni, nj = L.nj;
   double volL, volR, mutf;
@@ -94,14 +139,16 @@ __device__ double visc_radius(const LevelDev& L, const PhysParams& ph, int i, in
     mutf = 0.5 * (L.mut[(j - 1) * ni + i] + L.mut[j * ni + i]);
   }
   const double mu = ph.inv_re;
-  const double nu = fmax(mu + mutf, GAM * (mu * ph.inv_pr + mutf * ph.inv_prt)) / rho;
+  const double num = fmax(mu + mutf, GAM * (mu * ph.inv_pr + mutf * ph.inv_prt));
   const int f = j * ni + i;
   const double sx = L.seta[f], sy = L.seta[L.nfe + f];
+  if (FAST) return num * rcp64(rho) * (sx * sx + sy * sy) * L.rvf[f];
+  const double nu = num / rho;
   return 2.0 * nu * (sx * sx + sy * sy) / (volL + volR);
 }
 
 template <typename T>
-__global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d) {
+__global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d, T rd) {
   pdl_entry();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   const int ni = L.ni;
@@ -116,7 +163,7 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d) {
     gR = gidx(L, i, j);
     sx = L.sxi[f];
     sy = L.sxi[L.nfx + f];
-    vf = L.vfx[f];
+    vf = ph.moving ? L.vfx[f] : 0.0;
     Ap = blk + f;
     Am = blk + 16 * L.nfx + f;
     stride = L.nfx;
@@ -127,7 +174,7 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d) {
     gR = gidx(L, i, j);
     sx = L.seta[e];
     sy = L.seta[L.nfe + e];
-    vf = L.vfe[e];
+    vf = ph.moving ? L.vfe[e] : 0.0;
     Ap = blk + 32 * L.nfx + e;
     Am = blk + 32 * L.nfx + 16 * L.nfe + e;
     stride = L.nfe;
@@ -137,13 +184,16 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     wd[k] = 0.5 * (L.u[k * L.Gn + gL] + L.u[k * L.Gn + gR]);
-    w[k] = T(wd[k]);
+    w[k] = from64<T>(wd[k]);
   }
   T P[16], M[16];
-  split_blocks<T>(w, T(sx), T(sy), T(vf), d, P, M);
+  if constexpr (sizeof(T) == 8)
+    split_blocks64(w, sx, sy, vf, ph.moving, d, rd, P, M);
+  else
+    split_blocks<T>(w, from64<T>(sx), from64<T>(sy), from64<T>(vf), d, P, M);
   if (ph.viscous && f >= L.nfx) {
     const int e = f - L.nfx;
-    const T V = T(visc_radius(L, ph, e % ni, e / ni, wd[0]));
+    const T V = from64<T>(visc_radius<sizeof(T) == 8>(L, ph, e % ni, e / ni, wd[0]));
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       P[5 * k] += V;
@@ -167,10 +217,11 @@ __global__ void k_diag_blocks(LevelDev L, const T* blk, T* dlu, int aw, double e
   const int ni = L.ni, i = c % ni, j = c / ni;
   double coef, sigma;
   if (aw) {
-    coef = eta * L.dts[c] / L.vol[c];
-    sigma = 1.0 + eta * L.dts[c] * L.a_t;
+    const double ed = eta * L.dts[c];
+    coef = sizeof(T) == 8 ? ed * L.rvol[c] : ed / L.vol[c];
+    sigma = is_zero(L.a_t) ? 1.0 : 1.0 + ed * L.a_t;
   } else {
-    coef = 1.0 / L.vol[c];
+    coef = L.rvol[c];
     sigma = L.a_t;
   }
   L.coef[c] = coef;
@@ -185,24 +236,38 @@ __global__ void k_diag_blocks(LevelDev L, const T* blk, T* dlu, int aw, double e
   const T* Aep = blk + 32 * L.nfx;
   const T* Aem = blk + 32 * L.nfx + 16 * L.nfe;
   T A[16];
-  const T cf = T(coef);
+  const T cf = from64<T>(coef), sg = from64<T>(sigma);
 #pragma unroll
   for (int e = 0; e < 16; ++e) {
     const T v = (Axp[e * L.nfx + fe] - Axm[e * L.nfx + fw]) + (Aep[e * L.nfe + fn] - Aem[e * L.nfe + fs]);
-    A[e] = ((e % 5 == 0) ? T(sigma) : T(0)) + cf * v;
+    A[e] = ((e % 5 == 0) ? sg : T(0)) + cf * v;
   }
+  if constexpr (sizeof(T) == 8) {  // each pivot's reciprocal once, for its column's multipliers too
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 4; ++k) {
+      A[5 * k] = rcp64(A[5 * k]);
 #pragma unroll
-    for (int r = k + 1; r < 4; ++r) {
-      const T m = A[4 * r + k] / A[4 * k + k];
-      A[4 * r + k] = m;
+      for (int r = k + 1; r < 4; ++r) {
+        const double m = A[4 * r + k] * A[5 * k];
+        A[4 * r + k] = m;
 #pragma unroll
-      for (int cc = k + 1; cc < 4; ++cc) A[4 * r + cc] -= m * A[4 * k + cc];
+        for (int cc = k + 1; cc < 4; ++cc) A[4 * r + cc] -= m * A[4 * k + cc];
+      }
     }
-  }
+  } else {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) A[5 * k] = T(1) / A[5 * k];
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+      for (int r = k + 1; r < 4; ++r) {
+        const T m = A[4 * r + k] / A[4 * k + k];
+        A[4 * r + k] = m;
+#pragma unroll
+        for (int cc = k + 1; cc < 4; ++cc) A[4 * r + cc] -= m * A[4 * k + cc];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) A[5 * k] = T(1) / A[5 * k];
+  }
 #pragma unroll
   for (int e = 0; e < 16; ++e) dlu[e * L.n + c] = A[e];
 }
@@ -305,9 +370,10 @@ __global__ void k_sgs_single(LevelDev L, const T* blk, const T* dlu, T* yz, cons
 void launch_face_blocks(const LevelDev& L, const PhysParams& ph, const SchemeParams& sc, int mixed, cudaStream_t st) {
   const int nf = L.nfx + L.nfe;
   if (mixed)
-    launch_pdl(k_face_blocks<float>, (nf + 63) / 64, 64, 0, st, L, ph, L.blk32, float(sc.d_cut));
+    launch_pdl(k_face_blocks<float>, (nf + 63) / 64, 64, 0, st, L, ph, L.blk32, float(sc.d_cut), 0.f);
   else
-    launch_pdl(k_face_blocks<double>, (nf + 63) / 64, 64, 0, st, L, ph, L.blk64, sc.d_cut);
+    launch_pdl(k_face_blocks<double>, (nf + 63) / 64, 64, 0, st, L, ph, L.blk64, sc.d_cut,
+               sc.d_cut > 0.0 ? 1.0 / sc.d_cut : 0.0);
 }
 
 void launch_diag_blocks(const LevelDev& L, const SchemeParams& sc, int mixed, cudaStream_t st) {

@@ -24,6 +24,7 @@
 //    chunk at once.  Every wait is bounded; on timeout the kernel raises an error flag and
 //    all strips return.
 #include <atomic>
+#include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 #include "fasw_sweep.cuh"
 
@@ -32,6 +33,9 @@ namespace fasw {
 namespace {
 
 __device__ __forceinline__ bool on_cut(const LevelDev& L, int i) { return L.nw > 0 && (i < L.nw || i >= L.ni - L.nw); }
+
+__device__ __forceinline__ float low(double x) { return d2f(x); }
+__device__ __forceinline__ float low(float x) { return x; }
 
 // Transfer blocks, entry-major: tb[(blk*16 + e) * n + c], blk 0 = D^-1, 1 = G_W, 2 = G_S,
 // 3 = H_E, 4 = H_N.  Blocks of absent neighbours are zero.  MODE 1 (HP, FP32 only): blocks 1-4
@@ -71,7 +75,7 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) Di[4 * r + col] = b[r];
   }
-  const T cf = T(L.coef[c]);
+  const T cf = from64<T>(L.coef[c]);
   const T* Axp = blk;
   const T* Axm = blk + 16 * L.nfx;
   const T* Aep = blk + 32 * L.nfx;
@@ -81,6 +85,14 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
   const bool hasS = j > 0 || on_cut(L, i);
 #pragma unroll
   for (int e = 0; e < 16; ++e) tb[e * n + c] = Di[e];
+  // FP64: the scale once on D^-1 instead of on every entry of the products (this kernel is bound by
+  // its FP64 instructions: 1024x256 level 220 -> 189 us with it and the conversions on the integer
+  // pipe); FP32 scales the sums
+  constexpr bool PRE = sizeof(T) == 8;
+  if constexpr (PRE) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) Di[e] *= cf;
+  }
   const size_t h = (size_t)(i + j) * nj + j;
   // MODE 2: this cell's forward / backward rows in the warp-strip layout
   const int jl = j % WS_ROWS, Mp = ws_steps(ni, nj);
@@ -100,7 +112,7 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
         if (present) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) acc += Di[4 * r + k] * B[(4 * k + cc) * sb + f];
-          acc *= s;
+          acc = PRE ? (s < T(0) ? -acc : acc) : acc * s;
         }
         row[cc] = acc;
       }
@@ -112,7 +124,7 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
         for (int cc = 0; cc < 4; ++cc) tb[(slot * 16 + 4 * r + cc) * n + c] = row[cc];
       }
       if constexpr (MODE == 2) {
-        const float4 f = make_float4(float(row[0]), float(row[1]), float(row[2]), float(row[3]));
+        const float4 f = make_float4(low(row[0]), low(row[1]), low(row[2]), low(row[3]));
         if (slot == 1) wf[r] = f;
         if (slot == 2) {
           wf[WS_F4_STEP / 2 + r] = gs_fwd ? f : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -123,10 +135,11 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
       }
     }
   };
-  prod(1, Axp, L.nfx, fw, cf, hasW);
-  prod(2, Aep, L.nfe, fs, cf, hasS);
-  prod(3, Axm, L.nfx, fe, -cf, hasE);
-  prod(4, Aem, L.nfe, fn, -cf, hasN);
+  const T sc = PRE ? T(1) : cf;
+  prod(1, Axp, L.nfx, fw, sc, hasW);
+  prod(2, Aep, L.nfe, fs, sc, hasS);
+  prod(3, Axm, L.nfx, fe, -sc, hasE);
+  prod(4, Aem, L.nfe, fn, -sc, hasN);
 }
 
 template <typename T>

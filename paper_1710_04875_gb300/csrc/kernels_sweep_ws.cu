@@ -42,6 +42,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 #include "fasw_sweep.cuh"
 
@@ -600,7 +601,7 @@ __device__ __forceinline__ double rhs_row(const LevelDev& L, const T* tb, const 
   const int n = L.n;
   double a = 0.0;
 #pragma unroll
-  for (int t = 0; t < 4; ++t) a += double(tb[(size_t)(4 * q + t) * n + c]) * rhs[(size_t)t * n + c];
+  for (int t = 0; t < 4; ++t) a += to64(tb[(size_t)(4 * q + t) * n + c]) * rhs[(size_t)t * n + c];
   return a;
 }
 
@@ -612,35 +613,43 @@ __global__ void k_ws_rhs(LevelDev L, const T* tb, const double* rhs, float4* C) 
   const int ni = L.ni, i = c % ni, j = c / ni;
   const int b = j / WS_ROWS, jl = j % WS_ROWS, Mp = ws_steps(ni, L.nj);
   float* out = reinterpret_cast<float*>(C + ((size_t)b * Mp + (i + jl)) * WS_ROWS + jl);
-  for (int q = q0; q < q1; ++q) out[q] = float(rhs_row(L, tb, rhs, c, q));
+  for (int q = q0; q < q1; ++q) out[q] = d2f(rhs_row(L, tb, rhs, c, q));
 }
 
 // ---------------------------------------------------------------- FP64 defect correction
 // t = (I + U~) z0: the vector the backward sweep would have started from to reach z0,
 //   t_c = z0_c - H_E z0_E - H_N z0_N (- G_S z0_mirror on row 0 of the lower wake).
-__device__ __forceinline__ double defect_t_row(const LevelDev& L, const double* tb, const float4* z0, int c, int q) {
-  const int ni = L.ni, nj = L.nj, n = L.n, i = c % ni, j = c / ni;
-  const int Mp = ws_steps(ni, nj);
-  const float4 zc = z0[ws_bpos(i, j, Mp)];
-  double acc = q == 0 ? zc.x : q == 1 ? zc.y : q == 2 ? zc.z : zc.w;
-  auto sub = [&](int blk, int cn) {
-    const float4 zn = z0[ws_bpos(cn % ni, cn / ni, Mp)];
-    const double x[4] = {zn.x, zn.y, zn.z, zn.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc -= tb[(size_t)(blk * 16 + 4 * q + k) * n + c] * x[k];
-  };
-  if (i < ni - 1) sub(3, c + 1);
-  if (j < nj - 1) sub(4, c + ni);
-  if (j == 0 && L.nw > 0 && i < L.nw && ni - 1 - i > i) sub(2, ni - 1 - i);
-  return acc;
+__device__ __forceinline__ void ws_load64(const float4* z, size_t pos, double x[4]) {
+  const float4 v = z[pos];
+  x[0] = f2d(v.x);
+  x[1] = f2d(v.y);
+  x[2] = f2d(v.z);
+  x[3] = f2d(v.w);
 }
 
+// rows q0 .. q1 - 1 of t (each neighbour's vector is converted once for all of them)
 template <bool SPLIT>
 __global__ void k_ws_defect_t(LevelDev L, const double* tb, const float4* z0, double* t) {
   pdl_entry();
   int c, q0, q1;
   if (!ws_thread<SPLIT>(L, c, q0, q1)) return;
-  for (int q = q0; q < q1; ++q) t[(size_t)q * L.n + c] = defect_t_row(L, tb, z0, c, q);
+  const int ni = L.ni, nj = L.nj, n = L.n, i = c % ni, j = c / ni, Mp = ws_steps(ni, nj);
+  double x[4];
+  ws_load64(z0, ws_bpos(i, j, Mp), x);
+  double acc[4] = {x[0], x[1], x[2], x[3]};
+  if (SPLIT) acc[0] = q0 == 0 ? x[0] : q0 == 1 ? x[1] : q0 == 2 ? x[2] : x[3];
+  auto sub = [&](int blk, int in, int jn) {
+    ws_load64(z0, ws_bpos(in, jn, Mp), x);
+#pragma unroll
+    for (int r = 0; r < (SPLIT ? 1 : 4); ++r)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[r] -= tb[(size_t)(blk * 16 + 4 * (q0 + r) + k) * n + c] * x[k];
+  };
+  if (i < ni - 1) sub(3, i + 1, j);
+  if (j < nj - 1) sub(4, i, j + 1);
+  if (j == 0 && L.nw > 0 && i < L.nw && ni - 1 - i > i) sub(2, ni - 1 - i, 0);
+#pragma unroll
+  for (int r = 0; r < (SPLIT ? 1 : 4); ++r) t[(size_t)(q0 + r) * n + c] = acc[r];
 }
 
 // d = D^-1 r - (I + L~) t = D^-1 r - t_c + G_W t_W + G_S t_S (t_S: the mirror on row 0 of the
@@ -669,7 +678,7 @@ __global__ void k_ws_defect_d(LevelDev L, const double* tb, const double* rhs, c
   const int ni = L.ni, i = c % ni, j = c / ni;
   const int b = j / WS_ROWS, jl = j % WS_ROWS, Mp = ws_steps(ni, L.nj);
   float* out = reinterpret_cast<float*>(C + ((size_t)b * Mp + (i + jl)) * WS_ROWS + jl);
-  for (int q = q0; q < q1; ++q) out[q] = float(defect_d_row(L, tb, rhs, t, c, q));
+  for (int q = q0; q < q1; ++q) out[q] = d2f(defect_d_row(L, tb, rhs, t, c, q));
 }
 
 // z = z0 (+ dz): the stage update u = u0 - alpha z (scaled by dt* for ARK), or z to the level's
@@ -681,14 +690,13 @@ __global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, int 
   if (c >= L.n) return;
   const int n = L.n, i = c % L.ni, j = c / L.ni;
   const size_t zp = ws_bpos(i, j, ws_steps(L.ni, L.nj));
-  const float4 a = z0[zp];
-  double z[4] = {a.x, a.y, a.z, a.w};
+  double z[4];
+  ws_load64(z0, zp, z);
   if (dz) {
-    const float4 d = dz[zp];
-    z[0] += d.x;
-    z[1] += d.y;
-    z[2] += d.z;
-    z[3] += d.w;
+    double d[4];
+    ws_load64(dz, zp, d);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) z[q] += d[q];
   }
   if (do_update) {
     const double sc = aw ? alpha : alpha * L.dts[c];
@@ -697,7 +705,7 @@ __global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, int 
     for (int q = 0; q < 4; ++q) L.u[q * (size_t)L.Gn + g] = L.u0[q * (size_t)n + c] - sc * z[q];
   } else if (mixed) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) L.yz32[q * (size_t)n + c] = float(z[q]);
+    for (int q = 0; q < 4; ++q) L.yz32[q * (size_t)n + c] = d2f(z[q]);
   } else {
 #pragma unroll
     for (int q = 0; q < 4; ++q) L.yz64[q * (size_t)n + c] = z[q];
@@ -716,14 +724,13 @@ __global__ void k_ws_accum(LevelDev L, const float4* z0, const float4* dz, doubl
   if (c >= L.n) return;
   const int i = c % L.ni, j = c / L.ni;
   const size_t zp = ws_bpos(i, j, ws_steps(L.ni, L.nj));
-  const float4 a = z0[zp];
-  double v[4] = {a.x, a.y, a.z, a.w};
+  double v[4];
+  ws_load64(z0, zp, v);
   if (dz) {
-    const float4 d = dz[zp];
-    v[0] += d.x;
-    v[1] += d.y;
-    v[2] += d.z;
-    v[3] += d.w;
+    double d[4];
+    ws_load64(dz, zp, d);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] += d[q];
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) x[4 * (size_t)c + q] = (init ? 0.0 : x[4 * (size_t)c + q]) + v[q];
@@ -744,14 +751,14 @@ __global__ void k_ws_exact_defect(LevelDev L, const T* tb, const double* rhs, co
   for (int q = 0; q < 4; ++q) {
     double a = -x[4 * (size_t)c + q];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) a += double(tb[(size_t)(4 * q + k) * n + c]) * r[k];
+    for (int k = 0; k < 4; ++k) a += to64(tb[(size_t)(4 * q + k) * n + c]) * r[k];
     acc[q] = a;
   }
   auto add = [&](int blk, int cn) {
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) acc[q] += double(tb[(size_t)(blk * 16 + 4 * q + k) * n + c]) * x[4 * (size_t)cn + k];
+      for (int k = 0; k < 4; ++k) acc[q] += to64(tb[(size_t)(blk * 16 + 4 * q + k) * n + c]) * x[4 * (size_t)cn + k];
   };
   if (i > 0) add(1, c - 1);
   if (j > 0) add(2, c - ni);
@@ -759,7 +766,7 @@ __global__ void k_ws_exact_defect(LevelDev L, const T* tb, const double* rhs, co
   if (i < ni - 1) add(3, c + 1);
   if (j < nj - 1) add(4, c + ni);
   const int b = j / WS_ROWS, jl = j % WS_ROWS, Mp = ws_steps(ni, L.nj);
-  C[((size_t)b * Mp + (i + jl)) * WS_ROWS + jl] = make_float4(float(acc[0]), float(acc[1]), float(acc[2]), float(acc[3]));
+  C[((size_t)b * Mp + (i + jl)) * WS_ROWS + jl] = make_float4(d2f(acc[0]), d2f(acc[1]), d2f(acc[2]), d2f(acc[3]));
 }
 
 // the stage update (or the result vector) from the accumulated x

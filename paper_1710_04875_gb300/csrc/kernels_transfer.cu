@@ -1,5 +1,6 @@
 // Grid metrics, agglomeration, FAS restriction / prolongation (section 3 of arXiv
 // 1710.04875) and small data-movement kernels.
+#include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 #include "fasw_transfer.cuh"
 
@@ -26,6 +27,25 @@ __device__ __forceinline__ void vert(const double* x, const double* y, int k, co
   const double dx = x[k] - m.xc, dy = y[k] - m.yc;
   px = m.xc + m.cs * dx - m.sn * dy;
   py = m.yc + m.sn * dx + m.cs * dy;
+}
+
+__device__ __forceinline__ double cell_vol(const double* x, const double* y, int V, int i, int j, const Motion& mo) {
+  double x00, y00, x10, y10, x11, y11, x01, y01;
+  vert(x, y, j * V + i, mo, x00, y00);
+  vert(x, y, j * V + i + 1, mo, x10, y10);
+  vert(x, y, (j + 1) * V + i + 1, mo, x11, y11);
+  vert(x, y, (j + 1) * V + i, mo, x01, y01);
+  const double d1x = x11 - x00, d1y = y11 - y00, d2x = x01 - x10, d2y = y01 - y10;
+  return 0.5 * (d1x * d2y - d1y * d2x);
+}
+
+// 1 / mean volume of the two cells at j-face (i, j) (thin-layer gradients): ghost volumes are the
+// interior neighbour's, across the wake cut the mirror cell's.  vol(i, j): a cell's volume.
+template <class Vol>
+__device__ __forceinline__ double face_rvol(const LevelDev& L, int i, int j, Vol vol) {
+  const double vL = j > 0 ? vol(i, j - 1) : vol(on_cut(L, i) ? L.ni - 1 - i : i, 0);
+  const double vR = j < L.nj ? vol(i, j) : vol(i, j - 1);
+  return 2.0 / (vL + vR);
 }
 
 __global__ void k_metrics_fine(LevelDev L, const double* x, const double* y, Motion mo) {
@@ -55,6 +75,7 @@ __global__ void k_metrics_fine(LevelDev L, const double* x, const double* y, Mot
     L.seta[L.nfe + t] = dx;
     const double mx = 0.5 * (xa + xb), my = 0.5 * (ya + yb);
     L.vfe[t] = vgx(mx, my) * (-dy) + vgy(mx, my) * dx;
+    L.rvf[t] = face_rvol(L, i, j, [&](int a, int b) { return cell_vol(x, y, V, a, b, mo); });
     if (j == 0) {
       L.wvx[i] = vgx(mx, my);
       L.wvy[i] = vgy(mx, my);
@@ -69,12 +90,23 @@ __global__ void k_metrics_fine(LevelDev L, const double* x, const double* y, Mot
     vert(x, y, (j + 1) * V + i, mo, x01, y01);
     vert(x, y, i, mo, xw0, yw0);
     vert(x, y, i + 1, mo, xw1, yw1);
-    const double d1x = x11 - x00, d1y = y11 - y00, d2x = x01 - x10, d2y = y01 - y10;
-    L.vol[t] = 0.5 * (d1x * d2y - d1y * d2x);
+    const double vol = cell_vol(x, y, V, i, j, mo);
+    L.vol[t] = vol;
+    L.rvol[t] = 1.0 / vol;
+    // the cell's mean face vectors, from the face vectors as stored
+    const double sx = 0.5 * ((y01 - y00) + (y11 - y10)), sy = 0.5 * (-(x01 - x00) + -(x11 - x10));
+    const double ex = 0.5 * (-(y10 - y00) + -(y11 - y01)), ey = 0.5 * ((x10 - x00) + (x11 - x01));
+    L.clen[t] = sqrt(fma(sx, sx, sy * sy));
+    L.clen[L.n + t] = sqrt(fma(ex, ex, ey * ey));
     const double cx = 0.25 * (x00 + x10 + x11 + x01), cy = 0.25 * (y00 + y10 + y11 + y01);
     const double mx = 0.5 * (xw0 + xw1), my = 0.5 * (yw0 + yw1);
     L.wdist[t] = sqrt((cx - mx) * (cx - mx) + (cy - my) * (cy - my));
   }
+}
+
+__device__ __forceinline__ double sum_vol(const LevelDev& F, int i, int j) {
+  const int a = (2 * j) * F.ni + 2 * i, b = (2 * j + 1) * F.ni + 2 * i;
+  return (F.vol[a] + F.vol[a + 1]) + (F.vol[b] + F.vol[b + 1]);
 }
 
 // Coarse metrics by agglomerating 2x2 fine cells: face vectors add, volumes add.
@@ -95,6 +127,7 @@ __global__ void k_agglomerate(LevelDev F, LevelDev C) {
     C.seta[t] = F.seta[fa] + F.seta[fb];
     C.seta[C.nfe + t] = F.seta[F.nfe + fa] + F.seta[F.nfe + fb];
     C.vfe[t] = F.vfe[fa] + F.vfe[fb];
+    C.rvf[t] = face_rvol(C, i, j, [&](int a, int b) { return sum_vol(F, a, b); });
     if (j == 0) {
       C.wvx[i] = 0.5 * (F.wvx[2 * i] + F.wvx[2 * i + 1]);
       C.wvy[i] = 0.5 * (F.wvy[2 * i] + F.wvy[2 * i + 1]);
@@ -102,8 +135,17 @@ __global__ void k_agglomerate(LevelDev F, LevelDev C) {
   }
   if (t < C.n) {
     const int i = t % ni, j = t / ni;
-    const int a = (2 * j) * F.ni + 2 * i, b = (2 * j + 1) * F.ni + 2 * i;
-    C.vol[t] = (F.vol[a] + F.vol[a + 1]) + (F.vol[b] + F.vol[b + 1]);
+    const int a = (2 * j) * F.ni + 2 * i;
+    const double vol = sum_vol(F, i, j);
+    C.vol[t] = vol;
+    C.rvol[t] = 1.0 / vol;
+    const int w = (2 * j) * (F.ni + 1) + 2 * i, n = a + 2 * F.ni;  // its west face's and its north face's first halves
+    auto xi = [&](int p, int f) { return F.sxi[p * F.nfx + f] + F.sxi[p * F.nfx + f + F.ni + 1]; };
+    auto eta = [&](int p, int f) { return F.seta[p * F.nfe + f] + F.seta[p * F.nfe + f + 1]; };
+    const double sx = 0.5 * (xi(0, w) + xi(0, w + 2)), sy = 0.5 * (xi(1, w) + xi(1, w + 2));
+    const double ex = 0.5 * (eta(0, a) + eta(0, n)), ey = 0.5 * (eta(1, a) + eta(1, n));
+    C.clen[t] = sqrt(fma(sx, sx, sy * sy));
+    C.clen[C.n + t] = sqrt(fma(ex, ex, ey * ey));
   }
 }
 
@@ -129,14 +171,15 @@ __global__ void k_copy_u0(LevelDev L) {
 
 // Volume-weighted agglomeration restriction of the state and of the FAS residual (rhs),
 // and of the eddy viscosity when requested; the coarse state starts at u~.
-__global__ void k_restrict(LevelDev F, LevelDev C, int restrict_mut) {
+__global__ void k_restrict(LevelDev F, LevelDev C, int restrict_mut, int fast) {
   pdl_entry();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= C.n) return;
   const int I = t % C.ni, J = t / C.ni;
   const int fi[4] = {2 * I, 2 * I + 1, 2 * I, 2 * I + 1};
   const int fj[4] = {2 * J, 2 * J, 2 * J + 1, 2 * J + 1};
-  const double vc = C.vol[t];
+  const double vc = C.vol[t], rvc = C.rvol[t];
+  auto over = [&](double a) { return fast ? a * rvc : a / vc; };
   double au[4] = {0, 0, 0, 0}, ar[4] = {0, 0, 0, 0}, am = 0.0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -153,12 +196,12 @@ __global__ void k_restrict(LevelDev F, LevelDev C, int restrict_mut) {
   const int cg = gidx(C, I, J);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const double v = au[k] / vc;
+    const double v = over(au[k]);
     C.u[k * C.Gn + cg] = v;
     C.ut[k * C.n + t] = v;
-    C.rhs[k * C.n + t] = ar[k] / vc;
+    C.rhs[k * C.n + t] = over(ar[k]);
   }
-  if (restrict_mut) C.mut[t] = am / vc;
+  if (restrict_mut) C.mut[t] = over(am);
 }
 
 // Correction u_{l-1} - u~_{l-1} at a possibly-ghost coarse cell: zero-gradient copy at the
@@ -255,8 +298,8 @@ cudaError_t launch_fill_state(const LevelDev& L, const double w[4], cudaStream_t
 
 void launch_copy_u0(const LevelDev& L, cudaStream_t st) { launch_pdl(k_copy_u0, (L.n + 255) / 256, 256, 0, st, L); }
 
-void launch_restrict(const LevelDev& F, const LevelDev& C, int restrict_mut, cudaStream_t st) {
-  launch_pdl(k_restrict, (C.n + 63) / 64, 64, 0, st, F, C, restrict_mut);
+void launch_restrict(const LevelDev& F, const LevelDev& C, int restrict_mut, int fast, cudaStream_t st) {
+  launch_pdl(k_restrict, (C.n + 63) / 64, 64, 0, st, F, C, restrict_mut, fast);
 }
 
 void launch_prolong(const LevelDev& F, const LevelDev& C, cudaStream_t st) {

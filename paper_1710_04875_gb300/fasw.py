@@ -107,6 +107,7 @@ def library(variant: str = "perf"):
             "fasw_pitching_objective": (i, [p, d, d, d, d, d, i, i, d, i, i, C.POINTER(d), C.POINTER(i)]),
             "fasw_checkpoint_schedule": (i, [i, i, dp, dp, i, C.POINTER(i), C.POINTER(ll)]),
             "fasw_check_math": (i, [i, p, p, p, i]),
+            "fasw_check_fp64": (i, [i, p, p]),
             "fasw_unsteady_adjoint": (i, [p, d, d, d, d, d, i, i, d, i, i, i, i, dp, d, d, d, i, i, d, C.POINTER(d),
                                           dp, dp, i, dp]),
             "fasw_residual_noalloc": (i, [i, i, i, dp, dp, dp, dp, C.POINTER(Params), p]),
@@ -515,6 +516,15 @@ def check_math(a, b):
         raise ValueError("a and b differ in size")
     out = np.zeros((a.size, 4))
     _check(library().fasw_check_math(a.size, a.ctypes.data, b.ctypes.data, out.ctypes.data, 0), "fasw_check_math")
+    return out[:, 0], out[:, 1], out[:, 2], out[:, 3]
+
+
+def check_fp64(a):
+    """(reciprocal, 1/a, FP32 rounding of a, widened FP32 of a) per element: the library's FP64 helpers
+    beside what they stand for, on the current GPU."""
+    a = np.ascontiguousarray(a, dtype=np.float64).ravel()
+    out = np.zeros((a.size, 4))
+    _check(library().fasw_check_fp64(a.size, a.ctypes.data, out.ctypes.data), "fasw_check_fp64")
     return out[:, 0], out[:, 1], out[:, 2], out[:, 3]
 
 

@@ -191,6 +191,7 @@ int alloc_level(fasw_ctx* c, LevelDev& L) {
     A(L.wsCut, 16 * (size_t)(L.nw > 0 ? L.nw : 1));
     A(L.wsZ, 2 * wv);
     A(L.wsT, 4 * n);
+    if (!c->mixed) A(L.wsR, 4 * n);
     A(L.wsX, 4 * n);
     // padding positions of the skewed arrays are never written: they must read as zero
     CKR(cudaMemsetAsync(L.wsF, 0, wf * sizeof(float), c->st));
@@ -247,25 +248,26 @@ int level_sweep_kind(const fasw_ctx* c, const LevelDev& L) {
   return k;
 }
 
-void run_sweep(fasw_ctx* c, const LevelDev& L, int do_update, double alpha, const double* rhs) {
+void run_sweep(fasw_ctx* c, const LevelDev& L, int do_update, double alpha, const double* rhs, WsPending* pending) {
   if (c->sweep_kind == SWEEP_LEGACY) {
     launch_sgs(L, c->sc, c->mixed, do_update, alpha, rhs, nullptr, c->st);
     ++c->launches;
     return;
   }
   c->launches += launch_sweep(L, c->mixed, level_sweep_kind(c, L), do_update, c->sc.aw, alpha, rhs, c->d_prog,
-                              c->d_err, c->spin_limit, c->st, c->exact_iters);
+                              c->d_err, c->spin_limit, c->st, c->exact_iters, pending);
 }
 
 void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts) {
   Prof p(c, FASW_K_CELL_AUX);
-  launch_bc_aux(c->lev[l], c->ph, cfl, want_dts, c->st);
+  launch_bc_aux(c->lev[l], c->ph, cfl, want_dts, c->st, &c->upd[l]);
+  c->upd[l] = WsPending{};
   ++c->launches;
 }
 
 // One smoothing step on level l: dt* and the preconditioner frozen at u^(0) (reading G19),
 // then the s-stage low-storage loop; AW applies W^-1 to (dt* r), ARK applies dt* P^-1 r.
-void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm) {
+void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next) {
   LevelDev& L = c->lev[l];
   const SchemeParams& sc = c->sc;
   bc_aux(c, l, cfl, 1);
@@ -277,6 +279,9 @@ void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm) {
     launch_sgs_prep(L, c->mixed, level_sweep_kind(c, L), c->st);
     ++c->launches;
   }
+  // With the warp strips the residual kernel writes the sweep's right-hand side, and the next cell
+  // auxiliaries make the stage update: two launches and two passes over the state fewer a stage.
+  const bool ws = c->sweep_kind != SWEEP_LEGACY && is_ws(level_sweep_kind(c, L)) && L.wsF && c->exact_iters == 0;
   for (int i = 1; i <= sc.nstages; ++i) {
     if (i > 1) bc_aux(c, l, cfl, 0);
     ResArgs a{};
@@ -286,20 +291,32 @@ void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm) {
     a.aw = sc.aw;
     a.want_norm = (record_norm && i == 1) ? 1 : 0;
     a.norm_all = c->prm.norm_all;
+    a.wsC = ws ? reinterpret_cast<float4*>(L.wsC) : nullptr;
+    a.tb32 = c->mixed;
     { Prof p(c, FASW_K_RESIDUAL); launch_residual(L, c->ph, a, c->st); }
     if (a.want_norm) {
       Prof p(c, FASW_K_NORM);
       launch_norm_final(L, residual_blocks(L), L.n * (c->prm.norm_all ? 4 : 1), c->d_norm, c->st);
       ++c->launches;
     }
-    { Prof p(c, FASW_K_SGS); run_sweep(c, L, 1, sc.alpha[i - 1], L.rhs); }
+    {
+      Prof p(c, FASW_K_SGS);
+      run_sweep(c, L, 1, sc.alpha[i - 1], ws ? nullptr : L.rhs,
+                ws && (i < sc.nstages || bc_next) ? &c->upd[l] : nullptr);
+    }
     ++c->launches;  // the residual
   }
   // no ghost refill here: every consumer of the ghosts starts with its own fill (bc_aux)
 }
 
-void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm) {
-  for (int k = 0; k < c->prm.nu1; ++k) smooth_step(c, l, cfl, record_norm && k == 0);
+// An update may wait for the bc_aux that begins the next smoothing step, which renews dt*, only where it
+// does not read dt* itself (AW).
+static bool may_wait(const fasw_ctx* c, bool step_next) { return step_next && c->sc.aw; }
+
+void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm, bool again) {
+  const int nu1 = c->prm.nu1;
+  for (int k = 0; k < nu1; ++k)
+    smooth_step(c, l, cfl, record_norm && k == 0, (k + 1 == nu1 && l > 0) || may_wait(c, again || k + 1 < nu1));
   if (l == 0) return;
   LevelDev& F = c->lev[l];
   LevelDev& C = c->lev[l - 1];
@@ -314,7 +331,7 @@ void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm) {
   b.mode = RES_FORCING;
   { Prof p(c, FASW_K_RESIDUAL); launch_residual(C, c->ph, b, c->st); }
   ++c->launches;
-  for (int g = 0; g < c->prm.gamma_cycle; ++g) fas_cycle_rec(c, l - 1, cfl, false);
+  for (int g = 0; g < c->prm.gamma_cycle; ++g) fas_cycle_rec(c, l - 1, cfl, false, g + 1 < c->prm.gamma_cycle);
   { Prof p(c, FASW_K_PROLONG); launch_prolong(F, C, c->st); }
   ++c->launches;
 }
@@ -465,6 +482,7 @@ int fasw_create(int ni, int nj, int n_wake, const double* x, const double* y, in
   c->sc.d_cut = p->d_cut;
   const int nl = p->nlevels;
   c->lev.resize(nl);
+  c->upd.assign(nl, WsPending{});
   for (int l = nl - 1; l >= 0; --l) {
     LevelDev& L = c->lev[l];
     std::memset(&L, 0, sizeof(L));
@@ -683,7 +701,7 @@ int fasw_face_blocks(fasw_ctx* c, int l, double* axp, double* axm, double* aep, 
 int fasw_smooth(fasw_ctx* c, int l, int nsteps, double cfl) {
   if (check_level(c, l) || nsteps < 0) return FASW_ERR_ARG;
   err_clear(c);
-  for (int k = 0; k < nsteps; ++k) smooth_step(c, l, cfl, false);
+  for (int k = 0; k < nsteps; ++k) smooth_step(c, l, cfl, false, may_wait(c, k + 1 < nsteps));
   int r = sync(c);
   return r ? r : err_read(c);
 }

@@ -60,6 +60,7 @@ struct fasw_ctx {
   double* d_un = nullptr;       // dual-time history of the finest level (4 x n)
   double* d_unm1 = nullptr;
   int steps_done = 0;
+  std::vector<fasw::WsPending> upd;  // per level: the stage update left to the next launch_bc_aux
   fasw::AdjointDev adj;               // discrete adjoint of the steady finest level (built on demand)
   int L() const { return (int)lev.size() - 1; }
 };
@@ -67,10 +68,13 @@ struct fasw_ctx {
 namespace fasw {
 // driver steps (fasw_api.cu)
 int level_sweep_kind(const fasw_ctx* c, const LevelDev& L);
-void run_sweep(fasw_ctx* c, const LevelDev& L, int do_update, double alpha, const double* rhs);
+void run_sweep(fasw_ctx* c, const LevelDev& L, int do_update, double alpha, const double* rhs,
+               WsPending* pending = nullptr);
 void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts);
-void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm);
-void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm);
+// bc_next: the level's next launch is a bc_aux that may make the last stage's update
+void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next);
+// again: the level is entered again before its state is used otherwise
+void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm, bool again = false);
 void enqueue_cycle(fasw_ctx* c, double cfl);
 void drop_graphs(fasw_ctx* c);
 int check_level(fasw_ctx* c, int l);

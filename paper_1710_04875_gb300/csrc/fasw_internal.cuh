@@ -105,6 +105,7 @@ struct LevelDev {
   float* wsCut;
   float* wsZ;
   double* wsT;
+  double* wsR;  // D^-1 r of the stage in FP64 (FP64 contexts)
   double* wsX;  // accumulated solution of the exact-preconditioner iterations (4 per cell)
 };
 
@@ -159,13 +160,20 @@ struct ResArgs {
   double* F;          // RES_FULL outputs (may be null), interior layout
   double* Fc;
   double* Fv;
+  // RES_STAGE with the warp-strip sweep: D^-1 rhs, skewed FP32, to wsC (and FP64 to L.wsR in FP64
+  // contexts) instead of rhs to L.rhs; tb32: the transfer blocks are FP32
+  float4* wsC;
+  int tb32;
 };
 
 // ---- launchers (kernels_residual.cu)
 cudaError_t launch_bc(const LevelDev& L, const PhysParams& ph, cudaStream_t st);
 cudaError_t launch_cell_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st);
 // ghost fill and cell auxiliaries in one launch
-void launch_bc_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st);
+// (pending: a stage update still to be made, which this launch makes first)
+struct WsPending;
+void launch_bc_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st,
+                   const WsPending* pending = nullptr);
 cudaError_t launch_residual(const LevelDev& L, const PhysParams& ph, const ResArgs& a, cudaStream_t st);
 int residual_blocks(const LevelDev& L);
 int residual_blocks_max(const LevelDev& L);  // the most tiles any tile height gives (height 1)

@@ -45,13 +45,15 @@ size_t carve(LevelDev& L, double* base) {
   take(L.sxi, 2 * (size_t)L.nfx);
   take(L.seta, 2 * (size_t)L.nfe);
   take(L.vol, (size_t)L.n);
-  take(L.rvol, (size_t)L.n);
-  take(L.clen, 2 * (size_t)L.n);
-  take(L.rvf, (size_t)L.nfe);
-  take(L.wdist, (size_t)L.n);
   take(L.mut, (size_t)L.n);
   take(L.s, 4 * (size_t)L.n);
-  L.src = L.s;  // both zero, and only read
+  L.src = L.s;      // both zero, and only read
+  L.wdist = L.dts;  // neither is read here: no turbulence model, no time steps
+  take(L.rvol, 5 * (size_t)L.n);  // 1/V, the cells' face lengths and the j-faces' 1/V: n + 2n + (n + ni)
+  if (base) {
+    L.clen = L.rvol + L.n;
+    L.rvf = L.clen + 2 * (size_t)L.n;
+  }
   take(L.norm_part, (size_t)residual_blocks(L));
   take(L.vfx, (size_t)L.nfx);
   take(L.vfe, (size_t)L.nfe);

@@ -1,5 +1,6 @@
 // Launchers of the transfer-block preparation and the SGS sweep kernels (kernels_sweep.cu).
 #pragma once
+#include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 
 namespace fasw {
@@ -25,9 +26,11 @@ void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st);
 // Forward and backward sweep of one stage: y = (D+L)^-1 rhs, z = (D+U)^-1 D y into L.yz64 /
 // L.yz32, with the stage update u = u0 - alpha z (AW) or u0 - alpha dt* z (ARK) when
 // do_update.  prog: 2 * sweep_strips(L) flags, err: device error word.  Returns the number of
-// kernels launched.
+// kernels launched.  Warp strips only: rhs null when D^-1 rhs is in place already (ResArgs::wsC);
+// pending non-null: the stage update is left to it.
 int launch_sweep(const LevelDev& L, int mixed, int kind, int do_update, int aw, double alpha, const double* rhs,
-                 long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters = 0);
+                 long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters = 0,
+                 struct WsPending* pending = nullptr);
 int sweep_strips(const LevelDev& L);
 // Warp-strip sweep (kernels_sweep_ws.cu): whether a level can use it, the sizes of its arrays
 // (floats of wsF / wsB; of wsC / wsY), its strips, and one application (refine: FP64 defect
@@ -44,6 +47,46 @@ __host__ __device__ __forceinline__ int ws_steps(int ni, int nj) {
   const int R = nj < WS_ROWS ? nj : WS_ROWS;
   return (ni + R - 1 + WS_U - 1) / WS_U * WS_U;
 }
+// Skewed index of cell (i, j) in the backward order (the layout of y as the backward pass reads
+// it and of its result z): strip j / WS_ROWS, step Mp - 1 - i - r, row r.
+__device__ __forceinline__ size_t ws_bpos(int i, int j, int Mp) {
+  const int jl = j & (WS_ROWS - 1);
+  return ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_ROWS + jl;
+}
+
+__device__ __forceinline__ void ws_load64(const float4* z, size_t pos, double x[4]) {
+  const float4 v = z[pos];
+  x[0] = f2d(v.x);
+  x[1] = f2d(v.y);
+  x[2] = f2d(v.z);
+  x[3] = f2d(v.w);
+}
+
+// A stage update u = u0 - alpha z (AW) or u0 - alpha dt* z (ARK), z = z0 (+ dz), that the sweep left to
+// the kernel that next reads the state, the cell auxiliaries' (launch_bc_aux).  z0 null: none.
+struct WsPending {
+  const float4 *z0, *dz;
+  double alpha;
+  int aw;
+};
+
+// the updated state of interior cell (i, j)
+__device__ __forceinline__ void ws_updated(const LevelDev& L, const WsPending& p, int i, int j, double w[4]) {
+  const int c = j * L.ni + i;
+  const size_t zp = ws_bpos(i, j, ws_steps(L.ni, L.nj));
+  double z[4];
+  ws_load64(p.z0, zp, z);
+  if (p.dz) {
+    double d[4];
+    ws_load64(p.dz, zp, d);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) z[q] += d[q];
+  }
+  const double sc = p.aw ? p.alpha : p.alpha * L.dts[c];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) w[q] = fma(-sc, z[q], L.u0[q * (size_t)L.n + c]);
+}
+
 bool ws_fits(int ni, int nj, int nw);
 size_t ws_floats(int ni, int nj);
 size_t ws_vec_floats(int ni, int nj);
@@ -52,7 +95,7 @@ int ws_strips(int nj);
 // deep: the deeper operand ring (false for SWEEP_WS8)
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,
                     long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters = 0,
-                    bool deep = true);
+                    bool deep = true, WsPending* pending = nullptr);
 // Hyperplane-staged FP32 sweep: whether a level fits (rows, shared memory), and the entries
 // (ni + nj - 1) * nj of its hyperplane-major arrays (hpF, hpB: 32 floats each; hpC, hpY: 4).
 bool hp_fits(int ni, int nj, int nw);

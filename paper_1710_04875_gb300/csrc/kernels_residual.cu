@@ -2,6 +2,7 @@
 // arXiv 1710.04875) and the Baldwin-Lomax closure, FP64.
 #include "fasw_internal.cuh"
 #include "fasw_roots.cuh"
+#include "fasw_sweep.cuh"
 
 namespace fasw {
 
@@ -88,22 +89,30 @@ __device__ void farfield(const double wi[4], const PhysParams& ph, double nx, do
   out[3] = p * (1.0 / (GAM - 1.0)) + 0.5 * rho * (u * u + v * v);
 }
 
+// State of an interior cell, the pending stage update made.
+__device__ __forceinline__ void cell_u(const LevelDev& L, const WsPending& up, int i, int j, double w[4]) {
+  if (up.z0)
+    ws_updated(L, up, i, j, w);
+  else
+    load4(L, gidx(L, i, j), w);
+}
+
 // Boundary value of ghost cell (gi, gj) (two layers on every side; corners excluded):
 // j < 0: wake-cut copy of the mirror cell or wall reflection (slip / no-slip, moving wall);
 // j >= nj, i < 0, i >= ni: Riemann far-field state (section 2, G9).
-__device__ void ghost_state(const LevelDev& L, const PhysParams& ph, int gi, int gj, double g[4]) {
+__device__ void ghost_state(const LevelDev& L, const PhysParams& ph, const WsPending& up, int gi, int gj, double g[4]) {
   const int ni = L.ni, nj = L.nj;
   if (gj < 0) {
     const int i = gi, k = -1 - gj;  // source row 0 or 1
     if (on_cut(L, i)) {
-      load4(L, gidx(L, ni - 1 - i, k), g);
+      cell_u(L, up, ni - 1 - i, k, g);
       return;
     }
     const double sx = L.seta[i], sy = L.seta[L.nfe + i];
     const double len = sqrt(sx * sx + sy * sy);
     const double nx = sx / len, ny = sy / len;
     double w[4];
-    load4(L, gidx(L, i, k), w);
+    cell_u(L, up, i, k, w);
     if (!ph.moving) {
       g[0] = w[0];
       g[3] = w[3];
@@ -139,19 +148,19 @@ __device__ void ghost_state(const LevelDev& L, const PhysParams& ph, int gi, int
     const int i = gi, f = nj * ni + i;
     const double sx = L.seta[f], sy = L.seta[L.nfe + f];
     const double il = 1.0 / sqrt(sx * sx + sy * sy);
-    load4(L, gidx(L, i, nj - 1), w);
+    cell_u(L, up, i, nj - 1, w);
     farfield(w, ph, sx * il, sy * il, L.vfe[f] * il, g);
   } else if (gi < 0) {  // outward -S_xi
     const int j = gj, f = j * (ni + 1);
     const double sx = L.sxi[f], sy = L.sxi[L.nfx + f];
     const double il = 1.0 / sqrt(sx * sx + sy * sy);
-    load4(L, gidx(L, 0, j), w);
+    cell_u(L, up, 0, j, w);
     farfield(w, ph, -sx * il, -sy * il, -L.vfx[f] * il, g);
   } else {  // gi >= ni, outward +S_xi
     const int j = gj, f = j * (ni + 1) + ni;
     const double sx = L.sxi[f], sy = L.sxi[L.nfx + f];
     const double il = 1.0 / sqrt(sx * sx + sy * sy);
-    load4(L, gidx(L, ni - 1, j), w);
+    cell_u(L, up, ni - 1, j, w);
     farfield(w, ph, sx * il, sy * il, L.vfx[f] * il, g);
   }
 }
@@ -184,7 +193,7 @@ __global__ void k_bc(LevelDev L, PhysParams ph) {
   int gi, gj;
   if (!ghost_of(L, blockIdx.x * blockDim.x + threadIdx.x, gi, gj)) return;
   double g[4];
-  ghost_state(L, ph, gi, gj, g);
+  ghost_state(L, ph, WsPending{}, gi, gj, g);
   store4(L, gidx(L, gi, gj), g);
 }
 
@@ -211,7 +220,10 @@ __device__ __forceinline__ void cell_thermo(const LevelDev& L, const PhysParams&
 // Martinelli radii, dt*), the blocks after them the ghost cells (with fill_ghosts their
 // boundary value first, which depends on interior cells only; then pressure, 1/rho, sensor).
 // Interior and ghost work never share a warp, so neither path waits on the other's FP64 chain.
-__global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, int fill_ghosts, int nbi) {
+// up: the stage update the sweep left (made here first: one launch and one pass over the state less;
+// a ghost thread makes it again for the cell it reflects).
+__global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, int fill_ghosts, int nbi,
+                           WsPending up) {
   pdl_entry();
   if ((int)blockIdx.x >= nbi) {
     int gi, gj;
@@ -219,7 +231,7 @@ __global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, 
     const int g = gidx(L, gi, gj);
     double w[4];
     if (fill_ghosts) {
-      ghost_state(L, ph, gi, gj, w);
+      ghost_state(L, ph, up, gi, gj, w);
       store4(L, g, w);
     } else {
       load4(L, g, w);
@@ -233,7 +245,8 @@ __global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, 
   const int ni = L.ni, i = c % ni, j = c / ni;
   const int g = gidx(L, i, j);
   double w[4];
-  load4(L, g, w);
+  cell_u(L, up, i, j, w);
+  if (up.z0) store4(L, g, w);
   double rr, u, v, p;
   cell_thermo(L, ph, g, w, rr, u, v, p);
   const double a = sqrt(GAM * p * rr);
@@ -555,6 +568,8 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
   }
   __syncthreads();
   double nacc = 0.0;
+  double r[4];  // this cell's stage right-hand side
+  bool have = false;
   if (warp < TY && lane < TX) {  // cell (i0 + lane, j0 + warp)
     const int tx = lane, ty = warp;
     const int i = i0 + tx, j = j0 + ty;
@@ -594,8 +609,10 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
             carry = a.beta * Fv[k] + (1.0 - a.beta) * L.fvc[k * n + c];
           }
           L.fvc[k * n + c] = carry;
-          L.rhs[k * n + c] = sc * (Fc[k] + carry);
+          r[k] = sc * (Fc[k] + carry);
+          if (!a.wsC) L.rhs[k * n + c] = r[k];
         }
+        have = true;
       } else if (a.mode == RES_FULL) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -610,6 +627,38 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
 #pragma unroll
         for (int k = 0; k < 4; ++k) L.rhs[k * n + c] = -(Fc[k] + Fv[k]);
       }
+    }
+  }
+  // The warp-strip sweep's right-hand side D^-1 r, where r is: a launch less, and D^-1 r of the defect
+  // with it.  The i-face warps take rows 0 and 1, the j-face warps rows 2 and 3 of the products.  Measured
+  // with the update moved to k_cell_aux: 1024x256 W-cycle FP64 11.43 -> 11.20 ms, mixed 7.18 -> 7.03;
+  // 64 cases of 64x16 ... 256x64 in a batch, mixed 10.7 -> 8.8 ms a cycle, FP64 17.9 -> 13.2.
+  if (a.wsC) {
+    __syncwarp();  // the warp has read its row of xc, which holds the right-hand sides now
+    if (have) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) xc[k][warp][lane] = r[k];
+    }
+    __syncthreads();
+    const int y = warp < TY ? warp : warp - TY, i = i0 + lane, j = j0 + y;
+    if (y < TY && lane < TX && i < ni && j < nj) {
+      const int c = j * ni + i, n = L.n, q0 = warp < TY ? 0 : 2;
+      double x[4], b[2];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[k] = xc[k][y][lane];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        b[q] = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const size_t e = (size_t)(4 * (q0 + q) + k) * n + c;
+          b[q] += (a.tb32 ? f2d(reinterpret_cast<const float*>(L.tb)[e]) : L.tb[e]) * x[k];
+        }
+        if (!a.tb32) L.wsR[(size_t)(q0 + q) * n + c] = b[q];
+      }
+      const int jl = j % WS_ROWS;
+      float4* out = a.wsC + ((size_t)(j / WS_ROWS) * ws_steps(ni, nj) + (i + jl)) * WS_ROWS + jl;
+      reinterpret_cast<float2*>(out)[q0 / 2] = make_float2(d2f(b[0]), d2f(b[1]));
     }
   }
   if (a.want_norm) {
@@ -789,12 +838,14 @@ cudaError_t launch_bc(const LevelDev& L, const PhysParams& ph, cudaStream_t st) 
 
 cudaError_t launch_cell_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st) {
   const int nbi = (L.n + 63) / 64, nbg = (4 * (L.ni + L.nj) + 63) / 64;
-  return launch_pdl(k_cell_aux, nbi + nbg, 64, 0, st, L, ph, cfl, want_dts, 0, nbi);
+  return launch_pdl(k_cell_aux, nbi + nbg, 64, 0, st, L, ph, cfl, want_dts, 0, nbi, WsPending{});
 }
 
-void launch_bc_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st) {
+void launch_bc_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st,
+                   const WsPending* pending) {
   const int nbi = (L.n + 63) / 64, nbg = (4 * (L.ni + L.nj) + 63) / 64;
-  launch_pdl(k_cell_aux, nbi + nbg, 64, 0, st, L, ph, cfl, want_dts, 1, nbi);
+  launch_pdl(k_cell_aux, nbi + nbg, 64, 0, st, L, ph, cfl, want_dts, 1, nbi,
+             pending ? *pending : WsPending{});
 }
 
 void launch_wall_force(const LevelDev& L, const PhysParams& ph, double* fx, double* fy, cudaStream_t st) {

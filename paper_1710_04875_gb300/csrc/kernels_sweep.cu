@@ -85,7 +85,7 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
   const bool hasS = j > 0 || on_cut(L, i);
 #pragma unroll
   for (int e = 0; e < 16; ++e) tb[e * n + c] = Di[e];
-  // FP64: the scale once on D^-1 instead of on every entry of the products (this kernel is bound by
+  // FP64 (MODE 0): the scale once on D^-1 instead of on every entry of the products (this kernel is bound by
   // its FP64 instructions: 1024x256 level 220 -> 189 us with it and the conversions on the integer
   // pipe); FP32 scales the sums
   constexpr bool PRE = sizeof(T) == 8;
@@ -786,10 +786,10 @@ bool hp_fits(int ni, int nj, int nw) {
 }
 
 int launch_sweep(const LevelDev& L, int mixed, int kind, int do_update, int aw, double alpha, const double* rhs,
-                 long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters) {
+                 long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, WsPending* pending) {
   if (is_ws(kind) && L.wsF)
     return launch_ws_sweep(L, mixed, 1, do_update, aw, alpha, rhs, prog, err, limit, st, exact_iters,
-                           kind != SWEEP_WS8);
+                           kind != SWEEP_WS8, pending);
   if (is_ws(kind)) kind = mixed ? SWEEP_AUTO : SWEEP_STRIPS;
   if (is_hp(kind) && mixed && L.hpF) {
     launch_pdl(k_hp_cy, (L.n + 127) / 128, 128, 0, st, L, reinterpret_cast<const float*>(L.tb), rhs);

@@ -228,13 +228,6 @@ int ws_strips(int nj) { return (nj + WS_ROWS - 1) / WS_ROWS; }
 
 namespace {
 
-// Skewed index of cell (i, j) in the backward order (the layout of y as the backward pass reads
-// it and of its result z): strip j / WS_ROWS, step Mp - 1 - i - r, row r.
-__device__ __forceinline__ size_t ws_bpos(int i, int j, int Mp) {
-  const int jl = j & (WS_ROWS - 1);
-  return ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_ROWS + jl;
-}
-
 // Ring bookkeeping: stage ch of a pass that starts at ring count `base` (0 forward, the number of
 // stages backward) is ring use n = base + ch: slot n % NS, phase n / NS.
 template <int NS>
@@ -605,28 +598,26 @@ __device__ __forceinline__ double rhs_row(const LevelDev& L, const T* tb, const 
   return a;
 }
 
+// D^-1 r of a given right-hand side (the stages' own comes from the residual kernel): FP32, skewed, and
+// in FP64 contexts FP64 in R for the defect.
 template <typename T, bool SPLIT>
-__global__ void k_ws_rhs(LevelDev L, const T* tb, const double* rhs, float4* C) {
+__global__ void k_ws_rhs(LevelDev L, const T* tb, const double* rhs, float4* C, double* R) {
   pdl_entry();
   int c, q0, q1;
   if (!ws_thread<SPLIT>(L, c, q0, q1)) return;
   const int ni = L.ni, i = c % ni, j = c / ni;
   const int b = j / WS_ROWS, jl = j % WS_ROWS, Mp = ws_steps(ni, L.nj);
   float* out = reinterpret_cast<float*>(C + ((size_t)b * Mp + (i + jl)) * WS_ROWS + jl);
-  for (int q = q0; q < q1; ++q) out[q] = d2f(rhs_row(L, tb, rhs, c, q));
+  for (int q = q0; q < q1; ++q) {
+    const double a = rhs_row(L, tb, rhs, c, q);
+    out[q] = d2f(a);
+    if (R) R[(size_t)q * L.n + c] = a;
+  }
 }
 
 // ---------------------------------------------------------------- FP64 defect correction
 // t = (I + U~) z0: the vector the backward sweep would have started from to reach z0,
 //   t_c = z0_c - H_E z0_E - H_N z0_N (- G_S z0_mirror on row 0 of the lower wake).
-__device__ __forceinline__ void ws_load64(const float4* z, size_t pos, double x[4]) {
-  const float4 v = z[pos];
-  x[0] = f2d(v.x);
-  x[1] = f2d(v.y);
-  x[2] = f2d(v.z);
-  x[3] = f2d(v.w);
-}
-
 // rows q0 .. q1 - 1 of t (each neighbour's vector is converted once for all of them)
 template <bool SPLIT>
 __global__ void k_ws_defect_t(LevelDev L, const double* tb, const float4* z0, double* t) {
@@ -654,12 +645,10 @@ __global__ void k_ws_defect_t(LevelDev L, const double* tb, const float4* z0, do
 
 // d = D^-1 r - (I + L~) t = D^-1 r - t_c + G_W t_W + G_S t_S (t_S: the mirror on row 0 of the
 // upper wake, none elsewhere on row 0), written as the next forward right-hand side (FP32).
-__device__ __forceinline__ double defect_d_row(const LevelDev& L, const double* tb, const double* rhs,
-                                               const double* t, int c, int q) {
+__device__ __forceinline__ double defect_d_row(const LevelDev& L, const double* tb, const double* R, const double* t,
+                                               int c, int q) {
   const int ni = L.ni, n = L.n, i = c % ni, j = c / ni;
-  double a = -t[(size_t)q * n + c];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) a += tb[(size_t)(4 * q + k) * n + c] * rhs[(size_t)k * n + c];
+  double a = R[(size_t)q * n + c] - t[(size_t)q * n + c];
   auto add = [&](int blk, int cn) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) a += tb[(size_t)(blk * 16 + 4 * q + k) * n + c] * t[(size_t)k * n + cn];
@@ -671,14 +660,14 @@ __device__ __forceinline__ double defect_d_row(const LevelDev& L, const double* 
 }
 
 template <bool SPLIT>
-__global__ void k_ws_defect_d(LevelDev L, const double* tb, const double* rhs, const double* t, float4* C) {
+__global__ void k_ws_defect_d(LevelDev L, const double* tb, const double* R, const double* t, float4* C) {
   pdl_entry();
   int c, q0, q1;
   if (!ws_thread<SPLIT>(L, c, q0, q1)) return;
   const int ni = L.ni, i = c % ni, j = c / ni;
   const int b = j / WS_ROWS, jl = j % WS_ROWS, Mp = ws_steps(ni, L.nj);
   float* out = reinterpret_cast<float*>(C + ((size_t)b * Mp + (i + jl)) * WS_ROWS + jl);
-  for (int q = q0; q < q1; ++q) out[q] = d2f(defect_d_row(L, tb, rhs, t, c, q));
+  for (int q = q0; q < q1; ++q) out[q] = d2f(defect_d_row(L, tb, R, t, c, q));
 }
 
 // z = z0 (+ dz): the stage update u = u0 - alpha z (scaled by dt* for ARK), or z to the level's
@@ -702,7 +691,7 @@ __global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, int 
     const double sc = aw ? alpha : alpha * L.dts[c];
     const size_t g = (size_t)(j + 2) * L.P + (i + 2);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) L.u[q * (size_t)L.Gn + g] = L.u0[q * (size_t)n + c] - sc * z[q];
+    for (int q = 0; q < 4; ++q) L.u[q * (size_t)L.Gn + g] = fma(-sc, z[q], L.u0[q * (size_t)n + c]);
   } else if (mixed) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) L.yz32[q * (size_t)n + c] = d2f(z[q]);
@@ -864,7 +853,8 @@ bool ws_fits(int ni, int nj, int nw) {
 }
 
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,
-                    long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, bool deep) {
+                    long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, bool deep,
+                    WsPending* pending) {
   (void)prog;  // the warp strips exchange their boundary rows in shared memory, not through progress words
   auto sweep = [&](float4* zout) {
     // An edge buffer per pass where two fit (1024x256 pair 171 us; with one, cleared between the
@@ -887,29 +877,33 @@ int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int
   const int g4 = (4 * L.n + 127) / 128;  // one thread per cell and row
   float4* wC = reinterpret_cast<float4*>(L.wsC);
   const double* tb64 = static_cast<const double*>(L.tb);
-  if (mixed) {
-    const float* tb32 = reinterpret_cast<const float*>(L.tb);
-    if (split)
-      launch_pdl(k_ws_rhs<float, true>, g4, 128, 0, st, L, tb32, rhs, wC);
-    else
-      launch_pdl(k_ws_rhs<float, false>, g, 128, 0, st, L, tb32, rhs, wC);
-  } else if (split) {
-    launch_pdl(k_ws_rhs<double, true>, g4, 128, 0, st, L, tb64, rhs, wC);
-  } else {
-    launch_pdl(k_ws_rhs<double, false>, g, 128, 0, st, L, tb64, rhs, wC);
+  double* noR = nullptr;
+  if (rhs) {
+    if (mixed) {
+      const float* tb32 = reinterpret_cast<const float*>(L.tb);
+      if (split)
+        launch_pdl(k_ws_rhs<float, true>, g4, 128, 0, st, L, tb32, rhs, wC, noR);
+      else
+        launch_pdl(k_ws_rhs<float, false>, g, 128, 0, st, L, tb32, rhs, wC, noR);
+    } else if (split) {
+      launch_pdl(k_ws_rhs<double, true>, g4, 128, 0, st, L, tb64, rhs, wC, L.wsR);
+    } else {
+      launch_pdl(k_ws_rhs<double, false>, g, 128, 0, st, L, tb64, rhs, wC, L.wsR);
+    }
+    ++launches;
   }
   sweep(z0);
-  launches += 2;
+  ++launches;
   const bool corr = refine && !mixed;
   if (corr) {
     const float4* z0c = z0;
-    const double* wT = L.wsT;
+    const double *wT = L.wsT, *wR = L.wsR;
     if (split) {
       launch_pdl(k_ws_defect_t<true>, g4, 128, 0, st, L, tb64, z0c, L.wsT);
-      launch_pdl(k_ws_defect_d<true>, g4, 128, 0, st, L, tb64, rhs, wT, wC);
+      launch_pdl(k_ws_defect_d<true>, g4, 128, 0, st, L, tb64, wR, wT, wC);
     } else {
       launch_pdl(k_ws_defect_t<false>, g, 128, 0, st, L, tb64, z0c, L.wsT);
-      launch_pdl(k_ws_defect_d<false>, g, 128, 0, st, L, tb64, rhs, wT, wC);
+      launch_pdl(k_ws_defect_d<false>, g, 128, 0, st, L, tb64, wR, wT, wC);
     }
     sweep(dz);
     launches += 3;
@@ -931,6 +925,10 @@ int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int
     }
     launch_pdl(k_ws_finish_x, g, 128, 0, st, L, static_cast<const double*>(L.wsX), do_update, aw, alpha, mixed);
     return launches + 1;
+  }
+  if (pending) {
+    *pending = WsPending{z0, corr ? dz : nullptr, alpha, aw};
+    return launches;
   }
   launch_pdl(k_ws_finish, g, 128, 0, st, L, static_cast<const float4*>(z0), corr ? static_cast<const float4*>(dz) : nullptr,
              do_update, aw, alpha, mixed);

@@ -41,7 +41,7 @@ __device__ __forceinline__ float low(float x) { return x; }
 // 3 = H_E, 4 = H_N.  Blocks of absent neighbours are zero.  MODE 1 (HP, FP32 only): blocks 1-4
 // go to the hyperplane-major arrays of k_sweep_hp instead: entry h = (i + j) * nj + j holds
 // hpF[32h..] = G_W, G_S and hpB[32h..] = H_E, H_N (row-major 4x4 each); D^-1 stays in tb.
-// MODE 2 (WS): tb as MODE 0, and blocks 1-4 also in FP32 in the skewed layout of the warp-strip
+// MODE 2 (WS; FP64: k_ws_prep64): tb as MODE 0, and blocks 1-4 also in FP32 in the skewed layout of the warp-strip
 // sweep (kernels_sweep_ws.cu): forward rows G_W, G_S at strip j / 8, step i + j % 8, row j % 8
 // (G_S zero on row 0 except the upper wake, whose mirror precedes it), backward rows H_E, H_N at
 // step Mp - 1 - i - j % 8; the lower wake's G_S (the backward coupling to its mirror) to wsCut.
@@ -737,14 +737,88 @@ __global__ void k_hp_finish(LevelDev L, int do_update, int aw, double alpha) {
   }
 }
 
+// k_sgs_prep for the warp strips in FP64, a row of the blocks per thread: warp r of a CTA forms row r of
+// D^-1 of its 32 cells (e_r^T U^-1 L^-1) and row r of the products with it; HALVES 2: warps 0-3 the
+// forward products (west, south), warps 4-7 the backward ones (east, north).  What bounds it is the
+// FP64 issue rate, one warp instruction per 64 clocks per scheduler: a thread per cell runs some 330 of
+// them in a row whatever the size, a row 84, a half row 52 (a quarter more in all: taken while every
+// warp has a scheduler of its own).  64x16 19.6 -> 7.5 us, 128x32 19.6 -> 10.9, 256x64 24.4 -> 16.3.
+constexpr int PREP_SCHEDULERS = 4 * 152;
+
+template <int HALVES>
+__global__ void __launch_bounds__(128 * HALVES) k_ws_prep64(LevelDev L, const double* blk, const double* dlu, double* tb) {
+  pdl_entry();
+  const int c = blockIdx.x * 32 + (threadIdx.x & 31), r = (threadIdx.x >> 5) & 3, half = threadIdx.x >> 7;
+  if (c >= L.n) return;
+  const int ni = L.ni, nj = L.nj, n = L.n, i = c % ni, j = c / ni;
+  auto A = [&](int row, int col) { return dlu[(size_t)(4 * row + col) * n + c]; };
+  // x = e_r^T U^-1 (reciprocal pivots on the diagonal; zero before column r), then L^-1 (unit lower)
+  double x[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    double s = k == r ? 1.0 : 0.0;
+#pragma unroll
+    for (int m = 0; m < k; ++m) s -= x[m] * A(m, k);
+    x[k] = s * A(k, k);
+  }
+#pragma unroll
+  for (int k = 2; k >= 0; --k)
+#pragma unroll
+    for (int m = k + 1; m < 4; ++m) x[k] -= x[m] * A(m, k);
+  if (half == 0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) tb[(size_t)(4 * r + k) * n + c] = x[k];
+  }
+  const double cf = L.coef[c];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) x[k] *= cf;
+  const double *Axp = blk, *Axm = blk + (size_t)16 * L.nfx, *Aep = blk + (size_t)32 * L.nfx, *Aem = Aep + (size_t)16 * L.nfe;
+  const int fw = j * (ni + 1) + i, fs = j * ni + i, jl = j % WS_ROWS, Mp = ws_steps(ni, nj);
+  const bool cut = on_cut(L, i), gs_fwd = j > 0 || (cut && ni - 1 - i < i), cut_lower = j == 0 && cut && ni - 1 - i > i;
+  // row r of sign D^-1 B (B entry-major with stride sb at face f), zero where there is no neighbour
+  auto prod = [&](int slot, const double* B, int sb, int f, bool neg, bool present) {
+    double row[4] = {0.0, 0.0, 0.0, 0.0};
+    if (present) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) row[q] += x[k] * B[(size_t)(4 * k + q) * sb + f];
+      }
+      if (neg) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) row[q] = -row[q];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tb[(size_t)(slot * 16 + 4 * r + q) * n + c] = row[q];
+    return make_float4(d2f(row[0]), d2f(row[1]), d2f(row[2]), d2f(row[3]));
+  };
+  if (HALVES == 1 || half == 0) {
+    float4* wf = reinterpret_cast<float4*>(L.wsF) + ((size_t)(j / WS_ROWS) * Mp + (i + jl)) * WS_F4_STEP + 4 * jl + r;
+    *wf = prod(1, Axp, L.nfx, fw, false, i > 0);
+    const float4 gs = prod(2, Aep, L.nfe, fs, false, j > 0 || cut);
+    wf[WS_F4_STEP / 2] = gs_fwd ? gs : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (cut_lower) *reinterpret_cast<float4*>(L.wsCut + 16 * i + 4 * r) = gs;
+  }
+  if (HALVES == 1 || half == 1) {
+    float4* wb =
+        reinterpret_cast<float4*>(L.wsB) + ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_F4_STEP + 4 * jl + r;
+    *wb = prod(3, Axm, L.nfx, fw + 1, true, i < ni - 1);
+    wb[WS_F4_STEP / 2] = prod(4, Aem, L.nfe, fs + ni, true, j < nj - 1);
+  }
+}
+
 }  // namespace
 
 void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st) {
   if (is_ws(kind) && L.wsF) {
+    const int g = (L.n + 31) / 32;
     if (mixed)
       launch_pdl(k_sgs_prep<float, 2>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, L.dlu32, reinterpret_cast<float*>(L.tb));
+    else if (8 * g <= PREP_SCHEDULERS)
+      launch_pdl(k_ws_prep64<2>, g, 256, 0, st, L, L.blk64, L.dlu64, L.tb);
     else
-      launch_pdl(k_sgs_prep<double, 2>, (L.n + 63) / 64, 64, 0, st, L, L.blk64, L.dlu64, L.tb);
+      launch_pdl(k_ws_prep64<1>, g, 128, 0, st, L, L.blk64, L.dlu64, L.tb);
     return;
   }
   if (mixed && is_hp(kind) && L.hpF)

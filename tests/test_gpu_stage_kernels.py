@@ -1,0 +1,57 @@
+"""The smoothing stage's kernels around the warp-strip sweep against the general path (the one-CTA sweep,
+whose blocks, right-hand side and update are kernels of their own): the stage update that waits for the
+next launch over schemes that read dt* in it (ARK) and that do not (AW), cycle shapes and repeated
+smoothing, and the FP64 block preparation where its split changes (up to 2,432 cells two threads a row)
+and where its last block is partly filled.
+
+Tolerance: in FP64 the two sweeps agree to 1e-14 of the state; a cycle of two levels amplifies that (ARK
+by up to 500, between any two FP64 sweeps): 1e-11."""
+import numpy as np
+import pytest
+
+import paper_1710_04875_gb300 as P
+from helpers import rel_err
+from synth.cgrid import make_cgrid
+
+pytestmark = pytest.mark.gpu
+
+
+def _solver(ni, nj, nw, kind, **kw):
+    s = P.Solver(make_cgrid(ni, nj, n_wake=nw, wall_spacing=1e-3),
+                 P.default_params(mach=0.6, alpha_deg=1.0, precision="fp64", cfl=2.0, **kw))
+    s.set_sweep(kind)  # from the free stream
+    return s
+
+
+@pytest.mark.parametrize("scheme", ["AW3", "ARK51"])
+@pytest.mark.parametrize("nlevels,nu1,gamma", [(1, 1, 1), (1, 3, 1), (2, 1, 2), (2, 2, 1)])
+def test_waiting_update_equals_the_update_kernel(scheme, nlevels, nu1, gamma):
+    u = []
+    for kind in ("warp", "cta"):
+        s = _solver(64, 16, 8, kind, scheme=scheme, nlevels=nlevels, nu1=nu1, gamma_cycle=gamma)
+        s.fas_cycle(0)
+        u.append(s.get_state())
+        s.close()
+    assert rel_err(u[0], u[1]) < 1e-11
+
+
+@pytest.mark.parametrize("scheme", ["AW51", "ARK3J"])
+def test_repeated_smoothing_equals_the_update_kernel(scheme):
+    u = []
+    for kind in ("warp", "cta"):
+        s = _solver(36, 9, 4, kind, scheme=scheme, nlevels=1)
+        s.smooth(3, 2.0)
+        u.append(s.get_state())
+        s.close()
+    assert rel_err(u[0], u[1]) < 1e-11
+
+
+@pytest.mark.parametrize("ni,nj,nw", [(10, 2, 2), (34, 3, 6), (152, 16, 20), (154, 16, 20)])
+def test_block_rows_equal_the_cell_kernel(ni, nj, nw):
+    r = np.random.default_rng(ni).standard_normal((4, nj, ni))
+    z = []
+    for kind in ("warp", "cta"):
+        s = _solver(ni, nj, nw, kind, nlevels=1)
+        z.append(s.precond_apply(r, 20.0))
+        s.close()
+    assert rel_err(z[0], z[1]) < 1e-11

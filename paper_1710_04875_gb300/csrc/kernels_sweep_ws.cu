@@ -247,18 +247,30 @@ struct WsGlobal {
   int nch;                         // stages of a pass
 };
 
-// Fills the slot of ring use n (the copying lane).  The right-hand sides of the first NS backward
-// stages are not fetched: they are the last forward stages' results, still in shared memory.
+// Fills the slot of ring use n (the copying lane): the blocks (ws_fill_blocks, which also announces
+// the bytes of both) and the right-hand sides (ws_fill_rhs).  The right-hand sides of the first NS
+// backward stages are not fetched: they are the last forward stages' results, still in shared memory.
 template <int NS>
-__device__ __forceinline__ void ws_fill(const WsSmem& S, const WsGlobal& G, unsigned n) {
+__device__ __forceinline__ bool ws_fetched(const WsGlobal& G, unsigned n) {
+  return n < (unsigned)G.nch || n - G.nch >= NS;
+}
+
+template <int NS>
+__device__ __forceinline__ void ws_fill_blocks(const WsSmem& S, const WsGlobal& G, unsigned n) {
   constexpr unsigned FB = WS_U * WS_STEP_BYTES, CB = WS_U * WS_VEC_BYTES;
   const unsigned sl = n % NS;
   const bool fwd = n < (unsigned)G.nch;
-  const size_t ch = fwd ? n : n - G.nch;
-  const bool rhs = fwd || ch >= NS;
-  mbar_expect_tx(&S.full[sl], rhs ? FB + CB : FB);
-  bulk_copy(S.F + sl * FB, (fwd ? G.F : G.B) + ch * FB, FB, &S.full[sl]);
-  if (rhs) bulk_copy(S.C + sl * CB, (fwd ? G.C : G.Y) + ch * CB, CB, &S.full[sl]);
+  mbar_expect_tx(&S.full[sl], ws_fetched<NS>(G, n) ? FB + CB : FB);
+  bulk_copy(S.F + sl * FB, (fwd ? G.F : G.B) + (size_t)(fwd ? n : n - G.nch) * FB, FB, &S.full[sl]);
+}
+
+template <int NS>
+__device__ __forceinline__ void ws_fill_rhs(const WsSmem& S, const WsGlobal& G, unsigned n) {
+  constexpr unsigned CB = WS_U * WS_VEC_BYTES;
+  const unsigned sl = n % NS;
+  const bool fwd = n < (unsigned)G.nch;
+  if (ws_fetched<NS>(G, n))
+    bulk_copy(S.C + sl * CB, (fwd ? G.C : G.Y) + (size_t)(fwd ? n : n - G.nch) * CB, CB, &S.full[sl]);
 }
 
 // The helper warps' loops are warp-uniform (a vote decides whether any lane still waits), so that a
@@ -287,7 +299,7 @@ __device__ __forceinline__ bool ws_copies(const WsSmem& S, const WsGlobal& G, un
   const unsigned nch = G.nch, all = 2 * nch, base = FWD ? 0 : nch, end = base + nch;
   if (FWD) {
     if (lane == 0)
-      for (unsigned n = 0; n < NS && n < all; ++n) ws_fill<NS>(S, G, n);
+      for (unsigned n = 0; n < NS && n < all; ++n) ws_fill_rhs<NS>(S, G, n);  // the blocks are on their way
   } else {
     // results of stage nch - 1 - k: right-hand sides of ring use nch + k
     for (int k = min(NS, G.nch) - 1; k >= 0; --k) {
@@ -320,7 +332,8 @@ __device__ __forceinline__ bool ws_copies(const WsSmem& S, const WsGlobal& G, un
         if (n == nch)  // from here on y comes back from global memory: its stores have completed
           asm volatile("cp.async.bulk.wait_group 1;\n\tfence.proxy.async.global;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-        ws_fill<NS>(S, G, n + NS);
+        ws_fill_blocks<NS>(S, G, n + NS);
+        ws_fill_rhs<NS>(S, G, n + NS);
       }
     }
     __syncwarp();
@@ -508,7 +521,11 @@ __global__ void __launch_bounds__(WS_THREADS)
   const bool compute = warp < 2, copier = (warp & ~1) == 2, watcher = (warp & ~1) == 6;
   const bool below = b > 0, above = b < nst - 1;  // neighbour strips
   const WsSmem S = ws_carve<NS, TWO>(ws_raw, w, Mp, nw);
-  // set-up that touches this CTA's shared memory only, before the wait for the kernel before
+  // Set-up while the kernel before still runs: this CTA's shared memory, the cluster's first barrier, and
+  // the first blocks.  The blocks are k_sgs_prep's, which is never the kernel before (the right-hand
+  // side's kernel is), and a kernel lets its successor start only once its own predecessors have
+  // completed (pdl_entry), so they are complete here (a
+  // sweep pair in an FP64 cycle: 64x16 13.2 -> 12.3 us, 128x32 23.4 -> 22.4).
   if (copier && lane == 0) {
     for (int k = 0; k < NS; ++k) {
       mbar_init(&S.full[k], 1);
@@ -517,21 +534,24 @@ __global__ void __launch_bounds__(WS_THREADS)
     *S.gave_up = 0;
     st_release(smem_addr(S.ready), 0);
     st_release(smem_addr(S.primed), 0);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n\tfence.proxy.async.shared::cta;" ::: "memory");
   }
   const int part = (warp >> 1) * 32 + lane;  // of the threads of this strip
   ws_clear(S.Ef, Mp, below, part, WS_THREADS / 2);
   if (TWO) ws_clear(S.Eb, Mp, above, part, WS_THREADS / 2);
-  pdl_entry();
   const size_t blk = (size_t)b * Mp * WS_STEP_BYTES, vec = (size_t)b * Mp * WS_VEC_BYTES;
   const WsGlobal G{reinterpret_cast<const unsigned char*>(Fb) + blk, reinterpret_cast<const unsigned char*>(Bb) + blk,
                    reinterpret_cast<const unsigned char*>(C) + vec,  reinterpret_cast<unsigned char*>(Y) + vec,
                    reinterpret_cast<unsigned char*>(Z) + vec,        Mp / WS_U};
+  if (b < nst && copier && lane == 0) {  // see above: written two launches ago or earlier
+    for (unsigned n = 0; n < NS && n < 2u * G.nch; ++n) ws_fill_blocks<NS>(S, G, n);
+  }
   if (b == 0)
     for (int x = part; x < 16 * nw; x += WS_THREADS / 2) reinterpret_cast<float*>(S.cutG)[x] = cutG[x];
   // every strip's edge buffer holds its sentinels before any neighbour stores into it
   cluster_arrive();
   cluster_wait();
+  pdl_entry();
   bool ok = b < nst;
   const WsSmem other = ws_carve<NS, TWO>(ws_raw, w ^ 1, Mp, nw);
   if (compute) {

@@ -143,26 +143,28 @@ __device__ void ghost_state(const LevelDev& L, const PhysParams& ph, const WsPen
     }
     return;
   }
-  double w[4];
-  if (gj >= nj) {  // outward +S_eta
-    const int i = gi, f = nj * ni + i;
-    const double sx = L.seta[f], sy = L.seta[L.nfe + f];
-    const double il = 1.0 / sqrt(sx * sx + sy * sy);
-    cell_u(L, up, i, nj - 1, w);
-    farfield(w, ph, sx * il, sy * il, L.vfe[f] * il, g);
-  } else if (gi < 0) {  // outward -S_xi
-    const int j = gj, f = j * (ni + 1);
-    const double sx = L.sxi[f], sy = L.sxi[L.nfx + f];
-    const double il = 1.0 / sqrt(sx * sx + sy * sy);
-    cell_u(L, up, 0, j, w);
-    farfield(w, ph, -sx * il, -sy * il, -L.vfx[f] * il, g);
-  } else {  // gi >= ni, outward +S_xi
-    const int j = gj, f = j * (ni + 1) + ni;
-    const double sx = L.sxi[f], sy = L.sxi[L.nfx + f];
-    const double il = 1.0 / sqrt(sx * sx + sy * sy);
-    cell_u(L, up, ni - 1, j, w);
-    farfield(w, ph, sx * il, sy * il, L.vfx[f] * il, g);
+  // Far field: one evaluation for the three sides, so that a warp with ghosts of several sides runs it
+  // once.  Outward is +S_eta at j = nj and +S_xi at i = ni, -S_xi at i = 0.
+  const bool top = gj >= nj, left = !top && gi < 0;
+  const int f = top ? nj * ni + gi : gj * (ni + 1) + (left ? 0 : ni);
+  double sx, sy, vb, w[4];
+  if (top) {
+    sx = L.seta[f];
+    sy = L.seta[L.nfe + f];
+    vb = L.vfe[f];
+  } else {
+    sx = L.sxi[f];
+    sy = L.sxi[L.nfx + f];
+    vb = L.vfx[f];
   }
+  if (left) {
+    sx = -sx;
+    sy = -sy;
+    vb = -vb;
+  }
+  cell_u(L, up, top ? gi : left ? 0 : ni - 1, top ? nj - 1 : gj, w);
+  const double il = 1.0 / sqrt(sx * sx + sy * sy);
+  farfield(w, ph, sx * il, sy * il, vb * il, g);
 }
 
 // Ghost cell t of the two layers around the domain (corners excluded): rows j = -1, -2, rows

@@ -66,6 +66,7 @@ int fasw_batch_create(int ncases, const int* ni, const int* nj, const int* n_wak
       return r;
     }
     c->in_batch = 1;
+    for (auto& L : c->lev) L.shared = ncases > 1;
     c->sweep_kind = SWEEP_WS;  // as a single case: the warp strips in both precisions
     b->cases.push_back(c);
   }

@@ -52,6 +52,7 @@ struct LevelDev {
   int nfe;      // j-faces ni*(nj+1)
   int finest;   // full JST (sensor + fourth differences) on the finest level only
   int res_ty;   // residual tile height (0: chosen from the level size)
+  int shared;   // other cases run beside this one (a batch)
   double a_t;   // time-derivative coefficient (0 = steady)
   double* u;    // 4*Gn ghosted conservative state
   double* u0;   // 4*n  state at the start of the smoothing step

@@ -47,6 +47,12 @@ __host__ __device__ __forceinline__ int ws_steps(int ni, int nj) {
   const int R = nj < WS_ROWS ? nj : WS_ROWS;
   return (ni + R - 1 + WS_U - 1) / WS_U * WS_U;
 }
+// Skewed index of cell (i, j) in the forward order: strip j / WS_ROWS, step i + r, row r.
+__device__ __forceinline__ size_t ws_fpos(int i, int j, int Mp) {
+  const int jl = j & (WS_ROWS - 1);
+  return ((size_t)(j / WS_ROWS) * Mp + (i + jl)) * WS_ROWS + jl;
+}
+
 // Skewed index of cell (i, j) in the backward order (the layout of y as the backward pass reads
 // it and of its result z): strip j / WS_ROWS, step Mp - 1 - i - r, row r.
 __device__ __forceinline__ size_t ws_bpos(int i, int j, int Mp) {

@@ -11,18 +11,25 @@ namespace {
 // Residual tile: TX x TY cells.  Warps 0..TY-1 compute the TX+1 = 32 i-faces of one tile row
 // each, warps TY..2TY compute the TX j-faces of one row of j-faces each (lane 31 idle), so no
 // warp mixes the two kinds of face and a j-face (with the viscous terms) is a thread of its
-// own: on GB300 an SM sub-partition issues one FP64 warp-instruction every few dozen cycles,
-// so the FP64 work of a launch is spread over as many warps and SMs as the grid allows.
-// Tile height 4 where that still gives at least half as many blocks as SMs, else 1: a coarse
-// level then spreads over four times as many SMs for 1.6 times the j-face work (its j-faces are
-// computed by both neighbouring tiles).
+// own: on GB300 an SM sub-partition issues one FP64 warp-instruction every 64 clocks,
+// so the FP64 work of a launch is spread over as many warps and SMs as the grid allows.  The cells'
+// phase takes two components of a cell per thread, on tile height 1 (with a fourth warp) one.
+//
+// Tile height 4 where that still gives a block per SM, else 1: a coarse level then spreads over four
+// times as many SMs for 1.6 times the j-face work (its j-faces are computed by both neighbouring tiles).
+// FP64, height 1 / 2 / 4 / 8: 64x16 5.3 / 7.0 / 10.3 / 17.8 us, 128x32 8.5 / 10.1 / 10.4 / 17.9, 256x64 (144
+// tiles of height 4) 13.9 / 18.2 / 17.5 / 18.1, 330x90 (253) 27.1 / 23.7 / 22.3 / 23.1, 512x128
+// 38.5 / 35.1 / 33.7 / 36.3, 1024x256 189 / 161 / 160 / 181.  Before the cells' phase was split and its
+// operands fetched ahead of the wait for the kernel before: 64x16 8.5, 128x32 10.1.  A case of a batch shares
+// the chip, so the extra work of height 1 counts there: height 4 from 76 tiles (64 cases, mixed: 8.7 ms
+// a cycle against 9.3 with the rule of a case alone).
 constexpr int TX = 31;
-constexpr int res_threads(int ty) { return 32 * (2 * ty + 1); }
-// Tile height: the level's setting (1, 2, 4 or 8, chosen by the batch autotuner or the caller),
-// else 4 rows where that still gives a grid of at least 76 tiles (half the SMs), else 1.
+constexpr int res_threads(int ty) { return ty == 1 ? 128 : 32 * (2 * ty + 1); }
+// Tile height: the level's setting (1, 2, 4 or 8, chosen by the batch autotuner or the caller), else
+// by the rule above.
 inline int res_ty(const LevelDev& L) {
   if (L.res_ty > 0) return L.res_ty;
-  return ((L.ni + TX - 1) / TX) * ((L.nj + 3) / 4) >= 76 ? 4 : 1;
+  return ((L.ni + TX - 1) / TX) * ((L.nj + 3) / 4) >= (L.shared ? 76 : 152) ? 4 : 1;
 }
 
 __device__ __forceinline__ int gidx(const LevelDev& L, int i, int j) { return (j + 2) * L.P + (i + 2); }
@@ -495,19 +502,66 @@ __device__ double block_sum(double v, double* wsum) {
 
 // One tile of TX x TY cells: every face of the tile is computed once into shared memory,
 // then each cell assembles F^c and F^v and writes what the mode asks for.
+// entry e of a cell's transfer blocks
+__device__ __forceinline__ double tb_entry(const LevelDev& L, int tb32, int e, int c) {
+  const size_t at = (size_t)e * L.n + c;
+  return tb32 ? f2d(reinterpret_cast<const float*>(L.tb)[at]) : L.tb[at];
+}
+
+// a cell's part of the squared norm
+__device__ __forceinline__ double norm_of(const double F[4], int all) {
+  double s = F[0] * F[0];
+  if (all) {
+    s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += F[k] * F[k];
+  }
+  return s;
+}
+
 template <int TY, bool FAST>
 __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysParams ph, ResArgs a) {
-  pdl_entry();
   __shared__ double xc[4][TY][TX + 1], xd[4][TY][TX + 1];
   __shared__ double ec[4][TY + 1][TX], ed[4][TY + 1][TX];
-  __shared__ double wsum[2 * TY + 1];
+  __shared__ double wsum[res_threads(TY) / 32];
   __shared__ double si[TY], sj[TY + 2][TX];  // sensors: along i of cell (i0 + TX, j0 + y), along j of rows j0 - 1 ..
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
-  const int ni = L.ni, nj = L.nj;
+  const int ni = L.ni, nj = L.nj, n = L.n;
+  // Before the wait for the kernel before: face vectors, volumes, forcing, history and carried viscous
+  // part.  Each was written two launches ago or earlier (between any of their kernels and a residual lies
+  // at least k_cell_aux), and a kernel lets its successor start only once its own predecessors have
+  // completed (pdl_entry).
+  const bool iface = warp < TY;
+  const int fi = i0 + lane, fj = j0 + (iface ? warp : warp - TY);  // this thread's face
+  const bool face = iface ? fi <= ni && fj < nj : lane < TX && warp <= 2 * TY && fi < ni && fj <= nj;
+  double sx = 0.0, sy = 0.0, fvol = 0.0;
+  if (face) {
+    const int f = iface ? fj * (ni + 1) + fi : fj * ni + fi;
+    sx = iface ? L.sxi[f] : L.seta[f];
+    sy = iface ? L.sxi[L.nfx + f] : L.seta[L.nfe + f];
+    if (ph.moving || ph.flux) fvol = iface ? L.vfx[f] : L.vfe[f];
+  }
+  // this thread's cell: one component of it (tile height 1, four warps) or two (a warp pair per row)
+  constexpr int NK = TY == 1 ? 1 : 2;
+  const int k0 = NK * (warp / TY), cy = warp % TY, c = (j0 + cy) * ni + fi;
+  const bool cell = k0 < 4 && lane < TX && fi < ni && j0 + cy < nj;
+  double rvol = 0.0, src[NK] = {}, frc[NK] = {}, old[NK] = {};
+  auto load_cell = [&] {
+    rvol = L.rvol[c];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      const int e = (k0 + k) * n + c;
+      if (L.finest) src[k] = L.src[e];  // coarse levels have no history source
+      frc[k] = a.mode == RES_FORCING ? L.rhs[e] : L.s[e];
+      if (a.mode == RES_STAGE && a.stage > 1) old[k] = L.fvc[e];
+    }
+  };
+  if (TY == 1 && cell) load_cell();
+  pdl_entry();
   // Each cell's pressure switch is formed once (finest level): an i-face warp's lane takes cell
   // i0 + lane - 1 of its row and passes it on, its last cell is the j-face warps' spare lane's; the
-  // j-face warps take a row each (the last one two).
+  // j-face warps take a row each (the last one two; tile height 1: the spare warp the last).
   double sl = 0.0;
   const bool sensors = L.finest && !ph.flux;
   if (sensors) {
@@ -519,148 +573,125 @@ __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysPa
       if (lane < TX ? i < ni && j <= nj : y < TY && i < ni + 1 && j < nj)
         (lane < TX ? sj[y][lane] : si[y]) =
             cell_sensor<FAST>(L, gidx(L, i, j), lane < TX ? L.P : 1);
-      if (y == TY && lane < TX && i < ni && j0 + TY <= nj) sj[TY + 1][lane] = cell_sensor<FAST>(L, gidx(L, i, j0 + TY), L.P);
+      if (TY > 1 && y == TY && lane < TX && i < ni && j0 + TY <= nj) sj[TY + 1][lane] = cell_sensor<FAST>(L, gidx(L, i, j0 + TY), L.P);
     }
     __syncthreads();
   }
-  if (warp < TY) {  // i-face (i0 + lane, j0 + warp)
+  // tile height 1: this thread's row of D^-1 and dt* are on their way early.  On larger tiles, whose other
+  // blocks hide the latency, the registers are worth more (64 cases, mixed: 9.2 ms a cycle early, 8.8 late).
+  double row[4], dt = 1.0;
+  if (TY == 1 && cell) {
+    if (a.mode == RES_STAGE && a.aw) dt = L.dts[c];
+    if (a.wsC) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) row[k] = tb_entry(L, a.tb32, 4 * k0 + k, c);
+    }
+  }
+  if (iface) {
     const double sdn = __shfl_down_sync(0xffffffffu, sl, 1), sr = lane < TX ? sdn : si[warp];
-    const int tx = lane, ty = warp;
-    const int i = i0 + tx, j = j0 + ty;
-    if (i <= ni && j < nj) {
-      const int f = j * (ni + 1) + i;
+    if (face) {
+      const int i = fi, j = fj;
       double hc[4], hd[4];
       if (ph.flux)
-        fvs_face(L, gidx(L, i - 1, j), gidx(L, i, j), L.sxi[f], L.sxi[L.nfx + f], L.vfx[f], ph.d_cut, hc, hd);
+        fvs_face(L, gidx(L, i - 1, j), gidx(L, i, j), sx, sy, fvol, ph.d_cut, hc, hd);
       else
-        jst_face<FAST>(L, gidx(L, i - 2, j), gidx(L, i - 1, j), gidx(L, i, j), gidx(L, i + 1, j), L.sxi[f],
-                 L.sxi[L.nfx + f], ph.moving ? L.vfx[f] : 0.0, ph.moving, rt_cell(L, i - 1, j, 0), rt_cell(L, i, j, 0),
-                 fmax(sl, sr), ph.s_coarse, hc, hd);
+        jst_face<FAST>(L, gidx(L, i - 2, j), gidx(L, i - 1, j), gidx(L, i, j), gidx(L, i + 1, j), sx, sy, fvol,
+                       ph.moving, rt_cell(L, i - 1, j, 0), rt_cell(L, i, j, 0), fmax(sl, sr), ph.s_coarse, hc, hd);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        xc[k][ty][tx] = hc[k];
-        xd[k][ty][tx] = hd[k];
+        xc[k][warp][lane] = hc[k];
+        xd[k][warp][lane] = hd[k];
       }
     }
-  } else if (lane < TX) {  // j-face (i0 + lane, j0 + warp - TY)
-    const int tx = lane, ty = warp - TY;
-    const int i = i0 + tx, j = j0 + ty;
-    if (i < ni && j <= nj) {
-      const int f = j * ni + i;
-      const double sx = L.seta[f], sy = L.seta[L.nfe + f];
-      double hc[4], hd[4];
-      if (ph.flux)
-        fvs_face(L, gidx(L, i, j - 1), gidx(L, i, j), sx, sy, L.vfe[f], ph.d_cut, hc, hd);
-      else
-        jst_face<FAST>(L, gidx(L, i, j - 2), gidx(L, i, j - 1), gidx(L, i, j), gidx(L, i, j + 1), sx, sy,
-                 ph.moving ? L.vfe[f] : 0.0, ph.moving, rt_cell(L, i, j - 1, 1), rt_cell(L, i, j, 1),
-                 sensors ? fmax(sj[ty][tx], sj[ty + 1][tx]) : 0.0, ph.s_coarse, hc, hd);
-      if (ph.viscous) {
-        double hv[4];
-        visc_face<FAST>(L, ph, i, j, sx, sy, hv);
+  } else if (face) {
+    const int i = fi, j = fj, ty = warp - TY;
+    double hc[4], hd[4];
+    if (ph.flux)
+      fvs_face(L, gidx(L, i, j - 1), gidx(L, i, j), sx, sy, fvol, ph.d_cut, hc, hd);
+    else
+      jst_face<FAST>(L, gidx(L, i, j - 2), gidx(L, i, j - 1), gidx(L, i, j), gidx(L, i, j + 1), sx, sy, fvol,
+                     ph.moving, rt_cell(L, i, j - 1, 1), rt_cell(L, i, j, 1),
+                     sensors ? fmax(sj[ty][lane], sj[ty + 1][lane]) : 0.0, ph.s_coarse, hc, hd);
+    if (ph.viscous) {
+      double hv[4];
+      visc_face<FAST>(L, ph, i, j, sx, sy, hv);
 #pragma unroll
-        for (int k = 1; k < 4; ++k) hd[k] += hv[k];
-      }
+      for (int k = 1; k < 4; ++k) hd[k] += hv[k];
+    }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        ec[k][ty][tx] = hc[k];
-        ed[k][ty][tx] = hd[k];
-      }
+    for (int k = 0; k < 4; ++k) {
+      ec[k][ty][lane] = hc[k];
+      ed[k][ty][lane] = hd[k];
     }
   }
   __syncthreads();
   double nacc = 0.0;
-  double r[4];  // this cell's stage right-hand side
-  bool have = false;
-  if (warp < TY && lane < TX) {  // cell (i0 + lane, j0 + warp)
-    const int tx = lane, ty = warp;
-    const int i = i0 + tx, j = j0 + ty;
-    if (i < ni && j < nj) {
-      const int c = j * ni + i;
-      const int n = L.n;
-      const double rvol = L.rvol[c];
-      const bool timed = !is_zero(L.a_t);
-      const int g = gidx(L, i, j);
-      double Fc[4], Fv[4];
+  double r[NK], F[NK];  // this thread's stage right-hand side and residual
+  if (cell) {
+    if (TY > 1) {
+      load_cell();
+      if (a.mode == RES_STAGE && a.aw) dt = L.dts[c];
+    }
+    const int tx = lane, ty = cy;
+    const bool timed = !is_zero(L.a_t);
+    const int g = gidx(L, fi, j0 + cy);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const double fc = (xc[k][ty][tx + 1] - xc[k][ty][tx]) + (ec[k][ty + 1][tx] - ec[k][ty][tx]);
-        const double fd = (xd[k][ty][tx] - xd[k][ty][tx + 1]) + (ed[k][ty][tx] - ed[k][ty + 1][tx]);
-        double fcv = timed ? fma(fc, rvol, __dmul_rn(L.a_t, L.u[k * L.Gn + g])) : fc * rvol;
-        if (L.finest) fcv += L.src[k * n + c];  // coarse levels have no history source
-        if (a.mode != RES_FORCING) fcv -= L.s[k * n + c];
-        Fc[k] = fcv;
-        Fv[k] = fd * rvol;
-      }
-      if (a.want_norm) {
-        if (a.norm_all) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) nacc += (Fc[k] + Fv[k]) * (Fc[k] + Fv[k]);
-        } else {
-          nacc = (Fc[0] + Fv[0]) * (Fc[0] + Fv[0]);
-        }
-      }
+    for (int q = 0; q < NK; ++q) {
+      const int k = k0 + q, e = k * n + c;
+      const double fc = (xc[k][ty][tx + 1] - xc[k][ty][tx]) + (ec[k][ty + 1][tx] - ec[k][ty][tx]);
+      const double fd = (xd[k][ty][tx] - xd[k][ty][tx + 1]) + (ed[k][ty][tx] - ed[k][ty + 1][tx]);
+      double Fc = timed ? fma(fc, rvol, __dmul_rn(L.a_t, L.u[k * L.Gn + g])) : fc * rvol;
+      if (L.finest) Fc += src[q];
+      if (a.mode != RES_FORCING) Fc -= frc[q];
+      const double Fv = fd * rvol;
+      F[q] = a.want_norm ? Fc + Fv : 0.0;
       if (a.mode == RES_STAGE) {
-        const double sc = a.aw ? L.dts[c] : 1.0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          double carry;
-          if (a.stage == 1) {
-            carry = Fv[k];
-          } else {
-            carry = a.beta * Fv[k] + (1.0 - a.beta) * L.fvc[k * n + c];
-          }
-          L.fvc[k * n + c] = carry;
-          r[k] = sc * (Fc[k] + carry);
-          if (!a.wsC) L.rhs[k * n + c] = r[k];
-        }
-        have = true;
+        const double carry = a.stage == 1 ? Fv : a.beta * Fv + (1.0 - a.beta) * old[q];
+        L.fvc[e] = carry;
+        r[q] = dt * (Fc + carry);
+        if (!a.wsC) L.rhs[e] = r[q];
       } else if (a.mode == RES_FULL) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (a.F) a.F[k * n + c] = Fc[k] + Fv[k];
-          if (a.Fc) a.Fc[k * n + c] = Fc[k];
-          if (a.Fv) a.Fv[k * n + c] = Fv[k];
-        }
+        if (a.F) a.F[e] = Fc + Fv;
+        if (a.Fc) a.Fc[e] = Fc;
+        if (a.Fv) a.Fv[e] = Fv;
       } else if (a.mode == RES_FORCING) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) L.s[k * n + c] = (Fc[k] + Fv[k]) + L.rhs[k * n + c];
+        L.s[e] = (Fc + Fv) + frc[q];
       } else {  // RES_FASRES
-#pragma unroll
-        for (int k = 0; k < 4; ++k) L.rhs[k * n + c] = -(Fc[k] + Fv[k]);
+        L.rhs[e] = -(Fc + Fv);
       }
     }
   }
   // The warp-strip sweep's right-hand side D^-1 r, where r is: a launch less, and D^-1 r of the defect
-  // with it.  The i-face warps take rows 0 and 1, the j-face warps rows 2 and 3 of the products.  Measured
-  // with the update moved to k_cell_aux: 1024x256 W-cycle FP64 11.43 -> 11.20 ms, mixed 7.18 -> 7.03;
-  // 64 cases of 64x16 ... 256x64 in a batch, mixed 10.7 -> 8.8 ms a cycle, FP64 17.9 -> 13.2.
-  if (a.wsC) {
-    __syncwarp();  // the warp has read its row of xc, which holds the right-hand sides now
-    if (have) {
+  // with it.  Measured with the update moved to k_cell_aux: 1024x256 W-cycle FP64 11.43 -> 11.20 ms, mixed
+  // 7.18 -> 7.03; 64 cases of 64x16 ... 256x64 in a batch, mixed 10.7 -> 8.8 ms a cycle, FP64 17.9 -> 13.2.
+  if (a.wsC || a.want_norm) {
+    // each warp has read its components' faces of its row: xc holds the right-hand sides now, xd the residuals
+    __syncwarp();
+    if (cell) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) xc[k][warp][lane] = r[k];
+      for (int q = 0; q < NK; ++q) {
+        xc[k0 + q][cy][lane] = r[q];
+        if (a.want_norm) xd[k0 + q][cy][lane] = F[q];
+      }
     }
     __syncthreads();
-    const int y = warp < TY ? warp : warp - TY, i = i0 + lane, j = j0 + y;
-    if (y < TY && lane < TX && i < ni && j < nj) {
-      const int c = j * ni + i, n = L.n, q0 = warp < TY ? 0 : 2;
-      double x[4], b[2];
+    if (cell && a.want_norm && k0 == 0) {
+      const double f[4] = {xd[0][cy][lane], xd[1][cy][lane], xd[2][cy][lane], xd[3][cy][lane]};
+      nacc = norm_of(f, a.norm_all);
+    }
+    if (cell && a.wsC) {
+      float* out = reinterpret_cast<float*>(a.wsC + ws_fpos(fi, j0 + cy, ws_steps(ni, nj))) + k0;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) x[k] = xc[k][y][lane];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        b[q] = 0.0;
+      for (int q = 0; q < NK; ++q) {
+        double b = 0.0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const size_t e = (size_t)(4 * (q0 + q) + k) * n + c;
-          b[q] += (a.tb32 ? f2d(reinterpret_cast<const float*>(L.tb)[e]) : L.tb[e]) * x[k];
+          const double d = TY == 1 ? row[k] : tb_entry(L, a.tb32, 4 * (k0 + q) + k, c);
+          b += d * xc[k][cy][lane];
         }
-        if (!a.tb32) L.wsR[(size_t)(q0 + q) * n + c] = b[q];
+        if (!a.tb32) L.wsR[(size_t)(k0 + q) * n + c] = b;
+        out[q] = d2f(b);
       }
-      const int jl = j % WS_ROWS;
-      float4* out = a.wsC + ((size_t)(j / WS_ROWS) * ws_steps(ni, nj) + (i + jl)) * WS_ROWS + jl;
-      reinterpret_cast<float2*>(out)[q0 / 2] = make_float2(d2f(b[0]), d2f(b[1]));
     }
   }
   if (a.want_norm) {

@@ -258,19 +258,19 @@ void run_sweep(fasw_ctx* c, const LevelDev& L, int do_update, double alpha, cons
                               c->d_err, c->spin_limit, c->st, c->exact_iters, pending);
 }
 
-void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts) {
+void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts, bool early) {
   Prof p(c, FASW_K_CELL_AUX);
-  launch_bc_aux(c->lev[l], c->ph, cfl, want_dts, c->st, &c->upd[l]);
+  launch_bc_aux(c->lev[l], c->ph, cfl, want_dts, c->st, &c->upd[l], early);
   c->upd[l] = WsPending{};
   ++c->launches;
 }
 
 // One smoothing step on level l: dt* and the preconditioner frozen at u^(0) (reading G19),
 // then the s-stage low-storage loop; AW applies W^-1 to (dt* r), ARK applies dt* P^-1 r.
-void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next) {
+void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next, bool early) {
   LevelDev& L = c->lev[l];
   const SchemeParams& sc = c->sc;
-  bc_aux(c, l, cfl, 1);
+  bc_aux(c, l, cfl, 1, early);
   { Prof p(c, FASW_K_FACE_BLOCKS); launch_face_blocks(L, c->ph, sc, c->mixed, c->st); }
   { Prof p(c, FASW_K_DIAG_BLOCKS); launch_diag_blocks(L, sc, c->mixed, c->st); }  // also saves u^(0)
   c->launches += 2;
@@ -283,7 +283,7 @@ void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next)
   // auxiliaries make the stage update: two launches and two passes over the state fewer a stage.
   const bool ws = c->sweep_kind != SWEEP_LEGACY && is_ws(level_sweep_kind(c, L)) && L.wsF && c->exact_iters == 0;
   for (int i = 1; i <= sc.nstages; ++i) {
-    if (i > 1) bc_aux(c, l, cfl, 0);
+    if (i > 1) bc_aux(c, l, cfl, 0, true);
     ResArgs a{};
     a.mode = RES_STAGE;
     a.stage = i;
@@ -316,17 +316,18 @@ static bool may_wait(const fasw_ctx* c, bool step_next) { return step_next && c-
 void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm, bool again) {
   const int nu1 = c->prm.nu1;
   for (int k = 0; k < nu1; ++k)
-    smooth_step(c, l, cfl, record_norm && k == 0, (k + 1 == nu1 && l > 0) || may_wait(c, again || k + 1 < nu1));
+    smooth_step(c, l, cfl, record_norm && k == 0, (k + 1 == nu1 && l > 0) || may_wait(c, again || k + 1 < nu1),
+                k > 0 || l < c->L());
   if (l == 0) return;
   LevelDev& F = c->lev[l];
   LevelDev& C = c->lev[l - 1];
-  bc_aux(c, l, cfl, 0);
+  bc_aux(c, l, cfl, 0, true);
   ResArgs a{};
   a.mode = RES_FASRES;
   { Prof p(c, FASW_K_RESIDUAL); launch_residual(F, c->ph, a, c->st); }
   { Prof p(c, FASW_K_RESTRICT); launch_restrict(F, C, c->prm.turb, c->ph.fast, c->st); }
   c->launches += 2;
-  bc_aux(c, l - 1, cfl, 0);
+  bc_aux(c, l - 1, cfl, 0, true);
   ResArgs b{};
   b.mode = RES_FORCING;
   { Prof p(c, FASW_K_RESIDUAL); launch_residual(C, c->ph, b, c->st); }
@@ -701,7 +702,7 @@ int fasw_face_blocks(fasw_ctx* c, int l, double* axp, double* axm, double* aep, 
 int fasw_smooth(fasw_ctx* c, int l, int nsteps, double cfl) {
   if (check_level(c, l) || nsteps < 0) return FASW_ERR_ARG;
   err_clear(c);
-  for (int k = 0; k < nsteps; ++k) smooth_step(c, l, cfl, false, may_wait(c, k + 1 < nsteps));
+  for (int k = 0; k < nsteps; ++k) smooth_step(c, l, cfl, false, may_wait(c, k + 1 < nsteps), k > 0);
   int r = sync(c);
   return r ? r : err_read(c);
 }

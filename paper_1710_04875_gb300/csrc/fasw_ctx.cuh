@@ -70,9 +70,10 @@ namespace fasw {
 int level_sweep_kind(const fasw_ctx* c, const LevelDev& L);
 void run_sweep(fasw_ctx* c, const LevelDev& L, int do_update, double alpha, const double* rhs,
                WsPending* pending = nullptr);
-void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts);
+// early: the kernel before is one of the cycle's (none of them writes the metrics)
+void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts, bool early = false);
 // bc_next: the level's next launch is a bc_aux that may make the last stage's update
-void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next);
+void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next, bool early);
 // again: the level is entered again before its state is used otherwise
 void fas_cycle_rec(fasw_ctx* c, int l, double cfl, bool record_norm, bool again = false);
 void enqueue_cycle(fasw_ctx* c, double cfl);

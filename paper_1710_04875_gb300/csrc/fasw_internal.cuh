@@ -171,10 +171,11 @@ struct ResArgs {
 cudaError_t launch_bc(const LevelDev& L, const PhysParams& ph, cudaStream_t st);
 cudaError_t launch_cell_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st);
 // ghost fill and cell auxiliaries in one launch
-// (pending: a stage update still to be made, which this launch makes first)
+// (pending: a stage update still to be made, which this launch makes first; early: the kernel before does
+// not write the metrics)
 struct WsPending;
 void launch_bc_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want_dts, cudaStream_t st,
-                   const WsPending* pending = nullptr);
+                   const WsPending* pending = nullptr, int early = 0);
 cudaError_t launch_residual(const LevelDev& L, const PhysParams& ph, const ResArgs& a, cudaStream_t st);
 int residual_blocks(const LevelDev& L);
 int residual_blocks_max(const LevelDev& L);  // the most tiles any tile height gives (height 1)

@@ -265,6 +265,19 @@ void bc_aux(fasw_ctx* c, int l, double cfl, int want_dts, bool early) {
   ++c->launches;
 }
 
+// The diagonal blocks, u^(0), and what the level's sweep needs of the blocks.
+static void prepare_blocks(fasw_ctx* c, const LevelDev& L) {
+  const int kind = level_sweep_kind(c, L);
+  if (c->sweep_kind == SWEEP_LEGACY || !prep_forms_diag(kind, L, c->mixed)) {
+    launch_diag_blocks(L, c->sc, c->mixed, c->st);
+    ++c->launches;
+  }
+  if (c->sweep_kind != SWEEP_LEGACY) {
+    launch_sgs_prep(L, c->mixed, kind, c->st, c->sc.aw, c->sc.eta);
+    ++c->launches;
+  }
+}
+
 // One smoothing step on level l: dt* and the preconditioner frozen at u^(0) (reading G19),
 // then the s-stage low-storage loop; AW applies W^-1 to (dt* r), ARK applies dt* P^-1 r.
 void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next, bool early) {
@@ -272,16 +285,14 @@ void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next,
   const SchemeParams& sc = c->sc;
   bc_aux(c, l, cfl, 1, early);
   { Prof p(c, FASW_K_FACE_BLOCKS); launch_face_blocks(L, c->ph, sc, c->mixed, c->st); }
-  { Prof p(c, FASW_K_DIAG_BLOCKS); launch_diag_blocks(L, sc, c->mixed, c->st); }  // also saves u^(0)
-  c->launches += 2;
-  if (c->sweep_kind != SWEEP_LEGACY) {
-    Prof p(c, FASW_K_DIAG_BLOCKS);
-    launch_sgs_prep(L, c->mixed, level_sweep_kind(c, L), c->st);
-    ++c->launches;
+  ++c->launches;
+  {
+    Prof p(c, FASW_K_DIAG_BLOCKS);  // also saves u^(0)
+    prepare_blocks(c, L);
   }
   // With the warp strips the residual kernel writes the sweep's right-hand side, and the next cell
   // auxiliaries make the stage update: two launches and two passes over the state fewer a stage.
-  const bool ws = c->sweep_kind != SWEEP_LEGACY && is_ws(level_sweep_kind(c, L)) && L.wsF && c->exact_iters == 0;
+  const bool ws = c->sweep_kind != SWEEP_LEGACY && ws_level(level_sweep_kind(c, L), L) && c->exact_iters == 0;
   for (int i = 1; i <= sc.nstages; ++i) {
     if (i > 1) bc_aux(c, l, cfl, 0, true);
     ResArgs a{};
@@ -657,14 +668,10 @@ int fasw_precond_apply(fasw_ctx* c, int l, double cfl, const double* rin, double
   const size_t m = 4 * (size_t)L.n;
   bc_aux(c, l, cfl, 1);
   launch_face_blocks(L, c->ph, c->sc, c->mixed, c->st);
-  launch_diag_blocks(L, c->sc, c->mixed, c->st);
-  c->launches += 2;
+  ++c->launches;
   int r = copy_in(c, c->d_tmp2, rin, m, on_device);
   if (r) return r;
-  if (c->sweep_kind != SWEEP_LEGACY) {
-    launch_sgs_prep(L, c->mixed, level_sweep_kind(c, L), c->st);
-    ++c->launches;
-  }
+  prepare_blocks(c, L);
   err_clear(c);
   run_sweep(c, L, 0, 0.0, c->d_tmp2);
   const double* zsrc = L.yz64;

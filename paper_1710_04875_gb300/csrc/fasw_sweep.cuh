@@ -22,7 +22,15 @@ inline bool is_ws(int kind) { return kind == SWEEP_WS || kind == SWEEP_WS8; }
 
 // kind: the resolved sweep kind of this level (SWEEP_HP writes the hyperplane-major blocks,
 // SWEEP_WS also the skewed FP32 blocks of the warp strips).
-void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st);
+// the level's sweep is the warp strips'
+inline bool ws_level(int kind, const LevelDev& L) { return is_ws(kind) && L.wsF; }
+// launch_sgs_prep forms the diagonal blocks itself (aw, eta as in launch_diag_blocks, which is left out);
+// the lines are at the kernels
+constexpr int PREP_SPLIT_CELLS = 16384;
+inline bool prep_forms_diag(int kind, const LevelDev& L, int mixed) {
+  return ws_level(kind, L) && (mixed || L.n <= PREP_SPLIT_CELLS);
+}
+void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st, int aw = 0, double eta = 0.0);
 // Forward and backward sweep of one stage: y = (D+L)^-1 rhs, z = (D+U)^-1 D y into L.yz64 /
 // L.yz32, with the stage update u = u0 - alpha z (AW) or u0 - alpha dt* z (ARK) when
 // do_update.  prog: 2 * sweep_strips(L) flags, err: device error word.  Returns the number of

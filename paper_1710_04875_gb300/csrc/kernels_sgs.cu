@@ -12,6 +12,7 @@
 // The sweeps follow the hyperplane order i + j = const; on a hyperplane the cells are
 // independent, and the lower/upper neighbour sets of every cell are those of the
 // lexicographic ordering, so the result equals the lexicographic Gauss-Seidel sweep.
+#include "fasw_blocks.cuh"
 #include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 
@@ -207,67 +208,14 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d, T rd) {
   }
 }
 
-// D_i = sigma I + c_i (A+_e - A-_w + B+_n - B-_s), LU without pivoting (unit L below the
-// diagonal, U on and above with the reciprocal of its diagonal stored on the diagonal).
+// The LU factors of D_i (fasw_blocks.cuh), c_i, and u^(0) of the smoothing step.
 template <typename T>
 __global__ void k_diag_blocks(LevelDev L, const T* blk, T* dlu, int aw, double eta) {
   pdl_entry();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= L.n) return;
-  const int ni = L.ni, i = c % ni, j = c / ni;
-  double coef, sigma;
-  if (aw) {
-    const double ed = eta * L.dts[c];
-    coef = sizeof(T) == 8 ? ed * L.rvol[c] : ed / L.vol[c];
-    sigma = is_zero(L.a_t) ? 1.0 : 1.0 + ed * L.a_t;
-  } else {
-    coef = L.rvol[c];
-    sigma = L.a_t;
-  }
-  L.coef[c] = coef;
-  {  // u^(0) of the smoothing step (the state the blocks are frozen at)
-    const int g = (j + 2) * L.P + (i + 2);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) L.u0[k * L.n + c] = L.u[k * L.Gn + g];
-  }
-  const int fw = j * (ni + 1) + i, fe = fw + 1, fs = j * ni + i, fn = fs + ni;
-  const T* Axp = blk;
-  const T* Axm = blk + 16 * L.nfx;
-  const T* Aep = blk + 32 * L.nfx;
-  const T* Aem = blk + 32 * L.nfx + 16 * L.nfe;
-  T A[16];
-  const T cf = from64<T>(coef), sg = from64<T>(sigma);
-#pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    const T v = (Axp[e * L.nfx + fe] - Axm[e * L.nfx + fw]) + (Aep[e * L.nfe + fn] - Aem[e * L.nfe + fs]);
-    A[e] = ((e % 5 == 0) ? sg : T(0)) + cf * v;
-  }
-  if constexpr (sizeof(T) == 8) {  // each pivot's reciprocal once, for its column's multipliers too
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      A[5 * k] = rcp64(A[5 * k]);
-#pragma unroll
-      for (int r = k + 1; r < 4; ++r) {
-        const double m = A[4 * r + k] * A[5 * k];
-        A[4 * r + k] = m;
-#pragma unroll
-        for (int cc = k + 1; cc < 4; ++cc) A[4 * r + cc] -= m * A[4 * k + cc];
-      }
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-#pragma unroll
-      for (int r = k + 1; r < 4; ++r) {
-        const T m = A[4 * r + k] / A[4 * k + k];
-        A[4 * r + k] = m;
-#pragma unroll
-        for (int cc = k + 1; cc < 4; ++cc) A[4 * r + cc] -= m * A[4 * k + cc];
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) A[5 * k] = T(1) / A[5 * k];
-  }
+  T A[16], cf;
+  cell_lu<T>(L, blk, aw, eta, c, A, cf);
 #pragma unroll
   for (int e = 0; e < 16; ++e) dlu[e * L.n + c] = A[e];
 }

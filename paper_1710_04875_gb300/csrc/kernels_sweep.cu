@@ -24,6 +24,7 @@
 //    chunk at once.  Every wait is bounded; on timeout the kernel raises an error flag and
 //    all strips return.
 #include <atomic>
+#include "fasw_blocks.cuh"
 #include "fasw_fp64.cuh"
 #include "fasw_internal.cuh"
 #include "fasw_sweep.cuh"
@@ -41,20 +42,27 @@ __device__ __forceinline__ float low(float x) { return x; }
 // 3 = H_E, 4 = H_N.  Blocks of absent neighbours are zero.  MODE 1 (HP, FP32 only): blocks 1-4
 // go to the hyperplane-major arrays of k_sweep_hp instead: entry h = (i + j) * nj + j holds
 // hpF[32h..] = G_W, G_S and hpB[32h..] = H_E, H_N (row-major 4x4 each); D^-1 stays in tb.
-// MODE 2 (WS; FP64: k_ws_prep64): tb as MODE 0, and blocks 1-4 also in FP32 in the skewed layout of the warp-strip
+// MODE 2 (WS; FP64 levels up to PREP_SPLIT_CELLS: k_ws_prep64): in FP32 forms D and its LU factors itself (a
+// launch and a pass over them less than with k_diag_blocks before it: 64x16 9.4 -> 7.2 us; in FP64 that
+// gains nothing, 1024x256 243 us against 245, 512x128 90 against 68), tb as MODE 0, and blocks 1-4 also in FP32 in the skewed layout of the warp-strip
 // sweep (kernels_sweep_ws.cu): forward rows G_W, G_S at strip j / 8, step i + j % 8, row j % 8
 // (G_S zero on row 0 except the upper wake, whose mirror precedes it), backward rows H_E, H_N at
 // step Mp - 1 - i - j % 8; the lower wake's G_S (the backward coupling to its mirror) to wsCut.
 template <typename T, int MODE>
-__global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
+__global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb, int aw, double eta) {
   constexpr bool HP = MODE == 1;
   pdl_entry();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= L.n) return;
   const int ni = L.ni, nj = L.nj, n = L.n, i = c % ni, j = c / ni;
-  T A[16];
+  T A[16], cf;
+  if constexpr (MODE == 2 && sizeof(T) == 4) {
+    cell_lu<T>(L, blk, aw, eta, c, A, cf);
+  } else {
+    cf = from64<T>(L.coef[c]);
 #pragma unroll
-  for (int e = 0; e < 16; ++e) A[e] = dlu[e * n + c];
+    for (int e = 0; e < 16; ++e) A[e] = dlu[e * n + c];
+  }
   // D^-1 column by column from the LU factors (unit lower, reciprocal pivots on the diagonal)
   T Di[16];
 #pragma unroll
@@ -75,7 +83,6 @@ __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) Di[4 * r + col] = b[r];
   }
-  const T cf = from64<T>(L.coef[c]);
   const T* Axp = blk;
   const T* Axm = blk + 16 * L.nfx;
   const T* Aep = blk + 32 * L.nfx;
@@ -737,21 +744,66 @@ __global__ void k_hp_finish(LevelDev L, int do_update, int aw, double alpha) {
   }
 }
 
-// k_sgs_prep for the warp strips in FP64, a row of the blocks per thread: warp r of a CTA forms row r of
-// D^-1 of its 32 cells (e_r^T U^-1 L^-1) and row r of the products with it; HALVES 2: warps 0-3 the
-// forward products (west, south), warps 4-7 the backward ones (east, north).  What bounds it is the
-// FP64 issue rate, one warp instruction per 64 clocks per scheduler: a thread per cell runs some 330 of
-// them in a row whatever the size, a row 84, a half row 52 (a quarter more in all: taken while every
-// warp has a scheduler of its own).  64x16 19.6 -> 7.5 us, 128x32 19.6 -> 10.9, 256x64 24.4 -> 16.3.
-constexpr int PREP_SCHEDULERS = 4 * 152;
+// k_diag_blocks and k_sgs_prep for the warp strips in FP64, half a row of the blocks per thread: warps r and
+// r + 4 of a CTA form row r of D of its 32 cells, warp 0 their LU factors, then warps r and r + 4 row r of
+// D^-1 (e_r^T U^-1 L^-1) and row r of the products with it, warp r the forward ones (west, south), warp
+// r + 4 the backward ones (east, north).  What bounds it is the FP64 issue rate, one warp instruction per
+// 64 clocks per scheduler: a thread per cell ran some 100 of them in a row for D and 330 for the products
+// whatever the size.  With D before in a launch of its own (k_diag_blocks) and a thread per cell, and now:
+// 64x16 26 -> 8.0 us, 128x32 28 -> 12.8, 256x64 32 -> 25, 512x128 68 -> 85, 1024x256 245 -> 327 (where every
+// scheduler has warps enough, the redundant factors and barriers cost more): up to PREP_SPLIT_CELLS.
+constexpr int PREP_THREADS = 256;
 
-template <int HALVES>
-__global__ void __launch_bounds__(128 * HALVES) k_ws_prep64(LevelDev L, const double* blk, const double* dlu, double* tb) {
-  pdl_entry();
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31), r = (threadIdx.x >> 5) & 3, half = threadIdx.x >> 7;
-  if (c >= L.n) return;
+__global__ void __launch_bounds__(PREP_THREADS) k_ws_prep64(LevelDev L, const double* blk, double* tb, int aw, double eta) {
+  __shared__ double lu[16][32];
+  const int lane = threadIdx.x & 31, r = (threadIdx.x >> 5) & 3, back = threadIdx.x >> 7;
+  const int c = blockIdx.x * 32 + lane;
   const int ni = L.ni, nj = L.nj, n = L.n, i = c % ni, j = c / ni;
-  auto A = [&](int row, int col) { return dlu[(size_t)(4 * row + col) * n + c]; };
+  const bool has = c < n;
+  // Before the wait for the kernel before, the face blocks': dt*, volumes and the state are k_cell_aux's
+  // or older (a kernel lets its successor start only once its own predecessors have completed).
+  double cf = 0.0, sg = 0.0;
+  if (has) {
+    diag_scales<double>(L, aw, eta, c, cf, sg);
+    if (back == 0) {
+      L.u0[(size_t)r * n + c] = L.u[(size_t)r * L.Gn + (j + 2) * L.P + (i + 2)];
+      if (r == 0) L.coef[c] = cf;
+    }
+  }
+  pdl_entry();
+  const double *Axp = blk, *Axm = blk + (size_t)16 * L.nfx, *Aep = blk + (size_t)32 * L.nfx, *Aem = Aep + (size_t)16 * L.nfe;
+  const int fw = j * (ni + 1) + i, fs = j * ni + i, jl = j % WS_ROWS, Mp = ws_steps(ni, nj);
+  const bool cut = on_cut(L, i);
+  // the neighbours' blocks that this thread multiplies: all on their way before the first barrier
+  const bool first = has && (back ? i < ni - 1 : i > 0), second = has && (back ? j < nj - 1 : j > 0 || cut);
+  const double *B1 = back ? Axm + fw + 1 : Axp + fw, *B2 = back ? Aem + fs + ni : Aep + fs;
+  double b1[16], b2[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    b1[e] = first ? B1[(size_t)e * L.nfx] : 0.0;
+    b2[e] = second ? B2[(size_t)e * L.nfe] : 0.0;
+  }
+  if (has) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int q = k + 2 * back, e = 4 * r + q;
+      const double v = (Axp[(size_t)e * L.nfx + fw + 1] - Axm[(size_t)e * L.nfx + fw]) +
+                       (Aep[(size_t)e * L.nfe + fs + ni] - Aem[(size_t)e * L.nfe + fs]);
+      lu[e][lane] = (q == r ? sg : 0.0) + cf * v;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double A[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) A[e] = lu[e][lane];
+    lu4<double>(A);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) lu[e][lane] = A[e];
+  }
+  __syncthreads();
+  if (!has) return;
+  auto A = [&](int row, int col) { return lu[4 * row + col][lane]; };
   // x = e_r^T U^-1 (reciprocal pivots on the diagonal; zero before column r), then L^-1 (unit lower)
   double x[4];
 #pragma unroll
@@ -765,68 +817,53 @@ __global__ void __launch_bounds__(128 * HALVES) k_ws_prep64(LevelDev L, const do
   for (int k = 2; k >= 0; --k)
 #pragma unroll
     for (int m = k + 1; m < 4; ++m) x[k] -= x[m] * A(m, k);
-  if (half == 0) {
+  if (back == 0) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) tb[(size_t)(4 * r + k) * n + c] = x[k];
   }
-  const double cf = L.coef[c];
+  const double scale = back ? -cf : cf;  // H = -c D^-1 A-
 #pragma unroll
-  for (int k = 0; k < 4; ++k) x[k] *= cf;
-  const double *Axp = blk, *Axm = blk + (size_t)16 * L.nfx, *Aep = blk + (size_t)32 * L.nfx, *Aem = Aep + (size_t)16 * L.nfe;
-  const int fw = j * (ni + 1) + i, fs = j * ni + i, jl = j % WS_ROWS, Mp = ws_steps(ni, nj);
-  const bool cut = on_cut(L, i), gs_fwd = j > 0 || (cut && ni - 1 - i < i), cut_lower = j == 0 && cut && ni - 1 - i > i;
-  // row r of sign D^-1 B (B entry-major with stride sb at face f), zero where there is no neighbour
-  auto prod = [&](int slot, const double* B, int sb, int f, bool neg, bool present) {
+  for (int k = 0; k < 4; ++k) x[k] *= scale;
+  auto prod = [&](int slot, const double b[16]) {
     double row[4] = {0.0, 0.0, 0.0, 0.0};
-    if (present) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) row[q] += x[k] * B[(size_t)(4 * k + q) * sb + f];
-      }
-      if (neg) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) row[q] = -row[q];
-      }
-    }
+      for (int q = 0; q < 4; ++q) row[q] += x[k] * b[4 * k + q];
 #pragma unroll
     for (int q = 0; q < 4; ++q) tb[(size_t)(slot * 16 + 4 * r + q) * n + c] = row[q];
     return make_float4(d2f(row[0]), d2f(row[1]), d2f(row[2]), d2f(row[3]));
   };
-  if (HALVES == 1 || half == 0) {
-    float4* wf = reinterpret_cast<float4*>(L.wsF) + ((size_t)(j / WS_ROWS) * Mp + (i + jl)) * WS_F4_STEP + 4 * jl + r;
-    *wf = prod(1, Axp, L.nfx, fw, false, i > 0);
-    const float4 gs = prod(2, Aep, L.nfe, fs, false, j > 0 || cut);
-    wf[WS_F4_STEP / 2] = gs_fwd ? gs : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (cut_lower) *reinterpret_cast<float4*>(L.wsCut + 16 * i + 4 * r) = gs;
-  }
-  if (HALVES == 1 || half == 1) {
-    float4* wb =
-        reinterpret_cast<float4*>(L.wsB) + ((size_t)(j / WS_ROWS) * Mp + (Mp - 1 - i - jl)) * WS_F4_STEP + 4 * jl + r;
-    *wb = prod(3, Axm, L.nfx, fw + 1, true, i < ni - 1);
-    wb[WS_F4_STEP / 2] = prod(4, Aem, L.nfe, fs + ni, true, j < nj - 1);
-  }
+  const float4 p1 = prod(back ? 3 : 1, b1), p2 = prod(back ? 4 : 2, b2);
+  const size_t strip = (size_t)(j / WS_ROWS) * Mp;
+  float4* w = back ? reinterpret_cast<float4*>(L.wsB) + (strip + (Mp - 1 - i - jl)) * WS_F4_STEP + 4 * jl + r
+                   : reinterpret_cast<float4*>(L.wsF) + (strip + (i + jl)) * WS_F4_STEP + 4 * jl + r;
+  *w = p1;
+  const bool upper = ni - 1 - i < i;  // the side of the cut whose mirror is processed first
+  w[WS_F4_STEP / 2] = back || j > 0 || (cut && upper) ? p2 : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!back && j == 0 && cut && !upper && ni - 1 - i > i) *reinterpret_cast<float4*>(L.wsCut + 16 * i + 4 * r) = p2;
 }
 
 }  // namespace
 
-void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st) {
-  if (is_ws(kind) && L.wsF) {
-    const int g = (L.n + 31) / 32;
+void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st, int aw, double eta) {
+  if (ws_level(kind, L)) {
+    const float* no32 = nullptr;
+    const double* lu64 = L.dlu64;
     if (mixed)
-      launch_pdl(k_sgs_prep<float, 2>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, L.dlu32, reinterpret_cast<float*>(L.tb));
-    else if (8 * g <= PREP_SCHEDULERS)
-      launch_pdl(k_ws_prep64<2>, g, 256, 0, st, L, L.blk64, L.dlu64, L.tb);
+      launch_pdl(k_sgs_prep<float, 2>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, no32, reinterpret_cast<float*>(L.tb), aw, eta);
+    else if (prep_forms_diag(kind, L, mixed))
+      launch_pdl(k_ws_prep64, (L.n + 31) / 32, PREP_THREADS, 0, st, L, L.blk64, L.tb, aw, eta);
     else
-      launch_pdl(k_ws_prep64<1>, g, 128, 0, st, L, L.blk64, L.dlu64, L.tb);
+      launch_pdl(k_sgs_prep<double, 2>, (L.n + 63) / 64, 64, 0, st, L, L.blk64, lu64, L.tb, aw, eta);
     return;
   }
   if (mixed && is_hp(kind) && L.hpF)
-    launch_pdl(k_sgs_prep<float, 1>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, L.dlu32, reinterpret_cast<float*>(L.tb));
+    launch_pdl(k_sgs_prep<float, 1>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, L.dlu32, reinterpret_cast<float*>(L.tb), 0, 0.0);
   else if (mixed)
-    launch_pdl(k_sgs_prep<float, 0>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, L.dlu32, reinterpret_cast<float*>(L.tb));
+    launch_pdl(k_sgs_prep<float, 0>, (L.n + 63) / 64, 64, 0, st, L, L.blk32, L.dlu32, reinterpret_cast<float*>(L.tb), 0, 0.0);
   else
-    launch_pdl(k_sgs_prep<double, 0>, (L.n + 63) / 64, 64, 0, st, L, L.blk64, L.dlu64, L.tb);
+    launch_pdl(k_sgs_prep<double, 0>, (L.n + 63) / 64, 64, 0, st, L, L.blk64, L.dlu64, L.tb, 0, 0.0);
 }
 
 namespace {
@@ -861,7 +898,7 @@ bool hp_fits(int ni, int nj, int nw) {
 
 int launch_sweep(const LevelDev& L, int mixed, int kind, int do_update, int aw, double alpha, const double* rhs,
                  long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, WsPending* pending) {
-  if (is_ws(kind) && L.wsF)
+  if (ws_level(kind, L))
     return launch_ws_sweep(L, mixed, 1, do_update, aw, alpha, rhs, prog, err, limit, st, exact_iters,
                            kind != SWEEP_WS8, pending);
   if (is_ws(kind)) kind = mixed ? SWEEP_AUTO : SWEEP_STRIPS;

@@ -1,8 +1,8 @@
 """The smoothing stage's kernels around the warp-strip sweep against the general path (the one-CTA sweep,
 whose blocks, right-hand side and update are kernels of their own): the stage update that waits for the
 next launch over schemes that read dt* in it (ARK) and that do not (AW), cycle shapes and repeated
-smoothing, and the FP64 block preparation where its split changes (up to 2,432 cells two threads a row)
-and where its last block is partly filled.
+smoothing, and the FP64 block preparation where its last block is partly filled and where it changes
+(up to 16,384 cells it forms the diagonal blocks too).
 
 Tolerance: in FP64 the two sweeps agree to 1e-14 of the state; a cycle of two levels amplifies that (ARK
 by up to 500, between any two FP64 sweeps): 1e-11."""
@@ -46,7 +46,7 @@ def test_repeated_smoothing_equals_the_update_kernel(scheme):
     assert rel_err(u[0], u[1]) < 1e-11
 
 
-@pytest.mark.parametrize("ni,nj,nw", [(10, 2, 2), (34, 3, 6), (152, 16, 20), (154, 16, 20)])
+@pytest.mark.parametrize("ni,nj,nw", [(10, 2, 2), (34, 3, 6), (152, 16, 20), (256, 64, 32), (258, 64, 32)])
 def test_block_rows_equal_the_cell_kernel(ni, nj, nw):
     r = np.random.default_rng(ni).standard_normal((4, nj, ni))
     z = []

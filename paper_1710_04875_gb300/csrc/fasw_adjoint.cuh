@@ -51,6 +51,10 @@ struct AdjointDev {
   double* mgt = nullptr;
   double* mgz = nullptr;   // start vector of a smoothing step
   double* tbt = nullptr;   // 80n transfer blocks of the transposed couplings (D' = I, G'_W, G'_S, H'_E, H'_N)
+  // the same blocks as the warp-strip sweep reads them (FP64 contexts, levels that it fits; null: the strips)
+  float* wsF = nullptr;
+  float* wsB = nullptr;
+  float* wsCut = nullptr;
   // FP32 transposed sweep (contexts in mixed precision): the transposed blocks in FP32, entry-major
   // (80n) and, where the level fits the hyperplane-staged sweep, hyperplane-major
   bool fp32 = false;

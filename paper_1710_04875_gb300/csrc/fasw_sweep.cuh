@@ -101,6 +101,8 @@ __device__ __forceinline__ void ws_updated(const LevelDev& L, const WsPending& p
   for (int q = 0; q < 4; ++q) w[q] = fma(-sc, z[q], L.u0[q * (size_t)L.n + c]);
 }
 
+// L.tb (FP64) into the warp-strip layout: L.wsF, L.wsB, L.wsCut
+void launch_ws_skew(const LevelDev& L, cudaStream_t st);
 bool ws_fits(int ni, int nj, int nw);
 size_t ws_floats(int ni, int nj);
 size_t ws_vec_floats(int ni, int nj);

@@ -203,6 +203,22 @@ __global__ void k_adj_wt_finish(LevelDev L, const double* b, double* z) {
   }
 }
 
+// z = S D^-T b of the warp-strip sweep's b = z0 + dz (skewed), a component per thread.
+__global__ void k_adj_ws_finish(LevelDev L, const float4* z0, const float4* dz, double* z) {
+  pdl_entry();
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
+  if (d >= L.n) return;
+  const int n = L.n;
+  const size_t at = ws_bpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj));
+  double b[4], c[4];
+  ws_load64(z0, at, b);
+  ws_load64(dz, at, c);
+  double s = 0.0;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) s += tbT(L.tb, n, 0, t, q, d) * (b[t] + c[t]);
+  z[q * n + d] = L.coef[d] * L.vol[d] * s;
+}
+
 // FP32 copies of the transposed transfer blocks for the FP32 sweeps: entry-major (all five
 // blocks; D' = I is what k_hp_cy reads) and, with hpF, hyperplane-major G'_W, G'_S | H'_E, H'_N
 // (entry h = (i + j) nj + j, 16 floats per block, row-major).
@@ -357,6 +373,16 @@ int adj_setup(AdjointDev& A, int ni, int nj, int nw, std::vector<void*>& allocs,
         return r;
     }
   }
+  if (!A.fp32 && ws_fits(ni, nj, nw)) {
+    const size_t wf = ws_floats(ni, nj), wc = 16 * (size_t)(nw > 0 ? nw : 1);
+    if ((r = adj_alloc(allocs, &A.wsB, wf)) || (r = adj_alloc(allocs, &A.wsCut, wc)) ||
+        (r = adj_alloc(allocs, &A.wsF, wf)))
+      return r;
+    // positions without a cell, or without a coupling, are never written: they must read as zero
+    cudaMemsetAsync(A.wsF, 0, wf * sizeof(float), st);
+    cudaMemsetAsync(A.wsB, 0, wf * sizeof(float), st);
+    cudaMemsetAsync(A.wsCut, 0, wc * sizeof(float), st);
+  }
   if (cudaMallocHost(&A.h_parts, MAXV * sizeof(double)) != cudaSuccess) return FASW_ERR_OOM;
   cudaMemcpyAsync(A.nbr, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(A.col, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice, st);
@@ -445,7 +471,21 @@ void adj_apply(const AdjointDev& A, const double* v, double* out, int transpose,
 
 namespace {
 
-// z = P^-T r (y: scratch of 4n): both triangular solves in one strip-pipelined FP64 sweep on
+// The FP64 sweep of a level: the warp strips with their defect correction where they fit (the adjoint of
+// 256x64: an application 494 us in the strip-pipelined FP64 sweep and 95 here, 32x8 42 and 21).
+int fp64_sweep(const AdjointDev& A, const LevelDev& L) { return A.wsF && L.wsF ? SWEEP_WS : SWEEP_STRIPS; }
+
+// the level with the transposed couplings in the place of its blocks
+LevelDev transposed(const AdjointDev& A, const LevelDev& L) {
+  LevelDev T = L;
+  T.tb = A.tbt;
+  T.wsF = A.wsF;
+  T.wsB = A.wsB;
+  T.wsCut = A.wsCut;
+  return T;
+}
+
+// z = P^-T r (y: scratch of 4n): both triangular solves in one FP64 sweep on
 // the transposed transfer blocks (into y), then z = S D^-T y.
 void precond(const AdjointDev& A, const double* r, double* y, double* z, cudaStream_t st) {
   LevelDev T = A.Lp;
@@ -460,8 +500,14 @@ void precond(const AdjointDev& A, const double* r, double* y, double* z, cudaStr
     launch_pdl(k_adj_wt_finish32, (A.n + 127) / 128, 128, 0, st, A.Lp, (const float*)A.yz32, z);
     return;
   }
-  T.tb = A.tbt;
+  T = transposed(A, A.Lp);
   T.yz64 = y;
+  if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
+    WsPending b{};  // the sweep's result, left in its own layout
+    launch_sweep(T, 0, SWEEP_WS, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st, 0, &b);
+    launch_pdl(k_adj_ws_finish, (4 * A.n + 127) / 128, 128, 0, st, A.Lp, b.z0, b.dz, z);
+    return;
+  }
   launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st);
   launch_pdl(k_adj_wt_finish, (A.n + 127) / 128, 128, 0, st, A.Lp, (const double*)y, z);
 }
@@ -547,10 +593,18 @@ void adj_build_precond(AdjointDev& A, const LevelDev& L, const PhysParams& ph, c
   aw.aw = 1;
   launch_bc_aux(L, ph, cfl, 1, st);
   launch_face_blocks(L, ph, aw, 0, st);
-  launch_diag_blocks(L, aw, 0, st);
-  launch_sgs_prep(L, 0, SWEEP_STRIPS, st);
+  const int kind = fp64_sweep(A, L);
+  if (!prep_forms_diag(kind, L, 0)) {
+    launch_diag_blocks(L, aw, 0, st);
+    ++launches;
+  }
+  launch_sgs_prep(L, 0, kind, st, aw.aw, aw.eta);
   launch_pdl(k_adj_tb_transpose, (A.n + 127) / 128, 128, 0, st, L, A.tbt);
-  launches += 5;
+  launches += 4;
+  if (ws_level(kind, L)) {
+    launch_ws_skew(transposed(A, L), st);
+    ++launches;
+  }
   if (A.fp32) {
     launch_pdl(k_adj_tb_lower, (A.n + 127) / 128, 128, 0, st, A.ni, A.nj, (const double*)A.tbt, A.tb32, A.hpF, A.hpB);
     ++launches;
@@ -756,7 +810,7 @@ void precond_fwd(const AdjointDev& A, double c, const double* t, double* s, doub
              s);
   LevelDev T = A.Lp;
   T.yz64 = x;
-  launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
+  launch_sweep(T, 0, fp64_sweep(A, A.Lp), 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
   const int m = 4 * A.n;
   lc(m, c, x, 0.0, nullptr, 0.0, nullptr, 0.0, nullptr, x, st);
 }

@@ -779,6 +779,29 @@ __global__ void __launch_bounds__(WD_THREADS) k_ws_defect(LevelDev L, const doub
   }
 }
 
+// Blocks 1-4 of tb in FP32 in the layout of the sweep, as k_sgs_prep writes them (a row per thread).
+__global__ void k_ws_skew(LevelDev L) {
+  pdl_entry();
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, c = x >> 2, r = x & 3;
+  if (c >= L.n) return;
+  const int ni = L.ni, n = L.n, i = c % ni, j = c / ni, Mp = ws_steps(ni, L.nj);
+  auto row = [&](int blk) {
+    const double* b = L.tb + (size_t)(16 * blk + 4 * r) * n + c;
+    return make_float4(d2f(b[0]), d2f(b[n]), d2f(b[2 * (size_t)n]), d2f(b[3 * (size_t)n]));
+  };
+  const int jl = j % WS_ROWS;
+  const size_t strip = (size_t)(j / WS_ROWS) * Mp;
+  float4* f = reinterpret_cast<float4*>(L.wsF) + (strip + i + jl) * WS_F4_STEP + 4 * jl + r;
+  float4* b = reinterpret_cast<float4*>(L.wsB) + (strip + Mp - 1 - i - jl) * WS_F4_STEP + 4 * jl + r;
+  const bool cut = L.nw > 0 && (i < L.nw || i >= ni - L.nw);
+  const float4 s = row(2);
+  f[0] = row(1);
+  f[WS_F4_STEP / 2] = j > 0 || (cut && ni - 1 - i < i) ? s : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (j == 0 && cut && ni - 1 - i > i) reinterpret_cast<float4*>(L.wsCut)[4 * i + r] = s;
+  b[0] = row(3);
+  b[WS_F4_STEP / 2] = row(4);
+}
+
 // z = z0 (+ dz): the stage update u = u0 - alpha z (scaled by dt* for ARK), or z to the level's
 // sweep vector (FP64 contexts: yz64; mixed: yz32).
 __global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, int do_update, int aw, double alpha,
@@ -1043,6 +1066,10 @@ int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int
   launch_pdl(k_ws_finish, g, 128, 0, st, L, static_cast<const float4*>(z0), corr ? static_cast<const float4*>(dz) : nullptr,
              do_update, aw, alpha, mixed);
   return launches + 1;
+}
+
+void launch_ws_skew(const LevelDev& L, cudaStream_t st) {
+  launch_pdl(k_ws_skew, (4 * L.n + 127) / 128, 128, 0, st, L);
 }
 
 size_t ws_floats(int ni, int nj) { return (size_t)ws_strips(nj) * ws_steps(ni, nj) * WS_F4_STEP * 4; }

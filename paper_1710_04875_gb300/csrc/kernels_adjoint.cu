@@ -66,21 +66,42 @@ __global__ void k_adj_get_state(LevelDev L, double* ub) {
   for (int q = 0; q < 4; ++q) ub[q * n + c] = L.u[q * L.Gn + g];
 }
 
-// Column m of the block of the unique colour-k dependency of every cell.
-__global__ void k_adj_extract(int n, const int* nbr, const int* col, int k, int m, const double* Fp,
-                              const double* Fm, const double* ub, double h_rel, double* J) {
+// Column m of the block of the unique colour-k dependency of every cell, in J (from Fp, Fm) and in the
+// dissipative part's Jv (from Gp, Gm; blockIdx.y 1).  What bounds it is the latency of its loads: all
+// slots' neighbours are on their way at once, then all their colours (a slot after the other, and a launch
+// for each of the two: 16 us on every level up to 256x64; now 5.5, 6.6 on 256x64).
+__global__ void k_adj_extract(int n, const int* nbr, const int* col, int k, int m, const double* Fp, const double* Fm,
+                              const double* Gp, const double* Gm, const double* ub, double h_rel, double* J,
+                              double* Jv) {
   pdl_entry();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
-  for (int s = 0; s < ADJ_SLOTS; ++s) {
-    const int d = nbr[c * ADJ_SLOTS + s];
-    if (d < 0 || col[d] != k) continue;
-    const double h2 = 2.0 * h_rel * fmax(1.0, fabs(ub[m * n + d]));
-    double* B = J + ((size_t)c * ADJ_SLOTS + s) * 16;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) B[4 * r + m] = (Fp[r * n + c] - Fm[r * n + c]) / h2;
-    return;
+  if (blockIdx.y) {
+    Fp = Gp;
+    Fm = Gm;
+    J = Jv;
   }
+  double df[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) df[r] = Fp[r * n + c] - Fm[r * n + c];
+  int d[ADJ_SLOTS], at = -1;
+#pragma unroll
+  for (int s = 0; s < ADJ_SLOTS; ++s) d[s] = nbr[c * ADJ_SLOTS + s];
+  bool hit[ADJ_SLOTS];
+#pragma unroll
+  for (int s = 0; s < ADJ_SLOTS; ++s) hit[s] = d[s] >= 0 && col[d[s]] == k;
+  int x = 0;
+#pragma unroll
+  for (int s = ADJ_SLOTS - 1; s >= 0; --s)
+    if (hit[s]) {
+      at = s;
+      x = d[s];
+    }
+  if (at < 0) return;
+  const double h2 = 2.0 * h_rel * fmax(1.0, fabs(ub[m * n + x]));
+  double* B = J + ((size_t)c * ADJ_SLOTS + at) * 16;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) B[4 * r + m] = df[r] / h2;
 }
 
 // Objective gradients: wall face i depends on cells (i, 0) and (i, 1) only.
@@ -99,47 +120,55 @@ __global__ void k_adj_extract_obj(int ni, int n, const int* col, int k, int m, c
   g[4 * (size_t)n + m * n + x] = 2.0 * (dfx * ca + dfy * sa);
 }
 
-// out = J v
+// out = J v, a component per thread (a row of every block: 44 FP64 instructions in a row instead of 176,
+// which bound it on the coarse levels).
 __global__ void k_jac_mv(int n, const int* nbr, const double* J, const double* v, double* out) {
   pdl_entry();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, c = t >> 2, r = t & 3;
   if (c >= n) return;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  int d[ADJ_SLOTS];
+#pragma unroll
+  for (int s = 0; s < ADJ_SLOTS; ++s) d[s] = nbr[c * ADJ_SLOTS + s];
+  double acc = 0.0;
+#pragma unroll
   for (int s = 0; s < ADJ_SLOTS; ++s) {
-    const int d = nbr[c * ADJ_SLOTS + s];
-    if (d < 0) continue;
-    const double* B = J + ((size_t)c * ADJ_SLOTS + s) * 16;
-    double vd[4];
+    if (d[s] < 0) continue;
+    const double* B = J + ((size_t)c * ADJ_SLOTS + s) * 16 + 4 * r;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) vd[m] = v[m * n + d];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) acc[r] += B[4 * r + m] * vd[m];
+    for (int m = 0; m < 4; ++m) acc += B[m] * v[m * n + d[s]];
   }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) out[r * n + c] = acc[r];
+  out[r * n + c] = acc;
 }
 
-// out = J^T v: every cell d gathers the blocks whose column is d.
+// out = J^T v, a component per thread: every cell d gathers the blocks whose column is d (32x8 11.6 us a
+// cell per thread, now 4.0; 256x64 21, now 5.3).
 __global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const double* J, const double* v, double* out) {
   pdl_entry();
-  const int d = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 2, m = t & 3;
   if (d >= n) return;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int e = rev_ptr[d]; e < rev_ptr[d + 1]; ++e) {
-    const int cs = rev[e], c = cs / ADJ_SLOTS;
-    const double* B = J + (size_t)cs * 16;
-    double vc[4];
+  const int end = rev_ptr[d + 1];
+  double acc = 0.0;
+  constexpr int U = 4;  // entries whose loads are in flight together
+  for (int e = rev_ptr[d]; e < end; e += U) {
+    int cs[U];
+    double b[U][4], x[U][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) vc[r] = v[r * n + c];
+    for (int u = 0; u < U; ++u) cs[u] = e + u < end ? rev[e + u] : -1;
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) acc[m] += B[4 * r + m] * vc[r];
+      for (int r = 0; r < 4; ++r) {
+        b[u][r] = cs[u] < 0 ? 0.0 : J[(size_t)cs[u] * 16 + 4 * r + m];
+        x[u][r] = cs[u] < 0 ? 0.0 : v[r * n + cs[u] / ADJ_SLOTS];
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (cs[u] < 0) break;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc += b[u][r] * x[u][r];
+    }
   }
-#pragma unroll
-  for (int m = 0; m < 4; ++m) out[m * n + d] = acc[m];
+  out[m * n + d] = acc;
 }
 
 // Preconditioner of the adjoint system: P = S^-1 W, with W the primal AW preconditioner
@@ -417,10 +446,9 @@ int adj_assemble(AdjointDev& A, const LevelDev& L, const PhysParams& ph, double 
         launch_tangent(L, A.tan, ph, nullptr, A.col, k, m, 2.0 * h_rel, A.Fp, A.Fvp, nullptr,
                        A.finest ? A.fw : nullptr, A.finest ? A.fw + A.ni : nullptr, st);
         launches += A.finest ? 6 : 5;
-        launch_pdl(k_adj_extract, nb, 128, 0, st, n, A.nbr, A.col, k, m, A.Fp, A.Fm, A.ub, h_rel, A.J);
-        launch_pdl(k_adj_extract, nb, 128, 0, st, n, A.nbr, A.col, k, m, (const double*)A.Fvp, (const double*)A.Fvm,
-                   (const double*)A.ub, h_rel, A.Jv);
-        launches += 2;
+        launch_pdl(k_adj_extract, dim3(nb, 2), 128, 0, st, n, A.nbr, A.col, k, m, A.Fp, A.Fm, A.Fvp, A.Fvm, A.ub, h_rel, A.J,
+                   A.Jv);
+        ++launches;
         if (A.finest) {
           launch_pdl(k_adj_extract_obj, nbf, 128, 0, st, A.ni, n, A.col, k, m, A.fw, A.ub, h_rel, sa, ca, A.g);
           ++launches;
@@ -445,10 +473,9 @@ int adj_assemble(AdjointDev& A, const LevelDev& L, const PhysParams& ph, double 
           ++launches;
         }
       }
-      launch_pdl(k_adj_extract, nb, 128, 0, st, n, A.nbr, A.col, k, m, A.Fp, A.Fm, A.ub, h_rel, A.J);
-      launch_pdl(k_adj_extract, nb, 128, 0, st, n, A.nbr, A.col, k, m, (const double*)A.Fvp, (const double*)A.Fvm,
-                 (const double*)A.ub, h_rel, A.Jv);
-      launches += 2;
+      launch_pdl(k_adj_extract, dim3(nb, 2), 128, 0, st, n, A.nbr, A.col, k, m, A.Fp, A.Fm, A.Fvp, A.Fvm, A.ub, h_rel, A.J,
+                   A.Jv);
+      ++launches;
       if (A.finest) {
         launch_pdl(k_adj_extract_obj, nbf, 128, 0, st, A.ni, n, A.col, k, m, A.fw, A.ub, h_rel, sa, ca, A.g);
         ++launches;
@@ -464,9 +491,9 @@ int adj_assemble(AdjointDev& A, const LevelDev& L, const PhysParams& ph, double 
 void adj_apply(const AdjointDev& A, const double* v, double* out, int transpose, cudaStream_t st) {
   const int nb = (A.n + 127) / 128;
   if (transpose)
-    launch_pdl(k_jac_tmv, nb, 128, 0, st, A.n, A.rev_ptr, A.rev, A.J, v, out);
+    launch_pdl(k_jac_tmv, (4 * A.n + 127) / 128, 128, 0, st, A.n, A.rev_ptr, A.rev, A.J, v, out);
   else
-    launch_pdl(k_jac_mv, nb, 128, 0, st, A.n, A.nbr, A.J, v, out);
+    launch_pdl(k_jac_mv, (4 * A.n + 127) / 128, 128, 0, st, A.n, A.nbr, A.J, v, out);
 }
 
 namespace {
@@ -799,9 +826,9 @@ void lc(int m, double a0, const double* x0, double a1, const double* x1, double 
 void jac(const AdjointDev& A, const double* blocks, const double* v, double* out, int transpose, cudaStream_t st) {
   const int nb = (A.n + 127) / 128;
   if (transpose)
-    launch_pdl(k_jac_tmv, nb, 128, 0, st, A.n, A.rev_ptr, A.rev, blocks, v, out);
+    launch_pdl(k_jac_tmv, (4 * A.n + 127) / 128, 128, 0, st, A.n, A.rev_ptr, A.rev, blocks, v, out);
   else
-    launch_pdl(k_jac_mv, nb, 128, 0, st, A.n, A.nbr, blocks, v, out);
+    launch_pdl(k_jac_mv, (4 * A.n + 127) / 128, 128, 0, st, A.n, A.nbr, blocks, v, out);
 }
 
 // x = c P^-1 t (forward: the level's own FP64 blocks; scratch s)

@@ -45,6 +45,7 @@ struct AdjointDev {
   double* kry = nullptr;   // (2 restart + 7) * 4n: Krylov basis V, preconditioned basis Z, work vectors
   int restart = 0;
   bool built = false;      // Jacobian assembled at the current state
+  bool cycled = false;     // the transposed cycle has run outside a capture
   LevelDev Lp{};           // level whose transfer blocks hold the preconditioner
   double* mgs = nullptr;   // smoother work vectors (4n each): residual, preconditioner scratch
   double* mgy = nullptr;   // and output

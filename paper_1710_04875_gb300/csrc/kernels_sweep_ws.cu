@@ -35,9 +35,11 @@
 // written.  Every wait is bounded; on timeout the kernel sets the error word, waits (bounded) for its
 // own copies in flight, and still meets the cluster's barriers, so that no strip waits forever.
 //
-// One sweep pair (launches back to back), against strips of 32 rows with a lane per cell that staged
-// and stored for themselves: 64x16 17.7 -> 13.3 us, 128x32 30.8 -> 24.2, 256x64 62.5 -> 45.3,
-// 1024x256 246 -> 171; about 45 ns a step (about 80 before) and 1.3 us from strip to strip.
+// One sweep pair in a cycle (from the end of the kernel before), against strips of 32 rows with a lane per
+// cell that staged and stored for themselves: 64x16 17.7 -> 12.5 us, 128x32 30.8 -> 22.2, 256x64 62.5 -> 42.5,
+// 512x128 83, 1024x256 246 -> 163; about 43 ns a step (about 80 before) and 1.1 us from strip to strip.
+// A tree instead of the chain of eight FMAs (FP64 contexts could take it) gains 1 %: the step waits for its
+// shared-memory instructions.
 #include <atomic>
 #include <cstdint>
 #include <type_traits>
@@ -375,14 +377,13 @@ __device__ __forceinline__ bool ws_watch(const WsSmem& S, int nch, unsigned base
 // row needs the neighbour's out row of the same column, which the neighbour computed at its step
 // s + 7: edge entry s + 7 (entries Mp ... are zero).  On row 0 of the upper wake the entry is the
 // mirror cell's vector, stored there by this strip's own row 0 when it passed that cell.
-// zero: always 0, unknown to the compiler.
 //
 // A taken branch costs this warp about 35 cycles and each test or vote as much as half a step, so
 // a stage is straight-line code: eight unrolled steps, one wait, asked for two steps ahead, and one
 // loop branch; everything else is the other warps' work.
 template <bool FWD, int NS>
 __device__ __forceinline__ bool ws_pass(const LevelDev& L, const WsSmem& S, int b, int Mp, unsigned base, int* err,
-                                        long long limit, unsigned zero) {
+                                        long long limit) {
   constexpr unsigned FB = WS_U * WS_STEP_BYTES, CB = WS_U * WS_VEC_BYTES;
   const int lane = threadIdx.x & 31, r = lane >> 2, q = lane & 3;
   const int ni = L.ni, nw = L.nw, nch = Mp / WS_U;
@@ -413,9 +414,9 @@ __device__ __forceinline__ bool ws_pass(const LevelDev& L, const WsSmem& S, int 
   float4 A[2], B[2];
   float c[2];
   auto load = [&](int z, unsigned sl, int u) {
+    c[z] = lds1(ca + sl * CB + u * WS_VEC_BYTES);  // first: the sum starts with it
     A[z] = lds4(fa + sl * FB + u * WS_STEP_BYTES);
     B[z] = lds4(fa + sl * FB + u * WS_STEP_BYTES + WS_STEP_BYTES / 2);
-    c[z] = lds1(ca + sl * CB + u * WS_VEC_BYTES);
   };
   float y = 0.f;            // this lane's component at the previous step
   unsigned sl = base % NS;  // ring slot
@@ -434,10 +435,7 @@ __device__ __forceinline__ bool ws_pass(const LevelDev& L, const WsSmem& S, int 
       unsigned landed = 0;
 #pragma unroll
       for (int u = 0; u < WS_U; ++u) {
-        // The address depends (by an AND with zero) on the operands loaded during the last step:
-        // without it they are scheduled right before this store and delay the exchange behind them
-        // (67 -> 80 cycles per step).
-        sts1(x_put | (__float_as_uint(c[u & 1]) & zero), y);
+        sts1(x_put, y);
         __syncwarp();
         const float4 x = lds4(x_own), w = lds4(nb + u * nb_step);
         if (u > 0) sts1(h + (FWD ? WS_U - u : u - 1) * WS_VEC_BYTES, y);  // the previous step's result
@@ -514,7 +512,7 @@ constexpr int WS_THREADS = 256;
 template <int NS, bool TWO>
 __global__ void __launch_bounds__(WS_THREADS)
     k_sweep_ws(LevelDev L, const float4* Fb, const float4* Bb, const float4* C, float4* Y, const float* cutG, float4* Z,
-               int* err, long long limit, unsigned zero) {
+               int* err, long long limit) {
   extern __shared__ __align__(128) unsigned char ws_raw[];
   const int nw = L.nw, Mp = ws_steps(L.ni, L.nj), nst = (L.nj + WS_ROWS - 1) / WS_ROWS;
   const int warp = threadIdx.x >> 5, w = warp & 1, b = 2 * blockIdx.x + w, lane = threadIdx.x & 31;
@@ -555,7 +553,7 @@ __global__ void __launch_bounds__(WS_THREADS)
   bool ok = b < nst;
   const WsSmem other = ws_carve<NS, TWO>(ws_raw, w ^ 1, Mp, nw);
   if (compute) {
-    ok = ok && ws_pass<true, NS>(L, S, b, Mp, 0, err, limit, zero);
+    ok = ok && ws_pass<true, NS>(L, S, b, Mp, 0, err, limit);
   } else if (copier) {
     ok = ok && ws_copies<true, NS>(S, G, above ? cluster_addr(other.Ef, (unsigned)(b + 1) >> 1) : 0u);
   } else if (watcher) {
@@ -570,7 +568,7 @@ __global__ void __launch_bounds__(WS_THREADS)
     cluster_wait();
   }
   if (compute) {
-    if (ok) ws_pass<false, NS>(L, S, b, Mp, G.nch, err, limit, zero);
+    if (ok) ws_pass<false, NS>(L, S, b, Mp, G.nch, err, limit);
   } else if (copier) {
     if (ok) ws_copies<false, NS>(S, G, below ? cluster_addr(other.Eb, (unsigned)(b - 1) >> 1) : 0u);
   } else if (watcher) {
@@ -955,7 +953,7 @@ cudaError_t ws_sweep_launch(const LevelDev& L, float4* zout, int* err, long long
   const cudaLaunchConfig_t cfg = ws_config<NS, TWO>(L, at, st);
   return cudaLaunchKernelEx(&cfg, k_sweep_ws<NS, TWO>, L, reinterpret_cast<const float4*>(L.wsF),
                             reinterpret_cast<const float4*>(L.wsB), reinterpret_cast<const float4*>(L.wsC),
-                            reinterpret_cast<float4*>(L.wsY), static_cast<const float*>(L.wsCut), zout, err, limit, 0u);
+                            reinterpret_cast<float4*>(L.wsY), static_cast<const float*>(L.wsCut), zout, err, limit);
 }
 
 template <int NS, bool TWO>

@@ -83,9 +83,19 @@ int dalloc(fasw_ctx* c, T** p, size_t count) {
 }
 
 // The device error word records a bounded wait that ran out.  Each call that runs sweeps clears
-// it first (on the stream, so a captured cycle clears it too) and reads it at its end, so a
-// timeout is reported by the call in which it happened and later calls start clean.
-void err_clear(fasw_ctx* c) { cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st); }
+// it first and reads it at its end, so a
+// timeout is reported by the call in which it happened and later calls start clean.  A cycle ends with a
+// kernel that reports the word and clears it for the next one; what other calls may have left in it is
+// cleared before the cycle (err_ready), outside its graph.
+void err_clear(fasw_ctx* c) {
+  cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+  c->err_used = true;
+}
+
+void err_ready(fasw_ctx* c, cudaStream_t st) {
+  if (c->err_used) cudaMemsetAsync(c->d_err, 0, sizeof(int), st);
+  c->err_used = false;
+}
 
 int err_read(fasw_ctx* c) {
   CKR(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st));
@@ -307,7 +317,7 @@ void smooth_step(fasw_ctx* c, int l, double cfl, bool record_norm, bool bc_next,
     { Prof p(c, FASW_K_RESIDUAL); launch_residual(L, c->ph, a, c->st); }
     if (a.want_norm) {
       Prof p(c, FASW_K_NORM);
-      launch_norm_final(L, residual_blocks(L), L.n * (c->prm.norm_all ? 4 : 1), c->d_norm, c->st);
+      launch_norm_final(L, residual_blocks(L), L.n * (c->prm.norm_all ? 4 : 1), c->h_norm, c->st);
       ++c->launches;
     }
     {
@@ -377,21 +387,21 @@ int sync(fasw_ctx* c) {
 
 void enqueue_cycle(fasw_ctx* c, double cfl) {
   const int Lf = c->L();
-  err_clear(c);
   if (c->prm.turb && !c->mut_frozen) {
     bc_aux(c, Lf, cfl, 0);
     { Prof p(c, FASW_K_BL); launch_bl(c->lev[Lf], c->ph, c->st); }
     c->launches += 2;
   }
   fas_cycle_rec(c, Lf, cfl, true);
-  cudaMemcpyAsync(c->h_norm, c->d_norm, sizeof(double), cudaMemcpyDeviceToHost, c->st);
-  cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+  launch_report_error(c->d_err, c->h_err, c->st);
+  ++c->launches;
 }
 
 // The launch sequence of a cycle depends only on c*, so each distinct c* is captured once
 // into a CUDA graph and replayed (no per-kernel launch overhead).  Not used while profiling
 // or on the legacy default stream, where capture is not possible.
 int run_cycle(fasw_ctx* c, double cfl) {
+  err_ready(c, c->st);
   if (!c->use_graphs || c->profiling || c->st == nullptr) {
     enqueue_cycle(c, cfl);
     return FASW_OK;
@@ -516,7 +526,7 @@ int fasw_create(int ni, int nj, int n_wake, const double* x, const double* y, in
     }
   }
   int r = FASW_OK;
-  if ((r = dalloc(c, &c->d_norm, 1)) != FASW_OK || (r = dalloc(c, &c->d_tmp, 4 * (size_t)ni * nj)) != FASW_OK ||
+  if ((r = dalloc(c, &c->d_tmp, 4 * (size_t)ni * nj)) != FASW_OK ||
       (r = dalloc(c, &c->d_tmp2, 4 * (size_t)ni * nj)) != FASW_OK ||
       (r = dalloc(c, &c->d_tmp3, 32 * (size_t)(ni + 1) * (nj + 1))) != FASW_OK) {
     fasw_destroy(c);
@@ -639,9 +649,8 @@ int fasw_residual(fasw_ctx* c, int l, double* F, double* Fc, double* Fv, int on_
   launch_residual(L, c->ph, a, c->st);
   ++c->launches;
   if (norm) {
-    launch_norm_final(L, residual_blocks(L), L.n * (c->prm.norm_all ? 4 : 1), c->d_norm, c->st);
+    launch_norm_final(L, residual_blocks(L), L.n * (c->prm.norm_all ? 4 : 1), c->h_norm, c->st);
     ++c->launches;
-    CKR(cudaMemcpyAsync(c->h_norm, c->d_norm, sizeof(double), cudaMemcpyDeviceToHost, c->st));
   }
   if (!on_device) {
     if (F) CKR(cudaMemcpyAsync(F, c->d_tmp, m * sizeof(double), cudaMemcpyDeviceToHost, c->st));

@@ -128,6 +128,7 @@ int fasw_batch_cycle(fasw_batch* b, int cycle_index, double* norms) {
     b->graphs.push_back({phase, exec, after - before});
     b->launches += after - before;
   }
+  for (fasw_ctx* c : b->cases) err_ready(c, b->st);
   CKR(cudaGraphLaunch(exec, b->st));
   CKR(cudaStreamSynchronize(b->st));
   CKR(cudaGetLastError());

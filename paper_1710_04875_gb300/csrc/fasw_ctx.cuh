@@ -30,8 +30,7 @@ struct fasw_ctx {
   std::vector<void*> allocs;
   cudaStream_t st = nullptr;
   int mixed = 0;
-  double* d_norm = nullptr;
-  double* h_norm = nullptr;    // pinned
+  double* h_norm = nullptr;    // pinned; written by the norm's kernel
   double* d_tmp = nullptr;     // 4 * n_finest scratch for host copies
   double* d_tmp2 = nullptr;
   double* d_tmp3 = nullptr;
@@ -55,6 +54,7 @@ struct fasw_ctx {
   long long* d_prog = nullptr;  // strip progress flags
   int* d_err = nullptr;         // device error word (bounded waits)
   int* h_err = nullptr;         // pinned copy
+  bool err_used = true;         // a call other than a cycle has used the word since it was last cleared for one
   double* d_x0 = nullptr;       // reference vertices (the grid at rest)
   double* d_y0 = nullptr;
   double* d_un = nullptr;       // dual-time history of the finest level (4 x n)
@@ -85,5 +85,6 @@ int sync(fasw_ctx* c);
 // device error word of the bounded waits: cleared on the stream at the start of a call that runs
 // sweeps, read (with a stream synchronize) at its end
 void err_clear(fasw_ctx* c);
+void err_ready(fasw_ctx* c, cudaStream_t st);
 int err_read(fasw_ctx* c);
 }  // namespace fasw

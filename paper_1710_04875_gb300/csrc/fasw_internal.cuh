@@ -179,7 +179,10 @@ void launch_bc_aux(const LevelDev& L, const PhysParams& ph, double cfl, int want
 cudaError_t launch_residual(const LevelDev& L, const PhysParams& ph, const ResArgs& a, cudaStream_t st);
 int residual_blocks(const LevelDev& L);
 int residual_blocks_max(const LevelDev& L);  // the most tiles any tile height gives (height 1)
+// out: pinned host memory
 void launch_norm_final(const LevelDev& L, int nparts, int ncomp_cells, double* out, cudaStream_t st);
+// the device error word to pinned host memory, then cleared
+void launch_report_error(int* err, int* host, cudaStream_t st);
 void launch_bl(const LevelDev& L, const PhysParams& ph, cudaStream_t st);
 // the auxiliaries' FP64 powers beside pow()/cbrt(), n values (device pointers)
 void launch_check_math(int n, const double* a, const double* b, double* out, cudaStream_t st);

@@ -787,6 +787,15 @@ __global__ void k_norm_final(const double* part, int nparts, double count, doubl
   if (threadIdx.x == 0) out[0] = sqrt(t / count);
 }
 
+// A cycle's norm and error word go to pinned host memory from kernels (k_norm_final, k_report_error) instead of
+// by a copy each after the last kernel, and the word is cleared here instead of by a fill before the next
+// cycle: 64x16, a residual with its norm 28.7 -> 24.1 us, a cycle 268 -> 265.
+__global__ void k_report_error(int* err, int* host) {
+  pdl_entry();
+  *host = *err;
+  *err = 0;
+}
+
 // ---- Baldwin-Lomax (finest level): vorticity by Green-Gauss, then one thread per i-line.
 __global__ void k_vorticity(LevelDev L) {
   pdl_entry();
@@ -962,6 +971,8 @@ int residual_blocks_max(const LevelDev& L) { return ((L.ni + TX - 1) / TX) * L.n
 void launch_norm_final(const LevelDev& L, int nparts, int ncomp_cells, double* out, cudaStream_t st) {
   launch_pdl(k_norm_final, 1, 256, 0, st, L.norm_part, nparts, (double)ncomp_cells, out);
 }
+
+void launch_report_error(int* err, int* host, cudaStream_t st) { launch_pdl(k_report_error, 1, 1, 0, st, err, host); }
 
 void launch_bl(const LevelDev& L, const PhysParams& ph, cudaStream_t st) {
   launch_pdl(k_vorticity, (L.n + 63) / 64, 64, 0, st, L);

@@ -53,21 +53,21 @@ HBM_FALLBACK_GBS = 6800.0
 #     D^-1 r: D^-1 (16 doubles) and r (4 doubles) read, the FP32 right-hand side written (4 floats)  176 B
 #     each sweep: forward blocks G_W G_S and backward blocks H_E H_N (64 floats), its right-hand
 #       side read, y written and read back, z written (4 x 4 floats)                            2 x 320 B
-#     defect: z read (4 floats), H_E H_N (32 doubles) read, t written (4 doubles); D^-1 G_W G_S
-#       (48 doubles), r and t (8 doubles) read, the defect written (4 floats)                  304 + 464 B
-#     update: z and dz read (8 floats), u^(0) read and u written (8 doubles)                      96 B
-#   mixed (one warp-strip sweep): D^-1 (16 floats) and r read, right-hand side written, the
-#     sweep, z and u^(0) read, u written: 112 + 320 + 80                                            512 B
+#     defect: z read (4 floats), H_E H_N (32 doubles) read, t written (4 doubles); G_W G_S
+#       (32 doubles), D^-1 r and t (8 doubles) read, the defect written (4 floats)             304 + 336 B
+#   mixed: one warp-strip sweep                                                                   320 B
+#   (D^-1 r is formed by the residual, the update made by the next cell auxiliaries)
 #   residual: ghosted u (4), p, q, 1/rho, radii (2), dt*, volume, mu_t, face vectors (4) read,
-#     the stage right-hand side and the F^v carry written and the carry read (12)                 232 B
-BYTES_PER_CELL = {"fp64": {"sgs": 1680.0, "residual": 232.0}, "mixed": {"sgs": 512.0, "residual": 232.0}}
+#     D^-1 (16 doubles; mixed 16 floats) read, D^-1 r written (4 floats; FP64 4 doubles too), the
+#     F^v carry written and read (8): 200 + 128 + 16 + 32, mixed 200 + 64 + 16                376, 280 B
+BYTES_PER_CELL = {"fp64": {"sgs": 1280.0, "residual": 376.0}, "mixed": {"sgs": 320.0, "residual": 280.0}}
 # DRAM traffic per cell of one launch of the dominant kernel, from an ncu capture of a finest-level
 # launch (dram__bytes_read.sum + dram__bytes_write.sum over the cells of that launch); None where
 # no capture of the current kernel exists.
-# FP64: 395.1 MB read + 1.2 MB written by one finest-level application on the 262,144 cells of
-# the 1024x256 grid (rhs, two sweep pairs, the defect kernels, the update), captured by ncu with
+# FP64: 299.4 MB read + 2.4 MB written by one finest-level application on the 262,144 cells of
+# the 1024x256 grid (two sweep pairs, the defect kernels), captured by ncu with
 # dram__bytes_read.sum and dram__bytes_write.sum.
-DRAM_BYTES_PER_CELL = {"fp64": {"sgs": 396.25e6 / 262144}, "mixed": {"sgs": None}}
+DRAM_BYTES_PER_CELL = {"fp64": {"sgs": 301.8e6 / 262144}, "mixed": {"sgs": None}}
 
 
 def level_visits(nlevels, gamma):

@@ -180,7 +180,7 @@ __global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const doubl
 // H_U^T couples d to its west and south cells (their H_E, H_N) and, on the upper wake, to its
 // mirror (its G_S); G_L^T couples d to its east and north cells (their G_W, G_S) and, on the
 // lower wake, to its mirror.  That is the primal sweep's own dependence pattern, so the two
-// triangular solves run in the primal's FP64 strip-pipelined sweep on transfer blocks built for
+// triangular solves run in the primal's sweep (fp64_sweep) on transfer blocks built for
 // the transposed couplings:
 //   D' = I, G'_W(d) = H_E(w)^T, G'_S(d) = H_N(s)^T (on the wake cut: G_S(mirror)^T),
 //   H'_E(d) = G_W(e)^T, H'_N(d) = G_S(n)^T,

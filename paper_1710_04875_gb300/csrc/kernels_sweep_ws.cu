@@ -580,10 +580,9 @@ __global__ void __launch_bounds__(WS_THREADS)
 }
 
 // ---------------------------------------------------------------- operand layout
-// Skewed position of cell (i, j): strip b = j / 32, lane jl = j % 32, forward step s = i + jl,
-// backward step Mp - 1 - i - jl (Mp: the ni + R - 1 steps that hold a cell, R = min(nj, 32), padded to whole chunks).
+// Skewed position of cell (i, j): strip b = j / 8, row jl = j % 8, forward step s = i + jl, backward step
+// Mp - 1 - i - jl (Mp: the steps that hold a cell, padded to whole stages; ws_fpos, ws_bpos).
 
-// Forward right-hand side D^-1 r (FP32), skewed.
 // The FP64 kernels of one application, written per row q of their block products: a thread
 // takes one cell and all four rows (SPLIT false: the loads of a warp coalesce along the cells, for
 // levels whose time is their memory traffic), or one cell and one row (SPLIT true: a quarter of

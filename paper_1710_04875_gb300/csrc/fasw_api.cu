@@ -82,24 +82,27 @@ int dalloc(fasw_ctx* c, T** p, size_t count) {
   return FASW_OK;
 }
 
-// The device error word records a bounded wait that ran out.  Each call that runs sweeps clears
-// it first and reads it at its end, so a
-// timeout is reported by the call in which it happened and later calls start clean.  A cycle ends with a
-// kernel that reports the word and clears it for the next one; what other calls may have left in it is
-// cleared before the cycle (err_ready), outside its graph.
-void err_clear(fasw_ctx* c) {
-  cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-  c->err_used = true;
-}
-
+// The device error word records a bounded wait that ran out.  Each call that runs sweeps starts with the word
+// clear (err_clear) and reads it at its end (err_read; a cycle: the same kernel at the end of its graph), so a
+// timeout is reported by the call in which it happened and later calls start clean.  Reading clears it: a
+// fill is only needed after a call that ended before its read.
 void err_ready(fasw_ctx* c, cudaStream_t st) {
   if (c->err_used) cudaMemsetAsync(c->d_err, 0, sizeof(int), st);
   c->err_used = false;
 }
 
+void err_clear(fasw_ctx* c) {
+  err_ready(c, c->st);
+  c->err_used = true;
+}
+
+// Waits for the call's work; its first error, or the device's.
 int err_read(fasw_ctx* c) {
-  CKR(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st));
-  CKR(cudaStreamSynchronize(c->st));
+  launch_report_error(c->d_err, c->h_err, c->st);
+  ++c->launches;
+  const int r = sync(c);
+  if (r) return r;
+  c->err_used = false;
   return *c->h_err ? FASW_ERR_DEVICE_TIMEOUT : FASW_OK;
 }
 
@@ -377,6 +380,19 @@ int copy_out(fasw_ctx* c, double* dst, const double* src, size_t count, int on_d
   return FASW_OK;
 }
 
+// Whether a kernel may use the caller's device buffer itself, without a copy: aligned, and memory of the
+// current device (a copy takes any).
+bool in_place(const double* p) {
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
+  cudaPointerAttributes a{};
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();  // not this call's error: the copy decides
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 int sync(fasw_ctx* c) {
   CKR(cudaGetLastError());
   CKR(cudaStreamSynchronize(c->st));
@@ -602,9 +618,12 @@ int fasw_level_dims(fasw_ctx* c, int l, int* ni, int* nj, int* nw) {
 int fasw_set_state(fasw_ctx* c, int l, const double* u, int on_device) {
   if (check_level(c, l) || !u) return FASW_ERR_ARG;
   LevelDev& L = c->lev[l];
-  int r = copy_in(c, c->d_tmp, u, 4 * (size_t)L.n, on_device);
-  if (r) return r;
-  launch_pack(L, c->d_tmp, 1, nullptr, c->st);
+  if (!on_device || !in_place(u)) {
+    int r = copy_in(c, c->d_tmp, u, 4 * (size_t)L.n, on_device);
+    if (r) return r;
+    u = c->d_tmp;
+  }
+  launch_pack(L, u, 1, nullptr, c->st);
   launch_bc(L, c->ph, c->st);
   c->launches += 2;
   return sync(c);
@@ -613,10 +632,13 @@ int fasw_set_state(fasw_ctx* c, int l, const double* u, int on_device) {
 int fasw_get_state(fasw_ctx* c, int l, double* u, int on_device) {
   if (check_level(c, l) || !u) return FASW_ERR_ARG;
   LevelDev& L = c->lev[l];
-  launch_pack(L, nullptr, 0, c->d_tmp, c->st);
+  const bool direct = on_device && in_place(u);
+  launch_pack(L, nullptr, 0, direct ? u : c->d_tmp, c->st);
   ++c->launches;
-  int r = copy_out(c, u, c->d_tmp, 4 * (size_t)L.n, on_device);
-  if (r) return r;
+  if (!direct) {
+    int r = copy_out(c, u, c->d_tmp, 4 * (size_t)L.n, on_device);
+    if (r) return r;
+  }
   return sync(c);
 }
 
@@ -675,24 +697,31 @@ int fasw_precond_apply(fasw_ctx* c, int l, double cfl, const double* rin, double
   if (check_level(c, l) || !rin || !z) return FASW_ERR_ARG;
   LevelDev& L = c->lev[l];
   const size_t m = 4 * (size_t)L.n;
+  // The warp strips read the right-hand side before they write the result, so they may use the caller's
+  // buffers, overlapping or not.
+  const bool ws = c->sweep_kind != SWEEP_LEGACY && ws_level(level_sweep_kind(c, L), L) && on_device;
   bc_aux(c, l, cfl, 1);
   launch_face_blocks(L, c->ph, c->sc, c->mixed, c->st);
   ++c->launches;
-  int r = copy_in(c, c->d_tmp2, rin, m, on_device);
-  if (r) return r;
+  int r;
+  if (!ws || !in_place(rin)) {
+    if ((r = copy_in(c, c->d_tmp2, rin, m, on_device))) return r;
+    rin = c->d_tmp2;
+  }
   prepare_blocks(c, L);
   err_clear(c);
-  run_sweep(c, L, 0, 0.0, c->d_tmp2);
-  const double* zsrc = L.yz64;
+  const bool direct = ws && in_place(z);
+  LevelDev T = L;
+  if (direct) T.yz64 = z;
+  run_sweep(c, T, 0, 0.0, rin);
+  const double* zsrc = T.yz64;
   if (c->mixed) {
-    launch_f2d(L.yz32, c->d_tmp, (int)m, c->st);
+    launch_f2d(L.yz32, direct ? z : c->d_tmp, (int)m, c->st);
     ++c->launches;
     zsrc = c->d_tmp;
   }
-  r = copy_out(c, z, zsrc, m, on_device);
-  if (r) return r;
-  r = sync(c);
-  return r ? r : err_read(c);
+  if (!direct && (r = copy_out(c, z, zsrc, m, on_device))) return r;
+  return err_read(c);
 }
 
 int fasw_face_blocks(fasw_ctx* c, int l, double* axp, double* axm, double* aep, double* aem, int on_device) {
@@ -719,8 +748,7 @@ int fasw_smooth(fasw_ctx* c, int l, int nsteps, double cfl) {
   if (check_level(c, l) || nsteps < 0) return FASW_ERR_ARG;
   err_clear(c);
   for (int k = 0; k < nsteps; ++k) smooth_step(c, l, cfl, false, may_wait(c, k + 1 < nsteps), k > 0);
-  int r = sync(c);
-  return r ? r : err_read(c);
+  return err_read(c);
 }
 
 int fasw_fas_cycle(fasw_ctx* c, int cycle_index, double* res_norm) {

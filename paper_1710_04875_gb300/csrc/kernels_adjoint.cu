@@ -140,12 +140,9 @@ __global__ void k_jac_mv(int n, const int* nbr, const double* J, const double* v
   out[r * n + c] = acc;
 }
 
-// out = J^T v, a component per thread: every cell d gathers the blocks whose column is d (32x8 11.6 us a
-// cell per thread, now 4.0; 256x64 21, now 5.3).
-__global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const double* J, const double* v, double* out) {
-  pdl_entry();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 2, m = t & 3;
-  if (d >= n) return;
+// Component m of J^T v at cell d, which gathers the blocks whose column it is.
+__device__ __forceinline__ double jac_t_row(int n, const int* rev_ptr, const int* rev, const double* J, const double* v,
+                                            int d, int m) {
   const int end = rev_ptr[d + 1];
   double acc = 0.0;
   constexpr int U = 4;  // entries whose loads are in flight together
@@ -168,7 +165,26 @@ __global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const doubl
       for (int r = 0; r < 4; ++r) acc += b[u][r] * x[u][r];
     }
   }
-  out[m * n + d] = acc;
+  return acc;
+}
+
+// out = J^T v, a component per thread (32x8 11.6 us a cell per thread, now 4.0; 256x64 21, now 5.3).
+__global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const double* J, const double* v, double* out) {
+  pdl_entry();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 2, m = t & 3;
+  if (d >= n) return;
+  out[m * n + d] = jac_t_row(n, rev_ptr, rev, J, v, d, m);
+}
+
+// J^v^T s - J^T w as the warp-strip sweep's right-hand side (D' = I): skewed FP32, and FP64 for the defect.
+__global__ void k_jac_tmv_rhs(LevelDev L, const int* rev_ptr, const int* rev, const double* J, const double* w,
+                              const double* Jv, const double* s) {
+  pdl_entry();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 2, m = t & 3;
+  if (d >= L.n) return;
+  const double x = jac_t_row(L.n, rev_ptr, rev, Jv, s, d, m) - jac_t_row(L.n, rev_ptr, rev, J, w, d, m);
+  L.wsR[(size_t)m * L.n + d] = x;
+  L.wsC[4 * ws_fpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj)) + m] = d2f(x);
 }
 
 // Preconditioner of the adjoint system: P = S^-1 W, with W the primal AW preconditioner
@@ -232,11 +248,8 @@ __global__ void k_adj_wt_finish(LevelDev L, const double* b, double* z) {
   }
 }
 
-// z = S D^-T b of the warp-strip sweep's b = z0 + dz (skewed), a component per thread.
-__global__ void k_adj_ws_finish(LevelDev L, const float4* z0, const float4* dz, double* z) {
-  pdl_entry();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
-  if (d >= L.n) return;
+// Component q of z = S D^-T b at cell d, b = z0 + dz the warp-strip sweep's result (skewed).
+__device__ __forceinline__ double ws_result_row(const LevelDev& L, const float4* z0, const float4* dz, int d, int q) {
   const int n = L.n;
   const size_t at = ws_bpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj));
   double b[4], c[4];
@@ -245,7 +258,32 @@ __global__ void k_adj_ws_finish(LevelDev L, const float4* z0, const float4* dz, 
   double s = 0.0;
 #pragma unroll
   for (int t = 0; t < 4; ++t) s += tbT(L.tb, n, 0, t, q, d) * (b[t] + c[t]);
-  z[q * n + d] = L.coef[d] * L.vol[d] * s;
+  return L.coef[d] * L.vol[d] * s;
+}
+
+__global__ void k_adj_ws_finish(LevelDev L, const float4* z0, const float4* dz, double* z) {
+  pdl_entry();
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
+  if (d >= L.n) return;
+  z[(size_t)q * L.n + d] = ws_result_row(L, z0, dz, d, q);
+}
+
+// One stage of the transposed smoothing step (smooth_T) after its sweep: w = c S D^-T b, out += w,
+// fbar -= w (the first stage: out = w, fbar = -w), and where a stage follows s = w + beta fbar and
+// fbar *= 1 - beta.
+__global__ void k_adj_ws_stage(LevelDev L, const float4* z0, const float4* dz, double c, int first, int last, double be,
+                               double* w, double* out, double* fb, double* s) {
+  pdl_entry();
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
+  if (d >= L.n) return;
+  const double v = c * ws_result_row(L, z0, dz, d, q);
+  const size_t at = (size_t)q * L.n + d;
+  w[at] = v;
+  out[at] = first ? v : out[at] + v;
+  if (last) return;
+  const double f = first ? -v : fb[at] - v;
+  s[at] = fma(be, f, v);
+  fb[at] = (1.0 - be) * f;
 }
 
 // FP32 copies of the transposed transfer blocks for the FP32 sweeps: entry-major (all five
@@ -866,8 +904,28 @@ void smooth_fwd(AdjointDev& A, const double* b, double* x, cudaStream_t st) {
   }
 }
 
+// smooth_T where the warp strips run the transposed sweep: a stage is the sweep's four launches, one for all
+// vector updates and one for both products, which writes the next sweep's right-hand side (17 launches for
+// a step of three stages instead of 35; 256x64 RANS adjoint 35.9 -> 30.3 ms).
+void smooth_T_ws(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
+  const int m = 4 * A.n, g = (4 * A.n + 127) / 128;
+  double *fb = A.mgw + (size_t)m, *w = A.mgw + 2 * (size_t)m, *s = A.mgw + 3 * (size_t)m;
+  const LevelDev T = transposed(A, A.Lp);
+  for (int i = A.nstages - 1; i >= 0; --i) {
+    const bool first = i == A.nstages - 1;
+    WsPending b{};
+    launch_sweep(T, 0, SWEEP_WS, 0, 1, 0.0, first ? v : nullptr, A.prog, A.err, A.spin_limit, st, 0, &b);
+    launch_pdl(k_adj_ws_stage, g, 128, 0, st, A.Lp, b.z0, b.dz, A.stage_c[i], (int)first, (int)(i == 0), A.stage_b[i], w,
+               out, fb, s);
+    if (i > 0)
+      launch_pdl(k_jac_tmv_rhs, g, 128, 0, st, T, A.rev_ptr, A.rev, (const double*)A.J, (const double*)w,
+                 (const double*)A.Jv, (const double*)s);
+  }
+}
+
 // out = S^T v (reverse of smooth_fwd).  Work: A.mgw vectors 0-4, A.mgy.
 void smooth_T(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
+  if (!A.fp32 && fp64_sweep(A, A.Lp) == SWEEP_WS) return smooth_T_ws(A, v, out, st);
   const int m = 4 * A.n;
   double* xb = A.mgw;
   double* fb = A.mgw + (size_t)m;

@@ -623,9 +623,8 @@ int fasw_set_state(fasw_ctx* c, int l, const double* u, int on_device) {
     if (r) return r;
     u = c->d_tmp;
   }
-  launch_pack(L, u, 1, nullptr, c->st);
-  launch_bc(L, c->ph, c->st);
-  c->launches += 2;
+  launch_pack(L, u, 1, nullptr, c->st);  // no ghost fill: every consumer of the ghosts starts with its own (bc_aux)
+  ++c->launches;
   return sync(c);
 }
 

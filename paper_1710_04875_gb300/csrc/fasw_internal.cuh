@@ -12,11 +12,13 @@ constexpr double GAM = 1.4;
 // Ghosted arrays have two ghost layers on every side: cell (i, j), -2 <= i < ni+2,
 // -2 <= j < nj+2, at (j+2)*P + (i+2) with pitch P = ni + 4.  Interior arrays hold
 // cell (i, j) at j*ni + i.  Vector fields are component-major (4 planes).
-// Programmatic dependent launch.  Every kernel of the library starts with pdl_entry(): it waits
-// until the kernel before it on the stream has completed and its writes are visible, then lets
-// the next kernel be launched, so that launch overlaps this kernel's run instead of following
-// its completion.  launch_pdl() launches with the attribute that allows this overlap; without
-// it griddepcontrol.wait returns at once.
+// Programmatic dependent launch.  Every kernel of the library calls pdl_entry() in every thread before
+// anything that depends on the kernel before it on the stream: it waits until that kernel has completed and
+// its writes are visible, then lets the next kernel be launched, so that launch overlaps this kernel's run
+// instead of following its completion.  Since a kernel lets its successor start only after its own wait,
+// all launches but the last are complete and visible when a kernel starts: what they wrote may be read
+// before pdl_entry() (and memory that the last one does not touch may be written).  launch_pdl() launches with
+// the attribute that allows this overlap; without it griddepcontrol.wait returns at once.
 __device__ __forceinline__ void pdl_entry() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

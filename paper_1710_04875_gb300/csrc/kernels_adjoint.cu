@@ -177,12 +177,16 @@ __global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const doubl
 }
 
 // J^v^T s - J^T w as the warp-strip sweep's right-hand side (D' = I): skewed FP32, and FP64 for the defect.
+// Lanes 4-7 of every eight take the second product (both in one thread: 32x8 6.1 us, now 3.9; 256x64 15.2, now 14.2).
 __global__ void k_jac_tmv_rhs(LevelDev L, const int* rev_ptr, const int* rev, const double* J, const double* w,
                               const double* Jv, const double* s) {
   pdl_entry();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 2, m = t & 3;
-  if (d >= L.n) return;
-  const double x = jac_t_row(L.n, rev_ptr, rev, Jv, s, d, m) - jac_t_row(L.n, rev_ptr, rev, J, w, d, m);
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 3, m = t & 3;
+  const bool second = t & 4;
+  double x = 0.0;
+  if (d < L.n) x = jac_t_row(L.n, rev_ptr, rev, second ? J : Jv, second ? w : s, d, m);
+  x -= __shfl_down_sync(0xffffffffu, x, 4);
+  if (d >= L.n || second) return;
   L.wsR[(size_t)m * L.n + d] = x;
   L.wsC[4 * ws_fpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj)) + m] = d2f(x);
 }
@@ -918,7 +922,7 @@ void smooth_T_ws(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
     launch_pdl(k_adj_ws_stage, g, 128, 0, st, A.Lp, b.z0, b.dz, A.stage_c[i], (int)first, (int)(i == 0), A.stage_b[i], w,
                out, fb, s);
     if (i > 0)
-      launch_pdl(k_jac_tmv_rhs, g, 128, 0, st, T, A.rev_ptr, A.rev, (const double*)A.J, (const double*)w,
+      launch_pdl(k_jac_tmv_rhs, (8 * A.n + 127) / 128, 128, 0, st, T, A.rev_ptr, A.rev, (const double*)A.J, (const double*)w,
                  (const double*)A.Jv, (const double*)s);
   }
 }

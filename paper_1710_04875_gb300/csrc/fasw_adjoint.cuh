@@ -56,6 +56,7 @@ struct AdjointDev {
   float* wsF = nullptr;
   float* wsB = nullptr;
   float* wsCut = nullptr;
+  float* wsZ = nullptr;    // its result and two corrections
   // FP32 transposed sweep (contexts in mixed precision): the transposed blocks in FP32, entry-major
   // (80n) and, where the level fits the hyperplane-staged sweep, hyperplane-major
   bool fp32 = false;

@@ -77,9 +77,10 @@ __device__ __forceinline__ void ws_load64(const float4* z, size_t pos, double x[
 }
 
 // A stage update u = u0 - alpha z (AW) or u0 - alpha dt* z (ARK), z = z0 (+ dz), that the sweep left to
-// the kernel that next reads the state, the cell auxiliaries' (launch_bc_aux).  z0 null: none.
+// the kernel that next reads the state, the cell auxiliaries' (launch_bc_aux).  z0 null: none.  dz2: the
+// second correction (adjoint).
 struct WsPending {
-  const float4 *z0, *dz;
+  const float4 *z0, *dz, *dz2;
   double alpha;
   int aw;
 };
@@ -107,6 +108,7 @@ bool ws_fits(int ni, int nj, int nw);
 size_t ws_floats(int ni, int nj);
 size_t ws_vec_floats(int ni, int nj);
 int ws_strips(int nj);
+// refine: FP64 defect corrections of the FP32 sweep (FP64 levels; L.wsZ holds one vector more than that);
 // exact_iters > 0: that many block Gauss-Seidel corrections toward the exact (D + L + U)^-1;
 // deep: the deeper operand ring (false for SWEEP_WS8)
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,

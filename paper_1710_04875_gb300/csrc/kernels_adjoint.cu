@@ -252,35 +252,36 @@ __global__ void k_adj_wt_finish(LevelDev L, const double* b, double* z) {
   }
 }
 
-// Component q of z = S D^-T b at cell d, b = z0 + dz the warp-strip sweep's result (skewed).
-__device__ __forceinline__ double ws_result_row(const LevelDev& L, const float4* z0, const float4* dz, int d, int q) {
+// Component q of z = S D^-T b at cell d, b = z0 + dz + dz2 the warp-strip sweep's result (skewed).
+__device__ __forceinline__ double ws_result_row(const LevelDev& L, const WsPending& z, int d, int q) {
   const int n = L.n;
   const size_t at = ws_bpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj));
-  double b[4], c[4];
-  ws_load64(z0, at, b);
-  ws_load64(dz, at, c);
+  double b[4], c[4], e[4];
+  ws_load64(z.z0, at, b);
+  ws_load64(z.dz, at, c);
+  ws_load64(z.dz2, at, e);
   double s = 0.0;
 #pragma unroll
-  for (int t = 0; t < 4; ++t) s += tbT(L.tb, n, 0, t, q, d) * (b[t] + c[t]);
+  for (int t = 0; t < 4; ++t) s += tbT(L.tb, n, 0, t, q, d) * ((b[t] + c[t]) + e[t]);
   return L.coef[d] * L.vol[d] * s;
 }
 
-__global__ void k_adj_ws_finish(LevelDev L, const float4* z0, const float4* dz, double* z) {
+__global__ void k_adj_ws_finish(LevelDev L, WsPending b, double* z) {
   pdl_entry();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
   if (d >= L.n) return;
-  z[(size_t)q * L.n + d] = ws_result_row(L, z0, dz, d, q);
+  z[(size_t)q * L.n + d] = ws_result_row(L, b, d, q);
 }
 
 // One stage of the transposed smoothing step (smooth_T) after its sweep: w = c S D^-T b, out += w,
 // fbar -= w (the first stage: out = w, fbar = -w), and where a stage follows s = w + beta fbar and
 // fbar *= 1 - beta.
-__global__ void k_adj_ws_stage(LevelDev L, const float4* z0, const float4* dz, double c, int first, int last, double be,
-                               double* w, double* out, double* fb, double* s) {
+__global__ void k_adj_ws_stage(LevelDev L, WsPending b, double c, int first, int last, double be, double* w, double* out,
+                               double* fb, double* s) {
   pdl_entry();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
   if (d >= L.n) return;
-  const double v = c * ws_result_row(L, z0, dz, d, q);
+  const double v = c * ws_result_row(L, b, d, q);
   const size_t at = (size_t)q * L.n + d;
   w[at] = v;
   out[at] = first ? v : out[at] + v;
@@ -447,7 +448,7 @@ int adj_setup(AdjointDev& A, int ni, int nj, int nw, std::vector<void*>& allocs,
   if (!A.fp32 && ws_fits(ni, nj, nw)) {
     const size_t wf = ws_floats(ni, nj), wc = 16 * (size_t)(nw > 0 ? nw : 1);
     if ((r = adj_alloc(allocs, &A.wsB, wf)) || (r = adj_alloc(allocs, &A.wsCut, wc)) ||
-        (r = adj_alloc(allocs, &A.wsF, wf)))
+        (r = adj_alloc(allocs, &A.wsZ, 3 * ws_vec_floats(ni, nj))) || (r = adj_alloc(allocs, &A.wsF, wf)))
       return r;
     // positions without a cell, or without a coupling, are never written: they must read as zero
     cudaMemsetAsync(A.wsF, 0, wf * sizeof(float), st);
@@ -540,9 +541,14 @@ void adj_apply(const AdjointDev& A, const double* v, double* out, int transpose,
 
 namespace {
 
-// The FP64 sweep of a level: the warp strips with their defect correction where they fit (the adjoint of
-// 256x64: an application 494 us in the strip-pipelined FP64 sweep and 95 here, 32x8 42 and 21).
+// The FP64 sweep of a level: the warp strips with their defect corrections where they fit (the adjoint case of
+// 256x64 90 ms with the strip-pipelined FP64 sweep, 38 with the warp strips).
 int fp64_sweep(const AdjointDev& A, const LevelDev& L) { return A.wsF && L.wsF ? SWEEP_WS : SWEEP_STRIPS; }
+
+// FP64 corrections of the warp strips' FP32 result.  With two its error is that of the FP64 strips (P^-T r
+// against 80-bit arithmetic, rms relative, strips / one / two corrections: 64x16 Euler 4.3e-16 / 1.4e-14 /
+// 3.7e-16, 150x43 laminar 3.8e-16 / 1.5e-14 / 3.7e-16, 256x64 RANS 3.8e-16 / 1.5e-14 / 4.2e-16).
+constexpr int ADJ_REFINE = 2;
 
 // the level with the transposed couplings in the place of its blocks
 LevelDev transposed(const AdjointDev& A, const LevelDev& L) {
@@ -551,6 +557,7 @@ LevelDev transposed(const AdjointDev& A, const LevelDev& L) {
   T.wsF = A.wsF;
   T.wsB = A.wsB;
   T.wsCut = A.wsCut;
+  T.wsZ = A.wsZ;
   return T;
 }
 
@@ -573,8 +580,8 @@ void precond(const AdjointDev& A, const double* r, double* y, double* z, cudaStr
   T.yz64 = y;
   if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
     WsPending b{};  // the sweep's result, left in its own layout
-    launch_sweep(T, 0, SWEEP_WS, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st, 0, &b);
-    launch_pdl(k_adj_ws_finish, (4 * A.n + 127) / 128, 128, 0, st, A.Lp, b.z0, b.dz, z);
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st, 0, true, &b);
+    launch_pdl(k_adj_ws_finish, (4 * A.n + 127) / 128, 128, 0, st, A.Lp, b, z);
     return;
   }
   launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st);
@@ -879,7 +886,12 @@ void precond_fwd(const AdjointDev& A, double c, const double* t, double* s, doub
              s);
   LevelDev T = A.Lp;
   T.yz64 = x;
-  launch_sweep(T, 0, fp64_sweep(A, A.Lp), 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
+  if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
+    T.wsZ = A.wsZ;
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
+  } else {
+    launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
+  }
   const int m = 4 * A.n;
   lc(m, c, x, 0.0, nullptr, 0.0, nullptr, 0.0, nullptr, x, st);
 }
@@ -918,8 +930,8 @@ void smooth_T_ws(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
   for (int i = A.nstages - 1; i >= 0; --i) {
     const bool first = i == A.nstages - 1;
     WsPending b{};
-    launch_sweep(T, 0, SWEEP_WS, 0, 1, 0.0, first ? v : nullptr, A.prog, A.err, A.spin_limit, st, 0, &b);
-    launch_pdl(k_adj_ws_stage, g, 128, 0, st, A.Lp, b.z0, b.dz, A.stage_c[i], (int)first, (int)(i == 0), A.stage_b[i], w,
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, first ? v : nullptr, A.prog, A.err, A.spin_limit, st, 0, true, &b);
+    launch_pdl(k_adj_ws_stage, g, 128, 0, st, A.Lp, b, A.stage_c[i], (int)first, (int)(i == 0), A.stage_b[i], w,
                out, fb, s);
     if (i > 0)
       launch_pdl(k_jac_tmv_rhs, (8 * A.n + 127) / 128, 128, 0, st, T, A.rev_ptr, A.rev, (const double*)A.J, (const double*)w,

@@ -633,19 +633,32 @@ __global__ void k_ws_rhs(LevelDev L, const T* tb, const double* rhs, float4* C, 
 }
 
 // ---------------------------------------------------------------- FP64 defect correction
-// t = (I + U~) z0: the vector the backward sweep would have started from to reach z0,
-//   t_c = z0_c - H_E z0_E - H_N z0_N (- G_S z0_mirror on row 0 of the lower wake).
+// t = (I + U~) z: the vector the backward sweep would have started from to reach z,
+//   t_c = z_c - H_E z_E - H_N z_N (- G_S z_mirror on row 0 of the lower wake),
+// z = z0 (+ dz: SECOND, the second correction's).
 // One thread per cell, t and d in a launch each (grids above WS_SPLIT_CELLS).
-__global__ void k_ws_defect_t(LevelDev L, const double* tb, const float4* z0, double* t) {
+template <bool SECOND>
+__device__ __forceinline__ void load_z(const float4* z0, const float4* dz, size_t pos, double x[4]) {
+  ws_load64(z0, pos, x);
+  if constexpr (SECOND) {
+    double d[4];
+    ws_load64(dz, pos, d);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] += d[q];
+  }
+}
+
+template <bool SECOND>
+__global__ void k_ws_defect_t(LevelDev L, const double* tb, const float4* z0, const float4* dz, double* t) {
   pdl_entry();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= L.n) return;
   const int ni = L.ni, nj = L.nj, n = L.n, i = c % ni, j = c / ni, Mp = ws_steps(ni, nj);
   double x[4];
-  ws_load64(z0, ws_bpos(i, j, Mp), x);
+  load_z<SECOND>(z0, dz, ws_bpos(i, j, Mp), x);
   double acc[4] = {x[0], x[1], x[2], x[3]};
   auto sub = [&](int blk, int in, int jn) {
-    ws_load64(z0, ws_bpos(in, jn, Mp), x);
+    load_z<SECOND>(z0, dz, ws_bpos(in, jn, Mp), x);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -690,8 +703,9 @@ __global__ void k_ws_defect_d(LevelDev L, const double* tb, const double* R, con
 // are three eighths more work: 64x16 4.7 -> 3.0 us against a launch each, 256x64 7.1 -> 6.4; with blocks of
 // 32 x 8 cells (a sixth more) 512x128 takes 27 us against 20.6, 1024x256 76 against 53.
 constexpr int WD_X = 8, WD_Y = 4, WD_THREADS = 192;
+template <bool SECOND>
 __global__ void __launch_bounds__(WD_THREADS) k_ws_defect(LevelDev L, const double* tb, const double* R, const float4* z0,
-                                                          float4* C) {
+                                                          const float4* dz, float4* C) {
   constexpr int OWN = WD_X * WD_Y, ALL = OWN + WD_X + WD_Y;
   static_assert(4 * ALL <= WD_THREADS, "a row of the products per thread");
   __shared__ double ts[4][ALL];
@@ -741,18 +755,19 @@ __global__ void __launch_bounds__(WD_THREADS) k_ws_defect(LevelDev L, const doub
     const int i = it, j = jt, q = qt;
     double v[4];
     double a = f2d(reinterpret_cast<const float*>(z0 + ws_bpos(i, j, Mp))[q]);
+    if (SECOND) a += f2d(reinterpret_cast<const float*>(dz + ws_bpos(i, j, Mp))[q]);
     if (i < ni - 1) {
-      ws_load64(z0, ws_bpos(i + 1, j, Mp), v);
+      load_z<SECOND>(z0, dz, ws_bpos(i + 1, j, Mp), v);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a -= E[k] * v[k];
     }
     if (j < nj - 1) {
-      ws_load64(z0, ws_bpos(i, j + 1, Mp), v);
+      load_z<SECOND>(z0, dz, ws_bpos(i, j + 1, Mp), v);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a -= N[k] * v[k];
     }
     if (j == 0 && nw > 0 && i < nw && ni - 1 - i > i) {
-      ws_load64(z0, ws_bpos(ni - 1 - i, 0, Mp), v);
+      load_z<SECOND>(z0, dz, ws_bpos(ni - 1 - i, 0, Mp), v);
 #pragma unroll
       for (int k = 0; k < 4; ++k) a -= entry(2, q, k, i) * v[k];
     }
@@ -799,10 +814,10 @@ __global__ void k_ws_skew(LevelDev L) {
   b[WS_F4_STEP / 2] = row(4);
 }
 
-// z = z0 (+ dz): the stage update u = u0 - alpha z (scaled by dt* for ARK), or z to the level's
+// z = z0 (+ dz + dz2): the stage update u = u0 - alpha z (scaled by dt* for ARK), or z to the level's
 // sweep vector (FP64 contexts: yz64; mixed: yz32).
-__global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, int do_update, int aw, double alpha,
-                            int mixed) {
+__global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, const float4* dz2, int do_update, int aw,
+                            double alpha, int mixed) {
   pdl_entry();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= L.n) return;
@@ -810,9 +825,10 @@ __global__ void k_ws_finish(LevelDev L, const float4* z0, const float4* dz, int 
   const size_t zp = ws_bpos(i, j, ws_steps(L.ni, L.nj));
   double z[4];
   ws_load64(z0, zp, z);
-  if (dz) {
+  for (const float4* more : {dz, dz2}) {
+    if (!more) break;
     double d[4];
-    ws_load64(dz, zp, d);
+    ws_load64(more, zp, d);
 #pragma unroll
     for (int q = 0; q < 4; ++q) z[q] += d[q];
   }
@@ -1001,6 +1017,7 @@ int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int
   const int g = (L.n + 127) / 128;
   float4* z0 = reinterpret_cast<float4*>(L.wsZ);
   float4* dz = z0 + ws_vec_floats(L.ni, L.nj) / 4;
+  float4* dz2 = dz + ws_vec_floats(L.ni, L.nj) / 4;
   int launches = 0;
   const bool split = L.n <= WS_SPLIT_CELLS;
   const int g4 = (4 * L.n + 127) / 128;  // one thread per cell and row
@@ -1023,21 +1040,26 @@ int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int
   }
   sweep(z0);
   ++launches;
-  const bool corr = refine && !mixed;
-  if (corr) {
-    const float4* z0c = z0;
+  const bool corr = refine > 0 && !mixed;
+  if (!corr || refine < 2) dz2 = nullptr;
+  const float4 *z0c = z0, *none = nullptr;
+  auto correct = [&](auto second, float4* out) {
+    constexpr bool SECOND = decltype(second)::value;
+    const float4* dzc = SECOND ? dz : none;
     const double *wT = L.wsT, *wR = L.wsR;
     if (split) {
-      launch_pdl(k_ws_defect, dim3((L.ni + WD_X - 1) / WD_X, (L.nj + WD_Y - 1) / WD_Y), WD_THREADS, 0, st, L, tb64, wR,
-                 z0c, wC);
+      launch_pdl(k_ws_defect<SECOND>, dim3((L.ni + WD_X - 1) / WD_X, (L.nj + WD_Y - 1) / WD_Y), WD_THREADS, 0, st, L,
+                 tb64, wR, z0c, dzc, wC);
     } else {
-      launch_pdl(k_ws_defect_t, g, 128, 0, st, L, tb64, z0c, L.wsT);
+      launch_pdl(k_ws_defect_t<SECOND>, g, 128, 0, st, L, tb64, z0c, dzc, L.wsT);
       launch_pdl(k_ws_defect_d, g, 128, 0, st, L, tb64, wR, wT, wC);
       ++launches;
     }
-    sweep(dz);
+    sweep(out);
     launches += 2;
-  }
+  };
+  if (corr) correct(std::false_type{}, dz);
+  if (dz2) correct(std::true_type{}, dz2);
   if (exact_iters > 0) {
     launch_pdl(k_ws_accum, g, 128, 0, st, L, static_cast<const float4*>(z0),
                corr ? static_cast<const float4*>(dz) : nullptr, L.wsX, 1);
@@ -1057,11 +1079,11 @@ int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int
     return launches + 1;
   }
   if (pending) {
-    *pending = WsPending{z0, corr ? dz : nullptr, alpha, aw};
+    *pending = WsPending{z0, corr ? dz : nullptr, dz2, alpha, aw};
     return launches;
   }
-  launch_pdl(k_ws_finish, g, 128, 0, st, L, static_cast<const float4*>(z0), corr ? static_cast<const float4*>(dz) : nullptr,
-             do_update, aw, alpha, mixed);
+  launch_pdl(k_ws_finish, g, 128, 0, st, L, z0c, corr ? static_cast<const float4*>(dz) : none,
+             static_cast<const float4*>(dz2), do_update, aw, alpha, mixed);
   return launches + 1;
 }
 

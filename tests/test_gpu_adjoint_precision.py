@@ -1,0 +1,58 @@
+"""The transposed preconditioner P^-T r of FP64 contexts against the two block-triangular solves in FP64 on
+the oracle's blocks: P = S^-1 (D + L) D^-1 (D + U), S = eta dt*.
+
+Tolerance (largest error over largest entry): a cell's unknown is a sum of 16 products and a 4x4 solve, whose
+roundings (1.1e-16 each) and whose blocks' (up to 8e-16 an entry, theirs and the oracle's) the two solves
+amplify by up to three: 5e-15.  An FP32 solve with one FP64 correction leaves (1.2e-7)^2 = 1.4e-14 and more."""
+import numpy as np
+import pytest
+
+from helpers import make_pair, perturbed_state
+from synth.cgrid import make_cgrid
+
+pytestmark = pytest.mark.gpu
+
+
+def _solve_transposed(o, r, cfl, nw, eta=0.8):
+    axp, axm, aep, aem = o.face_blocks()
+    dts, vol = o.pseudo_dt(cfl), o.metrics(o.finest)[4]
+    nj, ni = dts.shape
+    c = (eta * dts / vol)[..., None, None]
+    W, E, S, N = -c * axp[:, :-1], c * axm[:, 1:], -c * aep[:-1], c * aem[1:]
+    DT = np.swapaxes(np.eye(4) + c * ((axp[:, 1:] - axm[:, :-1]) + (aep[1:] - aem[:-1])), -1, -2).copy()
+    r = r.transpose(1, 2, 0).copy()
+    a, z = np.zeros_like(r), np.zeros_like(r)
+    for j in range(nj):                      # (D + U)^T a = r
+        for i in range(ni):
+            x = a[j, i] = np.linalg.solve(DT[j, i], r[j, i])
+            if i < ni - 1:
+                r[j, i + 1] -= E[j, i].T @ x
+            if j < nj - 1:
+                r[j + 1, i] -= N[j, i].T @ x
+            if j == 0 and i < nw:            # the lower wake's cells come before their mirrors
+                r[0, ni - 1 - i] -= S[0, i].T @ x
+    r = (DT @ a[..., None])[..., 0]
+    for j in range(nj - 1, -1, -1):          # (D + L)^T z = D^T a
+        for i in range(ni - 1, -1, -1):
+            x = z[j, i] = np.linalg.solve(DT[j, i], r[j, i])
+            if i > 0:
+                r[j, i - 1] -= W[j, i].T @ x
+            if j > 0:
+                r[j - 1, i] -= S[j, i].T @ x
+            if j == 0 and i >= ni - nw:
+                r[0, ni - 1 - i] -= S[0, i].T @ x
+    return (eta * dts) * z.transpose(2, 0, 1)
+
+
+@pytest.mark.parametrize("ni,nj,nw,viscous", [(64, 16, 8, 0), (150, 43, 18, 1), (40, 9, 0, 0)])
+def test_transposed_preconditioner_is_exact_to_fp64(ni, nj, nw, viscous):
+    g = make_cgrid(ni, nj, n_wake=nw, wall_spacing=1e-3)
+    o, s = make_pair(g, nlevels=1, mach=0.6, alpha_deg=1.0, viscous=viscous, re=5e4)
+    u = perturbed_state(0.6, 1.0, nj, ni, amp=0.01, seed=ni)
+    r = np.random.default_rng(nj).standard_normal((4, nj, ni))
+    o.set_state(u)
+    s.set_state(u)
+    for cfl in (5.0, 100.0):
+        want = _solve_transposed(o, r, cfl, nw)
+        assert np.abs(s.adjoint_precond_apply(r, cfl) - want).max() < 5e-15 * np.abs(want).max()
+    s.close()

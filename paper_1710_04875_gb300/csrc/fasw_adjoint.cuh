@@ -150,6 +150,11 @@ void adj_build_precond(AdjointDev& A, const LevelDev& L, const PhysParams& ph, c
 void adj_mg_build_precond(AdjointDev& A, const std::vector<LevelDev>& lev, const PhysParams& ph,
                           const SchemeParams& sc, double cfl, cudaStream_t st, long long& launches);
 void adj_precond(const AdjointDev& A, const double* r, double* scratch, double* z, cudaStream_t st);
+// The operators applied below are linear, and their FP64 sweeps run in FP32 with corrections: a right-hand side
+// of any size goes in scaled by the power of two of its largest entry (r in place; no bit of the mantissas
+// changes), and the result is scaled back.  In between A.parts is the scale's.
+void adj_scale_in(AdjointDev& A, double* r, cudaStream_t st);
+void adj_scale_out(const AdjointDev& A, double* z, cudaStream_t st);
 // z = P^-T r (steps <= 0) or z = `steps` transposed stage-loop steps from zero; the
 // preconditioner must be built.
 void adj_steps_apply(AdjointDev& A, int steps, const double* r, double* z, cudaStream_t st);

@@ -57,6 +57,25 @@ __global__ void k_adj_set_state(LevelDev L, const double* ub, const int* col, in
   }
 }
 
+// The bit pattern of the largest |x| (of finite non-negative values the order of the patterns is the values').
+__global__ void k_max_bits(int m, const double* x, unsigned long long* out) {
+  pdl_entry();
+  unsigned long long b = 0;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x)
+    b = max(b, (unsigned long long)__double_as_longlong(fabs(x[t])));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, b);
+}
+
+// x times the power of two of the value in *bits to the power sgn; zero, infinity and NaN leave x as it is.
+__global__ void k_scale_pow2(int m, const unsigned long long* bits, int sgn, double* x) {
+  pdl_entry();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const double s = __longlong_as_double((long long)*bits);
+  if (t < m && s > 0.0 && s <= 1.7976931348623157e308) x[t] = ldexp(x[t], sgn * ilogb(s));
+}
+
 __global__ void k_adj_get_state(LevelDev L, double* ub) {
   pdl_entry();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -695,6 +714,19 @@ void adj_build_precond(AdjointDev& A, const LevelDev& L, const PhysParams& ph, c
 
 void adj_precond(const AdjointDev& A, const double* r, double* scratch, double* z, cudaStream_t st) {
   precond(A, r, scratch, z, st);
+}
+
+void adj_scale_in(AdjointDev& A, double* r, cudaStream_t st) {
+  auto* bits = reinterpret_cast<unsigned long long*>(A.parts);
+  const int m = 4 * A.n;
+  cudaMemsetAsync(bits, 0, sizeof(*bits), st);
+  launch_pdl(k_max_bits, RED_BLOCKS, 256, 0, st, m, (const double*)r, bits);
+  launch_pdl(k_scale_pow2, (m + 255) / 256, 256, 0, st, m, (const unsigned long long*)bits, -1, r);
+}
+
+void adj_scale_out(const AdjointDev& A, double* z, cudaStream_t st) {
+  const int m = 4 * A.n;
+  launch_pdl(k_scale_pow2, (m + 255) / 256, 256, 0, st, m, reinterpret_cast<const unsigned long long*>(A.parts), 1, z);
 }
 
 void adj_steps_apply(AdjointDev& A, int steps, const double* r, double* z, cudaStream_t st) {

@@ -56,3 +56,25 @@ def test_transposed_preconditioner_is_exact_to_fp64(ni, nj, nw, viscous):
         want = _solve_transposed(o, r, cfl, nw)
         assert np.abs(s.adjoint_precond_apply(r, cfl) - want).max() < 5e-15 * np.abs(want).max()
     s.close()
+
+
+@pytest.mark.parametrize("levels", [1, 2])
+def test_operators_take_right_hand_sides_of_any_size(levels):
+    """The operators are linear: of a right-hand side times a power of two they give the result times it, bit
+    for bit, beyond the range of FP32 too; a right-hand side of zeros gives zeros."""
+    import paper_1710_04875_gb300 as P
+    ni, nj = 64, 16
+    s = P.Solver(make_cgrid(ni, nj, n_wake=8, wall_spacing=1e-3),
+                 P.default_params(mach=0.6, alpha_deg=1.0, nlevels=levels, gamma_cycle=2))
+    s.set_state(perturbed_state(0.6, 1.0, nj, ni, amp=0.01, seed=1))
+    s.adjoint_jacobian()
+    r = np.random.default_rng(2).standard_normal((4, nj, ni))
+    kind = "cycle" if levels > 1 else "smoother"
+    for apply in (lambda v: s.adjoint_precond_apply(v, 5.0), lambda v: s.adjoint_precond_apply(v, 5.0, steps=1),
+                  lambda v: s.adjoint_cycle_apply(v, 5.0, kind=kind), lambda v: s.adjoint_cycle_apply(v, 5.0, kind=kind, transpose=False)):
+        z = apply(r)
+        assert np.all(np.isfinite(z)) and np.any(z)
+        for e in (-700.0, -130.0, 130.0, 700.0):
+            assert np.array_equal(apply(r * 2.0**e), z * 2.0**e)
+        assert not np.any(apply(0.0 * r))
+    s.close()

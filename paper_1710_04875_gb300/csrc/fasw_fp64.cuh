@@ -52,16 +52,20 @@ __device__ __forceinline__ float from64<float>(double x) {
 __device__ __forceinline__ double to64(double x) { return x; }
 __device__ __forceinline__ double to64(float x) { return f2d(x); }
 
-// The larger of two non-negative values, the smaller of x and a positive c: on the bit patterns, whose
-// order as signed integers is that of the values.
+// fmax of two non-negative values, fmin of x and a positive c: on the bit patterns, whose order as signed
+// integers is that of the values.  As with fmax and fmin a NaN gives way to the other (a cell of negative
+// pressure has a NaN for its sound speed; its faces take their neighbours' radii).  The upper word of a
+// NaN that an operation returns is above that of infinity, with either sign.
 __device__ __forceinline__ double max_nn(double a, double b) {
-  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+  const bool nan = (unsigned)__double2hiint(a) > 0x7ff00000u, other = (unsigned)__double2hiint(b) > 0x7ff00000u;
+  return !nan && (other || __double_as_longlong(a) > __double_as_longlong(b)) ? a : b;
 }
 __device__ __forceinline__ double min_pos(double x, double c) {
-  return __double_as_longlong(x) < __double_as_longlong(c) ? x : c;
+  const bool nan = (unsigned)__double2hiint(x) > 0xfff00000u;  // a negative one; a positive one is above c
+  return !nan && __double_as_longlong(x) < __double_as_longlong(c) ? x : c;
 }
-// max(x, 0)
-__device__ __forceinline__ double relu64(double x) { return __double2hiint(x) < 0 ? 0.0 : x; }
+// fmax(x, 0)
+__device__ __forceinline__ double relu64(double x) { return (unsigned)__double2hiint(x) > 0x7ff00000u ? 0.0 : x; }
 __device__ __forceinline__ bool is_zero(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) == 0; }
 
 }  // namespace fasw

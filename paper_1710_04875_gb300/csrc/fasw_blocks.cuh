@@ -10,7 +10,7 @@ template <typename T>
 __device__ __forceinline__ void diag_scales(const LevelDev& L, int aw, double eta, int c, double& coef, double& sigma) {
   if (aw) {
     const double ed = eta * L.dts[c];
-    coef = sizeof(T) == 8 ? ed * L.rvol[c] : ed / L.vol[c];
+    coef = sizeof(T) == 8 ? div64(ed, L.vol[c], L.rvol[c]) : ed / L.vol[c];
     sigma = is_zero(L.a_t) ? 1.0 : 1.0 + ed * L.a_t;
   } else {
     coef = L.rvol[c];
@@ -25,10 +25,11 @@ __device__ __forceinline__ void lu4(T A[16]) {
   if constexpr (sizeof(T) == 8) {  // each pivot's reciprocal once, for its column's multipliers too
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      A[5 * k] = rcp64(A[5 * k]);
+      const double d = A[5 * k];
+      A[5 * k] = rcp64(d);
 #pragma unroll
       for (int r = k + 1; r < 4; ++r) {
-        const double m = A[4 * r + k] * A[5 * k];
+        const double m = div64(A[4 * r + k], d, A[5 * k]);
         A[4 * r + k] = m;
 #pragma unroll
         for (int cc = k + 1; cc < 4; ++cc) A[4 * r + cc] -= m * A[4 * k + cc];

@@ -42,6 +42,14 @@ __device__ __forceinline__ double rcp64(double x) {
   return fma(fma(-x, y, 1.0), y, y);
 }
 
+// a / b, rb = rcp64(b): the product with the reciprocal and one correction by its remainder (Markstein, IBM J. Res.
+// Dev. 34, 1990), which give the division's rounding where the product alone is off by up to one and a half units in
+// the last place.  Where there is no remainder (zero or infinite b, overflow) the product stands.
+__device__ __forceinline__ double div64(double a, double b, double rb) {
+  const double q = a * rb, c = fma(fma(-q, b, a), rb, q);
+  return ((unsigned)__double2hiint(c) & 0x7fffffffu) > 0x7ff00000u ? q : c;
+}
+
 // x in the precision of T
 template <typename T>
 __device__ __forceinline__ T from64(double x);

@@ -86,7 +86,7 @@ __device__ void farfield(const double wi[4], const PhysParams& ph, double nx, do
     ut = uf - vnf * nx;
     vt = vf - vnf * ny;
   }
-  const double ra = ph.fast ? ab * rcp64(aup) : ab / aup, ra2 = ra * ra;
+  const double ra = ph.fast ? div64(ab, aup, rcp64(aup)) : ab / aup, ra2 = ra * ra;
   const double rho = rup * (ra2 * ra2 * ra);
   const double p = rho * ab * ab * (1.0 / GAM);
   const double u = ut + vnb * nx, v = vt + vnb * ny;
@@ -326,7 +326,7 @@ __global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, 
   L.rt[L.n + c] = reta + rxi * cr;
   if (want_dts) {
     const double r = rxi + reta;
-    L.dts[c] = ph.fast ? cv * rcp64(r) : cv / r;
+    L.dts[c] = ph.fast ? div64(cv, r, rcp64(r)) : cv / r;
   }
 }
 
@@ -346,7 +346,7 @@ __device__ __forceinline__ double rt_cell(const LevelDev& L, int i, int j, int d
 template <bool FAST>
 __device__ __forceinline__ double sensor_val(double qm, double q0, double qp) {
   const double d = fabs(qp - 2.0 * q0 + qm), s = qp + 2.0 * q0 + qm + 0.001;
-  return FAST ? d * rcp64(s) : d / s;
+  return FAST ? div64(d, s, rcp64(s)) : d / s;
 }
 
 // JST flux through a face with area vector (sx, sy) from L to R; stencil LL, L, R, RR

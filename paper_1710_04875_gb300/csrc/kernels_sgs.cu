@@ -79,12 +79,12 @@ __device__ __forceinline__ void split_blocks64(const double w[4], double nx, dou
                                                double vf, int moving, double d, double rd, double Ap[16],
                                                double Am[16]) {
   constexpr double g1 = GAM - 1.0;
-  const double rr = rcp64(w[0]), u = w[1] * rr, v = w[2] * rr;
+  const double rr = rcp64(w[0]), u = div64(w[1], w[0], rr), v = div64(w[2], w[0], rr);
   const double q2 = u * u + v * v;
   const double p = g1 * (w[3] - 0.5 * w[0] * q2);
-  const double a = sqrt(GAM * p * rr), ia = rcp64(a);
-  const double H = (w[3] + p) * rr;
-  const double vn = u * nx + v * ny, vr = moving ? vn - vf * rl : vn;
+  const double a = sqrt(div64(GAM * p, w[0], rr)), ia = rcp64(a);
+  const double H = div64(w[3] + p, w[0], rr);
+  const double vn = u * nx + v * ny, vr = moving ? vn - div64(vf, len, rl) : vn;
   const double dp[3] = {0.5 * g1 * q2, -g1 * u, -g1 * v};  // dp[3] = g1; dvn = (-vn, nx, ny, 0)
   const double lam[3] = {vr, vr + a, vr - a}, ad = a * d, iad = ia * rd, hl = 0.5 * len;
   double P[3], Q[3];  // halves of the eigenvalues and of their cutoff moduli, times the length
@@ -187,8 +187,8 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d, T rd) {
   if (F64) {
     len = sqrt(sx * sx + sy * sy);
     rl = rcp64(len);
-    nx = sx * rl;
-    ny = sy * rl;
+    nx = div64(sx, len, rl);
+    ny = div64(sy, len, rl);
     if (ph.viscous && has && f >= L.nfx) vr = visc_radius<true>(L, ph, (f - L.nfx) % ni, (f - L.nfx) / ni, 0.0);
   }
   pdl_entry();
@@ -207,7 +207,7 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d, T rd) {
     split_blocks<T>(w, from64<T>(sx), from64<T>(sy), from64<T>(vf), d, P, M);
   if (ph.viscous && f >= L.nfx) {
     const int e = f - L.nfx;
-    const T V = F64 ? T(vr * rcp64(wd[0])) : from64<T>(visc_radius<false>(L, ph, e % ni, e / ni, wd[0]));
+    const T V = F64 ? T(div64(vr, wd[0], rcp64(wd[0]))) : from64<T>(visc_radius<false>(L, ph, e % ni, e / ni, wd[0]));
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       P[5 * k] += V;

@@ -179,7 +179,7 @@ __global__ void k_restrict(LevelDev F, LevelDev C, int restrict_mut, int fast) {
   const int fi[4] = {2 * I, 2 * I + 1, 2 * I, 2 * I + 1};
   const int fj[4] = {2 * J, 2 * J, 2 * J + 1, 2 * J + 1};
   const double vc = C.vol[t], rvc = C.rvol[t];
-  auto over = [&](double a) { return fast ? a * rvc : a / vc; };
+  auto over = [&](double a) { return fast ? div64(a, vc, rvc) : a / vc; };
   double au[4] = {0, 0, 0, 0}, ar[4] = {0, 0, 0, 0}, am = 0.0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {

@@ -429,11 +429,12 @@ __device__ __forceinline__ void jst_face(const LevelDev& L, int gLL, int gL, int
     const double qL = (uL[1] * hx + uL[2] * hy) * L.rinv[gL];
     const double qR = (uR[1] * hx + uR[2] * hy) * L.rinv[gR];
     if (FAST) {
-      const double aL = moving ? qL - hf : qL, aR = moving ? qR - hf : qR, ps = pL + pR;
+      const double aL = moving ? qL - hf : qL, aR = moving ? qR - hf : qR;
       hc[0] = uL[0] * aL + uR[0] * aR;
-      hc[1] = uL[1] * aL + (uR[1] * aR + ps * hx);
-      hc[2] = uL[2] * aL + (uR[2] * aR + ps * hy);
-      hc[3] = uL[3] * aL + (uR[3] * aR + (pL * qL + pR * qR));
+      hc[1] = pR * hx + (pL * hx + (uL[1] * aL + uR[1] * aR));  // the pressure's part, the largest, last
+      hc[2] = pR * hy + (pL * hy + (uL[2] * aL + uR[2] * aR));
+      hc[3] = wL3 * qL + wR3 * qR;
+      if (moving) hc[3] -= hf * (uL[3] + uR[3]);
     } else if (moving) {
       const double qnL = (uL[1] * sx + uL[2] * sy) * L.rinv[gL];
       const double qnR = (uR[1] * sx + uR[2] * sy) * L.rinv[gR];

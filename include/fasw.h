@@ -457,6 +457,15 @@ int fasw_check_math(int n, const double* a, const double* b, double* out, int on
  * FASW_ERR_ARG for n < 0 or null pointers, FASW_ERR_OOM / FASW_ERR_CUDA on device failures. */
 int fasw_check_fp64(int n, const double* a, double* out);
 
+/* Verification hook for the choice of the warp-strip sweep's form on a level of ni x nj cells with n_wake
+ * wake-cut columns: *stages of its operand ring (5 or 3; deep = 0: as kind 10, 3 only), *edges buffers of
+ * boundary rows (2 or 1) and *bytes of shared memory per CTA, all zero where the level takes another sweep.
+ * cluster_bytes > 0: as on a device that holds a cluster of more than eight CTAs (nj > 128) only with up to
+ * that much shared memory per CTA (host only, no device needed); 0: asks the current device.  FASW_ERR_ARG for
+ * sizes below one, negative cluster_bytes or null pointers. */
+int fasw_check_sweep_form(int ni, int nj, int n_wake, int deep, long long cluster_bytes, int* stages, int* edges,
+                          long long* bytes);
+
 /* Coefficients of the stage loop of a scheme, Table "RK smoothers" (section 4.1): *nstages
  * (3 or 5) and alpha[k], beta[k] for k < *nstages (alpha, beta nullable, 5 doubles each).  The
  * W methods use the ARK coefficients of the same name; AW51/AW52 and ARK51/ARK52 take the

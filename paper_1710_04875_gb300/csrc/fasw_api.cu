@@ -195,7 +195,8 @@ int alloc_level(fasw_ctx* c, LevelDev& L) {
     A(L.hpC, 4 * h);
     A(L.hpY, 4 * h);
   }
-  if (ws_fits(L.ni, L.nj, L.nw)) {
+  for (int deep = 0; deep < 2; ++deep) L.wsForm[deep] = ws_form(L.ni, L.nj, L.nw, deep);
+  if (L.wsForm[0] >= 0) {
     const size_t wf = ws_floats(L.ni, L.nj), wv = ws_vec_floats(L.ni, L.nj);
     A(L.wsF, wf);
     A(L.wsB, wf);
@@ -968,6 +969,13 @@ int fasw_check_fp64(int n, const double* a, double* out) {
   if (e == cudaSuccess) e = cudaMemcpy(out, d + m, 4 * m * sizeof(double), cudaMemcpyDeviceToHost);
   cudaFree(d);
   return e == cudaSuccess ? FASW_OK : cuda_fail(e);
+}
+
+int fasw_check_sweep_form(int ni, int nj, int n_wake, int deep, long long cluster_bytes, int* stages, int* edges,
+                          long long* bytes) {
+  if (ni < 1 || nj < 1 || n_wake < 0 || cluster_bytes < 0 || !stages || !edges || !bytes) return FASW_ERR_ARG;
+  ws_form_shape(ni, nj, n_wake, ws_form(ni, nj, n_wake, deep != 0, cluster_bytes), stages, edges, bytes);
+  return FASW_OK;
 }
 
 void fasw_fault_inject_alloc(long long n) { g_fail_alloc_in.store(n < 0 ? -1 : n); }

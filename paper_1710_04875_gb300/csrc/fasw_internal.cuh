@@ -110,6 +110,7 @@ struct LevelDev {
   double* wsT;
   double* wsR;  // D^-1 r of the stage in FP64 (FP64 contexts)
   double* wsX;  // accumulated solution of the exact-preconditioner iterations (4 per cell)
+  int wsForm[2];  // forms of the warp-strip sweep (ws_form): kind 10, kind 9
 };
 
 struct PhysParams {

@@ -104,7 +104,11 @@ __device__ __forceinline__ void ws_updated(const LevelDev& L, const WsPending& p
 
 // L.tb (FP64) into the warp-strip layout: L.wsF, L.wsB, L.wsCut
 void launch_ws_skew(const LevelDev& L, cudaStream_t st);
-bool ws_fits(int ni, int nj, int nw);
+// The form of the sweep (operand ring, edge buffers) for a level: the first, in order of speed, that the
+// device can launch, -1: none (another sweep).  deep: kind 9.  cluster_bytes: 0 asks the current device whether
+// it holds a cluster of more than eight CTAs; else only with up to that much shared memory a CTA.
+int ws_form(int ni, int nj, int nw, bool deep, long long cluster_bytes = 0);
+void ws_form_shape(int ni, int nj, int nw, int form, int* stages, int* edges, long long* bytes);
 size_t ws_floats(int ni, int nj);
 size_t ws_vec_floats(int ni, int nj);
 int ws_strips(int nj);

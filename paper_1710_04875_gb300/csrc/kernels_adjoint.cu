@@ -464,7 +464,7 @@ int adj_setup(AdjointDev& A, int ni, int nj, int nw, std::vector<void*>& allocs,
         return r;
     }
   }
-  if (!A.fp32 && ws_fits(ni, nj, nw)) {
+  if (!A.fp32 && ws_form(ni, nj, nw, false) >= 0) {
     const size_t wf = ws_floats(ni, nj), wc = 16 * (size_t)(nw > 0 ? nw : 1);
     if ((r = adj_alloc(allocs, &A.wsB, wf)) || (r = adj_alloc(allocs, &A.wsCut, wc)) ||
         (r = adj_alloc(allocs, &A.wsZ, 3 * ws_vec_floats(ni, nj))) || (r = adj_alloc(allocs, &A.wsF, wf)))

@@ -971,49 +971,78 @@ cudaError_t ws_sweep_launch(const LevelDev& L, float4* zout, int* err, long long
                             reinterpret_cast<float4*>(L.wsY), static_cast<const float*>(L.wsCut), zout, err, limit);
 }
 
+// The forms in order of speed: an edge buffer per pass (1024x256 pair 162 us; with one, cleared between
+// the passes, 3 % more), a ring of five stages (three: 1-3 % slower).
+struct WsForm {
+  int stages;
+  bool two;
+  size_t (*bytes)(int Mp, int nw);
+  cudaLaunchConfig_t (*config)(const LevelDev&, cudaLaunchAttribute*, cudaStream_t);
+  void (*attributes)();
+  const void* kernel;
+  cudaError_t (*launch)(const LevelDev&, float4*, int*, long long, cudaStream_t);
+};
+
 template <int NS, bool TWO>
-bool ws_smem_fits(int ni, int nj, int nw) {
-  return ws_cta_bytes<NS, TWO>(ws_steps(ni, nj), nw) <= kWsSmemMax;
+WsForm form_of() {
+  return {NS,
+          TWO,
+          [](int Mp, int nw) { return ws_cta_bytes<NS, TWO>(Mp, nw); },
+          ws_config<NS, TWO>,
+          ws_attributes<NS, TWO>,
+          reinterpret_cast<const void*>(k_sweep_ws<NS, TWO>),
+          ws_sweep_launch<NS, TWO>};
+}
+
+const WsForm kWsForms[] = {form_of<WS_STAGES, true>(), form_of<WS_STAGES, false>(), form_of<WS_SHALLOW, true>(),
+                           form_of<WS_SHALLOW, false>()};
+
+// whether the device can hold the cluster of this form's launch
+bool ws_cluster_fits(const WsForm& f, int ni, int nj, int nw) {
+  LevelDev L = {};
+  L.ni = ni;
+  L.nj = nj;
+  L.nw = nw;
+  f.attributes();
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t cfg = f.config(L, at, nullptr);
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, f.kernel, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();  // not this call's error: the level takes another form
+  return e == cudaSuccess && n >= 1;
 }
 
 }  // namespace
 
 // One cluster per sweep: at most 16 CTAs of two strips, a ring and an edge buffer that fit in shared
-// memory, and (beyond the portable 8 CTAs) a device that can hold such a cluster.
-bool ws_fits(int ni, int nj, int nw) {
+// memory, and (beyond the portable 8 CTAs) a device that can hold such a cluster.  The question is asked for
+// the very form that is launched: at 1024x256 the deepest takes 176 KB a CTA and 16 SMs, the shallowest 103 KB
+// and 8.
+int ws_form(int ni, int nj, int nw, bool deep, long long cluster_bytes) {
   const int nb = (ws_strips(nj) + 1) / 2;
-  if (nb > kWsCluster || !ws_smem_fits<WS_SHALLOW, false>(ni, nj, nw)) return false;
-  if (nb <= kWsPortable) return true;
-  LevelDev L = {};
-  L.ni = ni;
-  L.nj = nj;
-  L.nw = nw;
-  ws_attributes<WS_SHALLOW, false>();
-  cudaLaunchAttribute at[2];
-  const cudaLaunchConfig_t cfg = ws_config<WS_SHALLOW, false>(L, at, nullptr);
-  int n = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k_sweep_ws<WS_SHALLOW, false>, &cfg);
-  if (e != cudaSuccess) cudaGetLastError();  // not this call's error: the level takes another sweep
-  return e == cudaSuccess && n >= 1;
+  if (nb > kWsCluster) return -1;
+  for (int k = 0; k < 4; ++k) {
+    const WsForm& f = kWsForms[k];
+    const size_t bytes = f.bytes(ws_steps(ni, nj), nw);
+    if ((f.stages > WS_SHALLOW && !deep) || bytes > kWsSmemMax) continue;
+    if (nb <= kWsPortable || (cluster_bytes > 0 ? (long long)bytes <= cluster_bytes : ws_cluster_fits(f, ni, nj, nw)))
+      return k;
+  }
+  return -1;
+}
+
+void ws_form_shape(int ni, int nj, int nw, int form, int* stages, int* edges, long long* bytes) {
+  *stages = form < 0 ? 0 : kWsForms[form].stages;
+  *edges = form < 0 ? 0 : kWsForms[form].two ? 2 : 1;
+  *bytes = form < 0 ? 0 : (long long)kWsForms[form].bytes(ws_steps(ni, nj), nw);
 }
 
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,
                     long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, bool deep,
                     WsPending* pending) {
   (void)prog;  // the warp strips exchange their boundary rows in shared memory, not through progress words
-  auto sweep = [&](float4* zout) {
-    // An edge buffer per pass where two fit (1024x256 pair 171 us; with one, cleared between the
-    // passes, 177 us), a ring of five stages where it fits (three: 1-3 % slower).
-    const auto fits = [&](auto deep, auto two) {
-      return ws_smem_fits<decltype(deep)::value ? WS_STAGES : WS_SHALLOW, decltype(two)::value>(L.ni, L.nj, L.nw);
-    };
-    constexpr std::true_type yes{};
-    constexpr std::false_type no{};
-    if (deep && fits(yes, yes)) return ws_sweep_launch<WS_STAGES, true>(L, zout, err, limit, st);
-    if (deep && fits(yes, no)) return ws_sweep_launch<WS_STAGES, false>(L, zout, err, limit, st);
-    if (fits(no, yes)) return ws_sweep_launch<WS_SHALLOW, true>(L, zout, err, limit, st);
-    return ws_sweep_launch<WS_SHALLOW, false>(L, zout, err, limit, st);
-  };
+  const WsForm& form = kWsForms[L.wsForm[deep]];
+  auto sweep = [&](float4* zout) { return form.launch(L, zout, err, limit, st); };
   const int g = (L.n + 127) / 128;
   float4* z0 = reinterpret_cast<float4*>(L.wsZ);
   float4* dz = z0 + ws_vec_floats(L.ni, L.nj) / 4;

@@ -440,7 +440,8 @@ __device__ __forceinline__ bool ws_pass(const LevelDev& L, const WsSmem& S, int 
         const float4 x = lds4(x_own), w = lds4(nb + u * nb_step);
         if (u > 0) sts1(h + (FWD ? WS_U - u : u - 1) * WS_VEC_BYTES, y);  // the previous step's result
         if (u == WS_U - 2) landed = ld_relaxed(ready);
-        if (u == WS_U - 1 && __builtin_expect(landed <= next, 0) && !wait_stage(next)) {
+        // one decision for the warp: each lane reads the counter for itself, and wait_stage's votes take every lane
+        if (u == WS_U - 1 && __builtin_expect(!__all_sync(WS_ALL, landed > next), 0) && !wait_stage(next)) {
           ok = false;
           return;
         }

@@ -434,12 +434,16 @@ int fasw_batch_solve(fasw_batch* batch, double drop, int max_cycles, int* cycles
  * batch cycles: states are saved and restored; each candidate is timed beside the incumbent, the
  * faster of two timings each, and a switch must gain 2 %.  Candidates are the variants whose CTAs
  * never wait on a CTA that might not be resident beside the other cases' kernels: mixed precision
- * 7, 6, 2, 9 and 10 (the warp strips run as one thread-block cluster, which the hardware
- * schedules together); FP64 9, 10 and 2.  Tile heights 0 (size rule), 1, 2, 4, 8.  Results are cached per shape
+ * 7, 6, 2, 9 (the warp strips run as one thread-block cluster, which the hardware schedules
+ * together) and, where the cases' finest levels have more CTAs of strips than the device has SMs,
+ * 10; FP64 9, 10 and 2 (fasw_batch_candidates).  Tile heights 0 (size rule), 1, 2, 4, 8.  Results are cached per shape
  * and precision for the process, so a batch whose shapes are all cached is not timed again.
  * choice[k] (nullable) receives kind | (tile height << 8) for case k.  Batch cases start with
  * kind 9 (the warp strips); strip-pipelined kinds are never used inside a batch. */
 int fasw_batch_autotune(fasw_batch* batch, int* choice);
+/* The sweep kinds that fasw_batch_autotune compares for the batch's cases in mixed precision (mixed != 0) or in
+ * FP64: kinds (5 ints), *n of them.  FASW_ERR_ARG for null pointers. */
+int fasw_batch_candidates(fasw_batch* batch, int mixed, int* kinds, int* n);
 long long fasw_batch_launch_count(fasw_batch* batch);
 
 /* Verification hook for two FP64 powers the per-cell auxiliaries form by Newton's method (the

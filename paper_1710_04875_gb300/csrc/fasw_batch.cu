@@ -172,10 +172,14 @@ int fasw_batch_solve(fasw_batch* b, double drop, int max_cycles, int* cycles, do
   return diverged ? FASW_ERR_DIVERGED : FASW_ERR_NOT_CONVERGED;
 }
 
-// Autotuner.  Candidates are the sweep variants whose CTAs never wait on one another (strip
-// sweeps are not candidates: their CTAs wait on each other, which is safe only while all CTAs
-// of one sweep are resident, and concurrent branches of a batch graph do not guarantee that):
-// the hyperplane-staged FP32 sweep with a ring of 8 or 4 steps and the one-CTA sweep.  Which
+// Autotuner.  Candidates are the sweep variants whose CTAs never wait on a CTA that may not be resident (the
+// strip sweeps are not candidates: their CTAs wait on one another, and concurrent branches of a batch graph do
+// not guarantee that all CTAs of one sweep are resident): the one-CTA sweep, the warp strips, which run as one
+// cluster, and in mixed precision the hyperplane-staged FP32 sweep with a ring of 8 or 4 steps.  The warp strips
+// with the smaller ring (kind 10) exist so that strips of different cases share an SM; in mixed precision they are
+// a candidate where the cases' finest levels have more strip CTAs than the device SMs (mixed cycle, kind 9
+// against 10: 64 cases of 256x64, 256 CTAs, 5,195 / 5,094 us; 128 of 128x32, 256 CTAs, 3,296 / 3,288; 64 of
+// 128x32, 128 CTAs, 1,700 / 1,710; 16 of 512x128, 128 CTAs, 4,803 / 5,006; 4 of 256x64, 16 CTAs, 752 / 778).  Which
 // wins depends on the grid shape and on how full the GPU is, so the tuner times whole batch
 // cycles (all cases concurrently, CUDA events, states saved and restored) and improves the
 // choice one grid shape (ni, nj) at a time, keeping a change only when the batch gets faster.
@@ -195,7 +199,26 @@ TuneKey key_of(fasw_ctx* c) {
   const LevelDev& F = c->lev[c->L()];
   return TuneKey{F.ni, F.nj, c->mixed};
 }
+
+std::vector<int> candidates(const fasw_batch* b, bool mixed) {
+  if (!mixed) return {SWEEP_WS, SWEEP_WS8, SWEEP_CTA};
+  std::vector<int> k{SWEEP_HP8, SWEEP_HP4, SWEEP_CTA, SWEEP_WS};
+  int ctas = 0, dev = 0, sms = 0;
+  for (const fasw_ctx* c : b->cases) ctas += (ws_strips(c->lev[c->L()].nj) + 1) / 2;  // two strips a CTA
+  if (cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && ctas > sms)
+    k.push_back(SWEEP_WS8);
+  return k;
+}
 }  // namespace
+
+int fasw_batch_candidates(fasw_batch* b, int mixed, int* kinds, int* n) {
+  if (!b || !kinds || !n) return FASW_ERR_ARG;
+  const std::vector<int> k = candidates(b, mixed != 0);
+  std::copy(k.begin(), k.end(), kinds);
+  *n = (int)k.size();
+  return FASW_OK;
+}
 
 static void set_tile(fasw_ctx* c, int rows) {
   for (auto& L : c->lev) L.res_ty = rows;
@@ -271,10 +294,6 @@ int fasw_batch_autotune(fasw_batch* b, int* choice) {
       if ((r = batch_time(b, kinds, tys, saved, reps, e0, e1, &c2))) return;
       *out = std::min(a, c2);
     };
-    // sweep variants whose CTAs never wait on a CTA that may not be resident (one CTA, or the
-    // warp strips launched as one cluster); the FP32 staged kinds only in mixed precision
-    const int cand_mixed[4] = {SWEEP_HP8, SWEEP_HP4, SWEEP_CTA, SWEEP_WS};
-    const int cand_fp64[3] = {SWEEP_WS, SWEEP_WS8, SWEEP_CTA};
     const int tile_cand[5] = {0, 1, 2, 4, 8};
     // larger shapes first: they dominate the batch time
     std::vector<std::pair<TuneKey, std::vector<size_t>>> order(groups.begin(), groups.end());
@@ -284,13 +303,9 @@ int fasw_batch_autotune(fasw_batch* b, int* choice) {
     // each candidate against the incumbent timed right beside it; a switch must gain 2 %
     for (size_t gi = 0; gi < order.size() && r == FASW_OK; ++gi) {
       const std::vector<size_t>& members = order[gi].second;
-      const bool mixed = order[gi].first.mixed != 0;
-      const int* cand = mixed ? cand_mixed : cand_fp64;
-      const int ncand = mixed ? 4 : 3;
       // sweep variant first (it dominates), then the residual tile height with it
       int keep = kinds[members[0]];
-      for (int ci = 0; ci < ncand; ++ci) {
-        const int k = cand[ci];
+      for (int k : candidates(b, order[gi].first.mixed != 0)) {
         if (k == keep || r) continue;
         float t_keep = 0.f, t_k = 0.f;
         timed(&t_keep);

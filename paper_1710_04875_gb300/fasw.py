@@ -119,6 +119,7 @@ def library(variant: str = "perf"):
             "fasw_batch_cycle": (i, [p, i, dp]),
             "fasw_batch_solve": (i, [p, d, i, dp, dp, C.POINTER(i)]),
             "fasw_batch_autotune": (i, [p, dp]),
+            "fasw_batch_candidates": (i, [p, i, p, C.POINTER(i)]),
             "fasw_batch_launch_count": (ll, [p]),
             "fasw_scheme_coefficients": (i, [i, C.POINTER(i), dp, dp]),
             "fasw_fault_inject_alloc": (None, [ll]),
@@ -581,6 +582,13 @@ class Batch:
         if with_tiles:
             return [(x & 0xFF, x >> 8) for x in ch]
         return [x & 0xFF for x in ch]
+
+    def candidates(self, precision="mixed"):
+        """The sweep kinds that autotune compares for the batch's cases of that precision."""
+        kinds, n = (C.c_int * 5)(), C.c_int()
+        _check(self.lib.fasw_batch_candidates(self.h, int(precision == "mixed"), C.cast(kinds, C.c_void_p), C.byref(n)),
+               "fasw_batch_candidates")
+        return list(kinds[:n.value])
 
     def get_state(self, k):
         g = self.grids[k]

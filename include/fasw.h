@@ -477,6 +477,12 @@ int fasw_check_sweep_form(int ni, int nj, int n_wake, int deep, long long cluste
  * only (no device needed).  FASW_ERR_ARG for an unknown scheme or nstages NULL. */
 int fasw_scheme_coefficients(int scheme, int* nstages, double* alpha, double* beta);
 
+/* Verification hook for the overlap of launches (programmatic dependent launch): with on != 0 the launches made,
+ * and the cycles captured, by the calling host thread from now on each wait for the one before to complete, as
+ * plain stream order has it; with 0 (the default) a kernel may start, and read what is complete, while the one
+ * before runs.  The results are the same bit for bit.  Returns the setting before.  Host only. */
+int fasw_ordered_launches(int on);
+
 /* Failure detection without a GPU fault (no counterpart in the paper).  After
  * fasw_fault_inject_alloc(n), the library's (n+1)-th following device allocation fails on the
  * host, before cudaMalloc is called, as if the device were out of memory (FASW_ERR_OOM); n < 0

@@ -978,6 +978,12 @@ int fasw_check_sweep_form(int ni, int nj, int n_wake, int deep, long long cluste
   return FASW_OK;
 }
 
+int fasw_ordered_launches(int on) {
+  const int was = t_ordered;
+  t_ordered = on != 0;
+  return was;
+}
+
 void fasw_fault_inject_alloc(long long n) { g_fail_alloc_in.store(n < 0 ? -1 : n); }
 
 long long fasw_live_allocations(void) { return g_live_allocs.load(); }

@@ -19,17 +19,31 @@ constexpr double GAM = 1.4;
 // all launches but the last are complete and visible when a kernel starts: what they wrote may be read
 // before pdl_entry() (and memory that the last one does not touch may be written).  launch_pdl() launches with
 // the attribute that allows this overlap; without it griddepcontrol.wait returns at once.
+//
+// The kernels that do so, and what the launch directly before them on the stream may therefore not write:
+//   k_cell_aux with `early`        metrics (face vectors, grid fluxes, volumes, face lengths)
+//   k_residual                     metrics; with tiles of one row also s, src, rhs (forcing evaluations) and, from
+//                                  the second stage on, the carried viscous part: between any of their writers and a
+//                                  residual lies at least k_cell_aux
+//   k_face_blocks (FP64)           metrics and the eddy viscosity: k_cell_aux is between
+//   k_ws_prep64                    state and dt* (read), u0 and coef (written: not to be read by it either):
+//                                  k_face_blocks is between
+//   k_sweep_ws                     the skewed blocks: the right-hand side's or the defect's kernel is between
+//   k_ws_defect                    tb and D^-1 r: the sweep is between
+// fasw_ordered_launches() turns the overlap off, so that results with and without it can be compared.
 __device__ __forceinline__ void pdl_entry() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+
+inline thread_local bool t_ordered = false;  // fasw_ordered_launches
 
 template <typename... KP, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               Args... args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].val.programmaticStreamSerializationAllowed = !t_ordered;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;

@@ -947,7 +947,7 @@ template <int NS, bool TWO>
 cudaLaunchConfig_t ws_config(const LevelDev& L, cudaLaunchAttribute* at, cudaStream_t st) {
   const int nb = (ws_strips(L.nj) + 1) / 2;
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].val.programmaticStreamSerializationAllowed = !t_ordered;
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = nb;
   at[1].val.clusterDim.y = 1;

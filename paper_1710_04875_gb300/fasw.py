@@ -108,6 +108,7 @@ def library(variant: str = "perf"):
             "fasw_checkpoint_schedule": (i, [i, i, dp, dp, i, C.POINTER(i), C.POINTER(ll)]),
             "fasw_check_math": (i, [i, p, p, p, i]),
             "fasw_check_fp64": (i, [i, p, p]),
+            "fasw_ordered_launches": (i, [i]),
             "fasw_check_sweep_form": (i, [i, i, i, i, ll, C.POINTER(i), C.POINTER(i), C.POINTER(ll)]),
             "fasw_unsteady_adjoint": (i, [p, d, d, d, d, d, i, i, d, i, i, i, i, dp, d, d, d, i, i, d, C.POINTER(d),
                                           dp, dp, i, dp]),

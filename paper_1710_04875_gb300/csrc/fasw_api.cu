@@ -204,7 +204,7 @@ int alloc_level(fasw_ctx* c, LevelDev& L) {
     A(L.wsY, wv);
     A(L.wsCut, 16 * (size_t)(L.nw > 0 ? L.nw : 1));
     A(L.wsZ, 2 * wv);
-    A(L.wsT, 4 * n);
+    if (!c->mixed && L.n > WS_SPLIT_CELLS) A(L.wsT, 4 * n);  // smaller levels form it in shared memory
     if (!c->mixed) A(L.wsR, 4 * n);
     A(L.wsX, 4 * n);
     // padding positions of the skewed arrays are never written: they must read as zero

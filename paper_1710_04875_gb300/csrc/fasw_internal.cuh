@@ -216,7 +216,6 @@ void launch_sgs(const LevelDev& L, const SchemeParams& sc, int mixed, int do_upd
                 const double* r_in, double* z_out, cudaStream_t st);
 
 // ---- launchers (kernels_transfer.cu)
-void launch_copy_u0(const LevelDev& L, cudaStream_t st);
 // fast: PhysParams::fast
 void launch_restrict(const LevelDev& F, const LevelDev& C, int restrict_mut, int fast, cudaStream_t st);
 void launch_prolong(const LevelDev& F, const LevelDev& C, cudaStream_t st);

@@ -27,6 +27,7 @@ inline bool ws_level(int kind, const LevelDev& L) { return is_ws(kind) && L.wsF;
 // launch_sgs_prep forms the diagonal blocks itself (aw, eta as in launch_diag_blocks, which is left out);
 // the lines are at the kernels
 constexpr int PREP_SPLIT_CELLS = 16384;
+constexpr int WS_SPLIT_CELLS = 16384;  // the defect kernels' and the right-hand side's
 inline bool prep_forms_diag(int kind, const LevelDev& L, int mixed) {
   return ws_level(kind, L) && (mixed || L.n <= PREP_SPLIT_CELLS);
 }
@@ -116,8 +117,8 @@ int ws_strips(int nj);
 // exact_iters > 0: that many block Gauss-Seidel corrections toward the exact (D + L + U)^-1;
 // deep: the deeper operand ring (false for SWEEP_WS8)
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,
-                    long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters = 0,
-                    bool deep = true, WsPending* pending = nullptr);
+                    int* err, long long limit, cudaStream_t st, int exact_iters = 0, bool deep = true,
+                    WsPending* pending = nullptr);
 // Hyperplane-staged FP32 sweep: whether a level fits (rows, shared memory), and the entries
 // (ni + nj - 1) * nj of its hyperplane-major arrays (hpF, hpB: 32 floats each; hpC, hpY: 4).
 bool hp_fits(int ni, int nj, int nw);

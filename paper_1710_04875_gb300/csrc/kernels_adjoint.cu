@@ -551,7 +551,6 @@ int adj_assemble(AdjointDev& A, const LevelDev& L, const PhysParams& ph, double 
 }
 
 void adj_apply(const AdjointDev& A, const double* v, double* out, int transpose, cudaStream_t st) {
-  const int nb = (A.n + 127) / 128;
   if (transpose)
     launch_pdl(k_jac_tmv, (4 * A.n + 127) / 128, 128, 0, st, A.n, A.rev_ptr, A.rev, A.J, v, out);
   else
@@ -599,7 +598,7 @@ void precond(const AdjointDev& A, const double* r, double* y, double* z, cudaStr
   T.yz64 = y;
   if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
     WsPending b{};  // the sweep's result, left in its own layout
-    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st, 0, true, &b);
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, r, A.err, A.spin_limit, st, 0, true, &b);
     launch_pdl(k_adj_ws_finish, (4 * A.n + 127) / 128, 128, 0, st, A.Lp, b, z);
     return;
   }
@@ -905,7 +904,6 @@ void lc(int m, double a0, const double* x0, double a1, const double* x1, double 
 }
 
 void jac(const AdjointDev& A, const double* blocks, const double* v, double* out, int transpose, cudaStream_t st) {
-  const int nb = (A.n + 127) / 128;
   if (transpose)
     launch_pdl(k_jac_tmv, (4 * A.n + 127) / 128, 128, 0, st, A.n, A.rev_ptr, A.rev, blocks, v, out);
   else
@@ -920,7 +918,7 @@ void precond_fwd(const AdjointDev& A, double c, const double* t, double* s, doub
   T.yz64 = x;
   if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
     T.wsZ = A.wsZ;
-    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, s, A.err, A.spin_limit, st);
   } else {
     launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
   }
@@ -962,7 +960,7 @@ void smooth_T_ws(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
   for (int i = A.nstages - 1; i >= 0; --i) {
     const bool first = i == A.nstages - 1;
     WsPending b{};
-    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, first ? v : nullptr, A.prog, A.err, A.spin_limit, st, 0, true, &b);
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, first ? v : nullptr, A.err, A.spin_limit, st, 0, true, &b);
     launch_pdl(k_adj_ws_stage, g, 128, 0, st, A.Lp, b, A.stage_c[i], (int)first, (int)(i == 0), A.stage_b[i], w,
                out, fb, s);
     if (i > 0)

@@ -525,11 +525,6 @@ __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc, bool va
   const int sz = valid ? 16 : 0;  // 0: zero-fill without reading
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gsrc), "r"(sz) : "memory");
 }
-__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc, bool valid) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
-  const int sz = valid ? 8 : 0;
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gsrc), "r"(sz) : "memory");
-}
 __device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc, bool valid) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
   const int sz = valid ? 4 : 0;
@@ -899,7 +894,7 @@ bool hp_fits(int ni, int nj, int nw) {
 int launch_sweep(const LevelDev& L, int mixed, int kind, int do_update, int aw, double alpha, const double* rhs,
                  long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, WsPending* pending) {
   if (ws_level(kind, L))
-    return launch_ws_sweep(L, mixed, 1, do_update, aw, alpha, rhs, prog, err, limit, st, exact_iters,
+    return launch_ws_sweep(L, mixed, 1, do_update, aw, alpha, rhs, err, limit, st, exact_iters,
                            kind != SWEEP_WS8, pending);
   if (is_ws(kind)) kind = mixed ? SWEEP_AUTO : SWEEP_STRIPS;
   if (is_hp(kind) && mixed && L.hpF) {

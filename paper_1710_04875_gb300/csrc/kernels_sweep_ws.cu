@@ -589,7 +589,6 @@ __global__ void __launch_bounds__(WS_THREADS)
 // levels whose time is their memory traffic), or one cell and one row (SPLIT true: a quarter of
 // the FP64 chain per thread, for the small levels whose time is that chain).  Every row is summed
 // in the same order either way.
-constexpr int WS_SPLIT_CELLS = 16384;  // levels up to this many cells take one thread per row
 
 template <bool SPLIT>
 __device__ __forceinline__ bool ws_thread(const LevelDev& L, int& c, int& q0, int& q1) {
@@ -1039,9 +1038,7 @@ void ws_form_shape(int ni, int nj, int nw, int form, int* stages, int* edges, lo
 }
 
 int launch_ws_sweep(const LevelDev& L, int mixed, int refine, int do_update, int aw, double alpha, const double* rhs,
-                    long long* prog, int* err, long long limit, cudaStream_t st, int exact_iters, bool deep,
-                    WsPending* pending) {
-  (void)prog;  // the warp strips exchange their boundary rows in shared memory, not through progress words
+                    int* err, long long limit, cudaStream_t st, int exact_iters, bool deep, WsPending* pending) {
   const WsForm& form = kWsForms[L.wsForm[deep]];
   auto sweep = [&](float4* zout) { return form.launch(L, zout, err, limit, st); };
   const int g = (L.n + 127) / 128;

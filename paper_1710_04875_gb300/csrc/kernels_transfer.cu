@@ -159,16 +159,6 @@ __global__ void k_fill_state(LevelDev L, double w0, double w1, double w2, double
   L.u[3 * L.Gn + t] = w3;
 }
 
-__global__ void k_copy_u0(LevelDev L) {
-  pdl_entry();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= L.n) return;
-  const int i = c % L.ni, j = c / L.ni;
-  const int g = gidx(L, i, j);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) L.u0[k * L.n + c] = L.u[k * L.Gn + g];
-}
-
 // Volume-weighted agglomeration restriction of the state and of the FAS residual (rhs),
 // and of the eddy viscosity when requested; the coarse state starts at u~.
 __global__ void k_restrict(LevelDev F, LevelDev C, int restrict_mut, int fast) {
@@ -295,8 +285,6 @@ void launch_agglomerate(const LevelDev& F, const LevelDev& C, cudaStream_t st) {
 cudaError_t launch_fill_state(const LevelDev& L, const double w[4], cudaStream_t st) {
   return launch_pdl(k_fill_state, (L.Gn + 255) / 256, 256, 0, st, L, w[0], w[1], w[2], w[3]);
 }
-
-void launch_copy_u0(const LevelDev& L, cudaStream_t st) { launch_pdl(k_copy_u0, (L.n + 255) / 256, 256, 0, st, L); }
 
 void launch_restrict(const LevelDev& F, const LevelDev& C, int restrict_mut, int fast, cudaStream_t st) {
   launch_pdl(k_restrict, (C.n + 63) / 64, 64, 0, st, F, C, restrict_mut, fast);

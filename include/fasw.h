@@ -262,7 +262,8 @@ int fasw_adjoint_objective_gradient(fasw_ctx* ctx, int which, double* g, int on_
  * additive-W preconditioner (D+L) D^-1 (D+U) (section 4), S = eta dt* per cell.  steps = 0:
  * z = P^-T r = S (D+L)^-T D^T (D+U)^-T r; steps > 0: z = that many steps from zero of the
  * transposed primal stage loop x_i = x_0 + (alpha_i / eta) P^-T (r - J^T x_{i-1}) (needs
- * fasw_adjoint_jacobian first).  Rebuilds the finest level's preconditioner blocks and dt*. */
+ * fasw_adjoint_jacobian first).  FP64 contexts apply it to FP64 accuracy and take r of any size; mixed ones
+ * in FP32, within its range.  Rebuilds the finest level's preconditioner blocks and dt*. */
 int fasw_adjoint_precond_apply(fasw_ctx* ctx, double cfl, int steps, const double* r, double* z, int on_device);
 /* Preconditioner of the adjoint GMRES (the Jacobian must be assembled again after a change):
  *   0: steps of the primal stage loop run on J^T, x_i = x_0 + (alpha_i/eta) P^-T (r - J^T x_(i-1));

@@ -241,17 +241,15 @@ void free_stream(double mach, double alpha_deg, double w[4]) {
 }
 
 // ---- driver steps
-// Sweep kind used on a level: automatic = hyperplane-staged FP32 sweep where the level fits
-// (mixed), else one CTA (mixed) or strips (FP64); a requested kind that does not apply to the
-// level or precision falls back the same way.
+// Sweep kind used on a level: automatic = the warp strips where the level fits, else (mixed) the
+// hyperplane-staged FP32 sweep or one CTA, (FP64) strips; a requested kind that does not apply to the
+// level or precision falls back the same way, but for the staged sweep.
 int level_sweep_kind(const fasw_ctx* c, const LevelDev& L) {
   if (c->exact_iters > 0 && L.wsF) return SWEEP_WS;  // the exact-preconditioner iterations run on it
   int k = c->sweep_kind;
   if (k == SWEEP_AUTO) {
-    // measured per level on GB300: the warp strips win on every level in both precisions (mixed,
-    // one application, before their strips went from 32 to 8 rows: 64x16 28.6 against 32.3 us for
-    // the one-CTA hyperplane-staged sweep, 128x32 41.9 against 58.3 us; the sweep alone is a quarter
-    // faster since)
+    // measured per level on GB300: the warp strips win on every level in both precisions (mixed, one
+    // sweep pair: 64x16 14 us, 128x32 24; an application of the hyperplane-staged sweep 32 and 58 us)
     if (L.wsF) return SWEEP_WS;
     return c->mixed ? (L.hpF ? SWEEP_HP : SWEEP_CTA) : SWEEP_STRIPS;
   }

@@ -3,7 +3,7 @@
 // are bound by it (ncu: FP64 pipe active 70-85 % of the active cycles in every one of them).
 // Conversions between FP32 and FP64 and comparisons of FP64 values count as such instructions; the
 // integer pipe takes one per two clocks.  So exact conversions are done on the bit patterns, and a
-// reciprocal is four FP64 instructions instead of the nine of an IEEE division.
+// reciprocal is four FP64 instructions (a quotient with it three more) instead of the nine of an IEEE division.
 #pragma once
 #include <cuda_runtime.h>
 

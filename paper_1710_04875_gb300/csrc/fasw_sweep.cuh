@@ -20,17 +20,22 @@ inline bool is_hp(int kind) { return kind == SWEEP_HP || kind == SWEEP_HP4 || ki
 // that strips of different cases of a batch can share an SM)
 inline bool is_ws(int kind) { return kind == SWEEP_WS || kind == SWEEP_WS8; }
 
-// kind: the resolved sweep kind of this level (SWEEP_HP writes the hyperplane-major blocks,
-// SWEEP_WS also the skewed FP32 blocks of the warp strips).
 // the level's sweep is the warp strips'
 inline bool ws_level(int kind, const LevelDev& L) { return is_ws(kind) && L.wsF; }
-// launch_sgs_prep forms the diagonal blocks itself (aw, eta as in launch_diag_blocks, which is left out);
-// the lines are at the kernels
+// FP64 levels up to this many cells take the half rows of k_ws_prep64, and a block row per thread in the right-hand
+// side's and the defect's kernels; larger ones two kernels and a cell per thread.  A smoothing step (RANS), split
+// against not: preparation 18,432 cells 482 / 496 us, 20,736 475 / 480, 25,600 516 / 516, 36,864 643 / 637,
+// 65,536 881 / 885; right-hand side and defect 18,432 477 / 496, 25,600 513 / 516, 36,864 632 / 637, 50,176
+// 747 / 748, 65,536 885 / 885.  So the lines could lie at about 24,000 and 45,000 cells, for 1 to 4 % of a step
+// between; up to 16,384 cells the split forms win by more (256x64 preparation 32 -> 25 us, defect 7.1 -> 6.4).
 constexpr int PREP_SPLIT_CELLS = 16384;
-constexpr int WS_SPLIT_CELLS = 16384;  // the defect kernels' and the right-hand side's
+constexpr int WS_SPLIT_CELLS = 16384;
+// launch_sgs_prep forms the diagonal blocks itself (aw, eta as in launch_diag_blocks, which is left out)
 inline bool prep_forms_diag(int kind, const LevelDev& L, int mixed) {
   return ws_level(kind, L) && (mixed || L.n <= PREP_SPLIT_CELLS);
 }
+// kind: the resolved sweep kind of this level (SWEEP_HP writes the hyperplane-major blocks,
+// SWEEP_WS also the skewed FP32 blocks of the warp strips).
 void launch_sgs_prep(const LevelDev& L, int mixed, int kind, cudaStream_t st, int aw = 0, double eta = 0.0);
 // Forward and backward sweep of one stage: y = (D+L)^-1 rhs, z = (D+U)^-1 D y into L.yz64 /
 // L.yz32, with the stage update u = u0 - alpha z (AW) or u0 - alpha dt* z (ARK) when

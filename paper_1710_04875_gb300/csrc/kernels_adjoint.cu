@@ -950,9 +950,9 @@ void smooth_fwd(AdjointDev& A, const double* b, double* x, cudaStream_t st) {
   }
 }
 
-// smooth_T where the warp strips run the transposed sweep: a stage is the sweep's four launches, one for all
-// vector updates and one for both products, which writes the next sweep's right-hand side (17 launches for
-// a step of three stages instead of 35; 256x64 RANS adjoint 35.9 -> 30.3 ms).
+// smooth_T where the warp strips run the transposed sweep: a stage is the sweep's five launches, one for all
+// vector updates and one for both products, which writes the next sweep's right-hand side (21 launches for a
+// step of three stages, 18 fewer than with a launch for each update and product; 256x64 RANS adjoint 5 ms less).
 void smooth_T_ws(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
   const int m = 4 * A.n, g = (4 * A.n + 127) / 128;
   double *fb = A.mgw + (size_t)m, *w = A.mgw + 2 * (size_t)m, *s = A.mgw + 3 * (size_t)m;

@@ -15,21 +15,24 @@ namespace {
 // so the FP64 work of a launch is spread over as many warps and SMs as the grid allows.  The cells'
 // phase takes two components of a cell per thread, on tile height 1 (with a fourth warp) one.
 //
-// Tile height 4 where that still gives a block per SM, else 1: a coarse level then spreads over four
+// Tile height 4 where that still gives a block per SM of the GB300, else 1: a coarse level then spreads over four
 // times as many SMs for 1.6 times the j-face work (its j-faces are computed by both neighbouring tiles).
-// FP64, height 1 / 2 / 4 / 8: 64x16 5.3 / 7.0 / 10.3 / 17.8 us, 128x32 8.5 / 10.1 / 10.4 / 17.9, 256x64 (144
-// tiles of height 4) 13.9 / 18.2 / 17.5 / 18.1, 330x90 (253) 27.1 / 23.7 / 22.3 / 23.1, 512x128
-// 38.5 / 35.1 / 33.7 / 36.3, 1024x256 189 / 161 / 160 / 181.  Before the cells' phase was split and its
-// operands fetched ahead of the wait for the kernel before: 64x16 8.5, 128x32 10.1.  A case of a batch shares
-// the chip, so the extra work of height 1 counts there: height 4 from 76 tiles (64 cases, mixed: 8.7 ms
-// a cycle against 9.3 with the rule of a case alone).
+// FP64, a finest level (with sensors), height 1 / 2 / 4 / 8: 64x16 7.9 / 10.2 / 14.7 / 23.4 us, 128x32 12.3 / 14.3 /
+// 14.7 / 23.7, 256x64 (144 tiles of height 4) 20.0 / 25.4 / 24.0 / 23.5, 330x90 (253) 29.3 / 25.6 / 24.1 / 23.7,
+// 512x128 54.7 / 49.2 / 46.5 / 47.8, 1024x256 201 / 170 / 168 / 190.  As coarse levels 64x16 takes 5.4 us, 128x32
+// 8.8, 256x64 14.3 (8.5 and 10.1 on the first two before the cells' phase was split and its operands fetched ahead
+// of the wait for the kernel before).  A case of a batch shares the chip, so the extra work of height 1 counts
+// there: height 4 from half as many tiles, also with few cases (FP64 cycle, this rule / height 1 / height 4
+// everywhere: 2 cases of 256x64 982 / 1,054 / 1,027 us, 4 of them 1,268 / 1,300 / 1,310, 16 2,598 / 2,703 / 2,606;
+// at its worst 2 cases of 192x48 692 / 678 / 716).
 constexpr int TX = 31;
+constexpr int SMS = 152;
 constexpr int res_threads(int ty) { return ty == 1 ? 128 : 32 * (2 * ty + 1); }
 // Tile height: the level's setting (1, 2, 4 or 8, chosen by the batch autotuner or the caller), else
 // by the rule above.
 inline int res_ty(const LevelDev& L) {
   if (L.res_ty > 0) return L.res_ty;
-  return ((L.ni + TX - 1) / TX) * ((L.nj + 3) / 4) >= (L.shared ? 76 : 152) ? 4 : 1;
+  return ((L.ni + TX - 1) / TX) * ((L.nj + 3) / 4) >= (L.shared ? SMS / 2 : SMS) ? 4 : 1;
 }
 
 __device__ __forceinline__ int gidx(const LevelDev& L, int i, int j) { return (j + 2) * L.P + (i + 2); }
@@ -264,7 +267,7 @@ __device__ __forceinline__ void cell_thermo(const LevelDev& L, const PhysParams&
 // early: the geometry is read, and what depends on it alone formed, before the wait for the kernel before
 // (which must not be one that writes the metrics; a kernel lets its successor start only once its own
 // predecessors have completed): a quarter of an interior cell's FP64 chain and a third of a ghost's.  With a
-// stage update 32x8 5.4 -> 3.7 us, 64x16 5.3 -> 4.1, 128x32 5.8 -> 4.3, 256x64 6.0 -> 5.3.
+// stage update 32x8 5.4 -> 4.2 us, 64x16 5.3 -> 4.0, 128x32 5.8 -> 4.0, 256x64 6.0 -> 5.2.
 __global__ void k_cell_aux(LevelDev L, PhysParams ph, double cfl, int want_dts, int fill_ghosts, int nbi,
                            WsPending up, int early) {
   if (!early) pdl_entry();
@@ -349,9 +352,6 @@ __device__ __forceinline__ double sensor_val(double qm, double q0, double qp) {
   return FAST ? div64(d, s, rcp64(s)) : d / s;
 }
 
-// JST flux through a face with area vector (sx, sy) from L to R; stencil LL, L, R, RR
-// given as ghosted indices.  hc: central part; hd: dissipation d (section 2).
-// On a moving face (grid volume flux vf) the convective flux is F . S - u vf.
 // First-order flux-vector-split face flux (the discretization section 4.4 linearizes for the
 // preconditioner): h = A+(u_bar) u_L + A-(u_bar) u_R at the mean state u_bar, with the cutoff
 // eigenvalues of eq. (cutoff), split as the JST flux is (h = hc - hd): hc = A(u_bar)(u_L + u_R)/2,
@@ -408,6 +408,9 @@ __device__ void fvs_face(const LevelDev& L, int gL, int gR, double sx, double sy
   }
 }
 
+// JST flux through a face with area vector (sx, sy) from L to R; stencil LL, L, R, RR
+// given as ghosted indices.  hc: central part; hd: dissipation d (section 2).
+// On a moving face (grid volume flux vf) the convective flux is F . S - u vf.
 // The factor 1/2 of the averages goes on the face vector, and on a fixed grid (moving 0) the terms in vf
 // are left out: both leave every bit as it is.  FAST (PhysParams::fast) takes the grid's flux off the
 // normal velocities once, sums the two cells' terms in chains, and forms the third difference as
@@ -550,8 +553,6 @@ __device__ double block_sum(double v, double* wsum) {
   return s;
 }
 
-// One tile of TX x TY cells: every face of the tile is computed once into shared memory,
-// then each cell assembles F^c and F^v and writes what the mode asks for.
 // entry e of a cell's transfer blocks
 __device__ __forceinline__ double tb_entry(const LevelDev& L, int tb32, int e, int c) {
   const size_t at = (size_t)e * L.n + c;
@@ -569,6 +570,8 @@ __device__ __forceinline__ double norm_of(const double F[4], int all) {
   return s;
 }
 
+// One tile of TX x TY cells: every face of the tile is computed once into shared memory,
+// then each cell assembles F^c and F^v and writes what the mode asks for.
 template <int TY, bool FAST>
 __global__ void __launch_bounds__(res_threads(TY)) k_residual(LevelDev L, PhysParams ph, ResArgs a) {
   __shared__ double xc[4][TY][TX + 1], xd[4][TY][TX + 1];

@@ -72,9 +72,10 @@ __device__ void split_blocks(const T w[4], T sx, T sy, T vf, T d, T Ap[16], T Am
 }
 
 // The same in FP64 with one reciprocal each of length, density, sound speed and cutoff (rd = 1/d), the
-// length folded into the eigenvalues, and the zeros and ones of r0, r1, dp and dvn left out: about 175
+// length folded into the eigenvalues, and the zeros and ones of r0, r1, dp and dvn left out: about 190
 // FP64 instructions a face against 300 of the form above, which is what bounds the kernel (1024x256
-// level 305 -> 185 us at the pipe's rate).  FP32 keeps the form above, operation by operation.
+// level 305 -> 204 us at the pipe's rate; 185 with products by reciprocals in the quotients' place, whose
+// error is up to three times a quotient's).  FP32 keeps the form above, operation by operation.
 __device__ __forceinline__ void split_blocks64(const double w[4], double nx, double ny, double len, double rl,
                                                double vf, int moving, double d, double rd, double Ap[16],
                                                double Am[16]) {
@@ -180,8 +181,8 @@ __global__ void k_face_blocks(LevelDev L, PhysParams ph, T* blk, T d, T rd) {
     stride = L.nfe;
   }
   // What depends on the grid and the eddy viscosity alone comes before the wait for the kernel before,
-  // k_cell_aux (a kernel lets its successor start only once its own predecessors have completed): FP64
-  // 64x16 7.9 -> 7.1 us, 256x64 14.9 -> 13.4.
+  // k_cell_aux (a kernel lets its successor start only once its own predecessors have completed): -0.8 us on
+  // FP64 64x16 (now 7.4), -1.5 on 256x64 (18.5).
   constexpr bool F64 = sizeof(T) == 8;
   double len = 0.0, rl = 0.0, nx = 0.0, ny = 0.0, vr = 0.0;
   if (F64) {

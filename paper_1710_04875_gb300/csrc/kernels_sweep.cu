@@ -42,12 +42,12 @@ __device__ __forceinline__ float low(float x) { return x; }
 // 3 = H_E, 4 = H_N.  Blocks of absent neighbours are zero.  MODE 1 (HP, FP32 only): blocks 1-4
 // go to the hyperplane-major arrays of k_sweep_hp instead: entry h = (i + j) * nj + j holds
 // hpF[32h..] = G_W, G_S and hpB[32h..] = H_E, H_N (row-major 4x4 each); D^-1 stays in tb.
-// MODE 2 (WS; FP64 levels up to PREP_SPLIT_CELLS: k_ws_prep64): in FP32 forms D and its LU factors itself (a
-// launch and a pass over them less than with k_diag_blocks before it: 64x16 9.4 -> 7.2 us; in FP64 that
-// gains nothing, 1024x256 243 us against 245, 512x128 90 against 68), tb as MODE 0, and blocks 1-4 also in FP32 in the skewed layout of the warp-strip
-// sweep (kernels_sweep_ws.cu): forward rows G_W, G_S at strip j / 8, step i + j % 8, row j % 8
-// (G_S zero on row 0 except the upper wake, whose mirror precedes it), backward rows H_E, H_N at
-// step Mp - 1 - i - j % 8; the lower wake's G_S (the backward coupling to its mirror) to wsCut.
+// MODE 2 (WS; FP64 levels up to PREP_SPLIT_CELLS: k_ws_prep64): tb as MODE 0, and blocks 1-4 also in FP32 in
+// the skewed layout of the warp-strip sweep (kernels_sweep_ws.cu): forward rows G_W, G_S at strip j / 8, step
+// i + j % 8, row j % 8 (G_S zero on row 0 except the upper wake, whose mirror precedes it), backward rows H_E,
+// H_N at step Mp - 1 - i - j % 8; the lower wake's G_S (the backward coupling to its mirror) to wsCut.  In FP32
+// it forms D and its LU factors itself (a launch and a pass over them less: 64x16 9.4 -> 7.2 us); in FP64 that
+// gains nothing (1024x256 243 us against 245, 512x128 90 against 68, a cell per thread both).
 template <typename T, int MODE>
 __global__ void k_sgs_prep(LevelDev L, const T* blk, const T* dlu, T* tb, int aw, double eta) {
   constexpr bool HP = MODE == 1;

@@ -35,9 +35,9 @@
 // written.  Every wait is bounded; on timeout the kernel sets the error word, waits (bounded) for its
 // own copies in flight, and still meets the cluster's barriers, so that no strip waits forever.
 //
-// One sweep pair in a cycle (from the end of the kernel before), against strips of 32 rows with a lane per
-// cell that staged and stored for themselves: 64x16 17.7 -> 12.5 us, 128x32 30.8 -> 22.2, 256x64 62.5 -> 42.5,
-// 512x128 83, 1024x256 246 -> 163; about 43 ns a step (about 80 before) and 1.1 us from strip to strip.
+// One sweep pair in an FP64 cycle (from the end of the kernel before), strips of 32 rows with a lane per cell
+// that staged and stored for themselves against these: 64x16 17.7 -> 12 us, 128x32 30.8 -> 22, 256x64 62.5 -> 42,
+// 512x128 82, 1024x256 246 -> 162; about 43 ns a step (about 80 before) and 1.1 us from strip to strip.
 // A tree instead of the chain of eight FMAs (FP64 contexts could take it) gains 1 %: the step waits for its
 // shared-memory instructions.
 #include <atomic>
@@ -523,8 +523,7 @@ __global__ void __launch_bounds__(WS_THREADS)
   // Set-up while the kernel before still runs: this CTA's shared memory, the cluster's first barrier, and
   // the first blocks.  The blocks are k_sgs_prep's, which is never the kernel before (the right-hand
   // side's kernel is), and a kernel lets its successor start only once its own predecessors have
-  // completed (pdl_entry), so they are complete here (a
-  // sweep pair in an FP64 cycle: 64x16 13.2 -> 12.3 us, 128x32 23.4 -> 22.4).
+  // completed (pdl_entry), so they are complete here (a sweep pair 1 us less).
   if (copier && lane == 0) {
     for (int k = 0; k < NS; ++k) {
       mbar_init(&S.full[k], 1);
@@ -580,10 +579,7 @@ __global__ void __launch_bounds__(WS_THREADS)
   cluster_wait();
 }
 
-// ---------------------------------------------------------------- operand layout
-// Skewed position of cell (i, j): strip b = j / 8, row jl = j % 8, forward step s = i + jl, backward step
-// Mp - 1 - i - jl (Mp: the steps that hold a cell, padded to whole stages; ws_fpos, ws_bpos).
-
+// ---------------------------------------------------------------- the kernels around the sweep
 // The FP64 kernels of one application, written per row q of their block products: a thread
 // takes one cell and all four rows (SPLIT false: the loads of a warp coalesce along the cells, for
 // levels whose time is their memory traffic), or one cell and one row (SPLIT true: a quarter of

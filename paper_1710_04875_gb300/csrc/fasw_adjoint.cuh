@@ -24,6 +24,8 @@ enum AdjPrecond {
   ADJ_FAS_VCYCLE_T = 3    // the same with one coarse cycle per level (V) whatever the primal's gamma
 };
 
+constexpr int ADJ_SIZES = 8;  // more than the stages of any scheme
+
 struct AdjointDev {
   int ni = 0, nj = 0, n = 0, ncolours = 0;
   int* nbr = nullptr;      // n * ADJ_SLOTS neighbour cell or -1
@@ -57,6 +59,9 @@ struct AdjointDev {
   float* wsB = nullptr;
   float* wsCut = nullptr;
   float* wsZ = nullptr;    // its result and two corrections
+  // Sizes of its right-hand sides: the upper word of a largest magnitude each.  [0, ADJ_SIZES): of the stages of
+  // a transposed smoothing step (word 0 is zero between two steps); [ADJ_SIZES]: of a single application.
+  unsigned* size = nullptr;
   // FP32 transposed sweep (contexts in mixed precision): the transposed blocks in FP32, entry-major
   // (80n) and, where the level fits the hyperplane-staged sweep, hyperplane-major
   bool fp32 = false;
@@ -150,11 +155,6 @@ void adj_build_precond(AdjointDev& A, const LevelDev& L, const PhysParams& ph, c
 void adj_mg_build_precond(AdjointDev& A, const std::vector<LevelDev>& lev, const PhysParams& ph,
                           const SchemeParams& sc, double cfl, cudaStream_t st, long long& launches);
 void adj_precond(const AdjointDev& A, const double* r, double* scratch, double* z, cudaStream_t st);
-// The operators applied below are linear, and their FP64 sweeps run in FP32 with corrections: a right-hand side
-// of any size goes in scaled by the power of two of its largest entry (r in place; no bit of the mantissas
-// changes), and the result is scaled back.  In between A.parts is the scale's.
-void adj_scale_in(AdjointDev& A, double* r, cudaStream_t st);
-void adj_scale_out(const AdjointDev& A, double* z, cudaStream_t st);
 // z = P^-T r (steps <= 0) or z = `steps` transposed stage-loop steps from zero; the
 // preconditioner must be built.
 void adj_steps_apply(AdjointDev& A, int steps, const double* r, double* z, cudaStream_t st);

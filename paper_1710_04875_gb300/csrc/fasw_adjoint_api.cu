@@ -19,17 +19,6 @@ PhysParams adj_ph(const fasw_ctx* c) {
   p.fast = 0;
   return p;
 }
-
-// z (c->d_tmp2) = the linear operator apply() of r (c->d_tmp), r of any size in FP64 contexts.  Mixed contexts
-// apply it in FP32, with FP32's range.
-template <class Apply>
-void adj_scaled(fasw_ctx* c, Apply apply) {
-  const bool fp64 = !c->adj.fp32;
-  if (fp64) adj_scale_in(c->adj, c->d_tmp, c->st);
-  apply();
-  if (fp64) adj_scale_out(c->adj, c->d_tmp2, c->st);
-  c->launches += fp64 ? 3 : 0;
-}
 }  // namespace
 
 
@@ -115,7 +104,7 @@ int fasw_adjoint_precond_apply(fasw_ctx* c, double cfl, int steps, const double*
   if ((e = copy_in(c, c->d_tmp, r, m, on_device))) return e;
   err_clear(c);
   adj_build_precond(c->adj, c->lev[c->L()], adj_ph(c), c->sc, cfl, c->st, c->launches);
-  adj_scaled(c, [&] { adj_steps_apply(c->adj, steps, c->d_tmp, c->d_tmp2, c->st); });
+  adj_steps_apply(c->adj, steps, c->d_tmp, c->d_tmp2, c->st);
   c->launches += 2;
   if ((e = adj_err_check(c))) return e;
   if ((e = copy_out(c, z, c->d_tmp2, m, on_device))) return e;
@@ -167,13 +156,12 @@ int fasw_adjoint_cycle_apply(fasw_ctx* c, double cfl, int kind, int transpose, c
   if (e) return e;
   err_clear(c);
   adj_build_precond(c->adj, c->lev[c->L()], adj_ph(c), c->sc, cfl, c->st, c->launches);
-  if (kind == 2) adj_mg_build_precond(c->adj, c->lev, adj_ph(c), c->sc, cfl, c->st, c->launches);
-  adj_scaled(c, [&] {
-    if (kind == 2)
-      adj_mg_apply(c->adj, transpose, c->d_tmp, c->d_tmp2, c->st);
-    else
-      adj_smoother_apply(c->adj, c->adj.smooth_steps, transpose, c->d_tmp, c->d_tmp2, c->st);
-  });
+  if (kind == 2) {
+    adj_mg_build_precond(c->adj, c->lev, adj_ph(c), c->sc, cfl, c->st, c->launches);
+    adj_mg_apply(c->adj, transpose, c->d_tmp, c->d_tmp2, c->st);
+  } else {
+    adj_smoother_apply(c->adj, c->adj.smooth_steps, transpose, c->d_tmp, c->d_tmp2, c->st);
+  }
   ++c->launches;
   if ((e = adj_err_check(c))) return e;
   if ((e = copy_out(c, z, c->d_tmp2, m, on_device))) return e;

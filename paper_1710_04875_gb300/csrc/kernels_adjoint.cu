@@ -57,23 +57,47 @@ __global__ void k_adj_set_state(LevelDev L, const double* ub, const int* col, in
   }
 }
 
-// The bit pattern of the largest |x| (of finite non-negative values the order of the patterns is the values').
-__global__ void k_max_bits(int m, const double* x, unsigned long long* out) {
-  pdl_entry();
-  unsigned long long b = 0;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x)
-    b = max(b, (unsigned long long)__double_as_longlong(fabs(x[t])));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, b);
+// Scaling by powers of two.  The FP64 operators run their sweeps in FP32 with FP64 corrections, and an operator
+// that amplifies (a stage loop or a cycle that does not converge, on a right-hand side of any size) leaves FP32's
+// range where FP64 does not.  So a sweep's right-hand side goes in divided by the power of two of the largest
+// entry of what it is formed from, and the result is multiplied by it: no bit of a mantissa changes.  The word is
+// the upper half of that entry; the power lies between 2^-1000 and 2^1000, and is 1 where an entry is infinite.
+__device__ __forceinline__ double pow2_of(unsigned word, int sgn) {
+  if (word >= 0x7ff00000u) return 1.0;
+  const int e = min(max((int)(word >> 20) - 1023, -1000), 1000);
+  return __hiloint2double((sgn * e + 1023) << 20, 0);
 }
 
-// x times the power of two of the value in *bits to the power sgn; zero, infinity and NaN leave x as it is.
-__global__ void k_scale_pow2(int m, const unsigned long long* bits, int sgn, double* x) {
+// the larger of *word and the upper word of x >= 0, over a warp
+__device__ __forceinline__ void add_size(unsigned* word, double x) {
+  const unsigned b = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(x));
+  if ((threadIdx.x & 31) == 0 && b > *(volatile unsigned*)word) atomicMax(word, b);
+}
+
+// *out: the size of x; clear: the words after it set to zero
+__global__ void k_adj_size(int m, const double* x, unsigned* out, int clear) {
+  pdl_entry();
+  if (blockIdx.x == 0 && threadIdx.x > 0 && (int)threadIdx.x <= clear) out[threadIdx.x] = 0;
+  double b = 0.0;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m; t += gridDim.x * blockDim.x) b = fmax(b, fabs(x[t]));
+  add_size(out, b);
+}
+
+// the scaled right-hand side x of a transposed sweep (D' = I): FP64 for the defects and skewed FP32
+__global__ void k_adj_rhs(LevelDev L, const double* x, const unsigned* size) {
+  pdl_entry();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 2, q = t & 3;
+  if (d >= L.n) return;
+  const double v = x[(size_t)q * L.n + d] * pow2_of(*size, -1);
+  L.wsR[(size_t)q * L.n + d] = v;
+  L.wsC[4 * ws_fpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj)) + q] = d2f(v);
+}
+
+// x *= c 2^size
+__global__ void k_adj_unscale(int m, double c, const unsigned* size, double* x) {
   pdl_entry();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const double s = __longlong_as_double((long long)*bits);
-  if (t < m && s > 0.0 && s <= 1.7976931348623157e308) x[t] = ldexp(x[t], sgn * ilogb(s));
+  if (t < m) x[t] *= c * pow2_of(*size, 1);
 }
 
 __global__ void k_adj_get_state(LevelDev L, double* ub) {
@@ -197,8 +221,9 @@ __global__ void k_jac_tmv(int n, const int* rev_ptr, const int* rev, const doubl
 
 // J^v^T s - J^T w as the warp-strip sweep's right-hand side (D' = I): skewed FP32, and FP64 for the defect.
 // Lanes 4-7 of every eight take the second product (both in one thread: 32x8 6.1 us, now 3.9; 256x64 15.2, now 14.2).
+// (divided by the power of two of w and s)
 __global__ void k_jac_tmv_rhs(LevelDev L, const int* rev_ptr, const int* rev, const double* J, const double* w,
-                              const double* Jv, const double* s) {
+                              const double* Jv, const double* s, const unsigned* size) {
   pdl_entry();
   const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t >> 3, m = t & 3;
   const bool second = t & 4;
@@ -206,6 +231,7 @@ __global__ void k_jac_tmv_rhs(LevelDev L, const int* rev_ptr, const int* rev, co
   if (d < L.n) x = jac_t_row(L.n, rev_ptr, rev, second ? J : Jv, second ? w : s, d, m);
   x -= __shfl_down_sync(0xffffffffu, x, 4);
   if (d >= L.n || second) return;
+  x *= pow2_of(*size, -1);
   L.wsR[(size_t)m * L.n + d] = x;
   L.wsC[4 * ws_fpos(d % L.ni, d / L.ni, ws_steps(L.ni, L.nj)) + m] = d2f(x);
 }
@@ -285,29 +311,38 @@ __device__ __forceinline__ double ws_result_row(const LevelDev& L, const WsPendi
   return L.coef[d] * L.vol[d] * s;
 }
 
-__global__ void k_adj_ws_finish(LevelDev L, WsPending b, double* z) {
+__global__ void k_adj_ws_finish(LevelDev L, WsPending b, const unsigned* size, double* z) {
   pdl_entry();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
   if (d >= L.n) return;
-  z[(size_t)q * L.n + d] = ws_result_row(L, b, d, q);
+  z[(size_t)q * L.n + d] = ws_result_row(L, b, d, q) * pow2_of(*size, 1);
 }
 
 // One stage of the transposed smoothing step (smooth_T) after its sweep: w = c S D^-T b, out += w,
 // fbar -= w (the first stage: out = w, fbar = -w), and where a stage follows s = w + beta fbar and
-// fbar *= 1 - beta.
+// fbar *= 1 - beta.  size: the right-hand side's; size[1] becomes that of w and s, and after the last stage
+// word 0 of the step, `size0`, zero.
 __global__ void k_adj_ws_stage(LevelDev L, WsPending b, double c, int first, int last, double be, double* w, double* out,
-                               double* fb, double* s) {
+                               double* fb, double* s, unsigned* size, unsigned* size0) {
   pdl_entry();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, d = x >> 2, q = x & 3;
-  if (d >= L.n) return;
-  const double v = c * ws_result_row(L, b, d, q);
-  const size_t at = (size_t)q * L.n + d;
-  w[at] = v;
-  out[at] = first ? v : out[at] + v;
-  if (last) return;
-  const double f = first ? -v : fb[at] - v;
-  s[at] = fma(be, f, v);
-  fb[at] = (1.0 - be) * f;
+  double v = 0.0, sv = 0.0;
+  if (d < L.n) {
+    v = c * ws_result_row(L, b, d, q) * pow2_of(*size, 1);
+    const size_t at = (size_t)q * L.n + d;
+    w[at] = v;
+    out[at] = first ? v : out[at] + v;
+    if (!last) {
+      const double f = first ? -v : fb[at] - v;
+      s[at] = sv = fma(be, f, v);
+      fb[at] = (1.0 - be) * f;
+    }
+  }
+  if (last) {
+    if (x == 0) *size0 = 0;  // size itself is another word: a scheme has three stages or more
+    return;
+  }
+  add_size(size + 1, fmax(fabs(v), fabs(sv)));
 }
 
 // FP32 copies of the transposed transfer blocks for the FP32 sweeps: entry-major (all five
@@ -467,8 +502,10 @@ int adj_setup(AdjointDev& A, int ni, int nj, int nw, std::vector<void*>& allocs,
   if (!A.fp32 && ws_form(ni, nj, nw, false) >= 0) {
     const size_t wf = ws_floats(ni, nj), wc = 16 * (size_t)(nw > 0 ? nw : 1);
     if ((r = adj_alloc(allocs, &A.wsB, wf)) || (r = adj_alloc(allocs, &A.wsCut, wc)) ||
-        (r = adj_alloc(allocs, &A.wsZ, 3 * ws_vec_floats(ni, nj))) || (r = adj_alloc(allocs, &A.wsF, wf)))
+        (r = adj_alloc(allocs, &A.wsZ, 3 * ws_vec_floats(ni, nj))) || (r = adj_alloc(allocs, &A.wsF, wf)) ||
+        (r = adj_alloc(allocs, &A.size, ADJ_SIZES + 1)))
       return r;
+    cudaMemsetAsync(A.size, 0, (ADJ_SIZES + 1) * sizeof(unsigned), st);
     // positions without a cell, or without a coupling, are never written: they must read as zero
     cudaMemsetAsync(A.wsF, 0, wf * sizeof(float), st);
     cudaMemsetAsync(A.wsB, 0, wf * sizeof(float), st);
@@ -579,6 +616,14 @@ LevelDev transposed(const AdjointDev& A, const LevelDev& L) {
   return T;
 }
 
+// the size of a single application's right-hand side
+const unsigned* size_of(const AdjointDev& A, const double* x, cudaStream_t st) {
+  unsigned* size = A.size + ADJ_SIZES;
+  cudaMemsetAsync(size, 0, sizeof(unsigned), st);
+  launch_pdl(k_adj_size, RED_BLOCKS, 256, 0, st, 4 * A.n, x, size, 0);
+  return size;
+}
+
 // z = P^-T r (y: scratch of 4n): both triangular solves in one FP64 sweep on
 // the transposed transfer blocks (into y), then z = S D^-T y.
 void precond(const AdjointDev& A, const double* r, double* y, double* z, cudaStream_t st) {
@@ -598,8 +643,10 @@ void precond(const AdjointDev& A, const double* r, double* y, double* z, cudaStr
   T.yz64 = y;
   if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
     WsPending b{};  // the sweep's result, left in its own layout
-    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, r, A.err, A.spin_limit, st, 0, true, &b);
-    launch_pdl(k_adj_ws_finish, (4 * A.n + 127) / 128, 128, 0, st, A.Lp, b, z);
+    const unsigned* size = size_of(A, r, st);
+    launch_pdl(k_adj_rhs, (4 * A.n + 127) / 128, 128, 0, st, T, r, size);
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, nullptr, A.err, A.spin_limit, st, 0, true, &b);
+    launch_pdl(k_adj_ws_finish, (4 * A.n + 127) / 128, 128, 0, st, A.Lp, b, size, z);
     return;
   }
   launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, r, A.prog, A.err, A.spin_limit, st);
@@ -715,19 +762,6 @@ void adj_precond(const AdjointDev& A, const double* r, double* scratch, double* 
   precond(A, r, scratch, z, st);
 }
 
-void adj_scale_in(AdjointDev& A, double* r, cudaStream_t st) {
-  auto* bits = reinterpret_cast<unsigned long long*>(A.parts);
-  const int m = 4 * A.n;
-  cudaMemsetAsync(bits, 0, sizeof(*bits), st);
-  launch_pdl(k_max_bits, RED_BLOCKS, 256, 0, st, m, (const double*)r, bits);
-  launch_pdl(k_scale_pow2, (m + 255) / 256, 256, 0, st, m, (const unsigned long long*)bits, -1, r);
-}
-
-void adj_scale_out(const AdjointDev& A, double* z, cudaStream_t st) {
-  const int m = 4 * A.n;
-  launch_pdl(k_scale_pow2, (m + 255) / 256, 256, 0, st, m, reinterpret_cast<const unsigned long long*>(A.parts), 1, z);
-}
-
 void adj_steps_apply(AdjointDev& A, int steps, const double* r, double* z, cudaStream_t st) {
   if (steps <= 0)
     precond(A, r, A.mgy, z, st);
@@ -761,12 +795,13 @@ __global__ void k_lc(int m, double a0, const double* x0, double a1, const double
   out[t] = s;
 }
 
-// out = eta dt* t per cell (eta dt* = coef vol)
-__global__ void k_scale_dts(int n, const double* coef, const double* vol, const double* t, double* out) {
+// out = eta dt* t per cell (eta dt* = coef vol), with a size divided by its power of two
+__global__ void k_scale_dts(int n, const double* coef, const double* vol, const double* t, const unsigned* size,
+                            double* out) {
   pdl_entry();
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= n) return;
-  const double s = coef[d] * vol[d];
+  const double s = coef[d] * vol[d] * (size ? pow2_of(*size, -1) : 1.0);
   for (int k = 0; k < 4; ++k) out[(size_t)k * n + d] = s * t[(size_t)k * n + d];
 }
 
@@ -912,17 +947,20 @@ void jac(const AdjointDev& A, const double* blocks, const double* v, double* out
 
 // x = c P^-1 t (forward: the level's own FP64 blocks; scratch s)
 void precond_fwd(const AdjointDev& A, double c, const double* t, double* s, double* x, cudaStream_t st) {
+  const bool ws = fp64_sweep(A, A.Lp) == SWEEP_WS;
+  const unsigned* size = ws ? size_of(A, t, st) : nullptr;
   launch_pdl(k_scale_dts, (A.n + 127) / 128, 128, 0, st, A.n, (const double*)A.Lp.coef, (const double*)A.Lp.vol, t,
-             s);
+             size, s);
   LevelDev T = A.Lp;
   T.yz64 = x;
-  if (fp64_sweep(A, A.Lp) == SWEEP_WS) {
+  const int m = 4 * A.n;
+  if (ws) {
     T.wsZ = A.wsZ;
     launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, s, A.err, A.spin_limit, st);
-  } else {
-    launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
+    launch_pdl(k_adj_unscale, (m + 255) / 256, 256, 0, st, m, c, size, x);
+    return;
   }
-  const int m = 4 * A.n;
+  launch_sweep(T, 0, SWEEP_STRIPS, 0, 1, 0.0, s, A.prog, A.err, A.spin_limit, st);
   lc(m, c, x, 0.0, nullptr, 0.0, nullptr, 0.0, nullptr, x, st);
 }
 
@@ -951,21 +989,24 @@ void smooth_fwd(AdjointDev& A, const double* b, double* x, cudaStream_t st) {
 }
 
 // smooth_T where the warp strips run the transposed sweep: a stage is the sweep's five launches, one for all
-// vector updates and one for both products, which writes the next sweep's right-hand side (21 launches for a
-// step of three stages, 18 fewer than with a launch for each update and product; 256x64 RANS adjoint 5 ms less).
+// vector updates and one for both products, which writes the next sweep's right-hand side (22 launches for a
+// step of three stages, 17 fewer than with a launch for each update and product; 256x64 RANS adjoint 5 ms less).
 void smooth_T_ws(AdjointDev& A, const double* v, double* out, cudaStream_t st) {
   const int m = 4 * A.n, g = (4 * A.n + 127) / 128;
   double *fb = A.mgw + (size_t)m, *w = A.mgw + 2 * (size_t)m, *s = A.mgw + 3 * (size_t)m;
   const LevelDev T = transposed(A, A.Lp);
+  launch_pdl(k_adj_size, RED_BLOCKS, 256, 0, st, m, v, A.size, ADJ_SIZES - 1);
+  launch_pdl(k_adj_rhs, g, 128, 0, st, T, v, (const unsigned*)A.size);
   for (int i = A.nstages - 1; i >= 0; --i) {
     const bool first = i == A.nstages - 1;
+    unsigned* size = A.size + (A.nstages - 1 - i);
     WsPending b{};
-    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, first ? v : nullptr, A.err, A.spin_limit, st, 0, true, &b);
+    launch_ws_sweep(T, 0, ADJ_REFINE, 0, 1, 0.0, nullptr, A.err, A.spin_limit, st, 0, true, &b);
     launch_pdl(k_adj_ws_stage, g, 128, 0, st, A.Lp, b, A.stage_c[i], (int)first, (int)(i == 0), A.stage_b[i], w,
-               out, fb, s);
+               out, fb, s, size, A.size);
     if (i > 0)
       launch_pdl(k_jac_tmv_rhs, (8 * A.n + 127) / 128, 128, 0, st, T, A.rev_ptr, A.rev, (const double*)A.J, (const double*)w,
-                 (const double*)A.Jv, (const double*)s);
+                 (const double*)A.Jv, (const double*)s, (const unsigned*)(size + 1));
   }
 }
 

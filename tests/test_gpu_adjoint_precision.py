@@ -78,3 +78,24 @@ def test_operators_take_right_hand_sides_of_any_size(levels):
             assert np.array_equal(apply(r * 2.0**e), z * 2.0**e)
         assert not np.any(apply(0.0 * r))
     s.close()
+
+
+def test_stage_loops_that_amplify_stay_in_the_range_of_fp64():
+    """The stage loop on J^T is not a convergent iteration: many steps of it leave FP32's range, not FP64's.  The
+    result is finite, linear in the right-hand side, and the step after it is that of the steps' recurrence."""
+    import paper_1710_04875_gb300 as P
+    ni, nj = 64, 16
+    s = P.Solver(make_cgrid(ni, nj, n_wake=8, wall_spacing=1e-3), P.default_params(mach=0.6, alpha_deg=1.0, nlevels=1))
+    s.set_state(perturbed_state(0.6, 1.0, nj, ni, amp=0.01, seed=1))
+    s.adjoint_jacobian()
+    r = np.random.default_rng(2).standard_normal((4, nj, ni))
+    n = 1
+    while np.abs(z := s.adjoint_precond_apply(r, 200.0, steps=n)).max() < 1e60 and n < 4096:
+        n *= 2
+    assert np.all(np.isfinite(z)) and np.abs(z).max() > 1e60
+    assert np.array_equal(s.adjoint_precond_apply(r * 2.0**-60, 200.0, steps=n), z * 2.0**-60)
+    # x_(n+1) = x_n + S (r - J^T x_n), S the step from zero
+    more = s.adjoint_precond_apply(r, 200.0, steps=n + 1)
+    want = z + s.adjoint_precond_apply(r - s.adjoint_apply(z, transpose=True), 200.0, steps=1)
+    assert np.abs(more - want).max() < 1e-10 * np.abs(more).max()
+    s.close()

@@ -243,7 +243,7 @@ void free_stream(double mach, double alpha_deg, double w[4]) {
 // ---- driver steps
 // Sweep kind used on a level: automatic = the warp strips where the level fits, else (mixed) the
 // hyperplane-staged FP32 sweep or one CTA, (FP64) strips; a requested kind that does not apply to the
-// level or precision falls back the same way, but for the staged sweep.
+// level or precision falls back to one CTA (mixed) or strips (FP64).
 int level_sweep_kind(const fasw_ctx* c, const LevelDev& L) {
   if (c->exact_iters > 0 && L.wsF) return SWEEP_WS;  // the exact-preconditioner iterations run on it
   int k = c->sweep_kind;
